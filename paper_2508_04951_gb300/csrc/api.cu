@@ -1370,10 +1370,25 @@ extern "C" dc_status resample_exact_batch(dc_ctx* c, const dc_c64* x, long long 
     if (stride != 0 && stride != (long long)n_pulses * n)
       return fail(c, DC_EINVAL, "tensor-core exact mode needs x_alpha_stride 0 or n_pulses*n");
     const long long rows_c = stride ? (long long)n_pulses * n_alpha : n_pulses;
-    Arena ar;
+    double delta_max = 0.0;
+    for (int i = 0; i < n_alpha; ++i) delta_max = std::max(delta_max, std::fabs(alpha_minus_one(v_r[i])));
     const size_t plane = exact_tc_plane_bytes(2 * rows_c, (int)n);
-    const size_t hi_at = ar.take(plane), lo_at = ar.take(plane);
-    if ((st = ensure_ws(c, ar.off))) return st;
+    const size_t mom = exact_tc_far_plane_bytes(2 * rows_c, (int)n);
+    const size_t loc = exact_tc_far_plane_bytes(2 * rows_c, (int)n_out);
+    ExTcPlanes pl{};
+    size_t at[6] = {};
+    for (bool far : {true, false}) {
+      // the dense sum where the far field does not apply or its planes do not fit
+      if (far && !exact_tc_far((int)n, (int)n_out, delta_max)) continue;
+      Arena ar;
+      for (int i = 0; i < (far ? 6 : 2); ++i) at[i] = ar.take(i < 2 ? plane : i < 4 ? mom : loc);
+      pl.far = far;
+      if ((st = ensure_ws(c, ar.off)) == DC_OK) break;
+    }
+    if (st) return st;
+    pl.hi = c->ws + at[0], pl.lo = c->ws + at[1];
+    pl.mom_hi = c->ws + at[2], pl.mom_lo = c->ws + at[3];
+    pl.loc_hi = c->ws + at[4], pl.loc_lo = c->ws + at[5];
     if ((st = ensure_items(c, items_bytes_for(n_alpha)))) return st;
     std::vector<float> dl(2 * (size_t)n_alpha);
     for (int i = 0; i < n_alpha; ++i) split(alpha_minus_one(v_r[i]), dl[2 * i], dl[2 * i + 1]);
@@ -1383,7 +1398,7 @@ extern "C" dc_status resample_exact_batch(dc_ctx* c, const dc_c64* x, long long 
                reinterpret_cast<float2*>(y), ddl, c->err};
     Phase ph(c, PH_EXACT_TC, s, (long long)n_alpha * n_pulses * n_out);
     cudaError_t e = launch_exact_tc(mode == DC_EXACT_FP16X3, reinterpret_cast<const float2*>(x), rows_c,
-                                    (int)n, c->ws + hi_at, c->ws + lo_at, a, n_alpha, s);
+                                    (int)n, pl, a, n_alpha, s);
     if (e != cudaSuccess) return cuda_fail(c, e, "tensor-core exact launch");
     return DC_OK;
   }

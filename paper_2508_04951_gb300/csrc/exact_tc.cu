@@ -23,6 +23,35 @@
 //   epilogue   TMEM -> registers (tcgen05.ld) -> complex64 outputs
 // Three (bf16) or four (fp16) pipeline stages of 64 / 48 KiB, mbarriers
 // between the producers and the MMA thread, every wait bounded.
+//
+// Near and far field.  S is a Cauchy matrix, sigma_n (-1)^m / (t_n - m), so a
+// block of sources seen from a distance has low rank: the sum over it needs 16
+// numbers per pulse instead of its samples (Chebyshev interpolation of 1/(t - m)
+// in both arguments; Fong & Darve, "The black-box fast multipole method", J.
+// Comput. Phys. 228, 2009).  Inputs and outputs are cut into blocks of
+// kFarBlock = 256 samples, and output block b sums
+//   near   blocks b-1, b, b+1 (or b-3 .. b+3, below) term by term, as the dense
+//          contraction does;
+//   far    every other block B through its moments
+//            M_B[j] = sum_m l_j(m) (-1)^m x[m]           (16 source nodes s_j)
+//          turned into 16 values at the target nodes tau_i of block b,
+//            L_b[i] = sum_{B far} sum_j M_B[j] / (tau_i - s_j),
+//          and read at every output as sigma_n sum_i u_i(t_n) L_b[i].
+// The nodes are fixed in each block (the target interval is 64 samples wider
+// on both sides, so that t_n of any output stays inside while |delta| n_out <=
+// 63), so both interpolation errors are below 2e-9 of the far sum (Chebyshev
+// ratio rho >= 3.7 at 16 nodes), itself 3 % of a typical output.  Three
+// launches: far_split_kernel writes the 16-bit planes and, in FP32 from the
+// values the planes hold, the moments; the tile kernel runs the moments-to-nodes
+// product (JOB_FAR: the same Cauchy form, K = 16 per block); the tile kernel
+// runs the near chunks and one more K = 16 step for the far field (JOB_NEAR).
+//
+// The accumulators round toward zero at every MMA, so a long sum loses a little of
+// each output (about 3e-8 per K = 16 step after its largest terms): the dense
+// contraction of 8192 samples is 2.3e-5 off in bf16x3 and 9e-6 in fp16x3, the
+// near and far form 4e-6 and 9e-7.  bf16x3 above 4096 samples takes the blocks
+// within three of its own, its own first (1.0e-5 off): with one block either
+// side the results would be more than 2e-5 from the dense contraction's.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
@@ -85,6 +114,25 @@ template <bool FP16> DC_DEV void split8(const float (&v)[8], uint4& hi, uint4& l
   lo = make_uint4(l[0], l[1], l[2], l[3]);
 }
 
+// One value into its hi and lo halves (lo times 2^11 for fp16).
+template <bool FP16> DC_DEV void split1(float v, uint16_t& hi, uint16_t& lo) {
+  if constexpr (FP16) {
+    const __half a = __float2half_rn(v);
+    hi = __half_as_ushort(a);
+    lo = __half_as_ushort(__float2half_rn((v - __half2float(a)) * 2048.f));
+  } else {
+    const __nv_bfloat16 a = __float2bfloat16_rn(v);
+    hi = __bfloat16_as_ushort(a);
+    lo = __bfloat16_as_ushort(__float2bfloat16_rn(v - __bfloat162float(a)));
+  }
+}
+template <bool FP16> DC_DEV float join1(uint16_t hi, uint16_t lo) {
+  if constexpr (FP16)
+    return fmaf(__half2float(__ushort_as_half(lo)), 1.f / 2048, __half2float(__ushort_as_half(hi)));
+  else
+    return __bfloat162float(__ushort_as_bfloat16(hi)) + __bfloat162float(__ushort_as_bfloat16(lo));
+}
+
 // a n = m_n + e_n with a - 1 a double-float (same arithmetic as the FP32 path).
 DC_DEV void position(float dl_hi, float dl_lo, int n, int& m, float& e) {
   const float fi = (float)n;
@@ -104,16 +152,67 @@ DC_DEV void position(float dl_hi, float dl_lo, int n, int& m, float& e) {
   e = r;
 }
 
-template <bool FP16>
+// ------------------------------------------------ near and far field
+constexpr int kFarBlock = 256;                       // samples per block, both sides
+constexpr int kFarP = 16;                            // nodes per block, both sides
+constexpr int kFarMargin = 64;                       // widening of the target interval
+constexpr float kSrcHalf = 127.5f;                   // source interval [0, 255] about 127.5
+constexpr float kTgtHalf = 128.f + kFarMargin;       // target interval about 127.5
+// Powers of two that keep the 16-bit moments and node values inside fp16's
+// range for any pulse inside it (|M| <= 32 max|x|, |L| <= 17 max|x|):
+// planes hold M / 32 and L / 32, the Cauchy elements are taken times 256.
+constexpr float kMomScale = 1.f / 32, kCauchyScale = 256.f, kLocScale = 1.f / 32;
+
+// Chebyshev node i of kFarP on [-1, 1], and T_k there.
+DC_DEV float far_node(int i) { return cospif((2 * i + 1) / (2.f * kFarP)); }
+DC_DEV float far_cheb(int i, int k) {
+  return cospif((float)((2 * i + 1) * k % (4 * kFarP)) / (2.f * kFarP));
+}
+// Lagrange basis of the nodes at z from the Chebyshev polynomials T_k(z):
+// l_i(z) = (1/p) sum_k d_k T_k(z_i) T_k(z), d_0 = 1, d_k = 2; D[i][k] holds
+// d_k T_k(z_i) / p.
+DC_DEV void far_fill_table(float* D, int tid, int threads) {
+  for (int q = tid; q < kFarP * kFarP; q += threads) {
+    const int i = q / kFarP, k = q % kFarP;
+    D[q] = far_cheb(i, k) * ((k ? 2.f : 1.f) / kFarP);
+  }
+}
+DC_DEV void far_polys(float z, float (&T)[kFarP]) {
+  T[0] = 1.f;
+  T[1] = z;
+#pragma unroll
+  for (int k = 2; k < kFarP; ++k) T[k] = fmaf(2.f * z, T[k - 1], -T[k - 2]);
+}
+DC_DEV float far_basis(const float* D, int i, const float (&T)[kFarP]) {
+  float v = 0.f;
+#pragma unroll
+  for (int k = 0; k < kFarP; ++k) v = fmaf(D[i * kFarP + k], T[k], v);
+  return v;
+}
+
+constexpr int kFarMinIn = 1536;                      // see exact_tc_far
+constexpr int kFarWideIn = 4096;                     // bf16x3 above: near = 3 blocks either side
+
+// What one launch of the tile kernel contracts.
+enum Job : int {
+  JOB_DENSE = 0,   // every input sample
+  JOB_NEAR = 1,    // the blocks around the output's own, and the far field from the node values
+  JOB_FAR = 2,     // block moments -> node values (rows (b, i), columns of K (B, j))
+};
+
+template <bool FP16, int JOB>
 __global__ void __launch_bounds__(kThreads, 1)
     exact_tc_kernel(const __grid_constant__ CUtensorMap map_hi,
-                    const __grid_constant__ CUtensorMap map_lo, ExTcArgs a) {
+                    const __grid_constant__ CUtensorMap map_lo,
+                    const __grid_constant__ CUtensorMap map_far_hi,
+                    const __grid_constant__ CUtensorMap map_far_lo, ExTcArgs a) {
   using C = Cfg<FP16>;
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) unsigned long long full_bar[C::STAGES], empty_bar[C::STAGES], acc_bar;
   __shared__ uint32_t tmem_base;
   __shared__ float s_sig[C::BM], s_e[C::BM];
   __shared__ int s_m[C::BM];
+  __shared__ float s_far[JOB == JOB_DENSE ? 1 : kFarP * kFarP];   // basis table, or source nodes
 
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~(uintptr_t)1023);
@@ -121,7 +220,24 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int n0 = blockIdx.x * C::BM;
   const int c0 = blockIdx.y * BN;
   const int alpha = blockIdx.z;
-  const int nk = (a.n_in + BK - 1) / BK;
+  // the K chunks of this tile: all of the planes' chunks, or (JOB_NEAR) those
+  // of the blocks around the tile's own and then one chunk of node values
+  const int blk = n0 / kFarBlock;              // output block of the tile
+  int k0 = 0, nk = (a.n_in + BK - 1) / BK, own = 0;
+  if constexpr (JOB == JOB_NEAR) {
+    constexpr int kPer = kFarBlock / BK;
+    k0 = max(0, (blk - a.near) * kPer);
+    const int planes = max(0, min(nk, (blk + a.near + 1) * kPer) - k0);
+    if (a.own_first) own = min(blk * kPer - k0, planes);
+    nk = planes + 1;
+  }
+  // plane chunk of step kc (own_first: the output's own block first, then
+  // those above it, then those below)
+  auto chunk_of = [&](int kc) {
+    if constexpr (JOB != JOB_NEAR) return kc;
+    const int c = kc + own;
+    return k0 + (c < nk - 1 ? c : c - (nk - 1));
+  };
   constexpr uint32_t kCols = 512;
 
   if (threadIdx.x == 0) {
@@ -139,13 +255,23 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
   if (warp >= 2 && threadIdx.x - 64 < C::BM) {
     const int nl = threadIdx.x - 64;
-    int m;
-    float e;
-    position(a.dl[2 * alpha], a.dl[2 * alpha + 1], n0 + nl, m, e);
-    const float s = sinpif(e) * kInvPi;
-    s_m[nl] = m;
-    s_e[nl] = e;
-    s_sig[nl] = (m & 1) ? -s : s;
+    if constexpr (JOB == JOB_FAR) {
+      // row (b, i): target node i of block b, relative to the block's centre
+      s_m[nl] = (n0 + nl) / kFarP;
+      s_e[nl] = kTgtHalf * far_node((n0 + nl) % kFarP);
+    } else {
+      int m;
+      float e;
+      position(a.dl[2 * alpha], a.dl[2 * alpha + 1], n0 + nl, m, e);
+      const float s = sinpif(e) * kInvPi;
+      s_m[nl] = m;
+      s_e[nl] = e;
+      s_sig[nl] = (m & 1) ? -s : s;
+    }
+  }
+  if constexpr (JOB == JOB_NEAR) far_fill_table(s_far, threadIdx.x, kThreads);
+  if constexpr (JOB == JOB_FAR) {
+    if (threadIdx.x < kFarP) s_far[threadIdx.x] = kSrcHalf * far_node(threadIdx.x);
   }
   tc_fence_before();
   __syncthreads();
@@ -163,8 +289,13 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (!mbar_wait_bounded(&empty_bar[s], ph ^ 1, a.err)) { ok = false; break; }
         uint8_t* st = smem + s * C::STAGE;
         mbar_expect_tx(&full_bar[s], 2 * kBPlane);
-        tma_load_2d(st + C::A_BYTES, &map_hi, kc * BK, row0, &full_bar[s]);
-        tma_load_2d(st + C::A_BYTES + kBPlane, &map_lo, kc * BK, row0, &full_bar[s]);
+        if (JOB == JOB_NEAR && kc == nk - 1) {       // the block's 16 node values (the first half)
+          tma_load_2d(st + C::A_BYTES, &map_far_hi, blk * kFarP, row0, &full_bar[s]);
+          tma_load_2d(st + C::A_BYTES + kBPlane, &map_far_lo, blk * kFarP, row0, &full_bar[s]);
+        } else {
+          tma_load_2d(st + C::A_BYTES, &map_hi, chunk_of(kc) * BK, row0, &full_bar[s]);
+          tma_load_2d(st + C::A_BYTES + kBPlane, &map_lo, chunk_of(kc) * BK, row0, &full_bar[s]);
+        }
       }
     }
   } else if (warp == 1) {
@@ -180,6 +311,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         const uint32_t b_hi = st + C::A_BYTES, b_lo = b_hi + kBPlane;
 #pragma unroll
         for (int kk = 0; kk < BK / 16; ++kk) {
+          if (JOB == JOB_NEAR && kk > 0 && kc == nk - 1) break;   // 16 node values only
           const uint32_t off = kk * 32;     // 16 elements of K = 32 bytes inside the swizzle atom
           const uint32_t acc = (kc > 0 || kk > 0) ? 1u : 0u;
 #pragma unroll
@@ -219,11 +351,29 @@ __global__ void __launch_bounds__(kThreads, 1)
       const uint32_t ph = (kc / C::STAGES) & 1;
       if (!mbar_wait_bounded(&empty_bar[s], ph ^ 1, a.err)) { ok = false; break; }
       uint8_t* st = smem + s * C::STAGE;
+      const bool far = JOB == JOB_NEAR && kc == nk - 1;
 #pragma unroll
       for (int q = 0; q < CHUNKS; ++q) {
         const int k8 = cbase + q;              // 16-byte chunk of the 64-byte row
         float v[8];
-        const int m0 = kc * BK + k8 * 8;
+        const int m0 = chunk_of(kc) * BK + k8 * 8;
+        if (far) {
+          // sigma_n u_i(t_n), i = 8 k8 .. + 7, at t_n relative to the block's centre
+          if (k8 >= kFarP / 8) continue;       // the MMA reads 16 columns of this chunk
+          float T[kFarP];
+          far_polys(((float)(mn - blk * kFarBlock) - 127.5f + en) * (1.f / kTgtHalf), T);
+          const float sc = sg * (1.f / kLocScale);
+#pragma unroll
+          for (int i = 0; i < 8; ++i) v[i] = sc * far_basis(s_far, k8 * 8 + i, T);
+        } else if (JOB == JOB_FAR) {
+          // 1 / (tau_i - s_j) of blocks b (the row's) and B = m0 / 16, times 2^8
+          const int db = mn - m0 / kFarP;
+          const float c = exact_i2f(db * kFarBlock) + en;
+          const bool live = db < -a.near || db > a.near;
+#pragma unroll
+          for (int i = 0; i < 8; ++i)
+            v[i] = live ? __fdividef(kCauchyScale, c - s_far[(m0 + i) % kFarP]) : 0.f;
+        } else {
         // (m_n - m) + e_n with the integer part formed exactly first
         // ((m_n - m0) - i, integers below 2^22) and e_n added last, so the
         // denominator near m = m_n is e_n itself even when e_n is far below
@@ -238,6 +388,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             else val = __fdividef((i & 1) ? -sg : sg, (di0 - (float)i) + en);
           }
           v[i] = val;
+        }
         }
         // (-1)^m: m = kc*32 + k8*8 + i has the parity of i
         uint4 hi, lo;
@@ -270,7 +421,20 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
             for (int i = 0; i < 16; ++i) f[i] = fmaf(g[i], 1.0f / 2048.f, f[i]);
           }
-          if (n < a.n_out) {
+          if (JOB == JOB_FAR) {
+            if (n < a.n_out) {
+#pragma unroll
+              for (int i = 0; i < 16; ++i) {
+                const int col = c0 + cc * 16 + i;
+                if (col >= 2 * a.n_pulses) break;
+                uint16_t hi, lo;
+                split1<FP16>(f[i] * (kLocScale / (kMomScale * kCauchyScale)), hi, lo);
+                const size_t o = ((size_t)alpha * 2 * a.n_pulses + col) * a.n_out + n;
+                a.loc_hi[o] = hi;
+                a.loc_lo[o] = lo;
+              }
+            }
+          } else if (n < a.n_out) {
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
               const int pulse = (c0 + cc * 16) / 2 + i;
@@ -306,20 +470,129 @@ __global__ void split_planes_kernel(const float2* __restrict__ x, int n, long lo
 #pragma unroll
     for (int c = 0; c < 2; ++c) {
       uint16_t h, l;
-      if constexpr (FP16) {
-        const __half a = __float2half_rn(vv[c]);
-        const __half b = __float2half_rn((vv[c] - __half2float(a)) * 2048.f);
-        h = __half_as_ushort(a);
-        l = __half_as_ushort(b);
-      } else {
-        const __nv_bfloat16 a = __float2bfloat16_rn(vv[c]);
-        const __nv_bfloat16 b = __float2bfloat16_rn(vv[c] - __bfloat162float(a));
-        h = __bfloat16_as_ushort(a);
-        l = __bfloat16_as_ushort(b);
-      }
+      split1<FP16>(vv[c], h, l);
       const long long o = (2 * pr + c) * (long long)ld + m;
       hi[o] = h;
       lo[o] = l;
+    }
+  }
+}
+
+// The planes as split_planes_kernel writes them, and the block moments
+// M_B[j] = sum_m l_j(m) (-1)^m x[m] of the values the planes hold, in FP32,
+// written as planes too (row 2p / 2p + 1, element 16 B + j, times kMomScale).
+// One warp per two consecutive blocks of a pulse: a lane holds 2 x 8 samples,
+// forms its share of the 2 x 16 complex moments (packed FMAs, the weights
+// from shared memory), and a halving exchange over the lanes leaves moment
+// j = lane % 16 of block lane / 16 in each lane.
+constexpr int kFsWarps = 8;
+template <bool FP16>
+__global__ void __launch_bounds__(32 * kFsWarps, 2)
+    far_split_kernel(const float2* __restrict__ x, int n, long long rows_c, int ld, uint16_t* hi,
+                     uint16_t* lo, int ld_mom, uint16_t* mom_hi, uint16_t* mom_lo) {
+  __shared__ float s_w[kFarP * kFarBlock];             // l_j(m) (-1)^m kMomScale at [j][m]
+  __shared__ float s_D[kFarP * kFarP];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  far_fill_table(s_D, threadIdx.x, blockDim.x);
+  __syncthreads();
+  {
+    static_assert(32 * kFsWarps == kFarBlock, "one thread per sample of a block");
+    const int m = threadIdx.x;
+    float T[kFarP];
+    far_polys(((float)m - 127.5f) * (1.f / kSrcHalf), T);
+#pragma unroll 1
+    for (int j = 0; j < kFarP; ++j)
+      s_w[j * kFarBlock + m] = far_basis(s_D, j, T) * ((m & 1) ? -kMomScale : kMomScale);
+  }
+  __syncthreads();
+  const int nb = (n + kFarBlock - 1) / kFarBlock;
+  const int n_pair = (nb + 1) / 2;                     // block pairs of a pulse
+  const long long total = rows_c * n_pair;
+  for (long long g = blockIdx.x * (long long)kFsWarps + warp; g < total;
+       g += (long long)gridDim.x * kFsWarps) {
+    const long long pr = g / n_pair;
+    const int m0 = (int)(g - pr * n_pair) * 2 * kFarBlock + 2 * lane;
+    const float2* xp = x + pr * n;
+    float2 v[2][4][2];
+    const bool al = (reinterpret_cast<uintptr_t>(xp) & 15) == 0;   // m0 is even
+#pragma unroll
+    for (int b = 0; b < 2; ++b)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int m = m0 + b * kFarBlock + 64 * q;
+        v[b][q][0] = v[b][q][1] = make_float2(0.f, 0.f);
+        if (al && m + 1 < n) {
+          const float4 t = __ldcs(reinterpret_cast<const float4*>(xp + m));
+          v[b][q][0] = make_float2(t.x, t.y);
+          v[b][q][1] = make_float2(t.z, t.w);
+        } else {
+          if (m < n) v[b][q][0] = __ldcs(xp + m);
+          if (m + 1 < n) v[b][q][1] = __ldcs(xp + m + 1);
+        }
+      }
+#pragma unroll
+    for (int b = 0; b < 2; ++b)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int m = m0 + b * kFarBlock + 64 * q;
+        uint16_t h[2][2], l[2][2];                     // [re, im][sample]
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          split1<FP16>(v[b][q][i].x, h[0][i], l[0][i]);
+          split1<FP16>(v[b][q][i].y, h[1][i], l[1][i]);
+          v[b][q][i] = make_float2(join1<FP16>(h[0][i], l[0][i]), join1<FP16>(h[1][i], l[1][i]));
+        }
+        if (m < n) {                                   // m + 1 < ld: the row pitch is even
+#pragma unroll
+          for (int c = 0; c < 2; ++c) {
+            const long long o = (2 * pr + c) * (long long)ld + m;
+            *reinterpret_cast<uint32_t*>(hi + o) = h[c][0] | ((uint32_t)h[c][1] << 16);
+            *reinterpret_cast<uint32_t*>(lo + o) = l[c][0] | ((uint32_t)l[c][1] << 16);
+          }
+        }
+      }
+    float acc[64];                                     // [block][node][re, im]
+#pragma unroll
+    for (int j = 0; j < kFarP; ++j) {
+      float2 s[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const float2 w = *reinterpret_cast<const float2*>(s_w + j * kFarBlock + 64 * q + 2 * lane);
+        const float2 w0 = make_float2(w.x, w.x), w1 = make_float2(w.y, w.y);
+#pragma unroll
+        for (int b = 0; b < 2; ++b) {
+          s[b] = __ffma2_rn(v[b][q][0], w0, s[b]);
+          s[b] = __ffma2_rn(v[b][q][1], w1, s[b]);
+        }
+      }
+#pragma unroll
+      for (int b = 0; b < 2; ++b) {
+        acc[b * 32 + 2 * j] = s[b].x;
+        acc[b * 32 + 2 * j + 1] = s[b].y;
+      }
+    }
+    // halving exchange: after the step over lane bit o, a lane keeps the half
+    // of its values that its bit selects, summed with its partner's
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const bool up = lane & o;
+#pragma unroll
+      for (int i = 0; i < 2 * o; ++i) {
+        const float keep = up ? acc[i + 2 * o] : acc[i];
+        const float send = up ? acc[i] : acc[i + 2 * o];
+        acc[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+      }
+    }
+    const int e = (m0 - 2 * lane) / kFarBlock * kFarP + lane;   // node lane % 16 of block lane / 16
+    if (e < nb * kFarP) {
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        uint16_t h, l;
+        split1<FP16>(acc[c], h, l);
+        const long long o = (2 * pr + c) * (long long)ld_mom + e;
+        mom_hi[o] = h;
+        mom_lo[o] = l;
+      }
     }
   }
 }
@@ -352,39 +625,86 @@ bool make_map(CUtensorMap* m, void* base, bool fp16, long long rows, int n, int 
 
 }  // namespace
 
+namespace {
+
+int far_blocks(int n) { return (n + kFarBlock - 1) / kFarBlock; }
+
+template <bool FP16, int JOB>
+cudaError_t launch_tiles(const CUtensorMap& mh, const CUtensorMap& ml, const CUtensorMap& fh,
+                         const CUtensorMap& fl, const ExTcArgs& args, int n_alpha, cudaStream_t s) {
+  using C = Cfg<FP16>;
+  dim3 grid((args.n_out + C::BM - 1) / C::BM, (2 * args.n_pulses + BN - 1) / BN, n_alpha);
+  auto k = exact_tc_kernel<FP16, JOB>;
+  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
+  if (e != cudaSuccess) return e;
+  k<<<grid, kThreads, C::SMEM, s>>>(mh, ml, fh, fl, args);
+  return cudaGetLastError();
+}
+
+template <bool FP16>
+cudaError_t run_exact_tc(const float2* x, long long x_rows_c, int n, const ExTcPlanes& pl,
+                         const ExTcArgs& args, int n_alpha, cudaStream_t s) {
+  const int ld = (n + 7) / 8 * 8;
+  CUtensorMap mh, ml;
+  if (!make_map(&mh, pl.hi, FP16, 2 * x_rows_c, n, ld) || !make_map(&ml, pl.lo, FP16, 2 * x_rows_c, n, ld))
+    return cudaErrorInvalidValue;
+  if (!pl.far) {
+    const long long total = x_rows_c * n;
+    const int grid_c = (int)std::min<long long>((total + 255) / 256, 152LL * 32);
+    split_planes_kernel<FP16><<<grid_c, 256, 0, s>>>(x, n, x_rows_c, ld, (uint16_t*)pl.hi, (uint16_t*)pl.lo);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    return launch_tiles<FP16, JOB_DENSE>(mh, ml, mh, ml, args, n_alpha, s);
+  }
+  // moments of the pulses' blocks, node values of the outputs' blocks
+  const int kb = kFarP * far_blocks(n), ob = kFarP * far_blocks(args.n_out);
+  CUtensorMap qh, ql, fh, fl;
+  if (!make_map(&qh, pl.mom_hi, FP16, 2 * x_rows_c, kb, kb) || !make_map(&ql, pl.mom_lo, FP16, 2 * x_rows_c, kb, kb) ||
+      !make_map(&fh, pl.loc_hi, FP16, 2 * x_rows_c, ob, ob) || !make_map(&fl, pl.loc_lo, FP16, 2 * x_rows_c, ob, ob))
+    return cudaErrorInvalidValue;
+  const long long pairs = x_rows_c * ((far_blocks(n) + 1) / 2);
+  const int grid_c = (int)std::min<long long>((pairs + kFsWarps - 1) / kFsWarps, 152LL * 2);
+  far_split_kernel<FP16><<<grid_c, 32 * kFsWarps, 0, s>>>(x, n, x_rows_c, ld, (uint16_t*)pl.hi, (uint16_t*)pl.lo, kb,
+                                                          (uint16_t*)pl.mom_hi, (uint16_t*)pl.mom_lo);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  ExTcArgs g = args;
+  g.near = !FP16 && n > kFarWideIn ? 3 : 1;
+  g.own_first = g.near > 1;
+  ExTcArgs f = g;
+  f.n_in = kb;
+  f.n_out = ob;
+  f.loc_hi = (uint16_t*)pl.loc_hi;
+  f.loc_lo = (uint16_t*)pl.loc_lo;
+  // the node values depend on the pulses only: one set per group of pulses
+  if ((e = launch_tiles<FP16, JOB_FAR>(qh, ql, qh, ql, f, args.rows_per_alpha ? n_alpha : 1, s))) return e;
+  return launch_tiles<FP16, JOB_NEAR>(mh, ml, fh, fl, g, n_alpha, s);
+}
+
+}  // namespace
+
 size_t exact_tc_plane_bytes(long long rows, int n) {
   const long long ld = (n + 7) / 8 * 8;
   return (size_t)rows * ld * 2;
 }
 
-cudaError_t launch_exact_tc(bool fp16, const float2* x, long long x_rows_c, int n, void* hi, void* lo,
+// The near and far form replaces n_in / 32 chunks by at most 25 (bf16x3 above
+// 4096: 57) and adds two launches.  Measured, far against dense, in us (bf16x3;
+// 8 pulses x 1 rate, 512 x 1, 512 x 16): n = 1025: 62 / 63, 75 / 68, 168 / 197;
+// 1536: 62 / 86, 74 / 93, 195 / 275; 2048: 64 / 111, 76 / 119, 251 / 448; 8192 at
+// 512 x 16: 1478 / 5172.  fp16x3: 1300: 43 / 47, 56 / 51, 192 / 238; 1536: 43 / 53,
+// 56 / 59, 206 / 307; 6000: 51 / 170, 97 / 320, 761 / 3187.
+bool exact_tc_far(int n_in, int n_out, double delta_max) {
+  return n_in >= kFarMinIn && delta_max * (double)n_out <= (double)(kFarMargin - 1);
+}
+size_t exact_tc_far_plane_bytes(long long rows, int n) {
+  return (size_t)rows * kFarP * far_blocks(n) * 2;
+}
+
+cudaError_t launch_exact_tc(bool fp16, const float2* x, long long x_rows_c, int n, const ExTcPlanes& pl,
                             const ExTcArgs& args, int n_alpha, cudaStream_t s) {
-  const int ld = (n + 7) / 8 * 8;
-  const long long total = x_rows_c * n;
-  const int grid_c = (int)std::min<long long>((total + 255) / 256, 152LL * 32);
-  if (fp16)
-    split_planes_kernel<true><<<grid_c, 256, 0, s>>>(x, n, x_rows_c, ld, (uint16_t*)hi, (uint16_t*)lo);
-  else
-    split_planes_kernel<false><<<grid_c, 256, 0, s>>>(x, n, x_rows_c, ld, (uint16_t*)hi, (uint16_t*)lo);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  CUtensorMap mh, ml;
-  if (!make_map(&mh, hi, fp16, 2 * x_rows_c, n, ld) || !make_map(&ml, lo, fp16, 2 * x_rows_c, n, ld))
-    return cudaErrorInvalidValue;
-  if (fp16) {
-    using Cf = Cfg<true>;
-    dim3 grid((args.n_out + Cf::BM - 1) / Cf::BM, (2 * args.n_pulses + BN - 1) / BN, n_alpha);
-    auto k = exact_tc_kernel<true>;
-    if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, Cf::SMEM))) return e;
-    k<<<grid, kThreads, Cf::SMEM, s>>>(mh, ml, args);
-  } else {
-    using Cb = Cfg<false>;
-    dim3 grid((args.n_out + Cb::BM - 1) / Cb::BM, (2 * args.n_pulses + BN - 1) / BN, n_alpha);
-    auto k = exact_tc_kernel<false>;
-    if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, Cb::SMEM))) return e;
-    k<<<grid, kThreads, Cb::SMEM, s>>>(mh, ml, args);
-  }
-  return cudaGetLastError();
+  return fp16 ? run_exact_tc<true>(x, x_rows_c, n, pl, args, n_alpha, s)
+              : run_exact_tc<false>(x, x_rows_c, n, pl, args, n_alpha, s);
 }
 
 }  // namespace dc

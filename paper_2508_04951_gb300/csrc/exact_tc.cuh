@@ -12,14 +12,34 @@ struct ExTcArgs {
   float2* y;               // [n_alpha][n_pulses][n_out]
   const float* dl;         // per alpha: (alpha - 1) as hi, lo floats
   int* err;                // device error flag (bounded waits)
+  // far-field pass only: its output planes [rows of the pulses][n_out]
+  uint16_t *loc_hi, *loc_lo;
+  // near and far field: blocks either side taken term by term; whether the
+  // output's own block is summed first
+  int near, own_first;
+};
+
+// Device scratch of one call: the split planes (exact_tc_plane_bytes each)
+// and, with `far`, the planes of block moments (exact_tc_far_plane_bytes of
+// n) and of node values (exact_tc_far_plane_bytes of n_out).
+struct ExTcPlanes {
+  void *hi, *lo;
+  bool far;
+  void *mom_hi, *mom_lo, *loc_hi, *loc_lo;
 };
 
 // Bytes of one 16-bit split plane for `rows` real rows of n samples.
 size_t exact_tc_plane_bytes(long long rows, int n);
 
-// Split x (x_rows_c complex pulses of n samples) into hi / lo planes (two
-// buffers of exact_tc_plane_bytes(2 x_rows_c, n)), then run the contraction.
-cudaError_t launch_exact_tc(bool fp16, const float2* x, long long x_rows_c, int n, void* hi, void* lo,
+// Whether blocks away from an output are summed through their moments:
+// n_in long enough, and every output within 63 samples of its own index
+// (delta_max: the largest |alpha - 1|).
+bool exact_tc_far(int n_in, int n_out, double delta_max);
+size_t exact_tc_far_plane_bytes(long long rows, int n);
+
+// Split x (x_rows_c complex pulses of n samples) into the planes, then run the
+// contraction.
+cudaError_t launch_exact_tc(bool fp16, const float2* x, long long x_rows_c, int n, const ExTcPlanes& planes,
                             const ExTcArgs& args, int n_alpha, cudaStream_t s);
 
 }  // namespace dc
