@@ -56,6 +56,7 @@ struct dc_ctx {
   // While a plan is being recorded: item uploads go to this host staging
   // buffer (copied to the plan's device item buffer once the capture ends).
   std::vector<char>* rec = nullptr;
+  bool fixed_ws = false;      // the scratch is the caller's (a server's pool block): never grown
   // per-phase CUDA-event timing (dc_profile_enable / dc_profile_read)
   bool profiling = false;
   struct Rec { int phase; cudaEvent_t a, b; long long samples; };
@@ -246,6 +247,30 @@ dc_status ensure_ws(dc_ctx* c, size_t bytes) {
   c->ws = (char*)p;
   c->ws_bytes = want;
   return DC_OK;
+}
+
+// Scratch that only a faster form of a call wants: true when the context has
+// it or can grow to it, leaving no error behind when it cannot.
+bool try_ws(dc_ctx* c, size_t bytes) {
+  if (bytes <= c->ws_bytes) return true;
+  if (c->rec || c->fixed_ws) return false;
+  const std::string msg = c->last_error;
+  if (ensure_ws(c, bytes) == DC_OK) return true;
+  c->last_error = msg;
+  return false;
+}
+
+// Near and far scratch of an FP32 exact sum, taken at offset `at` of the
+// context's scratch where the form applies and the scratch can be had.
+void exact_far(dc_ctx* c, ExArgs& a, int n_alpha, double delta_max, size_t at) {
+  if (!exact_fp32_far(a.n_in, a.n_out, a.n_pulses, n_alpha, delta_max)) return;
+  const long long groups = a.shared ? 1 : n_alpha;
+  at = (at + 255) & ~(size_t)255;
+  const size_t mom = exact_fp32_far_elems(groups * a.n_pulses, a.n_in);
+  const size_t loc = exact_fp32_far_elems(groups * a.n_pulses, a.n_out);
+  if (!try_ws(c, at + (mom + loc) * sizeof(float2))) return;
+  a.mom = reinterpret_cast<float2*>(c->ws + at);
+  a.loc = a.mom + mom;
 }
 
 dc_status ensure_items(dc_ctx* c, size_t bytes) {
@@ -824,6 +849,7 @@ dc_status doppler_resample(dc_ctx* c, const dc_c64* x, long long n, dc_c64* y, d
   const ExItem* dev = nullptr;
   if ((st = upload(c, ex, 0, s, &dev))) return st;
   ExArgs a{dev, (int)n, (int)n_out, 1};
+  exact_far(c, a, 1, std::fabs(dl), 0);
   Phase ph(c, PH_EXACT, s, n_out);
   cudaError_t e = launch_exact_fp32(a, 1, s);
   if (e != cudaSuccess) return cuda_fail(c, e, "exact launch");
@@ -886,6 +912,17 @@ dc_status correct_batch(dc_ctx* c, const dc_c64* in, dc_c64* out, const dc_item*
   const std::vector<size_t>& class_chunk = lay.class_chunk;
   if ((st = ensure_ws(c, lay.bytes))) return st;
   if ((st = ensure_items(c, items_bytes_for((size_t)n_items * 4)))) return st;
+  if (o.mode == DC_EXACT_FP32) {
+    // the near and far scratch lies behind the batch's, one item's at a time;
+    // grown to the largest first, as the layout's pointers come from c->ws
+    size_t far = 0;
+    for (int i = 0; i < n_items; ++i) {
+      const int no = (int)(items[i].n_out ? items[i].n_out : items[i].n);
+      if (exact_fp32_far((int)items[i].n, no, 1, 1, std::fabs(alpha_minus_one(items[i].v_r))))
+        far = std::max(far, exact_fp32_far_elems(1, (int)items[i].n) + exact_fp32_far_elems(1, no));
+    }
+    if (far) try_ws(c, ((lay.bytes + 255) & ~(size_t)255) + far * sizeof(float2));
+  }
   char* ws = c->ws;
   size_t item_at = 0;
 
@@ -919,6 +956,7 @@ dc_status correct_batch(dc_ctx* c, const dc_c64* in, dc_c64* out, const dc_item*
       if ((st = upload(c, ex, item_at, s, &dev))) return st;
       item_at += 256;
       ExArgs a{dev, (int)it.n, (int)(it.n_out ? it.n_out : it.n), 1};
+      if (lay.bytes < c->ws_bytes) exact_far(c, a, 1, std::fabs(dl), lay.bytes);
       Phase ph(c, PH_EXACT, s, a.n_out);
       cudaError_t e = launch_exact_fp32(a, 1, s);
       if (e != cudaSuccess) return cuda_fail(c, e, "exact launch");
@@ -1258,6 +1296,9 @@ extern "C" dc_status correct_compress(dc_ctx* c, const dc_c64* x, long long n,
   const size_t t_at = ar.take(log2L > 12 ? L * sizeof(float2) : 0);
   if ((st = ensure_ws(c, ar.off))) return st;
   if ((st = ensure_items(c, items_bytes_for(16)))) return st;
+  const double dl = alpha_minus_one(v_r);
+  ExArgs ea{nullptr, (int)n, (int)n_out, 1};
+  if (o.mode == DC_EXACT_FP32) exact_far(c, ea, 1, std::fabs(dl), ar.off);   // before c->ws is read
   char* ws = c->ws;
   float2* Yr = reinterpret_cast<float2*>(ws + y_at);
   float2* H = reinterpret_cast<float2*>(ws + h_at);
@@ -1265,7 +1306,6 @@ extern "C" dc_status correct_compress(dc_ctx* c, const dc_c64* x, long long n,
   float2* T = reinterpret_cast<float2*>(ws + t_at);
   size_t item_at = 0;
   cudaError_t e;
-  const double dl = alpha_minus_one(v_r);
   // 1. resampling
   if (o.mode == DC_EXACT_FP32) {
     std::vector<ExItem> ex(1);
@@ -1277,9 +1317,9 @@ extern "C" dc_status correct_compress(dc_ctx* c, const dc_c64* x, long long n,
     const ExItem* dev = nullptr;
     if ((st = upload(c, ex, item_at, s, &dev))) return st;
     item_at += 256;
-    ExArgs a{dev, (int)n, (int)n_out, 1};
+    ea.items = dev;
     Phase ph(c, PH_EXACT, s, n_out);
-    if ((e = launch_exact_fp32(a, 1, s)) != cudaSuccess) return cuda_fail(c, e, "exact launch");
+    if ((e = launch_exact_fp32(ea, 1, s)) != cudaSuccess) return cuda_fail(c, e, "exact launch");
   } else {
     std::vector<RsItem> rs(1);
     rs[0] = RsItem{};
@@ -1413,6 +1453,10 @@ extern "C" dc_status resample_exact_batch(dc_ctx* c, const dc_c64* x, long long 
   const ExItem* dev = nullptr;
   if ((st = upload(c, ex, 0, s, &dev))) return st;
   ExArgs a{dev, (int)n, (int)n_out, n_pulses};
+  a.shared = stride == 0;
+  double delta_max = 0.0;
+  for (int i = 0; i < n_alpha; ++i) delta_max = std::max(delta_max, std::fabs(alpha_minus_one(v_r[i])));
+  exact_far(c, a, n_alpha, delta_max, 0);
   Phase ph(c, PH_EXACT, s, (long long)n_alpha * n_pulses * n_out);
   cudaError_t e = launch_exact_fp32(a, n_alpha, s);
   if (e != cudaSuccess) return cuda_fail(c, e, "exact launch");
@@ -1778,10 +1822,12 @@ dc_status dc_internal_correct_batch_ws(dc_ctx* c, const dc_c64* in, dc_c64* out,
   char* ws0 = c->ws;
   const size_t b0 = c->ws_bytes;
   c->ws = static_cast<char*>(ws);
+  c->fixed_ws = true;
   c->ws_bytes = ws_bytes;
   const dc_status st = correct_batch(c, in, out, items, n_items, opts, stream);
   c->ws = ws0;
   c->ws_bytes = b0;
+  c->fixed_ws = false;
   return st;
 }
 

@@ -60,6 +60,7 @@
 #include <algorithm>
 
 #include "exact_tc.cuh"
+#include "far.cuh"
 #include "tc.cuh"
 
 namespace dc {
@@ -152,43 +153,10 @@ DC_DEV void position(float dl_hi, float dl_lo, int n, int& m, float& e) {
   e = r;
 }
 
-// ------------------------------------------------ near and far field
-constexpr int kFarBlock = 256;                       // samples per block, both sides
-constexpr int kFarP = 16;                            // nodes per block, both sides
-constexpr int kFarMargin = 64;                       // widening of the target interval
-constexpr float kSrcHalf = 127.5f;                   // source interval [0, 255] about 127.5
-constexpr float kTgtHalf = 128.f + kFarMargin;       // target interval about 127.5
 // Powers of two that keep the 16-bit moments and node values inside fp16's
 // range for any pulse inside it (|M| <= 32 max|x|, |L| <= 17 max|x|):
 // planes hold M / 32 and L / 32, the Cauchy elements are taken times 256.
 constexpr float kMomScale = 1.f / 32, kCauchyScale = 256.f, kLocScale = 1.f / 32;
-
-// Chebyshev node i of kFarP on [-1, 1], and T_k there.
-DC_DEV float far_node(int i) { return cospif((2 * i + 1) / (2.f * kFarP)); }
-DC_DEV float far_cheb(int i, int k) {
-  return cospif((float)((2 * i + 1) * k % (4 * kFarP)) / (2.f * kFarP));
-}
-// Lagrange basis of the nodes at z from the Chebyshev polynomials T_k(z):
-// l_i(z) = (1/p) sum_k d_k T_k(z_i) T_k(z), d_0 = 1, d_k = 2; D[i][k] holds
-// d_k T_k(z_i) / p.
-DC_DEV void far_fill_table(float* D, int tid, int threads) {
-  for (int q = tid; q < kFarP * kFarP; q += threads) {
-    const int i = q / kFarP, k = q % kFarP;
-    D[q] = far_cheb(i, k) * ((k ? 2.f : 1.f) / kFarP);
-  }
-}
-DC_DEV void far_polys(float z, float (&T)[kFarP]) {
-  T[0] = 1.f;
-  T[1] = z;
-#pragma unroll
-  for (int k = 2; k < kFarP; ++k) T[k] = fmaf(2.f * z, T[k - 1], -T[k - 2]);
-}
-DC_DEV float far_basis(const float* D, int i, const float (&T)[kFarP]) {
-  float v = 0.f;
-#pragma unroll
-  for (int k = 0; k < kFarP; ++k) v = fmaf(D[i * kFarP + k], T[k], v);
-  return v;
-}
 
 constexpr int kFarMinIn = 1536;                      // see exact_tc_far
 constexpr int kFarWideIn = 4096;                     // bf16x3 above: near = 3 blocks either side
@@ -481,10 +449,7 @@ __global__ void split_planes_kernel(const float2* __restrict__ x, int n, long lo
 // The planes as split_planes_kernel writes them, and the block moments
 // M_B[j] = sum_m l_j(m) (-1)^m x[m] of the values the planes hold, in FP32,
 // written as planes too (row 2p / 2p + 1, element 16 B + j, times kMomScale).
-// One warp per two consecutive blocks of a pulse: a lane holds 2 x 8 samples,
-// forms its share of the 2 x 16 complex moments (packed FMAs, the weights
-// from shared memory), and a halving exchange over the lanes leaves moment
-// j = lane % 16 of block lane / 16 in each lane.
+// One warp per two consecutive blocks of a pulse (far_moments).
 constexpr int kFsWarps = 8;
 template <bool FP16>
 __global__ void __launch_bounds__(32 * kFsWarps, 2)
@@ -495,15 +460,8 @@ __global__ void __launch_bounds__(32 * kFsWarps, 2)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   far_fill_table(s_D, threadIdx.x, blockDim.x);
   __syncthreads();
-  {
-    static_assert(32 * kFsWarps == kFarBlock, "one thread per sample of a block");
-    const int m = threadIdx.x;
-    float T[kFarP];
-    far_polys(((float)m - 127.5f) * (1.f / kSrcHalf), T);
-#pragma unroll 1
-    for (int j = 0; j < kFarP; ++j)
-      s_w[j * kFarBlock + m] = far_basis(s_D, j, T) * ((m & 1) ? -kMomScale : kMomScale);
-  }
+  static_assert(32 * kFsWarps == kFarBlock, "one thread per sample of a block");
+  far_fill_weights(s_w, s_D, threadIdx.x, kMomScale);
   __syncthreads();
   const int nb = (n + kFarBlock - 1) / kFarBlock;
   const int n_pair = (nb + 1) / 2;                     // block pairs of a pulse
@@ -551,38 +509,9 @@ __global__ void __launch_bounds__(32 * kFsWarps, 2)
           }
         }
       }
-    float acc[64];                                     // [block][node][re, im]
-#pragma unroll
-    for (int j = 0; j < kFarP; ++j) {
-      float2 s[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const float2 w = *reinterpret_cast<const float2*>(s_w + j * kFarBlock + 64 * q + 2 * lane);
-        const float2 w0 = make_float2(w.x, w.x), w1 = make_float2(w.y, w.y);
-#pragma unroll
-        for (int b = 0; b < 2; ++b) {
-          s[b] = __ffma2_rn(v[b][q][0], w0, s[b]);
-          s[b] = __ffma2_rn(v[b][q][1], w1, s[b]);
-        }
-      }
-#pragma unroll
-      for (int b = 0; b < 2; ++b) {
-        acc[b * 32 + 2 * j] = s[b].x;
-        acc[b * 32 + 2 * j + 1] = s[b].y;
-      }
-    }
-    // halving exchange: after the step over lane bit o, a lane keeps the half
-    // of its values that its bit selects, summed with its partner's
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const bool up = lane & o;
-#pragma unroll
-      for (int i = 0; i < 2 * o; ++i) {
-        const float keep = up ? acc[i + 2 * o] : acc[i];
-        const float send = up ? acc[i] : acc[i + 2 * o];
-        acc[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
-      }
-    }
+    float2 mom;
+    far_moments(s_w, lane, v, mom);
+    const float acc[2] = {mom.x, mom.y};
     const int e = (m0 - 2 * lane) / kFarBlock * kFarP + lane;   // node lane % 16 of block lane / 16
     if (e < nb * kFarP) {
 #pragma unroll
@@ -626,8 +555,6 @@ bool make_map(CUtensorMap* m, void* base, bool fp16, long long rows, int n, int 
 }  // namespace
 
 namespace {
-
-int far_blocks(int n) { return (n + kFarBlock - 1) / kFarBlock; }
 
 template <bool FP16, int JOB>
 cudaError_t launch_tiles(const CUtensorMap& mh, const CUtensorMap& ml, const CUtensorMap& fh,

@@ -1,4 +1,4 @@
-// Windowed and exact Whittaker-Shannon resampling kernels (Eq. 17, Sec. III-B).
+// Windowed Whittaker-Shannon resampling kernels (Eq. 17, Sec. III-B).
 //
 // Windowed: y[n] = sum_i x[i] h(alpha n - i), h(u) = sinc(u) w(u), w a Kaiser
 // window of half width R, support |u| < R, x zero outside [0, N).  With
@@ -43,12 +43,6 @@ DC_DEV float tap_weight(const RsArgs& a, float e, float s_e, int k) {
   if (u == 0.f) return 1.f;
   const float sc = __fdividef((k & 1) ? -s_e : s_e, u);
   return sc * window_at(a.wpoly, k + a.half - 1, e);
-}
-
-// v exp(2 pi i g n) (the item's carrier rotation), or v when g = 0.
-DC_DEV float2 rotate(float2 v, float g_hi, float g_lo, int n) {
-  if (g_hi == 0.f && g_lo == 0.f) return v;
-  return cmul(v, cycles_rot(g_hi, g_lo, n));
 }
 
 // The item owning a tile: the last item with tile_begin <= tile (tile_begin
@@ -417,194 +411,6 @@ cudaError_t launch_freqconv(const RsArgs& a, cudaStream_t s) {
 cudaError_t launch_resample_direct(const RsArgs& a, cudaStream_t s) {
   if (a.n_tiles <= 0) return cudaSuccess;
   resample_direct_kernel<<<a.n_tiles, kRsThreads, 0, s>>>(a);
-  return cudaGetLastError();
-}
-
-// ------------------------------------------------- exact sinc, FP32 cores
-// Y[p][n] = sum_m X[p][m] S[n][m], S[n][m] = sinc(alpha n - m)
-//         = (-1)^(m + m_n) sin(pi e_n) / (pi ((m_n - m) + e_n)),  alpha n = m_n + e_n.
-// CTA tile: 64 outputs x 32 pulses, K chunks of 32 samples; S generated in
-// shared memory per chunk and reused by all 32 pulses.
-constexpr int kExBN = 64, kExBP = 32, kExBK = 32;
-
-__global__ void __launch_bounds__(256) exact_fp32_kernel(ExArgs a) {
-  const ExItem& I = a.items[blockIdx.z];
-  const int n0 = blockIdx.x * kExBN, p0 = blockIdx.y * kExBP;
-  __shared__ float Ss[kExBK][kExBN + 4];
-  __shared__ float2 Xs[kExBK][kExBP + 1];
-  __shared__ float sig[kExBN], en[kExBN];
-  __shared__ int mn[kExBN];
-  const int tid = threadIdx.x;
-  if (tid < kExBN) {
-    const int n = n0 + tid;
-    int fl;
-    float e;
-    rs_delay(I.dl_hi, I.dl_lo, (float)n, fl, e);
-    const int m = n + fl;
-    mn[tid] = m;
-    en[tid] = e;
-    const float s = sinpif(e) * kInvPi;
-    sig[tid] = (m & 1) ? -s : s;
-  }
-  const int tn = tid & 15, tp = tid >> 4;        // 4 outputs x 2 pulses per thread
-  float2 acc[4][2];
-#pragma unroll
-  for (int i = 0; i < 4; ++i) acc[i][0] = acc[i][1] = make_float2(0.f, 0.f);
-  __syncthreads();
-
-  for (int m0 = 0; m0 < a.n_in; m0 += kExBK) {
-    for (int idx = tid; idx < kExBK * kExBN; idx += 256) {
-      const int n = idx % kExBN, k = idx / kExBN;
-      const int m = m0 + k;
-      float v = 0.f;
-      if (m < a.n_in) {
-        if (en[n] == 0.f) {
-          v = (m == mn[n]) ? 1.f : 0.f;
-        } else {
-          const float den = (float)(mn[n] - m) + en[n];
-          v = __fdividef((m & 1) ? -sig[n] : sig[n], den);
-        }
-      }
-      Ss[k][n] = v;
-    }
-    for (int idx = tid; idx < kExBK * kExBP; idx += 256) {
-      const int k = idx % kExBK, p = idx / kExBK;
-      const int m = m0 + k, pp = p0 + p;
-      Xs[k][p] = (m < a.n_in && pp < a.n_pulses) ? __ldg(I.x + (size_t)pp * a.n_in + m)
-                                                  : make_float2(0.f, 0.f);
-    }
-    __syncthreads();
-#pragma unroll 8
-    for (int k = 0; k < kExBK; ++k) {
-      const float4 s4 = *reinterpret_cast<const float4*>(&Ss[k][tn * 4]);
-      const float2 x0 = Xs[k][tp * 2], x1 = Xs[k][tp * 2 + 1];
-      const float s[4] = {s4.x, s4.y, s4.z, s4.w};
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        acc[i][0].x = fmaf(x0.x, s[i], acc[i][0].x);
-        acc[i][0].y = fmaf(x0.y, s[i], acc[i][0].y);
-        acc[i][1].x = fmaf(x1.x, s[i], acc[i][1].x);
-        acc[i][1].y = fmaf(x1.y, s[i], acc[i][1].y);
-      }
-    }
-    __syncthreads();
-  }
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int n = n0 + tn * 4 + i;
-    if (n >= a.n_out) continue;
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      const int p = p0 + tp * 2 + j;
-      if (p < a.n_pulses) I.y[(size_t)p * a.n_out + n] = rotate(acc[i][j], I.rot_hi, I.rot_lo, n);
-    }
-  }
-}
-
-// The same sum for a few pulses (a matrix-vector product: one pulse per
-// call of the single-pulse entry points): one warp per output sample, lanes
-// striding the input, the weight computed once per (n, m) and applied to
-// every pulse, lanes combined by a fixed shuffle tree (deterministic).
-// One lane's share of the sum: terms m = lane, lane + 32, ... (FAST: m_n - m
-// converted by exact_i2f, valid for |m_n - m| < 2^22).  Four terms per round:
-// their weights, then their loads, issued together so that a warp has four
-// loads in flight instead of one (the kernel is bound by the load latency);
-// the terms are still added in the order m = lane, lane + 32, ...
-template <bool FAST> DC_DEV float gemv_weight(int mn, int m, float e, float sgl) {
-  const float den = (FAST ? exact_i2f(mn - m) : (float)(mn - m)) + e;
-  return __fdividef(sgl, den);
-}
-template <int P, bool FAST>
-DC_DEV void gemv_terms(const float2* __restrict__ x, int n_in, int np, int mn, float e, float sgl,
-                       int lane, float2 (&acc)[P]) {
-  int m = lane;
-  for (; m + 96 < n_in; m += 128) {
-    float w[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) w[u] = gemv_weight<FAST>(mn, m + 32 * u, e, sgl);
-#pragma unroll
-    for (int p = 0; p < P; ++p) {
-      if (p < np) {
-        float2 xv[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) xv[u] = __ldg(x + (size_t)p * n_in + m + 32 * u);
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          acc[p].x = fmaf(xv[u].x, w[u], acc[p].x);
-          acc[p].y = fmaf(xv[u].y, w[u], acc[p].y);
-        }
-      }
-    }
-  }
-  for (; m < n_in; m += 32) {
-    const float w = gemv_weight<FAST>(mn, m, e, sgl);
-#pragma unroll
-    for (int p = 0; p < P; ++p) {
-      if (p < np) {
-        const float2 xv = __ldg(x + (size_t)p * n_in + m);
-        acc[p].x = fmaf(xv.x, w, acc[p].x);
-        acc[p].y = fmaf(xv.y, w, acc[p].y);
-      }
-    }
-  }
-}
-
-template <int P>
-__global__ void __launch_bounds__(256) exact_gemv_kernel(ExArgs a) {
-  pdl_release();                        // the transform that follows may start its set-up
-  const ExItem& I = a.items[blockIdx.y];
-  const int n = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (n >= a.n_out) return;
-  const int np = a.n_pulses;
-  int fl;
-  float e;
-  rs_delay(I.dl_hi, I.dl_lo, (float)n, fl, e);
-  const int mn = n + fl;
-  if (e == 0.f) {                                  // alpha n on a sample: copy it
-    if (lane < np) {
-      const bool in = mn >= 0 && mn < a.n_in;
-      const float2 v = in ? __ldg(I.x + (size_t)lane * a.n_in + mn) : make_float2(0.f, 0.f);
-      I.y[(size_t)lane * a.n_out + n] = rotate(v, I.rot_hi, I.rot_lo, n);
-    }
-    return;
-  }
-  const float s = sinpif(e) * kInvPi;
-  const float sg = (mn & 1) ? -s : s;
-  const float sgl = (lane & 1) ? -sg : sg;         // (-1)^m: m steps by 32 from lane
-  float2 acc[P];
-#pragma unroll
-  for (int p = 0; p < P; ++p) acc[p] = make_float2(0.f, 0.f);
-  // m_n - m lies in (m_n - n_in, m_n]; below 2^22 in size (any Doppler
-  // range rate) it converts exactly without the quarter-rate instruction
-  if (mn < (1 << 22)) gemv_terms<P, true>(I.x, a.n_in, np, mn, e, sgl, lane, acc);
-  else gemv_terms<P, false>(I.x, a.n_in, np, mn, e, sgl, lane, acc);
-#pragma unroll
-  for (int p = 0; p < P; ++p) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      acc[p].x += __shfl_xor_sync(0xffffffffu, acc[p].x, o);
-      acc[p].y += __shfl_xor_sync(0xffffffffu, acc[p].y, o);
-    }
-  }
-  if (lane == 0) {
-#pragma unroll
-    for (int p = 0; p < P; ++p)
-      if (p < np) I.y[(size_t)p * a.n_out + n] = rotate(acc[p], I.rot_hi, I.rot_lo, n);
-  }
-}
-
-cudaError_t launch_exact_fp32(const ExArgs& a, int n_alpha, cudaStream_t s) {
-  if (n_alpha <= 0 || a.n_out <= 0 || a.n_pulses <= 0) return cudaSuccess;
-  if (a.n_pulses <= 8) {
-    dim3 grid((a.n_out + 7) / 8, n_alpha);
-    if (a.n_pulses == 1) exact_gemv_kernel<1><<<grid, 256, 0, s>>>(a);
-    else if (a.n_pulses <= 2) exact_gemv_kernel<2><<<grid, 256, 0, s>>>(a);
-    else if (a.n_pulses <= 4) exact_gemv_kernel<4><<<grid, 256, 0, s>>>(a);
-    else exact_gemv_kernel<8><<<grid, 256, 0, s>>>(a);
-    return cudaGetLastError();
-  }
-  dim3 grid((a.n_out + kExBN - 1) / kExBN, (a.n_pulses + kExBP - 1) / kExBP, n_alpha);
-  exact_fp32_kernel<<<grid, 256, 0, s>>>(a);
   return cudaGetLastError();
 }
 

@@ -44,7 +44,17 @@ struct ExItem {
 struct ExArgs {
   const ExItem* items; // one per alpha (grid.z)
   int n_in, n_out, n_pulses;
+  // Scratch of the near and far form (null: every sample term by term):
+  // block moments [groups][n_pulses][16 blocks(n_in)] and node values
+  // [groups][n_pulses][16 blocks(n_out)], groups = 1 when every alpha has
+  // the same pulses (`shared`), else one per alpha.
+  float2 *mom, *loc;
+  int shared;
 };
+// Float2 elements of that scratch for n samples a pulse, and whether a call
+// takes the form at all (delta_max: the largest |alpha - 1|).
+size_t exact_fp32_far_elems(long long pulses, int n);
+bool exact_fp32_far(int n_in, int n_out, int n_pulses, int n_alpha, double delta_max);
 
 // delta * fi = fl + e with fl integer and e in [0, 1), fi a float holding an
 // integer or half-integer output position (exact), delta a double-float.
@@ -63,6 +73,12 @@ DC_DEV void rs_delay(float dl_hi, float dl_lo, float fi, int& fl, float& e) {
   }
   fl = (int)f;
   e = r;
+}
+
+// v exp(2 pi i g n) (the item's carrier rotation), or v when g = 0.
+DC_DEV float2 rotate(float2 v, float g_hi, float g_lo, int n) {
+  if (g_hi == 0.f && g_lo == 0.f) return v;
+  return cmul(v, cycles_rot(g_hi, g_lo, n));
 }
 
 // One launch of the tensor-core bank resampler (rs_tc.cu): one pulse x[n_in]

@@ -71,6 +71,92 @@ def test_far_field_matches_oracle(dcg, mode_name, tol, n, n_out, P, shared):
     ctx.close()
 
 
+@pytest.mark.parametrize("n,n_out,P,shared", [
+    (1535, 1535, 9, False), (1536, 1536, 16, False), (1700, 2000, 17, True), (2000, 255, 40, False),
+    (3001, 3001, 48, False), (1793, 1537, 65, True), (17000, 300, 10, True),   # tiles of pulses
+    (4095, 4095, 1, False), (5793, 5793, 1, False), (4097, 5000, 2, False), (40001, 700, 3, True),
+    (4096, 4096, 8, False), (20000, 20000, 1, False),                          # one warp per output
+])
+def test_far_field_fp32_matches_oracle(dcg, n, n_out, P, shared):
+    # FP32 weights (2 ulp divide, sinpi) and sums of at most 4095 terms: 4e-6
+    ctx = dcg.Context(0)
+    v = [7500.0, v_of_delay(62.9, n_out), -v_of_delay(62.9, n_out)]
+    check(dcg, ctx, "DC_EXACT_FP32", n, n_out, P, v, shared, 4e-6)
+    check(dcg, ctx, "DC_EXACT_FP32", n, n_out, P, [v_of_delay(64.0, n_out), 0.0], shared, 4e-6)
+    ctx.close()
+
+
+@pytest.mark.parametrize("mode_name,n,P", [("DC_EXACT_FP32", 6200, 1), ("DC_EXACT_FP32", 2300, 20),
+                                           ("DC_EXACT_BF16X3", 2300, 4), ("DC_EXACT_FP16X3", 2300, 4)])
+@pytest.mark.parametrize("bad", [np.inf, -np.inf, np.nan, 3.3e38])
+def test_far_field_keeps_values_that_are_not_finite(dcg, mode_name, n, P, bad):
+    # one sample per pulse that is infinite, NaN or near the largest float: the
+    # same outputs are infinite, NaN and finite as in the dense sum (a context
+    # whose scratch budget leaves no room for the far field's)
+    import torch
+    rng = synth.rng_for(4, salt=n)
+    X = np.stack([synth.bandlimited_noise(n, rng) for _ in range(P)]).astype(np.complex64)
+    X[:, 300] = bad
+    xd = torch.from_numpy(X.reshape(-1)).cuda()
+    dense = {"DC_EXACT_FP32": 1}.get(mode_name, 2 * (2 * P * ((n + 7) // 8 * 8) * 2) + 512)
+    got = []
+    for budget in (0, dense):
+        ctx = dcg.Context(0, budget)
+        yd = torch.zeros(2 * P * n, dtype=torch.complex64, device="cuda")
+        dcg.resample_exact_batch(ctx, xd, n, P, [5000.0, 0.5], yd, n_out=n, mode=getattr(dcg, mode_name))
+        dcg.dc_check(ctx)
+        got.append(torch.view_as_real(yd).cpu().numpy())
+        ctx.close()
+    far, ref = got
+    np.testing.assert_array_equal(np.isnan(far), np.isnan(ref))
+    np.testing.assert_array_equal(np.isinf(far), np.isinf(ref))
+    np.testing.assert_array_equal(far[np.isinf(far)], ref[np.isinf(ref)])
+
+
+@pytest.mark.parametrize("n", [4096, 6000])
+def test_far_field_in_every_single_pulse_call(dcg, n):
+    # doppler_resample, correct_batch, a plan and correct_compress take their
+    # scratch from the context in different places: all against one oracle
+    import torch
+    rng = synth.rng_for(4, salt=n)
+    x = synth.bandlimited_noise(n, rng).astype(np.complex64)
+    h = synth.lfm(256, 20e6, 5e6).astype(np.complex64)
+    fs, fc, v, tec = 20e6, 1e9, -6100.0, 60.0
+    ctx = dcg.Context(0)
+    xd, hd = torch.from_numpy(x).cuda(), torch.from_numpy(h).cuda()
+    y, z, c = (torch.empty_like(xd) for _ in range(3))
+    E = dcg.DC_EXACT_FP32
+    items = np.zeros(2, dtype=dcg.ITEM_DTYPE)
+    items["in_off"], items["out_off"], items["n"], items["n_out"] = 0, [0, n], n, n
+    items["fs"], items["fc"], items["v_r"], items["tec_tecu"] = fs, fc, [v, 0.3 * v], tec
+    b = torch.empty(2 * n, dtype=torch.complex64, device="cuda")
+    pb = torch.empty_like(b)
+    dcg.doppler_resample(ctx, xd, y, fs, fc, v, mode=E)
+    dcg.correct_batch(ctx, xd, b, items, mode=E)
+    torch.cuda.synchronize()
+    plan = dcg.dc_plan_batch(ctx, xd, pb, items, mode=E)
+    for _ in range(3):
+        plan.execute()
+    dcg.correct_compress(ctx, xd, hd, c, fs, fc, v, tec, mode=E)
+    dcg.dc_check(ctx)
+    assert torch.equal(torch.view_as_real(b), torch.view_as_real(pb))
+    x64 = x.astype(np.complex128)
+    rel = lambda a, r: np.linalg.norm(a - r) / np.linalg.norm(r)
+    ref = oracle.resample(x64, fs, fc, v, "exact")
+    assert rel(y.cpu().numpy(), ref) <= 4e-6
+    assert rel(b[:n].cpu().numpy(), oracle.iono_correct(ref, fs, fc, tec)) <= 5e-6
+    ref2 = oracle.correct(x64, fs, fc, 0.3 * v, tec, mode="exact")
+    assert rel(b[n:].cpu().numpy(), ref2) <= 5e-6
+    L = 1 << (n - 1).bit_length()
+    H = np.fft.fft(h.astype(np.complex128), L)
+    want = np.fft.ifft(np.fft.fft(oracle.iono_correct(ref, fs, fc, tec, L=L) if n == L else
+                                  np.fft.ifft(np.fft.fft(ref, L) * np.exp(-1j * oracle.iono_phase(L, fs, fc, tec))), L)
+                       * H.conj())[:n]
+    assert rel(c.cpu().numpy(), want) <= 5e-6
+    plan.close()
+    ctx.close()
+
+
 def test_far_field_within_a_scratch_budget(dcg):
     # scratch capped at the dense sum's planes: the call is accepted and takes
     # the dense sum; capped below, it is refused
