@@ -206,24 +206,14 @@ double alpha_minus_one(double v_r) {
   return (2.0 * b) / (1.0 - b);
 }
 
-// Per-pulse ionospheric constants (Eq. 16): A = 4 pi kappa E / c.
+// Per-pulse ionospheric constants (Eq. 16): phi / 2 pi = C / f, C = 2 kappa E / c.
 PhaseParams phase_params(double fs, double fc, double tec_tecu, int log2L) {
   PhaseParams p{};
-  const double A = 4.0 * kPi * kKappa * tec_tecu * 1e16 / kC;
-  split(A, p.a_hi, p.a_lo);
+  split(2.0 * kKappa * tec_tecu * 1e16 / kC, p.c_hi, p.c_lo);
   split(fc, p.fc_hi, p.fc_lo);
   split(fs / (double)(1LL << log2L), p.d_hi, p.d_lo);
   p.log2L = log2L;
   p.enabled = tec_tecu != 0.0;
-  // Stepped phase runs (16 bins, s d = fs / 4096): the largest step over the
-  // band is |A| (fs / 4096) / f_min^2; 15 steps of relative error ~3.3e-7
-  // stay within 1e-7 rad while it is <= 0.02 rad.  RF sampling (a bin at
-  // f = 0) always evaluates every bin.
-  p.run = 1;
-  if (fc > 0.0) {
-    const double fmin = fc - 0.5 * fs;
-    if (fmin > 0.0 && std::fabs(A) * (fs / 4096.0) / (fmin * fmin) <= 0.02) p.run = 16;
-  }
   return p;
 }
 
@@ -630,7 +620,7 @@ dc_status run_iono_class(dc_ctx* c, std::vector<FftItem>& it, int log2L, float2*
     RowArgs a2{d2 + j0, cnt, log2L, log2L1, c->tw};
     {
       Phase ph(c, PH_ROW_MID, s, outs);
-      e = log2L >= 17 ? launch_row_mid_4096(a2, s) : launch_row(ROW_MID, a2, s);
+      e = launch_row(ROW_MID, a2, s);
       if (e != cudaSuccess) return cuda_fail(c, e, "row launch");
     }
     ColArgs a3{d3 + j0, cnt, log2L, log2L1, c->tw};
@@ -999,9 +989,9 @@ __global__ void stuck_wait_kernel(int* err, int polls) {
   atomicMax(err, 1);
 }
 
-// Factor tables P[t][.] in the spectrum layout (element k1*4096 + k2 holds
-// bin k1 + L1 k2, L1 = L/4096, for L > 4096; natural order for L <= 4096 --
-// the same formula with L1 = 1): exp(-i phi_k(TEC_t)) times `scale` (1/L
+// Factor tables P[t][.] in the spectrum layout (element k1*4096 +
+// spec_index(k2) holds bin k1 + L1 k2, L1 = L/4096, for L >= 4096; natural
+// order below): exp(-i phi_k(TEC_t)) times `scale` (1/L
 // for the spectrum-apply kernel, which folds in the inverse transform's
 // factor; else 1).  H (optional): a replica's spectrum in the same layout;
 // each factor is then multiplied by conj(H_k), the matched filter of pulse
@@ -1014,7 +1004,7 @@ __global__ void phase_table_kernel(const PhaseParams* ph, int n_tec, int log2L, 
   for (size_t g = blockIdx.x * (size_t)blockDim.x + threadIdx.x; g < total;
        g += (size_t)gridDim.x * blockDim.x) {
     const int t = (int)(g >> log2L), idx = (int)(g & (L - 1));
-    const int k = (idx >> 12) + ((idx & 4095) << log2L1);
+    const int k = log2L >= 12 ? (idx >> 12) + (spec_bin(idx & 4095) << log2L1) : idx;
     float2 w = ph[t].enabled ? iono_factor(ph[t], k) : make_float2(1.f, 0.f);
     if (H) {
       const float2 h = __ldg(H + idx);
@@ -1028,8 +1018,8 @@ __global__ void phase_table_kernel(const PhaseParams* ph, int n_tec, int log2L, 
 namespace {
 
 // Forward spectra of the items' sources (zero-padded past n_valid) into their
-// dst, length L = 2^log2L, in the spectrum layout (bin k1 + L1 k2 at
-// k1*4096 + k2 for L > 4096, natural order below): cluster-fused, one row
+// dst, length L = 2^log2L, in the spectrum layout (bin k1 + L1 k2 at k1*4096 +
+// spec_index(k2) for L >= 4096, natural order below): cluster-fused, one row
 // pass, or the first two passes of the four-step split (T: L samples per
 // item of scratch).
 dc_status run_spectra(dc_ctx* c, std::vector<FftItem>& sp, int log2L, float2* T, size_t& item_at,

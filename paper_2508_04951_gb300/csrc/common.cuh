@@ -67,32 +67,6 @@ DC_DEV df two_prod(float a, float b) {
   float p = __fmul_rn(a, b);
   return {p, fmaf(a, b, -p)};
 }
-DC_DEV df df_add(df a, df b) {
-  df s = two_sum(a.hi, b.hi);
-  float lo = __fadd_rn(s.lo, __fadd_rn(a.lo, b.lo));
-  return two_sum(s.hi, lo);
-}
-// (a.hi + a.lo) * k for a float k
-DC_DEV df df_mul_f(df a, float k) {
-  df p = two_prod(a.hi, k);
-  return two_sum(p.hi, fmaf(a.lo, k, p.lo));
-}
-// a / b, both double-float.  One reciprocal of b.hi serves both quotient
-// steps: q1 = a.hi / b.hi to a couple of ulps, the remainder
-// a - q1 b is formed exactly (two_prod, Sterbenz), and its quotient q2 only
-// needs float accuracy relative to itself (|q2| ~ 2^-23 |q1|).
-DC_DEV df df_div(df a, df b) {
-  const float rb = __frcp_rn(b.hi);
-  const float q1 = __fmul_rn(a.hi, rb);
-  df p = two_prod(q1, b.hi);
-  float r = __fsub_rn(a.hi, p.hi);          // exact: q1*b.hi is within a few ulps of a.hi
-  r = __fsub_rn(r, p.lo);
-  r = __fadd_rn(r, a.lo);
-  r = fmaf(-q1, b.lo, r);
-  const float q2 = __fmul_rn(r, rb);
-  return two_sum(q1, q2);
-}
-
 // exp(2 pi i g n) for a rotation rate g (cycles per sample) held as the
 // double-float g_hi + g_lo and an output index n < 2^24: g n is formed as a
 // double-float (two_prod, exact for the high part), its integer part removed

@@ -1,6 +1,7 @@
 // Stockham FFT passes with the fused ionospheric phase multiply.
 // Index conventions and the four-step split are described in fft.cuh.
 #include "fft.cuh"
+#include "fused.cuh"
 
 namespace dc {
 
@@ -113,7 +114,7 @@ __global__ void __launch_bounds__(kThreads) row_kernel(RowArgs a) {
       }
       if (OP == ROW_APPLY) {
         const int k = row + L1 * p;
-        // the table is in the spectrum's own layout: bin k at row * M + p
+        // the table is in the spectrum's own layout (natural below 4096)
         if (I.ptab) v = cmul(v, __ldg(I.ptab + (size_t)row * M + p));
         else if (I.ph.enabled) v = cmul(v, iono_factor(I.ph, k));
       }
@@ -133,7 +134,7 @@ __global__ void __launch_bounds__(kThreads) row_kernel(RowArgs a) {
         const FftItem& I = a.items[it];
         const int k = row + L1 * p;
         float2 w;
-        if (I.ptab) w = __ldg(I.ptab + (size_t)row * M + p);   // the spectrum's layout
+        if (I.ptab) w = __ldg(I.ptab + (size_t)row * M + (M == 4096 ? spec_index(p) : p));
         else if (I.ph.enabled) w = iono_factor(I.ph, k);
         else continue;
         sm[c * LP + rpad(p)] = cmul(sm[c * LP + rpad(p)], w);
@@ -342,7 +343,11 @@ static cudaError_t launch_row_op(const RowArgs& a, cudaStream_t s) {
     case 9: return launch_row_m<512, OP>(a, s);
     case 10: return launch_row_m<1024, OP>(a, s);
     case 11: return launch_row_m<2048, OP>(a, s);
-    case 12: return launch_row_m<4096, OP>(a, s);
+    case 12:
+      // one-pass rows of L = 4096 here; every other row of 4096 points in
+      // registers (fused.cu)
+      if constexpr (OP == ROW_FULL) return launch_row_m<4096, OP>(a, s);
+      else return launch_row_4096(OP, a, s);
     default: return cudaErrorInvalidValue;
   }
 }

@@ -6,8 +6,9 @@
 // L2 = 4096, n = n2 + L2 n1, k = k1 + L1 k2:
 //   F1  (column pass): DFT over n1 of x[n2 + L2 n1], times W_L^(n2 k1),
 //                      stored at T[n2 + L2 k1]
-//   F2  (row pass)   : DFT over n2 of row k1 of T  -> bin k1 + L1 k2 sits at
-//                      T[k1 L2 + k2] (transposed spectrum, never reordered)
+//   F2  (row pass)   : DFT over n2 of row k1 of T  -> bins k1 + L1 k2 of row k1
+//                      (transposed spectrum, never reordered; stored spectra and
+//                      factor tables keep bin k2 of a row at spec_index(k2))
 //   phase multiply on that layout, then the inverse in mirror order:
 //   A   (row pass)   : inverse DFT over k2, times W_L^(-n2 k1), back to T
 //   B   (column pass): inverse DFT over k1, times 1/L, out[n2 + L2 n1]
@@ -20,6 +21,14 @@
 
 namespace dc {
 
+// Order of the bins of a 4096-point row in stored spectra and factor tables: bin
+// k2 = s + 16 a + 256 r (nibbles r, a, s) at index 256 s + 16 r + a.  Thread
+// (s, a) of a row transform holds exactly those 16 bins (r = 0..15) after the
+// forward row and before the inverse one, so both read and write them straight
+// from registers.  Rows below 4096 points keep natural order.
+__host__ __device__ constexpr int spec_index(int k2) { return ((k2 & 15) << 8) | (k2 >> 4); }
+__host__ __device__ constexpr int spec_bin(int idx) { return ((idx & 255) << 4) | (idx >> 8); }
+
 // One transform of a launch.  All items of one launch share L.
 struct FftItem {
   const float2* src;     // input of this pass
@@ -27,8 +36,8 @@ struct FftItem {
   const float2* ptab;    // per-bin factors (length L): exp(-i phi_k), times a
                          // matched filter's conjugate replica spectrum when
                          // compressing, in the spectrum's layout (bin
-                         // k1 + L1 k2 at k1*4096 + k2 for L > 4096, natural
-                         // order below); null -> exp(-i phi_k) computed from
+                         // k1 + L1 k2 at k1*4096 + spec_index(k2) for L >=
+                         // 4096, natural order below); null -> exp(-i phi_k) computed from
                          // `ph`
   PhaseParams ph;
   int n_valid;           // samples of src that are data (zero beyond), first pass

@@ -17,224 +17,143 @@ constexpr int kRowPitch = kRowN + kRowN / 16;
 
 DC_DEV int pad16(int p) { return p + (p >> 4); }
 
-// Stage twiddles of a 4096-point row from the precomputed tables: stage 2
-// multiplies v[r] by W256^(r k), k = j mod 16; stage 3 by W4096^(r j).  Only
-// the table rows r = 1, 2, 4, 8 are read (coalesced across the warp); the
-// other powers are their products (apply_powers).  The one-buffer rows load
-// the bases ahead of the CTA barrier that precedes their use; the two-buffer
-// row of the single-CTA transform takes them loaded at kernel start.
-template <int DIR>
-DC_DEV void stage2_bases(float2 (&b)[4], const float2* __restrict__ tw, int k) {
-  const float2* t = tw + kTwS2 + k;             // row r at (r - 1) * 16
-  b[0] = conj_if<DIR>(__ldg(t));
-  b[1] = conj_if<DIR>(__ldg(t + 16));
-  b[2] = conj_if<DIR>(__ldg(t + 48));
-  b[3] = conj_if<DIR>(__ldg(t + 112));
-}
-template <int DIR>
-DC_DEV void stage3_bases(float2 (&b)[4], const float2* __restrict__ tw, int j) {
-  const float2* t = tw + kTwS3 + j;             // row r at (r - 1) * 256
-  b[0] = conj_if<DIR>(__ldg(t));
-  b[1] = conj_if<DIR>(__ldg(t + 256));
-  b[2] = conj_if<DIR>(__ldg(t + 768));
-  b[3] = conj_if<DIR>(__ldg(t + 1792));
+// Twiddles of a 4096-point row: W256^(r k), k = 0..15 (s2) and W4096^(r j), j =
+// 0..255 (s3), forward values.  Only the table rows r = 1, 2, 4, 8 are read;
+// the other powers are their products (apply_powers).
+struct GlobalTw {                 // the context's table (coalesced across the warp)
+  const float2* __restrict__ tw;
+  DC_DEV void s2(float2 (&b)[4], int k) const {
+    const float2* t = tw + kTwS2 + k;             // row r at (r - 1) * 16
+    b[0] = __ldg(t), b[1] = __ldg(t + 16), b[2] = __ldg(t + 48), b[3] = __ldg(t + 112);
+  }
+  DC_DEV void s3(float2 (&b)[4], int j) const {
+    const float2* t = tw + kTwS3 + j;             // row r at (r - 1) * 256
+    b[0] = __ldg(t), b[1] = __ldg(t + 256), b[2] = __ldg(t + 768), b[3] = __ldg(t + 1792);
+  }
+};
+struct SharedTw {                 // a persistent CTA's copies of those rows, [4][16] and [4][256]
+  const float2 *t2, *t3;
+  DC_DEV void s2(float2 (&b)[4], int k) const {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) b[q] = t2[q * 16 + k];
+  }
+  DC_DEV void s3(float2 (&b)[4], int j) const {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) b[q] = t3[q * 256 + j];
+  }
+};
+struct HeldTw {                   // loaded ahead by the caller, for this thread
+  const float2 (&f2)[4], (&f3)[4];
+  DC_DEV void s2(float2 (&b)[4], int) const {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) b[q] = f2[q];
+  }
+  DC_DEV void s3(float2 (&b)[4], int) const {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) b[q] = f3[q];
+  }
+};
+template <int DIR> DC_DEV void orient(float2 (&b)[4]) {
+#pragma unroll
+  for (int q = 0; q < 4; ++q) b[q] = conj_if<DIR>(b[q]);
 }
 
-// One 4096-point row, thread j of 256.  In: v[r] = x[j + 256 r].
-// Out: v[r] = X[j + 256 r].  Three radix-16 Stockham stages exchanging
-// through two padded shared-memory buffers (element p at p + p/16): stage 1
-// writes b1, stage 2 reads b1 and writes b2, stage 3 reads b2.  One CTA
-// barrier per exchange; the caller must make sure nobody still reads b1 when
-// this starts.  Every thread of the CTA calls this together.  f2, f3: the
-// forward transform's stage bases (stage2_bases / stage3_bases with DIR =
-// -1), loaded by the caller ahead of time; the inverse takes their
-// conjugates.
-template <int DIR>
-DC_DEV void row4096(float2 (&v)[16], float2* b1, float2* b2, int j, const float2 (&f2)[4],
-                    const float2 (&f3)[4]) {
+// 4096-point rows, thread j = 16 s + t of 256, with one CTA barrier each.  The
+// split 4096 = 16 x 16 x 16: n = 256 p + 16 u + w, k = s + 16 a + 256 r.
+//
+// Forward: v[p] = x[256 p + j] in, v[r] = X[s + 16 t + 256 r] out.
+//   length-16 DFT over p (thread q = 16 u + w), W4096^(q s); a CTA-wide exchange
+//   gives half-warp s the 256 values of its sub-problem; DFT over u in thread w =
+//   t, W256^(w a); a 16 x 16 transpose inside the half-warp; DFT over w in thread
+//   a = t.
+// Inverse: the mirror image, v[r] = Y[s + 16 t + 256 r] in, v[p] = y[256 p + j]
+// out: DFT over r, W256^(-w a), half-warp transpose, DFT over a, CTA-wide
+// exchange, W4096^(-q s), DFT over s.
+//
+// So a forward row, factors on the bins and an inverse row need two CTA barriers
+// between them, and the bins meet their factors in registers.  b is one padded
+// buffer (element n at n + n / 16): half-warp s keeps to its own 272 elements
+// except in the CTA-wide exchange, where the forward row writes element 256 p +
+// j (thread j of every p: what that thread may itself have read there before)
+// and the inverse row reads it.  Callers: before the forward row nobody else may
+// still read elements 256 p + j, before the inverse row nobody may still read
+// b; on return from the inverse row other threads may still read b.
+template <class TW>
+DC_DEV void row_forward(float2 (&v)[16], float2* b, int j, const TW& tw) {
+  const int s = j >> 4, t = j & 15;
   float2 w[4];
-  dft16<DIR>(v);                                           // Ns = 1
-#pragma unroll
-  for (int r = 0; r < 16; ++r) b1[pad16(16 * j + r)] = v[r];
-#pragma unroll
-  for (int b = 0; b < 4; ++b) w[b] = conj_if<DIR>(f2[b]);
-  __syncthreads();
-#pragma unroll
-  for (int r = 0; r < 16; ++r) v[r] = b1[pad16(j + 256 * r)];
-  apply_powers<16>(v, w);                                  // Ns = 16: W256^(r k)
-  dft16<DIR>(v);
-  const int base = (j >> 4) * 256 + (j & 15);
-#pragma unroll
-  for (int r = 0; r < 16; ++r) b2[pad16(base + 16 * r)] = v[r];
-#pragma unroll
-  for (int b = 0; b < 4; ++b) w[b] = conj_if<DIR>(f3[b]);
-  __syncthreads();
-#pragma unroll
-  for (int r = 0; r < 16; ++r) v[r] = b2[pad16(j + 256 * r)];
-  apply_powers<16>(v, w);                                  // Ns = 256: W4096^(r j)
-  dft16<DIR>(v);
-}
-
-// One 4096-point row, thread j of 256.  In: v[r] = x[j + 256 r].
-// Out: v[r] = X[j + 256 r].  Three radix-16 Stockham stages with the data in
-// registers, exchanging through one padded shared-memory buffer (element p
-// at p + p/16): a CTA barrier after each exchange's writes and one before
-// the second exchange's writes.  The caller must make sure nobody still
-// reads b when this starts; on
-// return other threads may still be reading b.  Every thread of the CTA
-// calls this together.
-template <int DIR>
-DC_DEV void row4096_1buf(float2 (&v)[16], float2* b, int j, const float2* __restrict__ tw) {
-  float2 w[4];
-  dft16<DIR>(v);
-#pragma unroll
-  for (int r = 0; r < 16; ++r) b[pad16(16 * j + r)] = v[r];
-  stage2_bases<DIR>(w, tw, j & 15);
-  __syncthreads();
-#pragma unroll
-  for (int r = 0; r < 16; ++r) v[r] = b[pad16(j + 256 * r)];
-  apply_powers<16>(v, w);
-  dft16<DIR>(v);
-  const int base = (j >> 4) * 256 + (j & 15);
-  stage3_bases<DIR>(w, tw, j);
-  __syncthreads();
-#pragma unroll
-  for (int r = 0; r < 16; ++r) b[pad16(base + 16 * r)] = v[r];
-  __syncthreads();
-#pragma unroll
-  for (int r = 0; r < 16; ++r) v[r] = b[pad16(j + 256 * r)];
-  apply_powers<16>(v, w);
-  dft16<DIR>(v);
-}
-
-// row4096_1buf with the stage bases read from shared-memory copies of the
-// table rows r = 1, 2, 4, 8 (s2: [4][16] of W256^(r k), s3: [4][256] of
-// W4096^(r j), forward values as in the table): a persistent kernel copies
-// them once, and the row's base loads then neither miss L1 nor wait on L2.
-template <int DIR>
-DC_DEV void row4096_1buf_sm(float2 (&v)[16], float2* b, int j, const float2* s2, const float2* s3) {
-  float2 w[4];
-  dft16<DIR>(v);
-#pragma unroll
-  for (int r = 0; r < 16; ++r) b[pad16(16 * j + r)] = v[r];
-#pragma unroll
-  for (int q = 0; q < 4; ++q) w[q] = conj_if<DIR>(s2[q * 16 + (j & 15)]);
-  __syncthreads();
-#pragma unroll
-  for (int r = 0; r < 16; ++r) v[r] = b[pad16(j + 256 * r)];
-  apply_powers<16>(v, w);                                  // Ns = 16: W256^(r k)
-  dft16<DIR>(v);
-  const int base = (j >> 4) * 256 + (j & 15);
-#pragma unroll
-  for (int q = 0; q < 4; ++q) w[q] = conj_if<DIR>(s3[q * 256 + j]);
-  __syncthreads();
-#pragma unroll
-  for (int r = 0; r < 16; ++r) b[pad16(base + 16 * r)] = v[r];
-  __syncthreads();
-#pragma unroll
-  for (int r = 0; r < 16; ++r) v[r] = b[pad16(j + 256 * r)];
-  apply_powers<16>(v, w);                                  // Ns = 256: W4096^(r j)
-  dft16<DIR>(v);
-}
-
-// row4096_1buf, and once every thread has read the buffer for the last time
-// (before the last stage's twiddles and DFT) the cluster barrier is arrived
-// at with release semantics: peers may overwrite the buffer after their wait,
-// while this CTA still finishes its last stage.
-template <int DIR>
-DC_DEV void row4096_1buf_arrive(float2 (&v)[16], float2* b, int j, const float2* __restrict__ tw) {
-  float2 w[4];
-  dft16<DIR>(v);
-#pragma unroll
-  for (int r = 0; r < 16; ++r) b[pad16(16 * j + r)] = v[r];
-  stage2_bases<DIR>(w, tw, j & 15);
-  __syncthreads();
-#pragma unroll
-  for (int r = 0; r < 16; ++r) v[r] = b[pad16(j + 256 * r)];
-  apply_powers<16>(v, w);
-  dft16<DIR>(v);
-  const int base = (j >> 4) * 256 + (j & 15);
-  stage3_bases<DIR>(w, tw, j);
-  __syncthreads();
-#pragma unroll
-  for (int r = 0; r < 16; ++r) b[pad16(base + 16 * r)] = v[r];
-  __syncthreads();
-#pragma unroll
-  for (int r = 0; r < 16; ++r) v[r] = b[pad16(j + 256 * r)];
-  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-  apply_powers<16>(v, w);
-  dft16<DIR>(v);
-}
-
-// One 4096-point row with a single CTA barrier, thread j of 256.  In:
-// v[p] = x[256 p + j].  Out: v[b] = X[hw_sigma(j) + 256 b].
-// The four-step split 4096 = 16 x 256 (n = 256 p + q, k = s + 16 t):
-//   X[s + 16 t] = sum_q W256^(q t) [W4096^(q s) sum_p x[256 p + q] W16^(p s)]
-// -- thread q takes the length-16 DFT over p and the twiddle W4096^(q s);
-// one CTA-wide exchange gives half-warp s the 256 values of sub-problem s;
-// its length-256 DFT (256 = 16 x 16: q = 16 u + w, t = a + 16 b) takes a
-// length-16 DFT over u in thread w, the twiddle W256^(w a), a 16 x 16
-// transpose inside the half-warp (shared memory, __syncwarp only) and a
-// length-16 DFT over w in thread a.  Half-warp s only ever touches its own
-// 272-element region of b after the barrier, so the transpose needs no CTA
-// barrier.  ARRIVE: arrive at the cluster barrier (release) once this
-// thread's last read of b is done.  The caller must make sure nobody still
-// reads b when this starts; on return other threads may still read b.
-DC_DEV int hw_sigma(int j) { return (j >> 4) + ((j & 15) << 4); }
-
-// Where a received row keeps column c (c < COLS) of the column owner:
-// rpos(c) = 256 (c >> 8) + sw16(hw_sigma(c & 255)), sw16(x) = x ^ ((x >> 4)
-// & 15).  The half-warp row leaves column hw_sigma(j) + 256 m in thread j,
-// which so stores at 256 m + sw16(j): a warp's 32 remote stores fill one
-// 256-byte block (the XOR only permutes inside each 16-element group), the
-// form the distributed-shared-memory path moves fastest (scattered
-// addresses cost far more), while the owner's lanes, reading columns
-// 16 h + a (+ 256 p) at 16 a + (h ^ a), meet 16 different bank pairs.
-DC_DEV int sw16(int x) { return x ^ ((x >> 4) & 15); }
-DC_DEV int rpos(int c) { return (c & ~255) + sw16(hw_sigma(c & 255)); }
-
-template <int DIR, bool ARRIVE>
-DC_DEV void row4096_hw(float2 (&v)[16], float2* b, int j, const float2* __restrict__ tw) {
-  float2 w[4];
-  stage3_bases<DIR>(w, tw, j);                             // issued ahead of the DFT
-  dft16<DIR>(v);                                           // over p
+  tw.s3(w, j);                                             // issued ahead of the DFT
+  dft16<-1>(v);                                            // over p
   apply_powers<16>(v, w);                                  // W4096^(q s), q = j
 #pragma unroll
   for (int r = 0; r < 16; ++r) b[pad16(256 * r + j)] = v[r];
-  const int s = j >> 4, t = j & 15;
-  stage2_bases<DIR>(w, tw, t);
+  tw.s2(w, t);
   __syncthreads();
+  float2* reg = b + 272 * s;                               // = pad16(256 s)
 #pragma unroll
-  for (int u = 0; u < 16; ++u) v[u] = b[pad16(256 * s + 16 * u + t)];   // q = 16 u + w, w = t
-  dft16<DIR>(v);                                           // over u
+  for (int u = 0; u < 16; ++u) v[u] = reg[17 * u + t];     // q = 16 u + t
+  dft16<-1>(v);                                            // over u
   apply_powers<16>(v, w);                                  // W256^(w a)
-  float2* reg = b + 272 * s;                               // = pad16(256 s): the half-warp's region
   __syncwarp();                                            // its reads of the region are done
 #pragma unroll
-  for (int a = 0; a < 16; ++a) reg[17 * a + t] = v[a];     // V[w][a]
+  for (int a = 0; a < 16; ++a) reg[17 * a + t] = v[a];     // V[w = t][a]
   __syncwarp();
 #pragma unroll
   for (int q = 0; q < 16; ++q) v[q] = reg[17 * t + q];     // thread a = t: V[w = q][a]
-  if constexpr (ARRIVE) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-  dft16<DIR>(v);                                           // over w
+  dft16<-1>(v);                                            // over w
 }
 
-// The per-bin factors of the full correction on 16 bins k0 + s i held by one
-// thread: the caller's table (I.ptab, in the four-step layout, entries
-// t0 .. t0 + 15: exp(-i phi_k) times anything else the call bundles into the
-// frequency domain, e.g. a matched filter's conjugate replica spectrum) when
-// there is one, else exp(-i phi_k) of Eq. 16 from the phase constants.
-DC_DEV void bin_factors(const FftItem& I, int k0, int s, int t0, float2 (&u)[16]) {
-  if (I.ptab) {
-    const float4* t = reinterpret_cast<const float4*>(I.ptab + t0);
+// ARRIVE: arrive at the cluster barrier (release) once this thread's last read
+// of b is done: peers may overwrite the buffer after their wait.
+template <bool ARRIVE, class TW>
+DC_DEV void row_inverse(float2 (&v)[16], float2* b, int j, const TW& tw) {
+  const int s = j >> 4, t = j & 15;
+  float2 w[4];
+  tw.s2(w, t);
+  dft16<+1>(v);                                            // over r
+  orient<+1>(w);
+  apply_powers<16>(v, w);                                  // W256^(-w a), a = t
+  float2* reg = b + 272 * s;
+  __syncwarp();                                            // a forward row's reads of the region
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const float4 w = __ldg(t + i);
-      u[2 * i] = cmul(u[2 * i], make_float2(w.x, w.y));
-      u[2 * i + 1] = cmul(u[2 * i + 1], make_float2(w.z, w.w));
-    }
-  } else {
-    iono_apply_run16(I.ph, k0, s, u);
+  for (int q = 0; q < 16; ++q) reg[17 * q + t] = v[q];     // V[a = t][w]
+  __syncwarp();
+#pragma unroll
+  for (int a = 0; a < 16; ++a) v[a] = reg[17 * t + a];     // thread w = t: V[a][w]
+  dft16<+1>(v);                                            // over a
+  __syncwarp();
+#pragma unroll
+  for (int u = 0; u < 16; ++u) reg[17 * u + t] = v[u];     // q = 16 u + t of sub-problem s
+  tw.s3(w, j);
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < 16; ++q) v[q] = b[pad16(256 * q + j)];
+  if constexpr (ARRIVE) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  orient<+1>(w);
+  apply_powers<16>(v, w);                                  // W4096^(-q s), q = j
+  dft16<+1>(v);                                            // over s
+}
+
+// Index of thread j's bin r in a stored row (spec_index(s + 16 t + 256 r)).
+DC_DEV int spec_pos(int j, int r) { return ((j >> 4) << 8) + (j & 15) + 16 * r; }
+
+// v[r] *= the factor of bin k1 + L1 (s + 16 t + 256 r), r = 0..15 (L1 =
+// 2^log2L1): the item's table (exp(-i phi_k) times anything else the call
+// bundles into the frequency domain, e.g. a matched filter's conjugate
+// replica spectrum) when there is one, else exp(-i phi_k) of Eq. 16.
+DC_DEV void bin_factors(const FftItem& I, int k1, int log2L1, int j, float2 (&v)[16]) {
+  if (I.ptab) {
+    const float2* t = I.ptab + (size_t)k1 * kRowN;
+#pragma unroll
+    for (int r = 0; r < 16; ++r) v[r] = cmul(v[r], __ldg(t + spec_pos(j, r)));
+  } else if (I.ph.enabled) {
+    // bins r >= 8 are the upper half of the transform: kt = k - L
+    const PhaseParams& P = I.ph;
+    const float kt0 = (float)(k1 + (((j >> 4) + ((j & 15) << 4)) << log2L1));
+    const float step = (float)(256 << log2L1);
+#pragma unroll
+    for (int r = 0; r < 16; ++r)
+      v[r] = cmul(v[r], iono_factor_kt(P, fmaf((float)(r < 8 ? r : r - 16), step, kt0)));
   }
 }
 
@@ -308,11 +227,10 @@ __global__ void __launch_bounds__(kRowThreads, 4) spec_kernel(FusedArgs a) {
     cluster_wait<L1>();
 #pragma unroll
     for (int r = 0; r < 16; ++r) v[r] = A[pad16(j + 256 * r)];
-    __syncthreads();                            // the row FFT overwrites A
   }
-  row4096_1buf<-1>(v, A, j, a.tw);
+  row_forward(v, A, j, GlobalTw{a.tw});
 #pragma unroll
-  for (int r = 0; r < 16; ++r) I.dst[(size_t)k1 * kRowN + j + 256 * r] = v[r];
+  for (int r = 0; r < 16; ++r) I.dst[(size_t)k1 * kRowN + spec_pos(j, r)] = v[r];
 }
 
 template <int LOG2L1>
@@ -343,17 +261,17 @@ cudaError_t launch_spec(const FusedArgs& a, cudaStream_t s) {
 }
 
 // Spectrum apply (FUSED_APPLY): G = 2^LOG2G rows of the transform per CTA
-// (256 threads per row), one cluster of CL = L1 / G CTAs per transform.  The
-// spectrum rows arrive by 32 KiB bulk copies, the phase rows by coalesced
-// loads; after the inverse row FFTs each thread writes its 16 outputs X[n2]
-// straight into the shared memory of the CTA that owns column n2 (plain
-// remote stores), so no CTA reads another's shared memory.  The rows are
-// received into the buffers the row FFTs used (one 34 KiB buffer per row,
-// 64 registers: 4 / G CTAs per SM): a first cluster barrier after the row
-// FFTs frees every buffer, a second one after the stores delivers them.
-// The owner then applies W_L^(-n2 q) from the table and runs its columns.
-// Two rows per CTA halve the cluster (8 CTAs at L = 65536): fewer peers per
-// barrier and exchange, which moves the same bytes faster.
+// (256 threads per row), one cluster of CL = L1 / G CTAs per transform.
+// Spectrum and factor rows come straight into registers (both stored in the
+// inverse row's order); after the inverse row FFTs each thread writes its 16
+// outputs X[n2] straight into the shared memory of the CTA that owns column n2
+// (plain remote stores, a warp's 32 into one 256-byte block), so no CTA reads
+// another's shared memory.  The rows are received into the buffers the row FFTs
+// used (one 34 KiB buffer per row, 64 registers: 4 / G CTAs per SM): a first
+// cluster barrier after the row FFTs frees every buffer, a second one after the
+// stores delivers them.  The owner then applies W_L^(-n2 q) from the table and
+// runs its columns.  Two rows per CTA halve the cluster (8 CTAs at L = 65536):
+// fewer peers per barrier and exchange, which moves the same bytes faster.
 template <int LOG2L1, int LOG2G>
 __global__ void __launch_bounds__(kRowThreads << LOG2G, 4 >> LOG2G) apply_kernel(FusedArgs a) {
   constexpr int L1 = 1 << LOG2L1;
@@ -361,15 +279,12 @@ __global__ void __launch_bounds__(kRowThreads << LOG2G, 4 >> LOG2G) apply_kernel
   constexpr int CL = L1 / G;                    // CTAs per transform
   constexpr int NT = kRowThreads * G;
   constexpr int COLS = kRowN / CL;              // columns owned by a CTA
-  constexpr int PCOLS = COLS;                   // received rows at rpos(c)
   constexpr int PER = COLS / kRowThreads;       // a row thread's output r goes to CTA r / PER
   constexpr int PERC = COLS / NT;               // columns per thread
   static_assert(G == 1 || CL > 1, "two rows per CTA need a cluster");
   static_assert(G == 1 || L1 * COLS <= G * kRowPitch, "received rows fit the row buffers");
   extern __shared__ __align__(128) float2 sm[];
-  float2* R = sm;                               // [L1][PCOLS] received rows (CL > 1), column c
-                                                // of row q at q * PCOLS + rpos(c)
-  __shared__ __align__(8) unsigned long long bar_in;
+  float2* R = sm;                               // [L1][COLS] received rows (CL > 1)
 
   const int rank = CL > 1 ? (int)cg::this_cluster().block_rank() : 0;
   const FftItem I = apply_item(a, blockIdx.x >> (LOG2L1 - LOG2G));
@@ -377,25 +292,14 @@ __global__ void __launch_bounds__(kRowThreads << LOG2G, 4 >> LOG2G) apply_kernel
   const int h = j / kRowThreads, jj = j % kRowThreads;   // row of the CTA, thread in the row
   const int k1 = rank * G + h;
   float2* A = sm + h * kRowPitch;               // this row's buffer
-  if (j == 0) mbar_init(&bar_in, 1);
-  __syncthreads();
-  if (j == 0) {
-    mbar_expect_tx(&bar_in, G * kRowN * sizeof(float2));
-#pragma unroll
-    for (int g = 0; g < G; ++g)
-      bulk_g2s(sm + g * kRowPitch, I.src + (size_t)(rank * G + g) * kRowN, kRowN * sizeof(float2), &bar_in);
-  }
   float2 v[16];
+  const float2* srow = I.src + (size_t)k1 * kRowN;
   const float2* prow = I.ptab + (size_t)k1 * kRowN;
 #pragma unroll
-  for (int r = 0; r < 16; ++r) v[r] = __ldg(prow + jj + 256 * r);
-  mbar_wait_bounded(&bar_in, 0, a.err);         // on a timeout: flag raised, keep going
+  for (int r = 0; r < 16; ++r) v[r] = __ldg(srow + spec_pos(jj, r));
 #pragma unroll
-  for (int r = 0; r < 16; ++r) v[r] = cmul(A[jj + 256 * r], v[r]);
-  __syncthreads();                              // the row FFT overwrites A
-  if constexpr (L1 == 1) row4096_1buf<+1>(v, A, jj, a.tw);
-  else row4096_hw<+1, true>(v, A, jj, a.tw);    // arrives at the cluster barrier; v[r] at
-                                                // n2 = hw_sigma(jj) + 256 r
+  for (int r = 0; r < 16; ++r) v[r] = cmul(v[r], __ldg(prow + spec_pos(jj, r)));
+  row_inverse<(L1 > 1)>(v, A, jj, GlobalTw{a.tw});   // arrives at the cluster barrier
 
   if constexpr (L1 == 1) {
 #pragma unroll
@@ -407,13 +311,13 @@ __global__ void __launch_bounds__(kRowThreads << LOG2G, 4 >> LOG2G) apply_kernel
     // every peer's row FFTs are done with their buffers (the release arrive
     // is inside the row FFT)
     cluster_wait<L1>();
-    const uint32_t r_loc = smem_addr(R + k1 * PCOLS + sw16(jj));   // rpos(hw_sigma(jj))
+    const uint32_t r_loc = smem_addr(R + k1 * COLS + jj);
     // the farthest element this thread writes in its owners' buffers
-    if (DC_IN_BOUNDS(k1 * PCOLS + sw16(jj) + 256 * (PER - 1) < L1 * PCOLS && 16 / PER <= CL, a.err)) {
+    if (DC_IN_BOUNDS(k1 * COLS + jj + 256 * (PER - 1) < L1 * COLS && 16 / PER <= CL, a.err)) {
 #pragma unroll
       for (int r = 0; r < 16; ++r) {
-        const int owner = r / PER;              // n2 = hw_sigma(jj) + 256 r -> owner n2 / COLS
-        const uint32_t off = (uint32_t)(256 * (r % PER) * sizeof(float2));   // rpos(c + 256 m)
+        const int owner = r / PER;              // n2 = jj + 256 r -> owner n2 / COLS
+        const uint32_t off = (uint32_t)(256 * (r % PER) * sizeof(float2));
         st_cluster_c64(dsmem_map(r_loc + off, owner), v[r]);
       }
     }
@@ -429,7 +333,7 @@ __global__ void __launch_bounds__(kRowThreads << LOG2G, 4 >> LOG2G) apply_kernel
       if (p == 0) cluster_wait<L1>();           // every peer's stores into R are visible
       float2 col[L1];
 #pragma unroll
-      for (int q = 0; q < L1; ++q) col[q] = R[q * PCOLS + rpos(c)];
+      for (int q = 0; q < L1; ++q) col[q] = R[q * COLS + c];
       apply_powers<L1>(col, w);
       dft<L1, +1>(col);
 #pragma unroll
@@ -534,7 +438,6 @@ __global__ void __launch_bounds__(kRowThreads, 4) apply_l2_kernel(FusedArgs a) {
   constexpr int COLS = kRowN / L1;              // columns of a column task
   constexpr int PER = COLS / kRowThreads;       // columns per thread
   extern __shared__ __align__(128) float2 sm[]; // [kRowPitch] the row buffer
-  __shared__ __align__(8) unsigned long long bar_in;
   __shared__ ApplyTask s_ti[2];                 // the task in hand and the next one
   __shared__ float2 s_tw2[64], s_tw3[1024];     // the row's stage-base table rows r = 1, 2, 4, 8
   const int j = threadIdx.x;
@@ -575,11 +478,7 @@ __global__ void __launch_bounds__(kRowThreads, 4) apply_l2_kernel(FusedArgs a) {
     return d;
   };
   int t_next = 0;                               // thread 0: the task taken ahead
-  if (j == 0) {
-    mbar_init(&bar_in, 1);
-    s_ti[0] = decode(atomicAdd(head, 1));
-  }
-  uint32_t phase = 0;
+  if (j == 0) s_ti[0] = decode(atomicAdd(head, 1));
   for (int it = 0;; ++it) {
     __syncthreads();                            // s_ti; the last task's reads of sm are done
     const ApplyTask T = s_ti[it & 1];
@@ -595,24 +494,17 @@ __global__ void __launch_bounds__(kRowThreads, 4) apply_l2_kernel(FusedArgs a) {
       I.dst = T.dst;
       I.n_out = T.n_out;
       if (!is_col) {
-        if (j == 0) {                           // the spectrum row first: its copy overlaps the rest
-          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");    // after the last generic reads
-          mbar_expect_tx(&bar_in, kRowN * sizeof(float2));
-          bulk_g2s(sm, I.src + (size_t)rq * kRowN, kRowN * sizeof(float2), &bar_in);
-        }
         float2 v[16];
+        const float2* srow = I.src + (size_t)rq * kRowN;
         const float2* prow = I.ptab + (size_t)rq * kRowN;
 #pragma unroll
-        for (int r = 0; r < 16; ++r) v[r] = __ldg(prow + j + 256 * r);
-        mbar_wait_bounded(&bar_in, phase, a.err);
-        phase ^= 1;
+        for (int r = 0; r < 16; ++r) v[r] = __ldg(srow + spec_pos(j, r));
 #pragma unroll
-        for (int r = 0; r < 16; ++r) v[r] = cmul(sm[j + 256 * r], v[r]);
-        // the slot is free; the CTA barrier orders thread 0's wait before
-        // every thread's stores (the others wait there, polling nothing)
+        for (int r = 0; r < 16; ++r) v[r] = cmul(v[r], __ldg(prow + spec_pos(j, r)));
+        // the slot is free: the row's CTA barrier orders thread 0's wait
+        // before every thread's stores (the others poll nothing)
         if (j == 0 && T.prev >= 0) wait_count(col_done + T.prev, L1, a.err);
-        __syncthreads();                        // also: the row FFT overwrites sm
-        row4096_1buf_sm<+1>(v, sm, j, s_tw2, s_tw3);   // v[r] = Y[j + 256 r]
+        row_inverse<false>(v, sm, j, SharedTw{s_tw2, s_tw3});   // v[r] = Y[j + 256 r]
         float2* yrow = slot + (size_t)rq * kRowN;
 #pragma unroll
         for (int r = 0; r < 16; ++r) __stcg(yrow + j + 256 * r, v[r]);
@@ -671,37 +563,34 @@ cudaError_t launch_apply_l2(const FusedArgs& a, cudaStream_t s) {
 // cluster of L1 CTAs per transform, one padded buffer per CTA.  The forward
 // columns run straight from global memory (zero past n_valid), take
 // W_L^(n2 k1) and go to the row owners by plain remote stores; the forward
-// row, exp(-i phi_k) / L at bin k1 + L1 k2 (regrouped so that each thread
-// owns 16 consecutive k2) and the inverse row follow in the same buffer; the
+// row, exp(-i phi_k) / L on the bins in registers and the inverse row (two CTA
+// barriers in all) follow in the same buffer; the
 // inverse row's outputs go to the column owners the same way, which apply
 // W_L^(-n2 q) and run the inverse columns (out truncated to n_out).  Cluster
 // barriers order it all: every CTA running before the first remote store,
 // each exchange delivered before it is read, every buffer free before the
 // second exchange overwrites it.  At L = 4096 one CTA holds the whole
-// transform and takes two buffers.
+// transform.
 template <int LOG2L1>
 __global__ void __launch_bounds__(kRowThreads, LOG2L1 == 0 ? 2 : 4) full_kernel(FusedArgs a) {
   constexpr int L1 = 1 << LOG2L1;
   constexpr int COLS = kRowN / L1;              // columns owned by a CTA
-  constexpr int PCOLS = COLS;                   // received rows at rpos(c) (as in apply_kernel)
   constexpr int PER = COLS / kRowThreads;       // columns per thread
   constexpr int LOG2L = 12 + LOG2L1;
   extern __shared__ __align__(128) float2 sm[];
   float2* A = sm;                               // [kRowPitch] received row, row FFTs,
-  float2* R = sm;                               // then [L1][PCOLS] received inverse rows
+  float2* R = sm;                               // then [L1][COLS] received inverse rows
   const int k1 = L1 > 1 ? (int)cg::this_cluster().block_rank() : 0;
   const FftItem I = a.items[blockIdx.x >> LOG2L1];
   const int j = threadIdx.x;
   float2 v[16];
   if constexpr (L1 == 1) {
-    // L = 4096: one CTA, no exchange; two buffers (a second [kRowPitch]
-    // after A) save a CTA barrier per row, which sets this latency path
-    float2* B = sm + kRowPitch;
-    // every stage base of both rows loaded up front, beside the input: one
-    // CTA per transform leaves nothing to hide a load issued per stage
+    // L = 4096: one CTA, no exchange.  Every stage base of both rows loaded
+    // up front, beside the input: one CTA per transform leaves nothing to hide
+    // a load issued per stage
     float2 f2[4], f3[4];
-    stage2_bases<-1>(f2, a.tw, j & 15);
-    stage3_bases<-1>(f3, a.tw, j);
+    GlobalTw{a.tw}.s2(f2, j & 15);
+    GlobalTw{a.tw}.s3(f3, j);
     pdl_wait();                                 // the input's producer has finished
     // plain loads: a non-coherent load may be scheduled ahead of the wait
 #pragma unroll
@@ -709,29 +598,12 @@ __global__ void __launch_bounds__(kRowThreads, LOG2L1 == 0 ? 2 : 4) full_kernel(
       const int n = j + 256 * r;
       v[r] = n < I.n_valid ? I.src[n] : make_float2(0.f, 0.f);
     }
-    row4096<-1>(v, A, B, j, f2, f3);            // last reads: B after its second barrier
-    const bool mult = I.ph.enabled || I.ptab;
-    if (mult) {
-      // regroup through A (last read before the forward's second barrier)
-#pragma unroll
-      for (int r = 0; r < 16; ++r) A[pad16(j + 256 * r)] = v[r];
-      __syncthreads();
-      float2 u[16];
-#pragma unroll
-      for (int i = 0; i < 16; ++i) u[i] = A[pad16(16 * j + i)];
-      bin_factors(I, 16 * j, 1, 16 * j, u);
-#pragma unroll
-      for (int i = 0; i < 16; ++i) A[pad16(16 * j + i)] = u[i];
-      __syncthreads();
-#pragma unroll
-      for (int r = 0; r < 16; ++r) v[r] = A[pad16(j + 256 * r)];
-    }
+    row_forward(v, A, j, HeldTw{f2, f3});
+    bin_factors(I, 0, 0, j, v);
     const float invL = 1.0f / (float)(1 << LOG2L);
 #pragma unroll
     for (int r = 0; r < 16; ++r) v[r] = cscale(v[r], invL);
-    // the inverse row writes first the buffer no thread can still be reading
-    if (mult) row4096<+1>(v, B, A, j, f2, f3);
-    else row4096<+1>(v, A, B, j, f2, f3);
+    row_inverse<false>(v, A, j, HeldTw{f2, f3});
 #pragma unroll
     for (int r = 0; r < 16; ++r) {
       const int n = j + 256 * r;
@@ -764,39 +636,18 @@ __global__ void __launch_bounds__(kRowThreads, LOG2L1 == 0 ? 2 : 4) full_kernel(
     cluster_wait<L1>();
 #pragma unroll
     for (int r = 0; r < 16; ++r) v[r] = A[pad16(j + 256 * r)];
-    __syncthreads();                            // the row FFT overwrites A
-    row4096_hw<-1, false>(v, A, j, a.tw);      // v[r] = X[hw_sigma(j) + 256 r]
-    {
-      // back to natural order through A (the inverse row takes v[r] =
-      // Y[j + 256 r]), with the factors on runs of 16 bins on the way
-      const int sj = hw_sigma(j);
-      __syncthreads();                          // every half-warp is done with its region
-#pragma unroll
-      for (int r = 0; r < 16; ++r) A[pad16(sj + 256 * r)] = v[r];
-      __syncthreads();
-      if (I.ph.enabled || I.ptab) {
-        float2 u[16];
-#pragma unroll
-        for (int i = 0; i < 16; ++i) u[i] = A[pad16(16 * j + i)];
-        bin_factors(I, k1 + L1 * 16 * j, L1, k1 * kRowN + 16 * j, u);
-#pragma unroll
-        for (int i = 0; i < 16; ++i) A[pad16(16 * j + i)] = u[i];
-        __syncthreads();
-      }
-#pragma unroll
-      for (int r = 0; r < 16; ++r) v[r] = A[pad16(j + 256 * r)];
-    }
+    row_forward(v, A, j, GlobalTw{a.tw});
+    bin_factors(I, k1, LOG2L1, j, v);
     const float invL = 1.0f / (float)(1 << LOG2L);
 #pragma unroll
     for (int r = 0; r < 16; ++r) v[r] = cscale(v[r], invL);
-    __syncthreads();                            // the inverse row writes A first
-    row4096_hw<+1, true>(v, A, j, a.tw);        // arrives at the cluster barrier
+    row_inverse<true>(v, A, j, GlobalTw{a.tw});   // arrives at the cluster barrier
     cluster_wait<L1>();                         // every peer's buffer is free
-    const uint32_t r_loc = smem_addr(R + k1 * PCOLS + sw16(j));    // rpos(hw_sigma(j))
+    const uint32_t r_loc = smem_addr(R + k1 * COLS + j);
 #pragma unroll
     for (int r = 0; r < 16; ++r) {
-      const int owner = r / PER;                // n2 = hw_sigma(j) + 256 r -> owner n2 / COLS
-      const uint32_t off = (uint32_t)(256 * (r % PER) * sizeof(float2));   // rpos(c + 256 m)
+      const int owner = r / PER;                // n2 = j + 256 r -> owner n2 / COLS
+      const uint32_t off = (uint32_t)(256 * (r % PER) * sizeof(float2));
       st_cluster_c64(dsmem_map(r_loc + off, owner), v[r]);
     }
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");   // rows delivered
@@ -810,7 +661,7 @@ __global__ void __launch_bounds__(kRowThreads, LOG2L1 == 0 ? 2 : 4) full_kernel(
       if (p == 0) cluster_wait<L1>();           // every peer's stores into R are visible
       float2 col[L1];
 #pragma unroll
-      for (int q = 0; q < L1; ++q) col[q] = R[q * PCOLS + rpos(c)];
+      for (int q = 0; q < L1; ++q) col[q] = R[q * COLS + c];
       apply_powers<L1>(col, w);
       dft<L1, +1>(col);
 #pragma unroll
@@ -826,7 +677,7 @@ template <int LOG2L1>
 cudaError_t launch_full(const FusedArgs& a, cudaStream_t s) {
   constexpr int L1 = 1 << LOG2L1;
   if (L1 > 1 && !a.t4) return cudaErrorInvalidValue;
-  const size_t smem = sizeof(float2) * kRowPitch * (L1 == 1 ? 2 : 1);
+  const size_t smem = sizeof(float2) * kRowPitch;
   auto k = full_kernel<LOG2L1>;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
@@ -856,67 +707,76 @@ cudaError_t launch_full(const FusedArgs& a, cudaStream_t s) {
 }
 
 
-// Middle pass of the three-pass four-step path for 65536 < L <= 2^20
-// (L1 = L / 4096 in 32..256 rows): one 4096-point row per CTA -- forward
-// row FFT, exp(-i phi_k) at bin k1 + L1 k2, inverse row FFT, four-step
-// twiddle W_L^(-n2 k1) -- in place on the scratch T between the column
-// passes.
-__global__ void __launch_bounds__(kRowThreads, 4) row_mid_kernel(RowArgs a) {
+// Row passes on 4096-point rows, one per CTA (launch_row_4096): the row comes
+// in and goes out coalesced (natural order on the four-step scratch, spec_index
+// order on stored spectra), everything between stays in registers and the one
+// padded buffer.  34 KiB and 64 registers: 4 CTAs per SM.
+template <int OP>
+__global__ void __launch_bounds__(kRowThreads, 4) row_4096_kernel(RowArgs a) {
   extern __shared__ __align__(128) float2 sm[];
   const int L1 = 1 << a.log2L1;
   const int g = blockIdx.x;
-  const int item = g >> a.log2L1, k1 = g & (L1 - 1);
-  const FftItem I = a.items[item];
+  const FftItem I = a.items[g >> a.log2L1];
+  const int k1 = g & (L1 - 1);
   const int j = threadIdx.x;
-  float2* bufA = sm;
+  const GlobalTw tw{a.tw};
   const float2* src = I.src + (size_t)k1 * kRowN;
+  float2* dst = I.dst + (size_t)k1 * kRowN;
   float2 v[16];
+  if constexpr (OP == ROW_APPLY) {
 #pragma unroll
-  for (int r = 0; r < 16; ++r) v[r] = src[j + 256 * r];
-  row4096_hw<-1, false>(v, bufA, j, a.tw);    // v[r] = X[hw_sigma(j) + 256 r]
-  {
-    // back to natural order through A, with the factor of bin k = k1 + L1 k2
-    // on the way (each thread on 16 consecutive k2)
-    const int sj = hw_sigma(j);
-    __syncthreads();                           // every half-warp is done with its region
+    for (int r = 0; r < 16; ++r) v[r] = __ldg(src + spec_pos(j, r));
+  } else {
+    // the zero-padded input itself when a row is the whole transform (L = 4096)
+    const int valid = OP == ROW_SPEC && L1 == 1 ? I.n_valid : kRowN;
 #pragma unroll
-    for (int r = 0; r < 16; ++r) bufA[pad16(sj + 256 * r)] = v[r];
-    __syncthreads();
-    if (I.ph.enabled || I.ptab) {
-      float2 u[16];
-#pragma unroll
-      for (int i = 0; i < 16; ++i) u[i] = bufA[pad16(16 * j + i)];
-      bin_factors(I, k1 + L1 * 16 * j, L1, k1 * kRowN + 16 * j, u);
-#pragma unroll
-      for (int i = 0; i < 16; ++i) bufA[pad16(16 * j + i)] = u[i];
-      __syncthreads();
-    }
-#pragma unroll
-    for (int r = 0; r < 16; ++r) v[r] = bufA[pad16(j + 256 * r)];
+    for (int r = 0; r < 16; ++r) v[r] = j + 256 * r < valid ? src[j + 256 * r] : make_float2(0.f, 0.f);
+    row_forward(v, sm, j, tw);
   }
-  __syncthreads();                             // the inverse row writes A first
-  row4096_1buf<+1>(v, bufA, j, a.tw);
+  if constexpr (OP == ROW_SPEC) {
+#pragma unroll
+    for (int r = 0; r < 16; ++r) dst[spec_pos(j, r)] = v[r];
+    return;
+  }
+  bin_factors(I, k1, a.log2L1, j, v);
+  row_inverse<false>(v, sm, j, tw);
+  if (OP == ROW_APPLY && L1 == 1) {
+    const float invL = 1.0f / (float)kRowN;
+#pragma unroll
+    for (int r = 0; r < 16; ++r)
+      if (j + 256 * r < I.n_out) __stcs(dst + j + 256 * r, cscale(v[r], invL));
+    return;
+  }
   if (k1) {
     const float2 a_j = tw_big<+1>(a.tw, (uint32_t)(j * k1), a.log2L);
     const int m16 = 16 * L1 - 1, step = 256 >> a.log2L1;
 #pragma unroll
     for (int r = 0; r < 16; ++r) v[r] = cmul(v[r], cmul(a_j, tw_m<+1>(a.tw, ((r * k1) & m16) * step)));
   }
-  float2* dst = I.dst + (size_t)k1 * kRowN;
 #pragma unroll
   for (int r = 0; r < 16; ++r) dst[j + 256 * r] = v[r];
 }
 
+template <int OP> cudaError_t launch_row_4096_op(const RowArgs& a, cudaStream_t s) {
+  const size_t smem = sizeof(float2) * kRowPitch;
+  auto k = row_4096_kernel<OP>;
+  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  k<<<(unsigned)(a.n_items << a.log2L1), kRowThreads, smem, s>>>(a);
+  return cudaGetLastError();
+}
+
 }  // namespace
 
-cudaError_t launch_row_mid_4096(const RowArgs& a, cudaStream_t s) {
+cudaError_t launch_row_4096(int op, const RowArgs& a, cudaStream_t s) {
   if (a.n_items <= 0) return cudaSuccess;
-  if (a.log2L - a.log2L1 != 12 || a.log2L1 < 5 || a.log2L1 > 8) return cudaErrorInvalidValue;
-  const size_t smem = sizeof(float2) * kRowPitch;
-  cudaError_t e = cudaFuncSetAttribute(row_mid_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  row_mid_kernel<<<(unsigned)(a.n_items << a.log2L1), kRowThreads, smem, s>>>(a);
-  return cudaGetLastError();
+  if (a.log2L - a.log2L1 != 12 || a.log2L1 < 0 || a.log2L1 > 8) return cudaErrorInvalidValue;
+  switch (op) {
+    case ROW_MID: return launch_row_4096_op<ROW_MID>(a, s);
+    case ROW_SPEC: return launch_row_4096_op<ROW_SPEC>(a, s);
+    case ROW_APPLY: return launch_row_4096_op<ROW_APPLY>(a, s);
+    default: return cudaErrorInvalidValue;
+  }
 }
 
 cudaError_t launch_fused(int op, const FusedArgs& a, cudaStream_t s) {

@@ -8,7 +8,8 @@
 // four-step intermediate never leaves the SMs, so a transform reads its input
 // once and writes its output once.
 //
-//   FUSED_APPLY : rows of a stored spectrum (bin k1 + L1 k2 at k1*4096 + k2)
+//   FUSED_APPLY : rows of a stored spectrum (bin k1 + L1 k2 at k1*4096 +
+//                 spec_index(k2))
 //                 times a phase table in the same layout (already scaled by
 //                 1/L) -> inverse rows -> written into the column owners'
 //                 shared memory (plain remote stores, delivered by a
@@ -79,9 +80,10 @@ constexpr int kApplyL2Slots = 4;
 // Launch; returns cudaErrorInvalidValue for L outside [4096, 65536].
 cudaError_t launch_fused(int op, const FusedArgs& a, cudaStream_t s);
 
-// Middle (row) pass of the three-pass path for 2^17 <= L <= 2^20: forward
-// row, phase, inverse row, four-step twiddle, in place (RowArgs as for
-// ROW_MID, rows of 4096).
-cudaError_t launch_row_mid_4096(const RowArgs& a, cudaStream_t s);
+// Row passes on 4096-point rows, one per CTA (RowArgs): ROW_MID (forward row,
+// factors, inverse row, four-step twiddle, in place), ROW_SPEC (forward row to
+// a stored spectrum) and ROW_APPLY (stored spectrum times factors, inverse row,
+// four-step twiddle; for L = 4096 itself 1/L and truncation).
+cudaError_t launch_row_4096(int op, const RowArgs& a, cudaStream_t s);
 
 }  // namespace dc

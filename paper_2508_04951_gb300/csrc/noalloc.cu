@@ -110,12 +110,11 @@ extern "C" dc_status iono_correct_noalloc(const dc_c64* x, long long n, dc_c64* 
   it.src = reinterpret_cast<const float2*>(x);
   it.dst = reinterpret_cast<float2*>(y);
   it.ptab = nullptr;
-  split(4.0 * kPi * kappa * tec_tecu * 1e16 / kC, it.ph.a_hi, it.ph.a_lo);
+  split(2.0 * kappa * tec_tecu * 1e16 / kC, it.ph.c_hi, it.ph.c_lo);
   split(fc, it.ph.fc_hi, it.ph.fc_lo);
   split(fs / (double)(1LL << log2L), it.ph.d_hi, it.ph.d_lo);
   it.ph.log2L = log2L;
   it.ph.enabled = tec_tecu != 0.0;
-  it.ph.run = 1;                               // every bin evaluated in full
   it.n_valid = (int)n;
   it.n_out = (int)n;
 
