@@ -556,6 +556,24 @@ BatchLayout batch_layout(const dc_ctx* c, const dc_item* items, int n_items) {
 }
 
 // ------------------------------------------------------ correction pipeline
+// Transforms of L <= 4096 in one launch, `it` ordered by class: class m's are
+// items [first[m], first[m + 1]).
+dc_status run_row_classes(dc_ctx* c, const std::vector<FftItem>& it, const int (&first)[14], size_t& item_at,
+                          cudaStream_t s) {
+  RowClasses a{};
+  dc_status st = upload(c, it, item_at, s, &a.items);
+  if (st) return st;
+  item_at += (it.size() * sizeof(FftItem) + 255) & ~(size_t)255;
+  std::copy(first, first + 14, a.first);
+  a.tw = c->tw;
+  long long outs = 0;
+  for (auto& f : it) outs += f.n_out;
+  Phase ph(c, PH_ROW_FULL, s, outs);
+  cudaError_t e = launch_row_classes(a, s);
+  if (e != cudaSuccess) return cuda_fail(c, e, "row launch");
+  return DC_OK;
+}
+
 // One L class of pulses already resampled into y; writes corrected outputs.
 // Four-step classes use T (L samples per item) from the scratch.
 dc_status run_iono_class(dc_ctx* c, std::vector<FftItem>& it, int log2L, float2* T,
@@ -576,7 +594,12 @@ dc_status run_iono_class(dc_ctx* c, std::vector<FftItem>& it, int log2L, float2*
     if (e != cudaSuccess) return cuda_fail(c, e, "fused launch");
     return DC_OK;
   }
-  if (log2L <= 12) {
+  if (log2L < 12) {
+    int first[14];
+    for (int m = 0; m < 14; ++m) first[m] = m > log2L ? (int)it.size() : 0;
+    return run_row_classes(c, it, first, item_at, s);
+  }
+  if (log2L == 12) {
     dc_status st = upload(c, it, item_at, s, &dev);
     if (st) return st;
     item_at += (it.size() * sizeof(FftItem) + 255) & ~(size_t)255;
@@ -952,21 +975,36 @@ dc_status correct_batch(dc_ctx* c, const dc_c64* in, dc_c64* out, const dc_item*
       if (e != cudaSuccess) return cuda_fail(c, e, "exact launch");
     }
   }
-  // 2. ionospheric correction per L class
-  for (int m = 0; m <= 20; ++m) {
-    if (by_L[m].empty()) continue;
-    std::vector<FftItem> fi(by_L[m].size());
-    for (size_t j = 0; j < by_L[m].size(); ++j) {
-      const int i = by_L[m][j];
+  // 2. ionospheric correction per L class; the classes below 4096, with that of
+  // 4096 itself when it runs on the same rows, in one launch
+  auto class_items = [&](int m, std::vector<FftItem>& fi) {
+    for (const int i : by_L[m]) {
       const dc_item& it = items[i];
-      const int no = (int)(it.n_out ? it.n_out : it.n);
-      fi[j].src = reinterpret_cast<const float2*>(ws + yoff[i]);
-      fi[j].dst = Y + it.out_off;
-      fi[j].ptab = nullptr;
-      fi[j].ph = phase_params(it.fs, it.fc, it.tec_tecu, m);
-      fi[j].n_valid = no;
-      fi[j].n_out = no;
+      FftItem f{};
+      f.src = reinterpret_cast<const float2*>(ws + yoff[i]);
+      f.dst = Y + it.out_off;
+      f.ph = phase_params(it.fs, it.fc, it.tec_tecu, m);
+      f.n_valid = f.n_out = (int)(it.n_out ? it.n_out : it.n);
+      fi.push_back(f);
     }
+  };
+  std::vector<FftItem> rows;
+  int first[14] = {}, m0 = 0;
+  for (; m0 < 12; ++m0) {
+    first[m0] = (int)rows.size();
+    class_items(m0, rows);
+  }
+  first[12] = (int)rows.size();
+  if (!rows.empty()) {
+    if (use_fused(c, 12)) class_items(m0++, rows);
+    first[13] = (int)rows.size();
+    if ((st = run_row_classes(c, rows, first, item_at, s))) return st;
+  }
+  for (int m = m0; m <= 20; ++m) {
+    if (by_L[m].empty()) continue;
+    std::vector<FftItem> fi;
+    fi.reserve(by_L[m].size());
+    class_items(m, fi);
     float2* T = reinterpret_cast<float2*>(ws + class_T[m]);
     if ((st = run_iono_class(c, fi, m, T, class_chunk[m], item_at, s))) return st;
   }

@@ -1,7 +1,10 @@
 // Stockham FFT passes with the fused ionospheric phase multiply.
 // Index conventions and the four-step split are described in fft.cuh.
+#include <algorithm>
+
 #include "fft.cuh"
 #include "fused.cuh"
+#include "rows.cuh"
 
 namespace dc {
 
@@ -84,85 +87,106 @@ DC_DEV void row_fft(float2* sm, const float2* __restrict__ tw) {
   }
 }
 
-// Row pass.  Line g of the launch is row (g mod L1) of item (g / L1).
+// Row pass of CTA `block`: its LINES transforms of length M, through shared
+// memory.  A thread's global loads are all issued before its first store to
+// shared memory, and items are read by non-coherent loads: otherwise every load
+// waits behind the store before it (a class of L <= 2048 took 20 us so).
 template <int M, int OP>
-__global__ void __launch_bounds__(kThreads) row_kernel(RowArgs a) {
+DC_DEV void row_pass(float2* sm, const FftItem* items, int n_items, int block, const float2* __restrict__ tw) {
   constexpr int LINES = RowShape<M>::LINES;
   constexpr int LP = M + (M >> 4) + 1;
-  extern __shared__ float2 sm[];
-  const int L1 = 1 << a.log2L1;
-  const int total = a.n_items * L1;
-  const int line0 = blockIdx.x * LINES;
-  const float invL = 1.0f / (float)(1 << a.log2L);
+  constexpr int PER = (LINES * M + kThreads - 1) / kThreads;   // elements per thread
+  const int line0 = block * LINES;
 
   // ---- load (coalesced along each line)
-  for (int idx = threadIdx.x; idx < LINES * M; idx += kThreads) {
-    const int c = idx / M, p = idx % M;
-    const int g = line0 + c;
-    float2 v = make_float2(0.f, 0.f);
-    if (g < total) {
-      const int it = g >> a.log2L1, row = g & (L1 - 1);
-      const FftItem& I = a.items[it];
-      if (a.log2L1 == 0) {
-        if (OP == ROW_FULL || OP == ROW_SPEC) {
-          if (p < I.n_valid) v = I.src[p];
-        } else {
-          v = I.src[p];
-        }
-      } else {
-        v = I.src[(size_t)row * M + p];
-      }
+  float2 v[PER];
+#pragma unroll
+  for (int q = 0; q < PER; ++q) {
+    const int idx = threadIdx.x + kThreads * q;
+    const int g = line0 + idx / M, p = idx % M;
+    v[q] = make_float2(0.f, 0.f);
+    if (g < n_items) {
+      const FftItem I = ldg_item(items + g);
+      if (OP == ROW_APPLY || p < I.n_valid) v[q] = I.src[p];
       if (OP == ROW_APPLY) {
-        const int k = row + L1 * p;
         // the table is in the spectrum's own layout (natural below 4096)
-        if (I.ptab) v = cmul(v, __ldg(I.ptab + (size_t)row * M + p));
-        else if (I.ph.enabled) v = cmul(v, iono_factor(I.ph, k));
+        if (I.ptab) v[q] = cmul(v[q], __ldg(I.ptab + p));
+        else if (I.ph.enabled) v[q] = cmul(v[q], iono_factor(I.ph, p));
       }
     }
-    sm[c * LP + rpad(p)] = v;
+  }
+#pragma unroll
+  for (int q = 0; q < PER; ++q) {
+    const int idx = threadIdx.x + kThreads * q;
+    sm[(idx / M) * LP + rpad(idx % M)] = v[q];
   }
   __syncthreads();
 
-  if (OP == ROW_FULL || OP == ROW_MID || OP == ROW_SPEC) row_fft<M, -1, LINES, LP>(sm, a.tw);
+  if (OP != ROW_APPLY) row_fft<M, -1, LINES, LP>(sm, tw);
 
-  if (OP == ROW_FULL || OP == ROW_MID) {
-    for (int idx = threadIdx.x; idx < LINES * M; idx += kThreads) {
+  if (OP == ROW_FULL) {
+#pragma unroll
+    for (int q = 0; q < PER; ++q) {
+      const int idx = threadIdx.x + kThreads * q;
       const int c = idx / M, p = idx % M;
-      const int g = line0 + c;
-      if (g < total) {
-        const int it = g >> a.log2L1, row = g & (L1 - 1);
-        const FftItem& I = a.items[it];
-        const int k = row + L1 * p;
-        float2 w;
-        if (I.ptab) w = __ldg(I.ptab + (size_t)row * M + (M == 4096 ? spec_index(p) : p));
-        else if (I.ph.enabled) w = iono_factor(I.ph, k);
-        else continue;
+      if (line0 + c < n_items) {
+        const FftItem I = ldg_item(items + line0 + c);
+        float2 w = make_float2(1.f, 0.f);
+        if (I.ptab) w = __ldg(I.ptab + (M == 4096 ? spec_index(p) : p));
+        else if (I.ph.enabled) w = iono_factor(I.ph, p);
         sm[c * LP + rpad(p)] = cmul(sm[c * LP + rpad(p)], w);
       }
     }
     __syncthreads();
   }
 
-  if (OP != ROW_SPEC) row_fft<M, +1, LINES, LP>(sm, a.tw);
+  if (OP != ROW_SPEC) row_fft<M, +1, LINES, LP>(sm, tw);
 
-  // ---- store
-  for (int idx = threadIdx.x; idx < LINES * M; idx += kThreads) {
+  // ---- store (scaled and truncated, or the whole spectrum)
+#pragma unroll
+  for (int q = 0; q < PER; ++q) {
+    const int idx = threadIdx.x + kThreads * q;
     const int c = idx / M, p = idx % M;
-    const int g = line0 + c;
-    if (g >= total) continue;
-    const int it = g >> a.log2L1, row = g & (L1 - 1);
-    const FftItem& I = a.items[it];
-    float2 v = sm[c * LP + rpad(p)];
-    if (OP == ROW_SPEC) {
-      I.dst[(size_t)row * M + p] = v;
-    } else if (a.log2L1 == 0) {
-      // single pass: scale and truncate
-      if (p < I.n_out) __stcs(I.dst + p, cscale(v, invL));
-    } else {
-      // four-step middle / apply: twiddle W_L^(-n2 k1), n2 = p, k1 = row
-      v = cmul(v, tw_big<+1>(a.tw, (uint32_t)(p * row) & ((1u << a.log2L) - 1), a.log2L));
-      I.dst[(size_t)row * M + p] = v;
-    }
+    if (line0 + c >= n_items) continue;
+    const FftItem I = ldg_item(items + line0 + c);
+    const float2 x = sm[c * LP + rpad(p)];
+    if (OP == ROW_SPEC) I.dst[p] = x;
+    else if (p < I.n_out) __stcs(I.dst + p, cscale(x, 1.0f / (float)M));
+  }
+}
+
+template <int M, int OP>
+__global__ void __launch_bounds__(kThreads) row_kernel(RowArgs a) {
+  extern __shared__ float2 sm[];
+  row_pass<M, OP>(sm, a.items, a.n_items, blockIdx.x, a.tw);
+}
+
+// Short transforms of several length classes in one launch: run one after the
+// other, the classes of a small batch leave the chip idle (each is one latency
+// chain of about 20 us on a few CTAs).
+template <int M>
+DC_DEV void class_pass(float2* sm, const RowClasses& a, int m) {
+  row_pass<M, ROW_FULL>(sm, a.items + a.first[m], a.first[m + 1] - a.first[m], blockIdx.x - a.block[m], a.tw);
+}
+__global__ void __launch_bounds__(kThreads) row_classes_kernel(const __grid_constant__ RowClasses a) {
+  extern __shared__ float2 sm[];
+  int m = 0;
+  while (m < 12 && (int)blockIdx.x >= a.block[m + 1]) ++m;
+  switch (m) {
+    case 0: class_pass<1>(sm, a, m); break;
+    case 1: class_pass<2>(sm, a, m); break;
+    case 2: class_pass<4>(sm, a, m); break;
+    case 3: class_pass<8>(sm, a, m); break;
+    case 4: class_pass<16>(sm, a, m); break;
+    case 5: class_pass<32>(sm, a, m); break;
+    case 6: class_pass<64>(sm, a, m); break;
+    case 7: class_pass<128>(sm, a, m); break;
+    case 8: class_pass<256>(sm, a, m); break;
+    case 9: class_pass<512>(sm, a, m); break;
+    case 10: class_pass<1024>(sm, a, m); break;
+    case 11: class_pass<2048>(sm, a, m); break;
+    default:
+      full_4096<false>(ldg_item(a.items + a.first[12] + blockIdx.x - a.block[12]), sm, threadIdx.x, a.tw);
   }
 }
 
@@ -352,10 +376,25 @@ static cudaError_t launch_row_op(const RowArgs& a, cudaStream_t s) {
   }
 }
 
+cudaError_t launch_row_classes(RowClasses a, cudaStream_t s) {
+  static constexpr int kLines[13] = {256, 256, 256, 256, 256, 128, 64, 32, 16, 8, 4, 2, 1};
+  size_t smem = 0;
+  a.block[0] = 0;
+  for (int m = 0; m <= 12; ++m) {
+    const int n = a.first[m + 1] - a.first[m];
+    a.block[m + 1] = a.block[m] + (n + kLines[m] - 1) / kLines[m];
+    const int M = 1 << m, line = m == 12 ? kRowPitch : M + (M >> 4) + 1;
+    if (n > 0) smem = std::max(smem, sizeof(float2) * kLines[m] * line);
+  }
+  if (a.block[13] == 0) return cudaSuccess;
+  row_classes_kernel<<<(unsigned)a.block[13], kThreads, smem, s>>>(a);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_row(int op, const RowArgs& a, cudaStream_t s) {
   switch (op) {
     case ROW_FULL: return launch_row_op<ROW_FULL>(a, s);
-    case ROW_MID: return launch_row_op<ROW_MID>(a, s);
+    case ROW_MID: return launch_row_4096(op, a, s);
     case ROW_SPEC: return launch_row_op<ROW_SPEC>(a, s);
     case ROW_APPLY: return launch_row_op<ROW_APPLY>(a, s);
     default: return cudaErrorInvalidValue;

@@ -29,20 +29,33 @@ namespace dc {
 __host__ __device__ constexpr int spec_index(int k2) { return ((k2 & 15) << 8) | (k2 >> 4); }
 __host__ __device__ constexpr int spec_bin(int idx) { return ((idx & 255) << 4) | (idx >> 8); }
 
-// One transform of a launch.  All items of one launch share L.
-struct FftItem {
+// One transform of a launch.  64 bytes: read whole by four 16-byte loads (ldg_item).
+struct alignas(16) FftItem {
+  PhaseParams ph;
   const float2* src;     // input of this pass
   float2* dst;           // output of this pass
   const float2* ptab;    // per-bin factors (length L): exp(-i phi_k), times a
                          // matched filter's conjugate replica spectrum when
                          // compressing, in the spectrum's layout (bin
                          // k1 + L1 k2 at k1*4096 + spec_index(k2) for L >=
-                         // 4096, natural order below); null -> exp(-i phi_k) computed from
-                         // `ph`
-  PhaseParams ph;
+                         // 4096, natural order below); null -> exp(-i phi_k)
+                         // computed from `ph`
   int n_valid;           // samples of src that are data (zero beyond), first pass
   int n_out;             // samples stored by the last pass (truncation)
 };
+static_assert(sizeof(FftItem) == 64, "four 16-byte loads");
+
+// An item by non-coherent loads, which the compiler may move over stores to
+// shared memory (it cannot prove those apart from a generic pointer's target).
+DC_DEV FftItem ldg_item(const FftItem* p) {
+  union {
+    uint4 q[4];
+    FftItem it;
+  } u = {};
+#pragma unroll
+  for (int i = 0; i < 4; ++i) u.q[i] = __ldg(reinterpret_cast<const uint4*>(p) + i);
+  return u.it;
+}
 
 enum RowOp : int {
   ROW_FULL = 0,   // L <= 4096: load (zero-pad), fwd, phase, inv, 1/L, store n < n_out
@@ -62,6 +75,14 @@ struct RowArgs {
   int log2L1;      // rows per transform (0 for L <= 4096)
   const float2* tw;
 };
+// The full correction (ROW_FULL) of several length classes L = 2^m, m <= 12, in
+// one launch: class m's transforms are items [first[m], first[m + 1]), its CTAs
+// blocks [block[m], block[m + 1]).
+struct RowClasses {
+  const FftItem* items;
+  int first[14], block[14];
+  const float2* tw;
+};
 struct ColArgs {
   const FftItem* items;
   int n_items;
@@ -72,6 +93,7 @@ struct ColArgs {
 
 // Launchers (fft.cu).  Return cudaSuccess or the launch error.
 cudaError_t launch_row(int op, const RowArgs& a, cudaStream_t s);
+cudaError_t launch_row_classes(RowClasses a, cudaStream_t s);   // block[] filled here
 cudaError_t launch_col(int op, const ColArgs& a, cudaStream_t s);
 
 }  // namespace dc

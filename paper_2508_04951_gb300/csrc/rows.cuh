@@ -1,0 +1,185 @@
+// 4096-point rows in registers: 256 threads, 16 points each, one padded
+// shared-memory buffer and one CTA barrier per direction.
+#pragma once
+
+#include "fft.cuh"
+
+namespace dc {
+
+constexpr int kRowN = 4096;             // row length
+constexpr int kRowThreads = 256;        // threads per row (one radix-16 butterfly each)
+constexpr int kRowPitch = kRowN + kRowN / 16;
+
+DC_DEV int pad16(int p) { return p + (p >> 4); }
+
+// Twiddles of a 4096-point row: W256^(r k), k = 0..15 (s2) and W4096^(r j), j =
+// 0..255 (s3), forward values.  Only the table rows r = 1, 2, 4, 8 are read;
+// the other powers are their products (apply_powers).
+struct GlobalTw {                 // the context's table (coalesced across the warp)
+  const float2* __restrict__ tw;
+  DC_DEV void s2(float2 (&b)[4], int k) const {
+    const float2* t = tw + kTwS2 + k;             // row r at (r - 1) * 16
+    b[0] = __ldg(t), b[1] = __ldg(t + 16), b[2] = __ldg(t + 48), b[3] = __ldg(t + 112);
+  }
+  DC_DEV void s3(float2 (&b)[4], int j) const {
+    const float2* t = tw + kTwS3 + j;             // row r at (r - 1) * 256
+    b[0] = __ldg(t), b[1] = __ldg(t + 256), b[2] = __ldg(t + 768), b[3] = __ldg(t + 1792);
+  }
+};
+struct SharedTw {                 // a persistent CTA's copies of those rows, [4][16] and [4][256]
+  const float2 *t2, *t3;
+  DC_DEV void s2(float2 (&b)[4], int k) const {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) b[q] = t2[q * 16 + k];
+  }
+  DC_DEV void s3(float2 (&b)[4], int j) const {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) b[q] = t3[q * 256 + j];
+  }
+};
+struct HeldTw {                   // loaded ahead by the caller, for this thread
+  const float2 (&f2)[4], (&f3)[4];
+  DC_DEV void s2(float2 (&b)[4], int) const {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) b[q] = f2[q];
+  }
+  DC_DEV void s3(float2 (&b)[4], int) const {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) b[q] = f3[q];
+  }
+};
+template <int DIR> DC_DEV void orient(float2 (&b)[4]) {
+#pragma unroll
+  for (int q = 0; q < 4; ++q) b[q] = conj_if<DIR>(b[q]);
+}
+
+// 4096-point rows, thread j = 16 s + t of 256, with one CTA barrier each.  The
+// split 4096 = 16 x 16 x 16: n = 256 p + 16 u + w, k = s + 16 a + 256 r.
+//
+// Forward: v[p] = x[256 p + j] in, v[r] = X[s + 16 t + 256 r] out.
+//   length-16 DFT over p (thread q = 16 u + w), W4096^(q s); a CTA-wide exchange
+//   gives half-warp s the 256 values of its sub-problem; DFT over u in thread w =
+//   t, W256^(w a); a 16 x 16 transpose inside the half-warp; DFT over w in thread
+//   a = t.
+// Inverse: the mirror image, v[r] = Y[s + 16 t + 256 r] in, v[p] = y[256 p + j]
+// out: DFT over r, W256^(-w a), half-warp transpose, DFT over a, CTA-wide
+// exchange, W4096^(-q s), DFT over s.
+//
+// So a forward row, factors on the bins and an inverse row need two CTA barriers
+// between them, and the bins meet their factors in registers.  b is one padded
+// buffer (element n at n + n / 16): half-warp s keeps to its own 272 elements
+// except in the CTA-wide exchange, where the forward row writes element 256 p +
+// j (thread j of every p: what that thread may itself have read there before)
+// and the inverse row reads it.  Callers: before the forward row nobody else may
+// still read elements 256 p + j, before the inverse row nobody may still read
+// b; on return from the inverse row other threads may still read b.
+template <class TW>
+DC_DEV void row_forward(float2 (&v)[16], float2* b, int j, const TW& tw) {
+  const int s = j >> 4, t = j & 15;
+  float2 w[4];
+  tw.s3(w, j);                                             // issued ahead of the DFT
+  dft16<-1>(v);                                            // over p
+  apply_powers<16>(v, w);                                  // W4096^(q s), q = j
+#pragma unroll
+  for (int r = 0; r < 16; ++r) b[pad16(256 * r + j)] = v[r];
+  tw.s2(w, t);
+  __syncthreads();
+  float2* reg = b + 272 * s;                               // = pad16(256 s)
+#pragma unroll
+  for (int u = 0; u < 16; ++u) v[u] = reg[17 * u + t];     // q = 16 u + t
+  dft16<-1>(v);                                            // over u
+  apply_powers<16>(v, w);                                  // W256^(w a)
+  __syncwarp();                                            // its reads of the region are done
+#pragma unroll
+  for (int a = 0; a < 16; ++a) reg[17 * a + t] = v[a];     // V[w = t][a]
+  __syncwarp();
+#pragma unroll
+  for (int q = 0; q < 16; ++q) v[q] = reg[17 * t + q];     // thread a = t: V[w = q][a]
+  dft16<-1>(v);                                            // over w
+}
+
+// ARRIVE: arrive at the cluster barrier (release) once this thread's last read
+// of b is done: peers may overwrite the buffer after their wait.
+template <bool ARRIVE, class TW>
+DC_DEV void row_inverse(float2 (&v)[16], float2* b, int j, const TW& tw) {
+  const int s = j >> 4, t = j & 15;
+  float2 w[4];
+  tw.s2(w, t);
+  dft16<+1>(v);                                            // over r
+  orient<+1>(w);
+  apply_powers<16>(v, w);                                  // W256^(-w a), a = t
+  float2* reg = b + 272 * s;
+  __syncwarp();                                            // a forward row's reads of the region
+#pragma unroll
+  for (int q = 0; q < 16; ++q) reg[17 * q + t] = v[q];     // V[a = t][w]
+  __syncwarp();
+#pragma unroll
+  for (int a = 0; a < 16; ++a) v[a] = reg[17 * t + a];     // thread w = t: V[a][w]
+  dft16<+1>(v);                                            // over a
+  __syncwarp();
+#pragma unroll
+  for (int u = 0; u < 16; ++u) reg[17 * u + t] = v[u];     // q = 16 u + t of sub-problem s
+  tw.s3(w, j);
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < 16; ++q) v[q] = b[pad16(256 * q + j)];
+  if constexpr (ARRIVE) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  orient<+1>(w);
+  apply_powers<16>(v, w);                                  // W4096^(-q s), q = j
+  dft16<+1>(v);                                            // over s
+}
+
+// Index of thread j's bin r in a stored row (spec_index(s + 16 t + 256 r)).
+DC_DEV int spec_pos(int j, int r) { return ((j >> 4) << 8) + (j & 15) + 16 * r; }
+
+// v[r] *= the factor of bin k1 + L1 (s + 16 t + 256 r), r = 0..15 (L1 =
+// 2^log2L1): the item's table (exp(-i phi_k) times anything else the call
+// bundles into the frequency domain, e.g. a matched filter's conjugate
+// replica spectrum) when there is one, else exp(-i phi_k) of Eq. 16.
+DC_DEV void bin_factors(const FftItem& I, int k1, int log2L1, int j, float2 (&v)[16]) {
+  if (I.ptab) {
+    const float2* t = I.ptab + (size_t)k1 * kRowN;
+#pragma unroll
+    for (int r = 0; r < 16; ++r) v[r] = cmul(v[r], __ldg(t + spec_pos(j, r)));
+  } else if (I.ph.enabled) {
+    // bins r >= 8 are the upper half of the transform: kt = k - L
+    const PhaseParams& P = I.ph;
+    const float kt0 = (float)(k1 + (((j >> 4) + ((j & 15) << 4)) << log2L1));
+    const float step = (float)(256 << log2L1);
+#pragma unroll
+    for (int r = 0; r < 16; ++r)
+      v[r] = cmul(v[r], iono_factor_kt(P, fmaf((float)(r < 8 ? r : r - 16), step, kt0)));
+  }
+}
+
+// The whole correction of one L = 4096 transform: zero-padded input, forward row,
+// factors, inverse row, 1 / L, truncation.  Every stage base of both rows is loaded up
+// front, beside the input: one CTA per transform leaves nothing to hide a load issued
+// per stage.  PDL: the input is read after pdl_wait, by plain loads (a
+// non-coherent load may be scheduled ahead of the wait).
+template <bool PDL>
+DC_DEV void full_4096(const FftItem& I, float2* b, int j, const float2* tw) {
+  float2 f2[4], f3[4];
+  GlobalTw{tw}.s2(f2, j & 15);
+  GlobalTw{tw}.s3(f3, j);
+  if constexpr (PDL) pdl_wait();                // the input's producer has finished
+  float2 v[16];
+#pragma unroll
+  for (int r = 0; r < 16; ++r) {
+    const int n = j + 256 * r;
+    v[r] = n < I.n_valid ? I.src[n] : make_float2(0.f, 0.f);
+  }
+  row_forward(v, b, j, HeldTw{f2, f3});
+  bin_factors(I, 0, 0, j, v);
+  const float invL = 1.0f / (float)kRowN;
+#pragma unroll
+  for (int r = 0; r < 16; ++r) v[r] = cscale(v[r], invL);
+  row_inverse<false>(v, b, j, HeldTw{f2, f3});
+#pragma unroll
+  for (int r = 0; r < 16; ++r) {
+    const int n = j + 256 * r;
+    if (n < I.n_out) __stcs(I.dst + n, v[r]);
+  }
+}
+
+}  // namespace dc
