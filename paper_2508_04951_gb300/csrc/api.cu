@@ -7,6 +7,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <functional>
 #include <mutex>
 #include <string>
 #include <vector>
@@ -53,7 +54,12 @@ struct dc_ctx {
   char* items = nullptr;      // device item arrays
   size_t items_bytes = 0;
   long long launches = 0;     // kernels launched by this context
-  // While a plan is being recorded: item uploads go to this host staging
+  // The call in hand: its lists staged for one copy to the item buffer, and the
+  // launches that follow it (enqueue, flush).
+  std::vector<char> stage;
+  size_t stage_lo = 0, stage_hi = 0;
+  std::vector<std::function<dc_status()>> todo;
+  // While a plan is being recorded: the lists go to this host staging
   // buffer (copied to the plan's device item buffer once the capture ends).
   std::vector<char>* rec = nullptr;
   bool fixed_ws = false;      // the scratch is the caller's (a server's pool block): never grown
@@ -76,6 +82,12 @@ struct dc_ctx {
     int apply_kind = 0;        // spectrum apply: 1 cluster, one row per CTA; 2 cluster, two rows
                                // per CTA (L >= 32768); 3 two passes through L2 (L >= 8192)
   } tune;
+  // Kaiser window tables on the device, by taps and beta, for the context's
+  // life: the first kPolySlots pairs it meets (later ones are uploaded per call).
+  static constexpr int kPolySlots = 16;
+  static constexpr size_t kPolyFloats = 2 * kMaxHalf * kWCoef + 32 * 3 * kWCoef;   // values, 32-tap derivatives
+  float* poly = nullptr;
+  std::vector<std::pair<int, double>> poly_keys;
   std::recursive_mutex mu;
 };
 
@@ -397,20 +409,115 @@ dc_status check_pulse(dc_ctx* c, long long n, long long n_out, double fs, double
 
 cudaStream_t S(void* s) { return reinterpret_cast<cudaStream_t>(s); }
 
-// Upload an item array to the context's device item buffer (stream-ordered;
-// the pageable source may be reused as soon as this returns).
+// Every entry point below stages its lists (upload) and queues its launches
+// (enqueue), then sends the lists in one copy and runs the launches (flush): a
+// call costs one copy instead of one per list, and none at all when its only
+// items travel in kernel arguments (a single pulse).
+//
+// Stage an item array at offset `at` of the context's device item buffer.
 template <class T>
-dc_status upload(dc_ctx* c, const std::vector<T>& v, size_t at, cudaStream_t s, const T** dev) {
+dc_status upload(dc_ctx* c, const std::vector<T>& v, size_t at, const T** dev) {
   const size_t bytes = v.size() * sizeof(T);
   if (at + bytes > c->items_bytes) return fail(c, DC_ENOMEM, "item list overflow");
-  if (c->rec) {
-    memcpy(c->rec->data() + at, v.data(), bytes);
-  } else {
-    cudaError_t e = cudaMemcpyAsync(c->items + at, v.data(), bytes, cudaMemcpyHostToDevice, s);
-    if (e != cudaSuccess) return cuda_fail(c, e, "item upload");
-  }
+  if (c->stage.size() < at + bytes) c->stage.resize(std::max(c->items_bytes, at + bytes));
+  if (bytes) memcpy(c->stage.data() + at, v.data(), bytes);
+  c->stage_lo = c->stage_hi ? std::min(c->stage_lo, at) : at;
+  c->stage_hi = std::max(c->stage_hi, at + bytes);
   *dev = reinterpret_cast<const T*>(c->items + at);
   return DC_OK;
+}
+
+// A launch's items: the one item into its arguments (`one`, the device pointer
+// stays null), several staged at `at`, which moves past them.
+template <class T>
+dc_status stage_items(dc_ctx* c, const std::vector<T>& v, size_t& at, const T** dev, T* one) {
+  if (v.size() == 1) {
+    *one = v[0];
+    return DC_OK;
+  }
+  dc_status st = upload(c, v, at, dev);
+  at += (v.size() * sizeof(T) + 255) & ~(size_t)255;
+  return st;
+}
+
+template <class F>
+void enqueue(dc_ctx* c, int phase, cudaStream_t s, long long samples, const char* what, F&& launch) {
+  c->todo.emplace_back([=]() -> dc_status {
+    Phase ph(c, phase, s, samples);
+    const cudaError_t e = launch();
+    return e == cudaSuccess ? DC_OK : cuda_fail(c, e, what);
+  });
+}
+
+// Drops what a call staged and queued, however it ends (the recursive calls of
+// plans and autotuning flush before they return).
+struct Call {
+  dc_ctx* c;
+  explicit Call(dc_ctx* c_) : c(c_) { reset(); }
+  ~Call() { reset(); }
+  void reset() {
+    c->todo.clear();
+    c->stage_lo = c->stage_hi = 0;
+  }
+};
+
+dc_status flush(dc_ctx* c, cudaStream_t s) {
+  if (c->stage_hi) {
+    const size_t n = c->stage_hi - c->stage_lo;
+    if (c->rec) {
+      memcpy(c->rec->data() + c->stage_lo, c->stage.data() + c->stage_lo, n);
+    } else {
+      // the pageable source may be reused as soon as this returns
+      const cudaError_t e = cudaMemcpyAsync(c->items + c->stage_lo, c->stage.data() + c->stage_lo, n,
+                                            cudaMemcpyHostToDevice, s);
+      if (e != cudaSuccess) return cuda_fail(c, e, "item upload");
+    }
+  }
+  for (auto& f : c->todo)
+    if (dc_status st = f()) return st;
+  return DC_OK;
+}
+
+// Window polynomials of (taps, beta) on the device: values and, for 32 taps, the
+// values with two derivatives.  Null when the context holds no table for the
+// pair and takes none (all slots used, or the stream is capturing: the copy would
+// become part of the graph); the caller then stages the polynomials itself.
+struct PolyTables { const float *w, *d012; };
+PolyTables poly_tables(dc_ctx* c, int taps, double beta, cudaStream_t s) {
+  size_t i = 0;
+  while (i < c->poly_keys.size() && !(c->poly_keys[i].first == taps && c->poly_keys[i].second == beta)) ++i;
+  float* dev = c->poly + i * dc_ctx::kPolyFloats;
+  if (i == c->poly_keys.size()) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (i == (size_t)dc_ctx::kPolySlots || c->rec ||
+        (s && (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone))) {
+      cudaGetLastError();
+      return {nullptr, nullptr};
+    }
+    std::vector<float> v(dc_ctx::kPolyFloats, 0.f);
+    const std::vector<float> w = window_poly(taps, beta);
+    std::copy(w.begin(), w.end(), v.begin());
+    if (taps == 32) {
+      const std::vector<float> d = window_poly_d012(taps, beta);
+      std::copy(d.begin(), d.end(), v.begin() + 2 * kMaxHalf * kWCoef);
+    }
+    // on a stream of its own, waited for: complete before any stream's launch
+    cudaStream_t up = nullptr;
+    if (cudaStreamCreateWithFlags(&up, cudaStreamNonBlocking) != cudaSuccess) {
+      cudaGetLastError();
+      return {nullptr, nullptr};
+    }
+    const bool ok = cudaMemcpyAsync(dev, v.data(), v.size() * sizeof(float), cudaMemcpyHostToDevice, up) ==
+                        cudaSuccess &&
+                    cudaStreamSynchronize(up) == cudaSuccess;
+    cudaStreamDestroy(up);
+    if (!ok) {
+      cudaGetLastError();
+      return {nullptr, nullptr};
+    }
+    c->poly_keys.emplace_back(taps, beta);
+  }
+  return {dev, taps == 32 ? dev + 2 * kMaxHalf * kWCoef : nullptr};
 }
 
 // ------------------------------------------------------------ resampling
@@ -418,65 +525,44 @@ dc_status upload(dc_ctx* c, const std::vector<T>& v, size_t at, cudaStream_t s, 
 dc_status run_windowed(dc_ctx* c, std::vector<RsItem>& items, const dc_opts& o, size_t item_at,
                        cudaStream_t s) {
   if (items.empty()) return DC_OK;
-  if (o.mode == DC_FREQCONV) {
-    int tiles = 0;
-    long long outs = 0;
-    for (auto& it : items) {
-      it.tile_begin = tiles;
-      tiles += (int)((it.n_out + kRsTile - 1) / kRsTile);
-      outs += it.n_out;
-    }
-    const RsItem* dev = nullptr;
-    dc_status st = upload(c, items, item_at, s, &dev);
-    if (st) return st;
-    RsArgs a{};
-    a.items = dev;
-    a.n_items = (int)items.size();
-    a.n_tiles = tiles;
-    a.err = c->err;
-    Phase ph(c, PH_FREQCONV, s, outs);
-    cudaError_t e = launch_freqconv(a, s);
-    if (e != cudaSuccess) return cuda_fail(c, e, "frequency conversion launch");
-    return DC_OK;
-  }
-  const std::vector<float> wp = window_poly(o.taps, o.kaiser_beta);
-  const float* dwp = nullptr;
-  dc_status st = upload(c, wp, item_at, s, &dwp);
-  if (st) return st;
-  size_t at = item_at + ((wp.size() * sizeof(float) + 255) & ~(size_t)255);
-  // Split into the tiled launches (32 taps, |delta| <= 0.01; 8 outputs per
-  // lane while the quadratic weights hold over 256 outputs, else 4) and the
-  // direct one.
-  std::vector<RsItem> tiled8, tiled4, direct;
+  // Frequency conversion is one launch; the windowed sum splits into the tiled
+  // launches (32 taps, |delta| <= 0.01; 8 outputs per lane while the quadratic
+  // weights hold over 256 outputs, else 4) and the direct one.
+  enum { TILED8, TILED4, DIRECT, CONVERT };
+  std::vector<RsItem> group[4];
   for (auto& it : items) {
     const double dl = std::fabs((double)it.dl_hi + (double)it.dl_lo);
-    if (o.taps != 32 || dl > kRsTiledMaxDelta) direct.push_back(it);
-    else (resample_q(dl) == 8 && c->tune.rs_q != 4 ? tiled8 : tiled4).push_back(it);
+    if (o.mode == DC_FREQCONV) group[CONVERT].push_back(it);
+    else if (o.taps != 32 || dl > kRsTiledMaxDelta) group[DIRECT].push_back(it);
+    else group[resample_q(dl) == 8 && c->tune.rs_q != 4 ? TILED8 : TILED4].push_back(it);
   }
-  for (int pass = 0; pass < 3; ++pass) {
-    auto& v = pass == 0 ? tiled8 : pass == 1 ? tiled4 : direct;
+  const float* dwp = nullptr;
+  size_t at = item_at;
+  if (o.mode != DC_FREQCONV && !(dwp = poly_tables(c, o.taps, o.kaiser_beta, s).w)) {
+    const std::vector<float> wp = window_poly(o.taps, o.kaiser_beta);
+    if (dc_status st = upload(c, wp, at, &dwp)) return st;
+    at += (wp.size() * sizeof(float) + 255) & ~(size_t)255;
+  }
+  for (int kind = TILED8; kind <= CONVERT; ++kind) {
+    auto& v = group[kind];
     if (v.empty()) continue;
-    int tiles = 0;
-    for (auto& it : v) {
-      it.tile_begin = tiles;
-      tiles += (int)((it.n_out + kRsTile - 1) / kRsTile);
-    }
-    const RsItem* dev = nullptr;
-    if ((st = upload(c, v, at, s, &dev))) return st;
-    at += (v.size() * sizeof(RsItem) + 255) & ~(size_t)255;
     RsArgs a{};
-    a.items = dev;
+    long long outs = 0;
+    for (auto& it : v) {
+      it.tile_begin = a.n_tiles;
+      a.n_tiles += (int)((it.n_out + kRsTile - 1) / kRsTile);
+      outs += it.n_out;
+    }
+    if (dc_status st = stage_items(c, v, at, &a.items, &a.one)) return st;
     a.n_items = (int)v.size();
-    a.n_tiles = tiles;
     a.half = o.taps / 2;
     a.wpoly = dwp;
     a.err = c->err;
-    long long outs = 0;
-    for (auto& it : v) outs += it.n_out;
-    Phase ph(c, pass < 2 ? PH_RS_TILED : PH_RS_DIRECT, s, outs);
-    cudaError_t e = pass < 2 ? launch_resample_tiled32(a, pass == 0 ? 8 : 4, s)
-                             : launch_resample_direct(a, s);
-    if (e != cudaSuccess) return cuda_fail(c, e, "resample launch");
+    enqueue(c, kind == CONVERT ? PH_FREQCONV : kind == DIRECT ? PH_RS_DIRECT : PH_RS_TILED, s, outs, "resample launch", [=] {
+      return kind == CONVERT ? launch_freqconv(a, s)
+             : kind == DIRECT ? launch_resample_direct(a, s)
+                              : launch_resample_tiled32(a, kind == TILED8 ? 8 : 4, s);
+    });
   }
   return DC_OK;
 }
@@ -500,26 +586,26 @@ dc_status run_resample_tc(dc_ctx* c, const float2* x, int n_in, int n_out, const
     const double spread = (dl[order[last]] - dl[order[g]]) * ((double)n_out + 64.0) + 2.0;
     if (spread > (double)rs_tc_max_span()) return DC_EINVAL;
   }
-  const std::vector<float> wp = window_poly_d012(o.taps, o.kaiser_beta);
   std::vector<float> dls(2 * (size_t)n_v);
   std::vector<int> vidx(n_v);
   for (int i = 0; i < n_v; ++i) {
     split(dl[order[i]], dls[2 * i], dls[2 * i + 1]);
     vidx[i] = order[i];
   }
-  const float* dwp = nullptr;
+  const float* dwp = poly_tables(c, o.taps, o.kaiser_beta, s).d012;
   const float* ddl = nullptr;
   const int* dvi = nullptr;
-  dc_status st = upload(c, wp, item_at, s, &dwp);
-  if (st) return st;
-  item_at += (wp.size() * sizeof(float) + 255) & ~(size_t)255;
-  if ((st = upload(c, dls, item_at, s, &ddl))) return st;
+  dc_status st;
+  if (!dwp) {
+    const std::vector<float> wp = window_poly_d012(o.taps, o.kaiser_beta);
+    if ((st = upload(c, wp, item_at, &dwp))) return st;
+    item_at += (wp.size() * sizeof(float) + 255) & ~(size_t)255;
+  }
+  if ((st = upload(c, dls, item_at, &ddl))) return st;
   item_at += (dls.size() * sizeof(float) + 255) & ~(size_t)255;
-  if ((st = upload(c, vidx, item_at, s, &dvi))) return st;
-  RsTcArgs a{x, n_in, n_out, Y, ddl, dvi, n_v, dwp, c->err};
-  Phase ph(c, PH_RS_TC, s, (long long)n_v * n_out);
-  cudaError_t e = launch_resample_tc(a, s);
-  if (e != cudaSuccess) return cuda_fail(c, e, "tensor-core resample launch");
+  if ((st = upload(c, vidx, item_at, &dvi))) return st;
+  const RsTcArgs a{x, n_in, n_out, Y, ddl, dvi, n_v, dwp, c->err};
+  enqueue(c, PH_RS_TC, s, (long long)n_v * n_out, "tensor-core resample launch", [=] { return launch_resample_tc(a, s); });
   return DC_OK;
 }
 
@@ -561,16 +647,13 @@ BatchLayout batch_layout(const dc_ctx* c, const dc_item* items, int n_items) {
 dc_status run_row_classes(dc_ctx* c, const std::vector<FftItem>& it, const int (&first)[14], size_t& item_at,
                           cudaStream_t s) {
   RowClasses a{};
-  dc_status st = upload(c, it, item_at, s, &a.items);
+  dc_status st = stage_items(c, it, item_at, &a.items, &a.one);
   if (st) return st;
-  item_at += (it.size() * sizeof(FftItem) + 255) & ~(size_t)255;
   std::copy(first, first + 14, a.first);
   a.tw = c->tw;
   long long outs = 0;
   for (auto& f : it) outs += f.n_out;
-  Phase ph(c, PH_ROW_FULL, s, outs);
-  cudaError_t e = launch_row_classes(a, s);
-  if (e != cudaSuccess) return cuda_fail(c, e, "row launch");
+  enqueue(c, PH_ROW_FULL, s, outs, "row launch", [=] { return launch_row_classes(a, s); });
   return DC_OK;
 }
 
@@ -579,19 +662,14 @@ dc_status run_row_classes(dc_ctx* c, const std::vector<FftItem>& it, const int (
 dc_status run_iono_class(dc_ctx* c, std::vector<FftItem>& it, int log2L, float2* T,
                          size_t chunk, size_t& item_at, cudaStream_t s) {
   if (it.empty()) return DC_OK;
-  const FftItem* dev = nullptr;
-  cudaError_t e;
+  long long all = 0;
+  for (auto& f : it) all += f.n_out;
+  dc_status st;
   if (use_fused(c, log2L)) {
-    dc_status st = upload(c, it, item_at, s, &dev);
-    if (st) return st;
-    item_at += (it.size() * sizeof(FftItem) + 255) & ~(size_t)255;
-    FusedArgs a{dev, (int)it.size(), log2L, c->tw, c->err, c->t4};
+    FusedArgs a{nullptr, (int)it.size(), log2L, c->tw, c->err, c->t4};
+    if ((st = stage_items(c, it, item_at, &a.items, &a.one))) return st;
     a.pdl = std::none_of(it.begin(), it.end(), [](const FftItem& f) { return f.ptab != nullptr; });
-    long long outs = 0;
-    for (auto& f : it) outs += f.n_out;
-    Phase ph(c, PH_FUSED_FULL, s, outs);
-    e = launch_fused(FUSED_FULL, a, s);
-    if (e != cudaSuccess) return cuda_fail(c, e, "fused launch");
+    enqueue(c, PH_FUSED_FULL, s, all, "fused launch", [=] { return launch_fused(FUSED_FULL, a, s); });
     return DC_OK;
   }
   if (log2L < 12) {
@@ -600,15 +678,9 @@ dc_status run_iono_class(dc_ctx* c, std::vector<FftItem>& it, int log2L, float2*
     return run_row_classes(c, it, first, item_at, s);
   }
   if (log2L == 12) {
-    dc_status st = upload(c, it, item_at, s, &dev);
-    if (st) return st;
-    item_at += (it.size() * sizeof(FftItem) + 255) & ~(size_t)255;
-    RowArgs a{dev, (int)it.size(), log2L, 0, c->tw};
-    long long outs = 0;
-    for (auto& f : it) outs += f.n_out;
-    Phase ph(c, PH_ROW_FULL, s, outs);
-    e = launch_row(ROW_FULL, a, s);
-    if (e != cudaSuccess) return cuda_fail(c, e, "row launch");
+    RowArgs a{nullptr, (int)it.size(), log2L, 0, c->tw};
+    if ((st = stage_items(c, it, item_at, &a.items, &a.one))) return st;
+    enqueue(c, PH_ROW_FULL, s, all, "row launch", [=] { return launch_row(ROW_FULL, a, s); });
     return DC_OK;
   }
   const int log2L1 = log2L - 12;
@@ -623,34 +695,21 @@ dc_status run_iono_class(dc_ctx* c, std::vector<FftItem>& it, int log2L, float2*
     p2[i].dst = Ti;
     p3[i].src = Ti;
   }
-  const FftItem *d1, *d2, *d3;
-  dc_status st;
-  if ((st = upload(c, p1, item_at, s, &d1))) return st;
-  item_at += (it.size() * sizeof(FftItem) + 255) & ~(size_t)255;
-  if ((st = upload(c, p2, item_at, s, &d2))) return st;
-  item_at += (it.size() * sizeof(FftItem) + 255) & ~(size_t)255;
-  if ((st = upload(c, p3, item_at, s, &d3))) return st;
-  item_at += (it.size() * sizeof(FftItem) + 255) & ~(size_t)255;
+  const FftItem *d1 = nullptr, *d2 = nullptr, *d3 = nullptr;
+  FftItem o1{}, o2{}, o3{};
+  if ((st = stage_items(c, p1, item_at, &d1, &o1)) || (st = stage_items(c, p2, item_at, &d2, &o2)) ||
+      (st = stage_items(c, p3, item_at, &d3, &o3)))
+    return st;
   for (size_t j0 = 0; j0 < it.size(); j0 += chunk) {
     const int cnt = (int)std::min(chunk, it.size() - j0);
     long long outs = 0;
     for (size_t i = j0; i < j0 + cnt; ++i) outs += it[i].n_out;
-    ColArgs a1{d1 + j0, cnt, log2L, log2L1, c->tw};
-    {
-      Phase ph(c, PH_COL_F1, s, outs);
-      if ((e = launch_col(COL_F1, a1, s)) != cudaSuccess) return cuda_fail(c, e, "col F1 launch");
-    }
-    RowArgs a2{d2 + j0, cnt, log2L, log2L1, c->tw};
-    {
-      Phase ph(c, PH_ROW_MID, s, outs);
-      e = launch_row(ROW_MID, a2, s);
-      if (e != cudaSuccess) return cuda_fail(c, e, "row launch");
-    }
-    ColArgs a3{d3 + j0, cnt, log2L, log2L1, c->tw};
-    {
-      Phase ph(c, PH_COL_B, s, outs);
-      if ((e = launch_col(COL_B, a3, s)) != cudaSuccess) return cuda_fail(c, e, "col B launch");
-    }
+    const ColArgs a1{d1 ? d1 + j0 : nullptr, cnt, log2L, log2L1, c->tw, o1};
+    const RowArgs a2{d2 ? d2 + j0 : nullptr, cnt, log2L, log2L1, c->tw, o2};
+    const ColArgs a3{d3 ? d3 + j0 : nullptr, cnt, log2L, log2L1, c->tw, o3};
+    enqueue(c, PH_COL_F1, s, outs, "col F1 launch", [=] { return launch_col(COL_F1, a1, s); });
+    enqueue(c, PH_ROW_MID, s, outs, "row launch", [=] { return launch_row(ROW_MID, a2, s); });
+    enqueue(c, PH_COL_B, s, outs, "col B launch", [=] { return launch_col(COL_B, a3, s); });
   }
   return DC_OK;
 }
@@ -712,15 +771,18 @@ dc_status dc_create(dc_ctx** out, int device, size_t budget) {
       (e = cudaMalloc(&c->t4, sizeof(float2) * kT4Size)) != cudaSuccess ||
       (e = cudaMemcpy(c->t4, t4.data(), sizeof(float2) * kT4Size, cudaMemcpyHostToDevice)) !=
           cudaSuccess ||
+      (e = cudaMalloc(&c->poly, dc_ctx::kPolySlots * dc_ctx::kPolyFloats * sizeof(float))) != cudaSuccess ||
       (e = cudaMalloc(&c->err, sizeof(int))) != cudaSuccess ||
       (e = cudaMemset(c->err, 0, sizeof(int))) != cudaSuccess) {
     cudaGetLastError();
     if (c->tw) cudaFree(c->tw);
     if (c->t4) cudaFree(c->t4);
+    if (c->poly) cudaFree(c->poly);
     if (c->err) cudaFree(c->err);
     delete c;
     return DC_ENOMEM;
   }
+  poly_tables(c, 32, 8.0, nullptr);           // the default window's tables
   // a schedule cache named by DC_TUNING_CACHE is loaded when it exists (a
   // missing or unreadable file leaves the built-in rules)
   if (const char* path = getenv("DC_TUNING_CACHE")) {
@@ -744,6 +806,7 @@ dc_status dc_destroy(dc_ctx* c) {
   if (c->items) cudaFree(c->items);
   if (c->tw) cudaFree(c->tw);
   if (c->t4) cudaFree(c->t4);
+  if (c->poly) cudaFree(c->poly);
   if (c->err) cudaFree(c->err);
   delete c;
   return DC_OK;
@@ -840,6 +903,7 @@ dc_status doppler_resample(dc_ctx* c, const dc_c64* x, long long n, dc_c64* y, d
   cudaSetDevice(c->device);
   const double dl = alpha_minus_one(v_r);
   cudaStream_t s = S(stream);
+  Call call(c);
   if ((st = ensure_items(c, items_bytes_for(4)))) return st;
   if (o.mode == DC_WINDOWED || o.mode == DC_FREQCONV) {
     std::vector<RsItem> items(1);
@@ -850,23 +914,18 @@ dc_status doppler_resample(dc_ctx* c, const dc_c64* x, long long n, dc_c64* y, d
     items[0].n_out = (int)n_out;
     split(dl, items[0].dl_hi, items[0].dl_lo);
     split(rotation_rate(o, dl, fs, fc), items[0].rot_hi, items[0].rot_lo);
-    return run_windowed(c, items, o, 0, s);
+    if ((st = run_windowed(c, items, o, 0, s))) return st;
+    return flush(c, s);
   }
   if (o.mode != DC_EXACT_FP32) return fail(c, DC_EINVAL, "single-pulse exact resampling uses FP32");
-  std::vector<ExItem> ex(1);
-  ex[0] = ExItem{};
-  ex[0].x = reinterpret_cast<const float2*>(x);
-  ex[0].y = reinterpret_cast<float2*>(y);
-  split(dl, ex[0].dl_hi, ex[0].dl_lo);
-  split(rotation_rate(o, dl, fs, fc), ex[0].rot_hi, ex[0].rot_lo);
-  const ExItem* dev = nullptr;
-  if ((st = upload(c, ex, 0, s, &dev))) return st;
-  ExArgs a{dev, (int)n, (int)n_out, 1};
+  ExArgs a{nullptr, (int)n, (int)n_out, 1};
+  a.one.x = reinterpret_cast<const float2*>(x);
+  a.one.y = reinterpret_cast<float2*>(y);
+  split(dl, a.one.dl_hi, a.one.dl_lo);
+  split(rotation_rate(o, dl, fs, fc), a.one.rot_hi, a.one.rot_lo);
   exact_far(c, a, 1, std::fabs(dl), 0);
-  Phase ph(c, PH_EXACT, s, n_out);
-  cudaError_t e = launch_exact_fp32(a, 1, s);
-  if (e != cudaSuccess) return cuda_fail(c, e, "exact launch");
-  return DC_OK;
+  enqueue(c, PH_EXACT, s, n_out, "exact launch", [=] { return launch_exact_fp32(a, 1, s); });
+  return flush(c, s);
 }
 
 dc_status iono_correct(dc_ctx* c, const dc_c64* x, long long n, dc_c64* y, double fs, double fc,
@@ -879,6 +938,7 @@ dc_status iono_correct(dc_ctx* c, const dc_c64* x, long long n, dc_c64* y, doubl
   cudaSetDevice(c->device);
   const int log2L = log2_ceil(n);
   const size_t L = (size_t)1 << log2L;
+  Call call(c);
   if ((st = ensure_ws(c, log2L > 12 ? L * sizeof(float2) : 256))) return st;
   if ((st = ensure_items(c, items_bytes_for(8)))) return st;
   std::vector<FftItem> it(1);
@@ -889,7 +949,8 @@ dc_status iono_correct(dc_ctx* c, const dc_c64* x, long long n, dc_c64* y, doubl
   it[0].n_valid = (int)n;
   it[0].n_out = (int)n;
   size_t at = 0;
-  return run_iono_class(c, it, log2L, reinterpret_cast<float2*>(c->ws), 1, at, S(stream));
+  if ((st = run_iono_class(c, it, log2L, reinterpret_cast<float2*>(c->ws), 1, at, S(stream)))) return st;
+  return flush(c, S(stream));
 }
 
 dc_status correct_batch(dc_ctx* c, const dc_c64* in, dc_c64* out, const dc_item* items,
@@ -915,6 +976,7 @@ dc_status correct_batch(dc_ctx* c, const dc_c64* in, dc_c64* out, const dc_item*
   }
   cudaSetDevice(c->device);
   cudaStream_t s = S(stream);
+  Call call(c);
   const float2* X = reinterpret_cast<const float2*>(in);
   float2* Y = reinterpret_cast<float2*>(out);
 
@@ -958,21 +1020,14 @@ dc_status correct_batch(dc_ctx* c, const dc_c64* in, dc_c64* out, const dc_item*
   } else {
     for (int i = 0; i < n_items; ++i) {
       const dc_item& it = items[i];
-      std::vector<ExItem> ex(1);
       const double dl = alpha_minus_one(it.v_r);
-      ex[0] = ExItem{};
-      ex[0].x = X + it.in_off;
-      ex[0].y = reinterpret_cast<float2*>(ws + yoff[i]);
-      split(dl, ex[0].dl_hi, ex[0].dl_lo);
-      split(rotation_rate(o, dl, it.fs, it.fc), ex[0].rot_hi, ex[0].rot_lo);
-      const ExItem* dev = nullptr;
-      if ((st = upload(c, ex, item_at, s, &dev))) return st;
-      item_at += 256;
-      ExArgs a{dev, (int)it.n, (int)(it.n_out ? it.n_out : it.n), 1};
+      ExArgs a{nullptr, (int)it.n, (int)(it.n_out ? it.n_out : it.n), 1};
+      a.one.x = X + it.in_off;
+      a.one.y = reinterpret_cast<float2*>(ws + yoff[i]);
+      split(dl, a.one.dl_hi, a.one.dl_lo);
+      split(rotation_rate(o, dl, it.fs, it.fc), a.one.rot_hi, a.one.rot_lo);
       if (lay.bytes < c->ws_bytes) exact_far(c, a, 1, std::fabs(dl), lay.bytes);
-      Phase ph(c, PH_EXACT, s, a.n_out);
-      cudaError_t e = launch_exact_fp32(a, 1, s);
-      if (e != cudaSuccess) return cuda_fail(c, e, "exact launch");
+      enqueue(c, PH_EXACT, s, a.n_out, "exact launch", [=] { return launch_exact_fp32(a, 1, s); });
     }
   }
   // 2. ionospheric correction per L class; the classes below 4096, with that of
@@ -1008,7 +1063,7 @@ dc_status correct_batch(dc_ctx* c, const dc_c64* in, dc_c64* out, const dc_item*
     float2* T = reinterpret_cast<float2*>(ws + class_T[m]);
     if ((st = run_iono_class(c, fi, m, T, class_chunk[m], item_at, s))) return st;
   }
-  return DC_OK;
+  return flush(c, s);
 }
 
 }  // extern "C"
@@ -1067,39 +1122,27 @@ dc_status run_spectra(dc_ctx* c, std::vector<FftItem>& sp, int log2L, float2* T,
   const size_t L = (size_t)1 << log2L;
   long long samples = 0;
   for (auto& f : sp) samples += f.n_valid;
-  const FftItem* dev = nullptr;
   dc_status st;
-  cudaError_t e;
   if (use_fused(c, log2L)) {
-    if ((st = upload(c, sp, item_at, s, &dev))) return st;
-    item_at += (n_sp * sizeof(FftItem) + 255) & ~(size_t)255;
-    FusedArgs a{dev, n_sp, log2L, c->tw, c->err, c->t4};
-    Phase ph(c, PH_FUSED_SPEC, s, samples);
-    if ((e = launch_fused(FUSED_SPEC, a, s)) != cudaSuccess) return cuda_fail(c, e, "spec launch");
+    FusedArgs a{nullptr, n_sp, log2L, c->tw, c->err, c->t4};
+    if ((st = stage_items(c, sp, item_at, &a.items, &a.one))) return st;
+    enqueue(c, PH_FUSED_SPEC, s, samples, "spec launch", [=] { return launch_fused(FUSED_SPEC, a, s); });
   } else if (!four) {
-    if ((st = upload(c, sp, item_at, s, &dev))) return st;
-    item_at += (n_sp * sizeof(FftItem) + 255) & ~(size_t)255;
-    RowArgs a{dev, n_sp, log2L, 0, c->tw};
-    Phase ph(c, PH_ROW_SPEC, s, samples);
-    if ((e = launch_row(ROW_SPEC, a, s)) != cudaSuccess) return cuda_fail(c, e, "spec launch");
+    RowArgs a{nullptr, n_sp, log2L, 0, c->tw};
+    if ((st = stage_items(c, sp, item_at, &a.items, &a.one))) return st;
+    enqueue(c, PH_ROW_SPEC, s, samples, "spec launch", [=] { return launch_row(ROW_SPEC, a, s); });
   } else {
     std::vector<FftItem> f1 = sp, f2 = sp;
     for (int i = 0; i < n_sp; ++i) {
       f1[i].dst = T + (size_t)i * L;
       f2[i].src = T + (size_t)i * L;
     }
-    if ((st = upload(c, f1, item_at, s, &dev))) return st;
-    item_at += (n_sp * sizeof(FftItem) + 255) & ~(size_t)255;
-    ColArgs a1{dev, n_sp, log2L, log2L - 12, c->tw};
-    {
-      Phase ph(c, PH_COL_F1, s, samples);
-      if ((e = launch_col(COL_F1, a1, s)) != cudaSuccess) return cuda_fail(c, e, "F1 launch");
-    }
-    if ((st = upload(c, f2, item_at, s, &dev))) return st;
-    item_at += (n_sp * sizeof(FftItem) + 255) & ~(size_t)255;
-    RowArgs a2{dev, n_sp, log2L, log2L - 12, c->tw};
-    Phase ph(c, PH_ROW_SPEC, s, samples);
-    if ((e = launch_row(ROW_SPEC, a2, s)) != cudaSuccess) return cuda_fail(c, e, "F2 launch");
+    ColArgs a1{nullptr, n_sp, log2L, log2L - 12, c->tw};
+    RowArgs a2{nullptr, n_sp, log2L, log2L - 12, c->tw};
+    if ((st = stage_items(c, f1, item_at, &a1.items, &a1.one)) || (st = stage_items(c, f2, item_at, &a2.items, &a2.one)))
+      return st;
+    enqueue(c, PH_COL_F1, s, samples, "F1 launch", [=] { return launch_col(COL_F1, a1, s); });
+    enqueue(c, PH_ROW_SPEC, s, samples, "F2 launch", [=] { return launch_row(ROW_SPEC, a2, s); });
   }
   return DC_OK;
 }
@@ -1161,7 +1204,7 @@ dc_status bank_impl(dc_ctx* c, const dc_c64* x, long long n, const dc_c64* rep, 
   float2* Sp = reinterpret_cast<float2*>(ws + s_at);
   float2* T = reinterpret_cast<float2*>(ws + t_at);
   size_t item_at = 0;
-  cudaError_t e;
+  Call call(c);
 
   // 1. resample per v_r
   std::vector<RsItem> rs(n_v);
@@ -1200,15 +1243,17 @@ dc_status bank_impl(dc_ctx* c, const dc_c64* x, long long n, const dc_c64* rep, 
   std::vector<PhaseParams> ph(n_tec);
   for (int t = 0; t < n_tec; ++t) ph[t] = phase_params(fs, fc, tec[t], log2L);
   const PhaseParams* dph = nullptr;
-  if ((st = upload(c, ph, item_at, s, &dph))) return st;
+  if ((st = upload(c, ph, item_at, &dph))) return st;
   item_at += (n_tec * sizeof(PhaseParams) + 255) & ~(size_t)255;
   {
     const size_t total = L * n_tec;
     const int grid = (int)std::min<size_t>((total + 255) / 256, 152 * 16);
-    Phase phs(c, PH_PHASE_TABLE, s, (long long)total);
-    phase_table_kernel<<<grid, 256, 0, s>>>(dph, n_tec, log2L, fused ? 1.0f / (float)L : 1.0f,
-                                            compress ? Sp + (size_t)n_v * L : nullptr, P);
-    if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(c, e, "phase table launch");
+    const float scale = fused ? 1.0f / (float)L : 1.0f;
+    const float2* H = compress ? Sp + (size_t)n_v * L : nullptr;
+    enqueue(c, PH_PHASE_TABLE, s, (long long)total, "phase table launch", [=] {
+      phase_table_kernel<<<grid, 256, 0, s>>>(dph, n_tec, log2L, scale, H, P);
+      return cudaGetLastError();
+    });
   }
   // 4. factors + inverse per (v_r, TEC), in chunks
   if (fused) {
@@ -1225,14 +1270,14 @@ dc_status bank_impl(dc_ctx* c, const dc_c64* x, long long n, const dc_c64* rep, 
       a.scratch = reinterpret_cast<float2*>(ws + q_at);
       a.ctr = reinterpret_cast<int*>(ws + k_at);
       a.chunk = l2_chunk;
-      if ((e = cudaMemsetAsync(a.ctr, 0, (1 + 2 * n_pairs) * sizeof(int), s)) != cudaSuccess)
-        return cuda_fail(c, e, "apply counters");
+      c->todo.emplace_back([=]() -> dc_status {
+        const cudaError_t e = cudaMemsetAsync(a.ctr, 0, (1 + 2 * n_pairs) * sizeof(int), s);
+        return e == cudaSuccess ? DC_OK : cuda_fail(c, e, "apply counters");
+      });
     }
-    Phase ph(c, PH_FUSED_APPLY, s, (long long)n_pairs * n_out);
-    if ((e = launch_fused(FUSED_APPLY, a, s)) != cudaSuccess) return cuda_fail(c, e, "apply launch");
-    return DC_OK;
+    enqueue(c, PH_FUSED_APPLY, s, (long long)n_pairs * n_out, "apply launch", [=] { return launch_fused(FUSED_APPLY, a, s); });
+    return flush(c, s);
   }
-  const FftItem* dev = nullptr;
   std::vector<FftItem> ap(n_pairs);
   for (int i = 0; i < n_v; ++i)
     for (int t = 0; t < n_tec; ++t) {
@@ -1245,11 +1290,10 @@ dc_status bank_impl(dc_ctx* c, const dc_c64* x, long long n, const dc_c64* rep, 
       f.n_out = (int)n_out;
     }
   if (!four) {
-    if ((st = upload(c, ap, item_at, s, &dev))) return st;
-    RowArgs a{dev, (int)n_pairs, log2L, 0, c->tw};
-    Phase ph(c, PH_ROW_APPLY, s, (long long)n_pairs * n_out);
-    if ((e = launch_row(ROW_APPLY, a, s)) != cudaSuccess) return cuda_fail(c, e, "apply launch");
-    return DC_OK;
+    RowArgs a{nullptr, (int)n_pairs, log2L, 0, c->tw};
+    if ((st = stage_items(c, ap, item_at, &a.items, &a.one))) return st;
+    enqueue(c, PH_ROW_APPLY, s, (long long)n_pairs * n_out, "apply launch", [=] { return launch_row(ROW_APPLY, a, s); });
+    return flush(c, s);
   }
   std::vector<FftItem> ra = ap, cb = ap;
   for (size_t j = 0; j < n_pairs; ++j) {
@@ -1258,23 +1302,16 @@ dc_status bank_impl(dc_ctx* c, const dc_c64* x, long long n, const dc_c64* rep, 
     cb[j].src = Tj;
   }
   const FftItem *dra = nullptr, *dcb = nullptr;
-  if ((st = upload(c, ra, item_at, s, &dra))) return st;
-  item_at += (n_pairs * sizeof(FftItem) + 255) & ~(size_t)255;
-  if ((st = upload(c, cb, item_at, s, &dcb))) return st;
+  FftItem ora{}, ocb{};
+  if ((st = stage_items(c, ra, item_at, &dra, &ora)) || (st = stage_items(c, cb, item_at, &dcb, &ocb))) return st;
   for (size_t j0 = 0; j0 < n_pairs; j0 += chunk) {
     const int cnt = (int)std::min<size_t>(chunk, n_pairs - j0);
-    RowArgs a{dra + j0, cnt, log2L, log2L - 12, c->tw};
-    {
-      Phase ph(c, PH_ROW_APPLY, s, (long long)cnt * n_out);
-      if ((e = launch_row(ROW_APPLY, a, s)) != cudaSuccess) return cuda_fail(c, e, "apply launch");
-    }
-    ColArgs b{dcb + j0, cnt, log2L, log2L - 12, c->tw};
-    {
-      Phase ph(c, PH_COL_B, s, (long long)cnt * n_out);
-      if ((e = launch_col(COL_B, b, s)) != cudaSuccess) return cuda_fail(c, e, "B launch");
-    }
+    const RowArgs a{dra ? dra + j0 : nullptr, cnt, log2L, log2L - 12, c->tw, ora};
+    const ColArgs b{dcb ? dcb + j0 : nullptr, cnt, log2L, log2L - 12, c->tw, ocb};
+    enqueue(c, PH_ROW_APPLY, s, (long long)cnt * n_out, "apply launch", [=] { return launch_row(ROW_APPLY, a, s); });
+    enqueue(c, PH_COL_B, s, (long long)cnt * n_out, "B launch", [=] { return launch_col(COL_B, b, s); });
   }
-  return DC_OK;
+  return flush(c, s);
 }
 
 }  // namespace
@@ -1333,21 +1370,14 @@ extern "C" dc_status correct_compress(dc_ctx* c, const dc_c64* x, long long n,
   float2* P = reinterpret_cast<float2*>(ws + p_at);
   float2* T = reinterpret_cast<float2*>(ws + t_at);
   size_t item_at = 0;
-  cudaError_t e;
+  Call call(c);
   // 1. resampling
   if (o.mode == DC_EXACT_FP32) {
-    std::vector<ExItem> ex(1);
-    ex[0] = ExItem{};
-    ex[0].x = reinterpret_cast<const float2*>(x);
-    ex[0].y = Yr;
-    split(dl, ex[0].dl_hi, ex[0].dl_lo);
-    split(rotation_rate(o, dl, fs, fc), ex[0].rot_hi, ex[0].rot_lo);
-    const ExItem* dev = nullptr;
-    if ((st = upload(c, ex, item_at, s, &dev))) return st;
-    item_at += 256;
-    ea.items = dev;
-    Phase ph(c, PH_EXACT, s, n_out);
-    if ((e = launch_exact_fp32(ea, 1, s)) != cudaSuccess) return cuda_fail(c, e, "exact launch");
+    ea.one.x = reinterpret_cast<const float2*>(x);
+    ea.one.y = Yr;
+    split(dl, ea.one.dl_hi, ea.one.dl_lo);
+    split(rotation_rate(o, dl, fs, fc), ea.one.rot_hi, ea.one.rot_lo);
+    enqueue(c, PH_EXACT, s, n_out, "exact launch", [=] { return launch_exact_fp32(ea, 1, s); });
   } else {
     std::vector<RsItem> rs(1);
     rs[0] = RsItem{};
@@ -1371,13 +1401,14 @@ extern "C" dc_status correct_compress(dc_ctx* c, const dc_c64* x, long long n,
   // 3. factors exp(-i phi_k) conj(H_k) in the spectrum layout
   std::vector<PhaseParams> ph(1, phase_params(fs, fc, tec, log2L));
   const PhaseParams* dph = nullptr;
-  if ((st = upload(c, ph, item_at, s, &dph))) return st;
+  if ((st = upload(c, ph, item_at, &dph))) return st;
   item_at += 256;
   {
     const int grid = (int)std::min<size_t>((L + 255) / 256, 152 * 16);
-    Phase phs(c, PH_PHASE_TABLE, s, (long long)L);
-    phase_table_kernel<<<grid, 256, 0, s>>>(dph, 1, log2L, 1.0f, H, P);
-    if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(c, e, "factor table launch");
+    enqueue(c, PH_PHASE_TABLE, s, (long long)L, "factor table launch", [=] {
+      phase_table_kernel<<<grid, 256, 0, s>>>(dph, 1, log2L, 1.0f, H, P);
+      return cudaGetLastError();
+    });
   }
   // 4. forward transform, factors, inverse transform, first n_out lags
   std::vector<FftItem> it(1);
@@ -1388,7 +1419,8 @@ extern "C" dc_status correct_compress(dc_ctx* c, const dc_c64* x, long long n,
   it[0].ph = ph[0];
   it[0].n_valid = (int)n_out;
   it[0].n_out = (int)n_out;
-  return run_iono_class(c, it, log2L, T, 1, item_at, s);
+  if ((st = run_iono_class(c, it, log2L, T, 1, item_at, s))) return st;
+  return flush(c, s);
 }
 
 extern "C" dc_status predistort_lfm(dc_ctx* c, dc_c64* y, long long n, double fs, double f0,
@@ -1461,7 +1493,8 @@ extern "C" dc_status resample_exact_batch(dc_ctx* c, const dc_c64* x, long long 
     std::vector<float> dl(2 * (size_t)n_alpha);
     for (int i = 0; i < n_alpha; ++i) split(alpha_minus_one(v_r[i]), dl[2 * i], dl[2 * i + 1]);
     const float* ddl = nullptr;
-    if ((st = upload(c, dl, 0, s, &ddl))) return st;
+    Call call(c);
+    if ((st = upload(c, dl, 0, &ddl)) || (st = flush(c, s))) return st;
     ExTcArgs a{(int)n, (int)n_out, n_pulses, stride ? 2 * n_pulses : 0,
                reinterpret_cast<float2*>(y), ddl, c->err};
     Phase ph(c, PH_EXACT_TC, s, (long long)n_alpha * n_pulses * n_out);
@@ -1478,17 +1511,16 @@ extern "C" dc_status resample_exact_batch(dc_ctx* c, const dc_c64* x, long long 
     ex[i].y = reinterpret_cast<float2*>(y) + (size_t)i * n_pulses * n_out;
     split(alpha_minus_one(v_r[i]), ex[i].dl_hi, ex[i].dl_lo);
   }
-  const ExItem* dev = nullptr;
-  if ((st = upload(c, ex, 0, s, &dev))) return st;
-  ExArgs a{dev, (int)n, (int)n_out, n_pulses};
+  Call call(c);
+  ExArgs a{nullptr, (int)n, (int)n_out, n_pulses};
+  size_t at = 0;
+  if ((st = stage_items(c, ex, at, &a.items, &a.one))) return st;
   a.shared = stride == 0;
   double delta_max = 0.0;
   for (int i = 0; i < n_alpha; ++i) delta_max = std::max(delta_max, std::fabs(alpha_minus_one(v_r[i])));
   exact_far(c, a, n_alpha, delta_max, 0);
-  Phase ph(c, PH_EXACT, s, (long long)n_alpha * n_pulses * n_out);
-  cudaError_t e = launch_exact_fp32(a, n_alpha, s);
-  if (e != cudaSuccess) return cuda_fail(c, e, "exact launch");
-  return DC_OK;
+  enqueue(c, PH_EXACT, s, (long long)n_alpha * n_pulses * n_out, "exact launch", [=] { return launch_exact_fp32(a, n_alpha, s); });
+  return flush(c, s);
 }
 
 // ================================================================ plans

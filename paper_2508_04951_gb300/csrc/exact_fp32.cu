@@ -68,7 +68,7 @@ __global__ void __launch_bounds__(kFarBlock, 2) ex_moments_kernel(ExArgs a, int 
   for (long long g = blockIdx.x * 8LL + warp; g < total; g += gridDim.x * 8LL) {
     const long long pr = g / n_pair;
     const int grp = (int)(pr / a.n_pulses);
-    const float2* x = a.items[grp].x + (pr - (long long)grp * a.n_pulses) * a.n_in;
+    const float2* x = ex_item(a, grp).x + (pr - (long long)grp * a.n_pulses) * a.n_in;
     const int m0 = (int)(g - pr * n_pair) * 2 * kFarBlock + 2 * lane;
     float2 v[2][4][2];
 #pragma unroll
@@ -113,7 +113,7 @@ __global__ void __launch_bounds__(4 * PT, (PT <= 32 ? 144 : 192) / PT) ex_tile_k
   __shared__ __align__(16) float2 Xs[kXS][kTK][PT + 2];
   __shared__ float s_D[JOB == EX_NEAR ? kFarP * kFarP : 1];
   const int al = blockIdx.z, n0 = blockIdx.x * kTN, p0 = blockIdx.y * PT;
-  const ExItem I = a.items[al];
+  const ExItem I = ex_item(a, al);
   const int tid = threadIdx.x;
   const int blk = n0 / kFarBlock;
   const int kb = (a.n_in + kFarBlock - 1) / kFarBlock * kFarP;
@@ -308,7 +308,7 @@ DC_DEV void gemv_terms(const float2* __restrict__ x, int n_in, int np, int m, in
 template <int P, int JOB>
 __global__ void __launch_bounds__(256) ex_gemv_kernel(ExArgs a) {
   pdl_release();                        // the kernel that follows may start its set-up
-  const ExItem& I = a.items[blockIdx.y];
+  const ExItem I = ex_item(a, blockIdx.y);
   const int n = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   const int kb = (a.n_in + kFarBlock - 1) / kFarBlock * kFarP;
   const int ob = (a.n_out + kFarBlock - 1) / kFarBlock * kFarP;

@@ -92,7 +92,8 @@ DC_DEV void row_fft(float2* sm, const float2* __restrict__ tw) {
 // shared memory, and items are read by non-coherent loads: otherwise every load
 // waits behind the store before it (a class of L <= 2048 took 20 us so).
 template <int M, int OP>
-DC_DEV void row_pass(float2* sm, const FftItem* items, int n_items, int block, const float2* __restrict__ tw) {
+DC_DEV void row_pass(float2* sm, const FftItem* items, const FftItem& one, int n_items, int block,
+                     const float2* __restrict__ tw) {
   constexpr int LINES = RowShape<M>::LINES;
   constexpr int LP = M + (M >> 4) + 1;
   constexpr int PER = (LINES * M + kThreads - 1) / kThreads;   // elements per thread
@@ -106,7 +107,7 @@ DC_DEV void row_pass(float2* sm, const FftItem* items, int n_items, int block, c
     const int g = line0 + idx / M, p = idx % M;
     v[q] = make_float2(0.f, 0.f);
     if (g < n_items) {
-      const FftItem I = ldg_item(items + g);
+      const FftItem I = items ? ldg_item(items + g) : one;
       if (OP == ROW_APPLY || p < I.n_valid) v[q] = I.src[p];
       if (OP == ROW_APPLY) {
         // the table is in the spectrum's own layout (natural below 4096)
@@ -130,7 +131,7 @@ DC_DEV void row_pass(float2* sm, const FftItem* items, int n_items, int block, c
       const int idx = threadIdx.x + kThreads * q;
       const int c = idx / M, p = idx % M;
       if (line0 + c < n_items) {
-        const FftItem I = ldg_item(items + line0 + c);
+        const FftItem I = items ? ldg_item(items + line0 + c) : one;
         float2 w = make_float2(1.f, 0.f);
         if (I.ptab) w = __ldg(I.ptab + (M == 4096 ? spec_index(p) : p));
         else if (I.ph.enabled) w = iono_factor(I.ph, p);
@@ -148,7 +149,7 @@ DC_DEV void row_pass(float2* sm, const FftItem* items, int n_items, int block, c
     const int idx = threadIdx.x + kThreads * q;
     const int c = idx / M, p = idx % M;
     if (line0 + c >= n_items) continue;
-    const FftItem I = ldg_item(items + line0 + c);
+    const FftItem I = items ? ldg_item(items + line0 + c) : one;
     const float2 x = sm[c * LP + rpad(p)];
     if (OP == ROW_SPEC) I.dst[p] = x;
     else if (p < I.n_out) __stcs(I.dst + p, cscale(x, 1.0f / (float)M));
@@ -158,7 +159,7 @@ DC_DEV void row_pass(float2* sm, const FftItem* items, int n_items, int block, c
 template <int M, int OP>
 __global__ void __launch_bounds__(kThreads) row_kernel(RowArgs a) {
   extern __shared__ float2 sm[];
-  row_pass<M, OP>(sm, a.items, a.n_items, blockIdx.x, a.tw);
+  row_pass<M, OP>(sm, a.items, a.one, a.n_items, blockIdx.x, a.tw);
 }
 
 // Short transforms of several length classes in one launch: run one after the
@@ -166,7 +167,8 @@ __global__ void __launch_bounds__(kThreads) row_kernel(RowArgs a) {
 // chain of about 20 us on a few CTAs).
 template <int M>
 DC_DEV void class_pass(float2* sm, const RowClasses& a, int m) {
-  row_pass<M, ROW_FULL>(sm, a.items + a.first[m], a.first[m + 1] - a.first[m], blockIdx.x - a.block[m], a.tw);
+  row_pass<M, ROW_FULL>(sm, a.items ? a.items + a.first[m] : nullptr, a.one, a.first[m + 1] - a.first[m],
+                        blockIdx.x - a.block[m], a.tw);
 }
 __global__ void __launch_bounds__(kThreads) row_classes_kernel(const __grid_constant__ RowClasses a) {
   extern __shared__ float2 sm[];
@@ -186,7 +188,8 @@ __global__ void __launch_bounds__(kThreads) row_classes_kernel(const __grid_cons
     case 10: class_pass<1024>(sm, a, m); break;
     case 11: class_pass<2048>(sm, a, m); break;
     default:
-      full_4096<false>(ldg_item(a.items + a.first[12] + blockIdx.x - a.block[12]), sm, threadIdx.x, a.tw);
+      full_4096<false>(a.items ? ldg_item(a.items + a.first[12] + blockIdx.x - a.block[12]) : a.one, sm,
+                       threadIdx.x, a.tw);
   }
 }
 
@@ -252,7 +255,7 @@ __global__ void __launch_bounds__(kThreads) col_kernel_smem(ColArgs a) {
   const int cta_per_item = L2 / C;
   const int it = blockIdx.x / cta_per_item;
   const int col0 = (blockIdx.x % cta_per_item) * C;
-  const FftItem& I = a.items[it];
+  const FftItem I = item_of(a, it);
   const float invL = 1.0f / (float)(1 << a.log2L);
 
   // all of a thread's loads first (the global source may not be proven
@@ -306,7 +309,7 @@ __global__ void __launch_bounds__(kThreads) col_kernel_reg(ColArgs a) {
   const int cta_per_item = L2 / kThreads;
   const int it = blockIdx.x / cta_per_item;
   const int n2 = (blockIdx.x % cta_per_item) * kThreads + threadIdx.x;
-  const FftItem& I = a.items[it];
+  const FftItem I = item_of(a, it);
   float2 v[M];
 #pragma unroll
   for (int p = 0; p < M; ++p) {

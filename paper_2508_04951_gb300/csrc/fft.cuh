@@ -68,12 +68,15 @@ enum ColOp : int {
   COL_B = 1,      // inverse last pass, from T to out (1/L, n < n_out)
 };
 
+// Items of a launch: an array on the device or, null, the one item in the
+// arguments themselves (a single transform: no upload, no load).
 struct RowArgs {
   const FftItem* items;
   int n_items;
   int log2L;       // transform length
   int log2L1;      // rows per transform (0 for L <= 4096)
   const float2* tw;
+  FftItem one;
 };
 // The full correction (ROW_FULL) of several length classes L = 2^m, m <= 12, in
 // one launch: class m's transforms are items [first[m], first[m + 1]), its CTAs
@@ -82,6 +85,7 @@ struct RowClasses {
   const FftItem* items;
   int first[14], block[14];
   const float2* tw;
+  FftItem one;
 };
 struct ColArgs {
   const FftItem* items;
@@ -89,7 +93,9 @@ struct ColArgs {
   int log2L;
   int log2L1;      // column length M = L1
   const float2* tw;
+  FftItem one;
 };
+template <class A> DC_DEV FftItem item_of(const A& a, int i) { return a.items ? a.items[i] : a.one; }
 
 // Launchers (fft.cu).  Return cudaSuccess or the launch error.
 cudaError_t launch_row(int op, const RowArgs& a, cudaStream_t s);

@@ -20,7 +20,7 @@ template <int CL> DC_DEV void cluster_wait() {
 // Transform p of a FUSED_APPLY launch: from the item list, or formed from
 // the grid description (FusedArgs::grid_src).
 DC_DEV FftItem apply_item(const FusedArgs& a, int p) {
-  if (!a.grid_src) return a.items[p];
+  if (!a.grid_src) return item_of(a, p);
   FftItem I = {};
   const int i = p / a.grid_n_tec, t = p - i * a.grid_n_tec;
   const size_t L = (size_t)1 << a.log2L;
@@ -47,7 +47,7 @@ __global__ void __launch_bounds__(kRowThreads, 4) spec_kernel(FusedArgs a) {
   extern __shared__ __align__(128) float2 sm[];
   float2* A = sm;                               // [kRowPitch] received row, row FFT buffer
   const int k1 = L1 > 1 ? (int)cg::this_cluster().block_rank() : 0;
-  const FftItem I = a.items[blockIdx.x >> LOG2L1];
+  const FftItem I = item_of(a, blockIdx.x >> LOG2L1);
   const int j = threadIdx.x;
   float2 v[16];
   if constexpr (L1 == 1) {
@@ -436,7 +436,7 @@ __global__ void __launch_bounds__(kRowThreads, LOG2L1 == 0 ? 2 : 4) full_kernel(
   float2* A = sm;                               // [kRowPitch] received row, row FFTs,
   float2* R = sm;                               // then [L1][COLS] received inverse rows
   const int k1 = L1 > 1 ? (int)cg::this_cluster().block_rank() : 0;
-  const FftItem I = a.items[blockIdx.x >> LOG2L1];
+  const FftItem I = item_of(a, blockIdx.x >> LOG2L1);
   const int j = threadIdx.x;
   if constexpr (L1 == 1) {
     full_4096<true>(I, A, j, a.tw);
@@ -548,7 +548,7 @@ __global__ void __launch_bounds__(kRowThreads, 4) row_4096_kernel(RowArgs a) {
   extern __shared__ __align__(128) float2 sm[];
   const int L1 = 1 << a.log2L1;
   const int g = blockIdx.x;
-  const FftItem I = a.items[g >> a.log2L1];
+  const FftItem I = item_of(a, g >> a.log2L1);
   const int k1 = g & (L1 - 1);
   const int j = threadIdx.x;
   const GlobalTw tw{a.tw};

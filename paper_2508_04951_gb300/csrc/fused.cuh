@@ -64,6 +64,7 @@ struct FusedArgs {
   // item has a factor table, so that everything the kernel reads from the
   // kernel before it -- the resampled input -- is read after pdl_wait).
   int pdl;
+  FftItem one;            // with items null: the single transform
 };
 
 // Four-step twiddle rows for L1 = 2, 4, 8, 16: log2(L1) rows of 4096 per L1.

@@ -51,6 +51,7 @@ DC_DEV float tap_weight(const RsArgs& a, float e, float s_e, int k) {
 // Every lane of the warp calls it and gets the answer.
 DC_DEV int find_item(const RsArgs& a, int tile) {
   const int lane = threadIdx.x & 31;
+  if (!a.items) return 0;
   int lo = 0, hi = a.n_items;                  // items[lo].tile_begin <= tile < items[hi]
   while (hi - lo > 1) {
     const int step = (hi - lo + 31) >> 5;
@@ -73,7 +74,7 @@ __global__ void __launch_bounds__(kRsThreads) resample_direct_kernel(RsArgs a) {
     if (threadIdx.x == 0) s_item = it;
   }
   __syncthreads();
-  const RsItem& I = a.items[s_item];
+  const RsItem I = rs_item(a, s_item);
   const int o0 = (tile - I.tile_begin) * kRsTile;
   for (int q = 0; q < kRsTile / kRsThreads; ++q) {
     const int i = o0 + q * kRsThreads + threadIdx.x;
@@ -110,7 +111,7 @@ __global__ void __launch_bounds__(kRsThreads) freqconv_kernel(RsArgs a) {
     if (threadIdx.x == 0) s_item = it;
   }
   __syncthreads();
-  const RsItem& I = a.items[s_item];
+  const RsItem I = rs_item(a, s_item);
   const int o0 = (tile - I.tile_begin) * kRsTile;
 #pragma unroll
   for (int q = 0; q < kRsTile / kRsThreads; ++q) {
@@ -201,7 +202,7 @@ __global__ void __launch_bounds__(kRsTile >> LQ) resample_tiled_kernel(RsArgs a)
   if (threadIdx.x < 32) {
     const int it = find_item(a, tile);
     if (threadIdx.x == 0) {
-      const RsItem& J = a.items[it];
+      const RsItem J = rs_item(a, it);
       const int p0 = (tile - J.tile_begin) * kRsTile;
       int flA, flB;
       float eA, eB;
@@ -241,7 +242,7 @@ __global__ void __launch_bounds__(kRsTile >> LQ) resample_tiled_kernel(RsArgs a)
     }
   }
   __syncthreads();
-  const RsItem& I = a.items[s_geo[0]];
+  const RsItem I = rs_item(a, s_geo[0]);
   const int o0 = (tile - I.tile_begin) * kRsTile;
   const int wlo = s_geo[1], t0 = s_geo[2], t1 = s_geo[3], sh = s_geo[4];
   if (s_geo[5]) {

@@ -32,7 +32,9 @@ struct RsArgs {
   // (fitted per tap in FP64 on the host; |error| <= 6e-8 for beta <= 20).
   const float* wpoly;
   int* err;            // device error flag (bounded waits)
+  RsItem one;          // with items null: the single pulse (no upload, no search)
 };
+DC_DEV RsItem rs_item(const RsArgs& a, int i) { return a.items ? a.items[i] : a.one; }
 
 // One alpha of an exact-sinc launch (config: n_pulses pulses share alpha).
 struct ExItem {
@@ -50,7 +52,9 @@ struct ExArgs {
   // the same pulses (`shared`), else one per alpha.
   float2 *mom, *loc;
   int shared;
+  ExItem one;          // with items null: the single alpha
 };
+DC_DEV ExItem ex_item(const ExArgs& a, int i) { return a.items ? a.items[i] : a.one; }
 // Float2 elements of that scratch for n samples a pulse, and whether a call
 // takes the form at all (delta_max: the largest |alpha - 1|).
 size_t exact_fp32_far_elems(long long pulses, int n);
