@@ -9,14 +9,15 @@
 //  * direct (any alpha): one output per thread, every weight evaluated.  This
 //    is the paper's Algorithm 1 shape and the library's general path.
 //  * tiled (|alpha - 1| <= 0.01, 32 taps): a CTA owns 1024 consecutive outputs;
-//    its input window is staged in shared memory by one TMA bulk copy; each
+//    each warp loads its own slice of the input into shared memory; each
 //    lane owns Q = 8 consecutive outputs (a warp 256) while e moves by at most
 //    0.015 of a sample across a warp tile (|alpha - 1| <= 5.8e-5, |v_r| <=
 //    8.7 km/s), else Q = 4 (|alpha - 1| <= 1.1e-4, |v_r| <= 17 km/s); each tap
 //    weight is then the quadratic through its exact values at the warp tile's
-//    first, middle and last output (error <= 2e-7).  Other warp tiles, and
-//    tiles where floor(delta n) steps, use exact per-output weights read
-//    against the same staged window.
+//    first, middle and last output (error <= 2e-7), with one more tap where
+//    floor(delta n) steps inside the tile.  Other warp tiles use exact
+//    per-output weights read against the same slice (Q = 8 used to take them at
+//    every step: 18.4 instead of 6.2 us for a short pulse).
 #include "resample.cuh"
 
 namespace dc {
@@ -123,11 +124,8 @@ __global__ void __launch_bounds__(kRsThreads) freqconv_kernel(RsArgs a) {
 }
 
 // ------------------------------------------------------------- tiled
-DC_DEV uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
 // Q consecutive outputs per lane (4 or 8): a warp tile is 32 Q outputs and
 // kRsTile / Q threads cover the 1024-output CTA tile.
-constexpr int kWaitLimit = 1 << 22;      // bounded mbarrier polls
 // Largest move of e across a warp tile for the quadratic weights: the
 // interpolation error is about 0.064 |h'''| (span/2)^3 <= 2e-7 per weight.
 constexpr float kQuadSpan = kRsQuadSpan;
@@ -177,6 +175,20 @@ DC_DEV void tap_loop(const float2* __restrict__ w0, const float4* __restrict__ w
   }
 }
 
+// h(e - k) for a tap of a warp tile whose nodes may lie in two unit cells: k is
+// relative to the node's own cell, and the taps just outside its support (k =
+// -R and R + 1) continue the neighbouring tap's window polynomial, so that a
+// tap's quadratic in the position is smooth across the step.
+DC_DEV float tap_weight_ext(const RsArgs& a, float e, float s_e, int k) {
+  const float u = e - (float)k;
+  if (u == 0.f) return 1.f;
+  const float sc = __fdividef((k & 1) ? -s_e : s_e, u);
+  const int t = k + a.half - 1;
+  if (t < 0) return sc * window_at(a.wpoly, 0, e + 1.f);
+  if (t >= 2 * a.half) return sc * window_at(a.wpoly, 2 * a.half - 1, e - 1.f);
+  return sc * window_at(a.wpoly, t, e);
+}
+
 template <int HALF, int LQ>
 __global__ void __launch_bounds__(kRsTile >> LQ) resample_tiled_kernel(RsArgs a) {
   pdl_release();                        // the transform that follows may start its set-up
@@ -185,103 +197,25 @@ __global__ void __launch_bounds__(kRsTile >> LQ) resample_tiled_kernel(RsArgs a)
   constexpr int W = 32 * Q;                // outputs per warp tile
   constexpr int TAPS = 2 * HALF;
   constexpr int NW = NT / 32;
-  constexpr int WINMAX = kRsTile + 2 * HALF + 40;
   constexpr int WWIN = W + TAPS + 3;                   // a warp's slice (|f2 - f0| <= 4)
   constexpr int WSTRIDE = ((WWIN + (WWIN >> LQ) + 1) | 1) + 1;   // even: 16-byte aligned slices
+  constexpr int NLD = (WWIN + 31) / 32;
   static_assert(WSTRIDE >= W, "a slice stages the warp's outputs");
-  __shared__ __align__(16) float2 stage[WINMAX + 2];   // the CTA's window, by TMA
   __shared__ __align__(16) float2 win[NW * WSTRIDE];
-  __shared__ float4 wts[NW][TAPS];
-  __shared__ __align__(8) unsigned long long mbar;
-  __shared__ int s_geo[6];                     // item, wlo, t0, t1, sh, window too long
-  __shared__ int s_done;
+  __shared__ float4 wts[NW][TAPS + 1];
+  __shared__ int s_item;
 
-  // Warp 0 finds the tile's item; its lane 0 sets out the CTA's input window
-  // and starts the TMA copy, alone (nothing in this is needed twice).
   const int tile = blockIdx.x;
-  if (threadIdx.x < 32) {
-    const int it = find_item(a, tile);
-    if (threadIdx.x == 0) {
-      const RsItem J = rs_item(a, it);
-      const int p0 = (tile - J.tile_begin) * kRsTile;
-      int flA, flB;
-      float eA, eB;
-      rs_delay(J.dl_hi, J.dl_lo, (float)p0, flA, eA);
-      rs_delay(J.dl_hi, J.dl_lo, (float)(p0 + kRsTile - 1), flB, eB);
-      const int flmin = min(flA, flB) - 2, flmax = max(flA, flB) + 2;
-      const int lo = p0 + flmin - HALF + 1;
-      const int hi = p0 + kRsTile - 1 + flmax + HALF;
-      const bool too_long = hi - lo + 1 > WINMAX;   // |delta| outside the tiled range
-      // the 16-byte-aligned interior of the valid part, by one bulk copy
-      const int vlo = max(lo, 0), vhi = min(hi, J.n_in - 1);
-      int u0 = vlo, u1 = vhi + 1;
-      if (u1 > u0 && (reinterpret_cast<uintptr_t>(J.x + u0) & 15)) ++u0;
-      if (u1 > u0 && ((u1 - u0) & 1)) --u1;
-      if (u1 < u0) u1 = u0;
-      const int shift = (u0 - lo) & 1;
-      s_geo[0] = it;
-      s_geo[1] = lo;
-      s_geo[2] = u0;
-      s_geo[3] = u1;
-      s_geo[4] = shift;
-      s_geo[5] = too_long;
-      const uint32_t bytes = (uint32_t)(u1 - u0) * 8u;
-      if (!too_long && bytes) {
-        const uint32_t mb = smem_u32(&mbar);
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(mb));
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(mb), "r"(bytes)
-                     : "memory");
-        asm volatile(
-            "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                smem_u32(stage + (u0 - lo + shift))),
-            "l"(J.x + u0), "r"(bytes), "r"(mb)
-            : "memory");
-      }
+  if (a.items) {
+    if (threadIdx.x < 32) {
+      const int it = find_item(a, tile);
+      if (threadIdx.x == 0) s_item = it;
     }
+    __syncthreads();                           // the only one: the warps go their own ways
   }
-  __syncthreads();
-  const RsItem I = rs_item(a, s_geo[0]);
-  const int o0 = (tile - I.tile_begin) * kRsTile;
-  const int wlo = s_geo[1], t0 = s_geo[2], t1 = s_geo[3], sh = s_geo[4];
-  if (s_geo[5]) {
-    if (threadIdx.x == 0) atomicMax(a.err, 2);
-    return;
-  }
-  if (t1 > t0) {
-    // thread 0 waits for the copy (bounded); the others wait at the barrier
-    if (threadIdx.x == 0) {
-      const uint32_t mb = smem_u32(&mbar);
-      uint32_t done = 0;
-      for (int it = 0; it < kWaitLimit && !done; ++it) {
-        asm volatile(
-            "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], 0;\n selp.u32 %0, 1, 0, p;\n}"
-            : "=r"(done)
-            : "r"(mb)
-            : "memory");
-      }
-      if (!done) {
-        atomicMax(a.err, 1);
-        for (int it = 0; it < kWaitLimit && !done; ++it) {   // the copy must land before the exit
-          asm volatile(
-              "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], 0;\n selp.u32 %0, 1, 0, p;\n}"
-              : "=r"(done)
-              : "r"(mb)
-              : "memory");
-        }
-      }
-      s_done = done;
-    }
-    __syncthreads();
-    if (!s_done) return;
-  }
-  // Each warp repacks its own slice of the window -- global positions
-  // G .. G + WWIN - 1, G = ow + min(f0, f2) - HALF + 1 -- into a private,
-  // bank-spread region, so tap offsets are compile-time constants and no CTA
-  // barrier follows; the region then stages the warp's outputs.
+  const RsItem I = rs_item(a, s_item);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int ow = o0 + warp * W;
+  const int ow = (tile - I.tile_begin) * kRsTile + warp * W;
   if (ow >= I.n_out) return;                   // warp-uniform: nothing to write
   constexpr float H = 0.5f * (W - 1);
   // the warp tile's first, centre and last positions: one per lane 0..2
@@ -298,45 +232,76 @@ __global__ void __launch_bounds__(kRsTile >> LQ) resample_tiled_kernel(RsArgs a)
     if (lane == 0) atomicMax(a.err, 2);
     return;
   }
+  // The warp's slice of the input -- positions G .. G + WWIN - 1, zero outside
+  // the pulse -- goes from global memory into a private, bank-spread region of
+  // shared memory (compile-time tap offsets, no CTA barrier; the region then
+  // stages the warp's outputs).  Its loads are in flight while the weights are
+  // formed.  (Staged for the whole CTA by one bulk copy first, as this kernel had
+  // it, the slice waited for the copy, a barrier and a second pass through
+  // shared memory.)
   const int fmin = min(f0, f2);
   const int G = ow + fmin - HALF + 1;
   float2* ww = win + warp * WSTRIDE;
-  for (int i = lane; i < WWIN; i += 32) {
-    const int gi = G + i;
-    float2 v = make_float2(0.f, 0.f);
-    if (gi >= t0 && gi < t1) {
-      if (DC_IN_BOUNDS(gi - wlo + sh >= 0 && gi - wlo + sh < WINMAX + 2, a.err)) v = stage[gi - wlo + sh];
-    } else if (gi >= 0 && gi < I.n_in) {
-      v = __ldg(I.x + gi);
+  float2 ld[NLD];
+#pragma unroll
+  for (int i = 0; i < NLD; ++i) {
+    const int gi = G + lane + 32 * i;
+    ld[i] = (lane + 32 * i < WWIN && gi >= 0 && gi < I.n_in) ? __ldg(I.x + gi) : make_float2(0.f, 0.f);
+  }
+  // Quadratic weights per tap through the three nodes s = -H, 0, +H, taps
+  // counted from the lower of the tile's (at most two) unit cells; a tile across
+  // a step of floor(delta n) has one more tap.
+  const bool step = f0 != f2;
+  const bool quad = abs(f2 - f0) <= 1 && fabsf((e2 - e0) + (float)(f2 - f0)) <= kQuadSpan;
+  if (quad) {
+    const float s0 = __shfl_sync(0xffffffffu, s_l, 0), s1 = __shfl_sync(0xffffffffu, s_l, 1),
+                s2 = __shfl_sync(0xffffffffu, s_l, 2);
+    for (int t = lane; t < TAPS + (step ? 1 : 0); t += 32) {
+      const int k = t - HALF + 1;
+      const float hA = tap_weight_ext(a, e0, s0, k - (f0 - fmin));
+      const float hB = tap_weight_ext(a, e1, s1, k - (f1 - fmin));
+      const float hC = tap_weight_ext(a, e2, s2, k - (f2 - fmin));
+      const float q1 = (hC - hA) * (0.5f / H);
+      const float q2 = (hC - 2.f * hB + hA) * (0.5f / (H * H));
+      wts[warp][t] = make_float4(hB, q1, q2, 2.f * q2);
     }
-    if (DC_IN_BOUNDS(wpad<LQ>(i) < WSTRIDE, a.err)) ww[wpad<LQ>(i)] = v;
+  }
+#pragma unroll
+  for (int i = 0; i < NLD; ++i) {
+    const int p = lane + 32 * i;
+    if (p < WWIN && DC_IN_BOUNDS(wpad<LQ>(p) < WSTRIDE, a.err)) ww[wpad<LQ>(p)] = ld[i];
   }
   __syncwarp();
 
   float2 acc[Q];
 #pragma unroll
   for (int q = 0; q < Q; ++q) acc[q] = make_float2(0.f, 0.f);
-  if (f0 == f2 && f0 == f1 && fabsf(e2 - e0) <= kQuadSpan) {
-    // Quadratic weights per tap through the three nodes s = -H, 0, +H.
-    const float s0 = __shfl_sync(0xffffffffu, s_l, 0), s1 = __shfl_sync(0xffffffffu, s_l, 1),
-                s2 = __shfl_sync(0xffffffffu, s_l, 2);
-    for (int t = lane; t < TAPS; t += 32) {
-      const int k = t - HALF + 1;
-      const float hA = tap_weight(a, e0, s0, k);
-      const float hB = tap_weight(a, e1, s1, k);
-      const float hC = tap_weight(a, e2, s2, k);
-      const float q1 = (hC - hA) * (0.5f / H);
-      const float q2 = (hC - 2.f * hB + hA) * (0.5f / (H * H));
-      wts[warp][t] = make_float4(hB, q1, q2, 2.f * q2);
-    }
-    __syncwarp();
+  if (quad) {
     // Output ow + Q lane + q at tap t reads slice position Q lane + q + t,
     // padded (Q + 1) lane + m + (m >> log2 Q) with m = q + t.
     const float sl = (float)(lane * Q) + 0.5f * (float)(Q - 1) - H;   // the lane's centre
     tap_loop<TAPS, LQ>(ww + (Q + 1) * lane, wts[warp], sl, acc);
+    if (step) {
+      // outputs in the upper cell: the lowest tap has left their support,
+      // one more has entered it
+      const float4 w0 = wts[warp][0], w1 = wts[warp][TAPS];
+#pragma unroll
+      for (int q = 0; q < Q; ++q) {
+        int fl;
+        float e;
+        rs_delay(I.dl_hi, I.dl_lo, (float)(ow + lane * Q + q), fl, e);
+        if (fl != fmin) {
+          const float s = (float)(lane * Q + q) - H;
+          const float h0 = fmaf(fmaf(w0.z, s, w0.y), s, w0.x), h1 = fmaf(fmaf(w1.z, s, w1.y), s, w1.x);
+          const float2 x0 = ww[wpad<LQ>(lane * Q + q)], x1 = ww[wpad<LQ>(lane * Q + q + TAPS)];
+          acc[q].x = fmaf(x1.x, h1, fmaf(-x0.x, h0, acc[q].x));
+          acc[q].y = fmaf(x1.y, h1, fmaf(-x0.y, h0, acc[q].y));
+        }
+      }
+    }
   } else {
-    // floor(delta n) steps inside this warp tile, or e moves too far:
-    // exact weights per output.
+    // floor(delta n) steps more than once inside this warp tile, or e moves
+    // too far: exact weights per output.
 #pragma unroll
     for (int q = 0; q < Q; ++q) {
       const int i = ow + lane * Q + q;
