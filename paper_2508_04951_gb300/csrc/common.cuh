@@ -221,6 +221,19 @@ template <int N> DC_DEV void apply_powers(float2 (&v)[N], const float2 (&b)[4]) 
   for (int q = 1; q < N; ++q) v[q] = cmul(v[q], p[q]);
 }
 
+// v[q] *= w0 w^q, q = 0 .. 15, bases as above: w0 goes into the bases' first
+// products (five more complex multiplies instead of sixteen).
+DC_DEV void apply_powers_from(float2 (&v)[16], float2 w0, const float2 (&b)[4]) {
+  float2 p[16];
+  p[0] = w0;
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int q = 0; q < (1 << i); ++q) p[(1 << i) + q] = cmul(b[i], p[q]);
+#pragma unroll
+  for (int q = 0; q < 16; ++q) v[q] = cmul(v[q], p[q]);
+}
+
 // --------------------------------------------------------------- twiddles
 // One device table of roots of unity, filled once per context in FP64 on the
 // host and rounded to float (fill_twiddles in twiddle_host.h):

@@ -194,80 +194,31 @@ __global__ void __launch_bounds__(kThreads) row_classes_kernel(const __grid_cons
 }
 
 // ------------------------------------------------------------ column pass
-// C = 4096 / M columns per CTA (32 KiB of shared memory for every M, and
-// 256 butterflies per radix-16 stage), element p of column c at sm[p*C + c];
-// consecutive threads take consecutive columns, so global rows of C complex
-// are read and written whole.
-template <int M> __host__ __device__ constexpr int col_width() { return 4096 / M; }
-
-template <int M, int R, int NS, int DIR>
-DC_DEV void col_stage(float2* sm, const float2* __restrict__ tw) {
-  constexpr int C = col_width<M>();
-  constexpr int NB = M / R;
-  constexpr int TOTAL = NB * C;
-  constexpr int PER = (TOTAL + kThreads - 1) / kThreads;
-  float2 v[PER][R];
-#pragma unroll
-  for (int q = 0; q < PER; ++q) {
-    const int b = threadIdx.x + kThreads * q;
-    if (TOTAL % kThreads == 0 || b < TOTAL) {
-      const int c = b % C, j = b / C;
-#pragma unroll
-      for (int r = 0; r < R; ++r) v[q][r] = sm[(j + r * NB) * C + c];
-      if constexpr (NS > 1) {
-        const int k = j % NS;
-#pragma unroll
-        for (int r = 1; r < R; ++r)
-          v[q][r] = cmul(v[q][r], tw_m<DIR>(tw, (r * k) * (4096 / (NS * R))));
-      }
-      dft<R, DIR>(v[q]);
-    }
-  }
-  __syncthreads();
-#pragma unroll
-  for (int q = 0; q < PER; ++q) {
-    const int b = threadIdx.x + kThreads * q;
-    if (TOTAL % kThreads == 0 || b < TOTAL) {
-      const int c = b % C, j = b / C;
-      const int k = j % NS;
-      const int base = (j / NS) * NS * R + k;
-#pragma unroll
-      for (int r = 0; r < R; ++r) sm[(base + r * NS) * C + c] = v[q][r];
-    }
-  }
-  __syncthreads();
-}
-
-template <int M, int DIR, int S = 0>
-DC_DEV void col_fft(float2* sm, const float2* __restrict__ tw) {
-  if constexpr (S < n_stages<M>()) {
-    col_stage<M, stage_radix<M>(S), stage_ns<M>(S), DIR>(sm, tw);
-    col_fft<M, DIR, S + 1>(sm, tw);
-  }
-}
-
-// Column pass for M = L1 in [32, 256] (shared memory).
+// Column pass for M = L1 in [32, 256]: M = 16 x R, R = M / 16.  A CTA takes C =
+// 4096 / M columns (32 KiB of shared memory for every M); consecutive threads take
+// consecutive columns, so global rows of C complex are read and written whole.
+// Thread (column c, p0 < R) loads rows p0 + R q straight into the radix-16
+// butterfly they form, exchanges once through shared memory (element p of column
+// c at sm[p*C + c]) and runs 16 / R butterflies of radix R, whose outputs again
+// are rows p0 + R i: four trips through the load/store path per element, which
+// bounds this pass (with both stages and the transfers through shared memory it
+// took eight, at 85 % of that path: 128 pulses of 2^18, forward 106 us, inverse 79).
 template <int M, int OP>
 __global__ void __launch_bounds__(kThreads) col_kernel_smem(ColArgs a) {
-  constexpr int C = col_width<M>();
-  __shared__ float2 sm[M * C];
+  constexpr int C = 4096 / M, R = M / 16, NB = 16 / R;
+  __shared__ float2 sm[4096];
   const int L2 = 1 << (a.log2L - a.log2L1);
   const int cta_per_item = L2 / C;
   const int it = blockIdx.x / cta_per_item;
   const int col0 = (blockIdx.x % cta_per_item) * C;
   const FftItem I = item_of(a, it);
-  const float invL = 1.0f / (float)(1 << a.log2L);
-
-  // all of a thread's loads first (the global source may not be proven
-  // apart from shared memory, which would serialise load/store pairs)
-  constexpr int PER = M * C / kThreads;
+  constexpr int DIR = OP == COL_F1 ? -1 : +1;
   const int c = threadIdx.x % C, p0 = threadIdx.x / C;
-  constexpr int PSTEP = kThreads / C;
   const int n2 = col0 + c;
-  float2 v[PER];
+  float2 v[16];
 #pragma unroll
-  for (int q = 0; q < PER; ++q) {
-    const int p = p0 + PSTEP * q;
+  for (int q = 0; q < 16; ++q) {
+    const int p = p0 + R * q;
     if (OP == COL_F1) {
       const int n = n2 + L2 * p;
       v[q] = n < I.n_valid ? __ldg(I.src + n) : make_float2(0.f, 0.f);
@@ -275,29 +226,38 @@ __global__ void __launch_bounds__(kThreads) col_kernel_smem(ColArgs a) {
       v[q] = __ldg(I.src + (size_t)p * L2 + n2);
     }
   }
+  dft16<DIR>(v);
 #pragma unroll
-  for (int q = 0; q < PER; ++q) sm[(p0 + PSTEP * q) * C + c] = v[q];
+  for (int r = 0; r < 16; ++r) sm[(16 * p0 + r) * C + c] = v[r];
   __syncthreads();
-  col_fft<M, OP == COL_F1 ? -1 : +1>(sm, a.tw);
 #pragma unroll
-  for (int q = 0; q < PER; ++q) v[q] = sm[(p0 + PSTEP * q) * C + c];
+  for (int q = 0; q < NB; ++q) {
+    const int k = p0 + R * q;                  // butterfly k: rows k + 16 r
+    float2 u[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) u[r] = sm[(k + 16 * r) * C + c];
+#pragma unroll
+    for (int r = 1; r < R; ++r) u[r] = cmul(u[r], tw_m<DIR>(a.tw, r * k * (4096 / M)));
+    dft<R, DIR>(u);
+#pragma unroll
+    for (int r = 0; r < R; ++r) v[q + NB * r] = u[r];   // row k + 16 r = p0 + R (q + NB r)
+  }
   if (OP == COL_F1) {
-    // twiddle W_L^(n2 k1), k1 = p0 + PSTEP q: W_L^(n2 p0) times the q-th
-    // power of W_L^(n2 PSTEP) (powers from the table values for 1, 2, 4, 8)
-    static_assert(PER == 16, "16 rows per thread");
+    // twiddle W_L^(n2 k1), k1 = p0 + R i: W_L^(n2 p0) times the i-th power of
+    // W_L^(n2 R) (powers from the table values for 1, 2, 4, 8)
     const uint32_t mask = (1u << a.log2L) - 1;
     float2 b[4];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) b[i] = tw_big<-1>(a.tw, (uint32_t)(n2 * (PSTEP << i)) & mask, a.log2L);
-    const float2 w0 = tw_big<-1>(a.tw, (uint32_t)(n2 * p0) & mask, a.log2L);
-    apply_powers<PER>(v, b);
+    for (int i = 0; i < 4; ++i) b[i] = tw_big<-1>(a.tw, (uint32_t)(n2 * (R << i)) & mask, a.log2L);
+    apply_powers_from(v, tw_big<-1>(a.tw, (uint32_t)(n2 * p0) & mask, a.log2L), b);
 #pragma unroll
-    for (int q = 0; q < PER; ++q) I.dst[(size_t)(p0 + PSTEP * q) * L2 + n2] = cmul(v[q], w0);
+    for (int i = 0; i < 16; ++i) I.dst[(size_t)(p0 + R * i) * L2 + n2] = v[i];
   } else {
+    const float invL = 1.0f / (float)(1 << a.log2L);
 #pragma unroll
-    for (int q = 0; q < PER; ++q) {
-      const int n = n2 + L2 * (p0 + PSTEP * q);
-      if (n < I.n_out) __stcs(I.dst + n, cscale(v[q], invL));
+    for (int i = 0; i < 16; ++i) {
+      const int n = n2 + L2 * (p0 + R * i);
+      if (n < I.n_out) __stcs(I.dst + n, cscale(v[i], invL));
     }
   }
 }
@@ -412,7 +372,7 @@ static cudaError_t launch_col_m(const ColArgs& a, cudaStream_t s) {
     const long long grid = (long long)a.n_items * (L2 / kThreads);
     col_kernel_reg<M, OP><<<(unsigned)grid, kThreads, 0, s>>>(a);
   } else {
-    const long long grid = (long long)a.n_items * (L2 / col_width<M>());
+    const long long grid = (long long)a.n_items * (L2 / (4096 / M));
     col_kernel_smem<M, OP><<<(unsigned)grid, kThreads, 0, s>>>(a);
   }
   return cudaGetLastError();

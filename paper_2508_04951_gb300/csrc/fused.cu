@@ -571,20 +571,20 @@ __global__ void __launch_bounds__(kRowThreads, 4) row_4096_kernel(RowArgs a) {
     return;
   }
   bin_factors(I, k1, a.log2L1, j, v);
-  row_inverse<false>(v, sm, j, tw);
   if (OP == ROW_APPLY && L1 == 1) {
+    row_inverse<false>(v, sm, j, tw);
     const float invL = 1.0f / (float)kRowN;
 #pragma unroll
     for (int r = 0; r < 16; ++r)
       if (j + 256 * r < I.n_out) __stcs(dst + j + 256 * r, cscale(v[r], invL));
     return;
   }
-  if (k1) {
-    const float2 a_j = tw_big<+1>(a.tw, (uint32_t)(j * k1), a.log2L);
-    const int m16 = 16 * L1 - 1, step = 256 >> a.log2L1;
+  // four-step twiddle W_L^(-k1 (j + 256 r)): the thread's own W_L^(-k1 j) inside
+  // the row, the CTA's W_(16 L1)^(-k1 r) after it
+  row_inverse<false, true>(v, sm, j, tw, tw_big<+1>(a.tw, (uint32_t)(j * k1), a.log2L));
+  const int m16 = 16 * L1 - 1, step = 256 >> a.log2L1;
 #pragma unroll
-    for (int r = 0; r < 16; ++r) v[r] = cmul(v[r], cmul(a_j, tw_m<+1>(a.tw, ((r * k1) & m16) * step)));
-  }
+  for (int r = 1; r < 16; ++r) v[r] = cmul(v[r], tw_m<+1>(a.tw, ((r * k1) & m16) * step));
 #pragma unroll
   for (int r = 0; r < 16; ++r) dst[j + 256 * r] = v[r];
 }

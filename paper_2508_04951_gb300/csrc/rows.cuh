@@ -100,8 +100,10 @@ DC_DEV void row_forward(float2 (&v)[16], float2* b, int j, const TW& tw) {
 
 // ARRIVE: arrive at the cluster barrier (release) once this thread's last read
 // of b is done: peers may overwrite the buffer after their wait.
-template <bool ARRIVE, class TW>
-DC_DEV void row_inverse(float2 (&v)[16], float2* b, int j, const TW& tw) {
+// FROM: the outputs of thread j also take the factor from (a thread's own
+// constant, folded into the last twiddle).
+template <bool ARRIVE, bool FROM = false, class TW>
+DC_DEV void row_inverse(float2 (&v)[16], float2* b, int j, const TW& tw, float2 from = float2{1.f, 0.f}) {
   const int s = j >> 4, t = j & 15;
   float2 w[4];
   tw.s2(w, t);
@@ -125,7 +127,8 @@ DC_DEV void row_inverse(float2 (&v)[16], float2* b, int j, const TW& tw) {
   for (int q = 0; q < 16; ++q) v[q] = b[pad16(256 * q + j)];
   if constexpr (ARRIVE) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
   orient<+1>(w);
-  apply_powers<16>(v, w);                                  // W4096^(-q s), q = j
+  if constexpr (FROM) apply_powers_from(v, from, w);       // W4096^(-q s), q = j
+  else apply_powers<16>(v, w);
   dft16<+1>(v);                                            // over s
 }
 
