@@ -43,6 +43,15 @@ DC_DEV float exact_i2f(int i) {
   return __int_as_float(i + 0x4B400000) - 12582912.0f;
 }
 
+// a / b to 2 ulp for normal b and quotient (the reciprocal instruction and one
+// product; without the flush of subnormals CUDA's __fdividef rescales around
+// them, four more instructions in loops that divide once per term).
+DC_DEV float fast_div(float a, float b) {
+  float r;
+  asm("div.approx.ftz.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+  return r;
+}
+
 // ------------------------------------------- programmatic dependent launch
 // A kernel launched with the programmatic-serialization attribute may start
 // while the kernel before it in the stream is still running; pdl_wait()

@@ -48,7 +48,7 @@ template <int JOB> DC_DEV ExRow ex_row(const ExItem& I, int n) {
 // 1 / (tau - s_j) of blocks b and B, s = the source node, zero for near blocks.
 DC_DEV float node_weight(const ExRow& r, int B, float s) {
   const int db = r.mn - B;
-  return db < -1 || db > 1 ? __fdividef(1.f, (float)(db * kFarBlock) + r.e - s) : 0.f;
+  return db < -1 || db > 1 ? fast_div(1.f, (float)(db * kFarBlock) + r.e - s) : 0.f;
 }
 
 // ------------------------------------------------------------- moments
@@ -175,7 +175,7 @@ __global__ void __launch_bounds__(4 * PT, (PT <= 32 ? 144 : 192) / PT) ex_tile_k
           // (m_n - m) exactly, then + e; samples past n_in are zero, their
           // weights finite; e = 0 (sigma = 0) leaves weight 1 at m = m_n alone
           const float den = (d0 - (float)(KS * r)) + row.e;
-          w = __fdividef((KS * r) & 1 ? -sgk : sgk, den);
+          w = fast_div((KS * r) & 1 ? -sgk : sgk, den);
           if (den == 0.f) w = 1.f;
         }
         Ss[c & 1][k][on] = make_float2(w, w);
@@ -263,32 +263,30 @@ __global__ void __launch_bounds__(4 * PT, (PT <= 32 ? 144 : 192) / PT) ex_tile_k
 // computed once per (n, m) and applied to every pulse, lanes combined by a fixed
 // shuffle tree (deterministic).
 // One lane's share of the sum: terms m = lo + lane, + 32, ... (FAST: m_n - m
-// converted by exact_i2f, valid for |m_n - m| < 2^22).  Four terms per round:
-// their weights, then their loads, issued together so that a warp has four
-// loads in flight instead of one (the kernel is bound by the load latency);
+// converted by exact_i2f, valid for |m_n - m| < 2^22).  A round's loads are
+// issued together, ahead of its weights (the kernel is bound by their latency);
 // the terms are still added in the order m = lo + lane, + 32, ...
 template <bool FAST> DC_DEV float gemv_weight(int mn, int m, float e, float sgl) {
   const float den = (FAST ? exact_i2f(mn - m) : (float)(mn - m)) + e;
-  return __fdividef(sgl, den);
+  return fast_div(sgl, den);
 }
 template <int P, class W>
 DC_DEV void gemv_terms(const float2* __restrict__ x, int n_in, int np, int m, int hi, W&& weight,
                        float2 (&acc)[P]) {
-  for (; m + 96 < hi; m += 128) {
-    float w[4];
+  constexpr int U = P <= 2 ? 8 : 4;                    // loads of a pulse in flight
+  for (; m + 32 * (U - 1) < hi; m += 32 * U) {
+    float2 xv[P][U];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) w[u] = weight(m + 32 * u);
+    for (int p = 0; p < P; ++p)
 #pragma unroll
-    for (int p = 0; p < P; ++p) {
-      if (p < np) {
-        float2 xv[4];
+      for (int u = 0; u < U; ++u) xv[p][u] = __ldg(x + (size_t)min(p, np - 1) * n_in + m + 32 * u);
 #pragma unroll
-        for (int u = 0; u < 4; ++u) xv[u] = __ldg(x + (size_t)p * n_in + m + 32 * u);
+    for (int u = 0; u < U; ++u) {
+      const float w = weight(m + 32 * u);
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          acc[p].x = fmaf(xv[u].x, w[u], acc[p].x);
-          acc[p].y = fmaf(xv[u].y, w[u], acc[p].y);
-        }
+      for (int p = 0; p < P; ++p) {
+        acc[p].x = fmaf(xv[p][u].x, w, acc[p].x);
+        acc[p].y = fmaf(xv[p][u].y, w, acc[p].y);
       }
     }
   }

@@ -340,22 +340,20 @@ __global__ void __launch_bounds__(kThreads, 1)
           const bool live = db < -a.near || db > a.near;
 #pragma unroll
           for (int i = 0; i < 8; ++i)
-            v[i] = live ? __fdividef(kCauchyScale, c - s_far[(m0 + i) % kFarP]) : 0.f;
+            v[i] = live ? fast_div(kCauchyScale, c - s_far[(m0 + i) % kFarP]) : 0.f;
         } else {
         // (m_n - m) + e_n with the integer part formed exactly first
         // ((m_n - m0) - i, integers below 2^22) and e_n added last, so the
         // denominator near m = m_n is e_n itself even when e_n is far below
         // the rounding unit of m_n - m0
+        // (samples past n_in are zero in X: their weights only need to be finite)
         const float di0 = exact_i2f(mn - m0);
+        if (en != 0.f) {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          const int m = m0 + i;
-          float val = 0.f;
-          if (m < a.n_in) {
-            if (en == 0.f) val = (m == mn) ? 1.f : 0.f;
-            else val = __fdividef((i & 1) ? -sg : sg, (di0 - (float)i) + en);
-          }
-          v[i] = val;
+          for (int i = 0; i < 8; ++i) v[i] = fast_div((i & 1) ? -sg : sg, (di0 - (float)i) + en);
+        } else {
+#pragma unroll
+          for (int i = 0; i < 8; ++i) v[i] = m0 + i == mn ? 1.f : 0.f;
         }
         }
         // (-1)^m: m = kc*32 + k8*8 + i has the parity of i

@@ -40,7 +40,7 @@ DC_DEV float iono_cycles(const PhaseParams& P, float kt) {
   const float fl = __fadd_rn(fmaf(P.d_lo, kt, p.lo), __fadd_rn(fe, P.fc_lo));
   // C / f = q1 + q2: q1 to a couple of ulps, the remainder C - q1 f formed
   // exactly, its quotient q2 to float accuracy relative to itself
-  const float rb = __fdividef(1.f, fh);
+  const float rb = fast_div(1.f, fh);
   const float q1 = __fmul_rn(P.c_hi, rb);
   float r = fmaf(-q1, fh, P.c_hi);
   r = fmaf(-q1, fl, __fadd_rn(r, P.c_lo));

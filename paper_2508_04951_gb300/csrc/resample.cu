@@ -42,7 +42,7 @@ DC_DEV float window_at(const float* __restrict__ wp, int t, float e) {
 DC_DEV float tap_weight(const RsArgs& a, float e, float s_e, int k) {
   const float u = e - (float)k;
   if (u == 0.f) return 1.f;
-  const float sc = __fdividef((k & 1) ? -s_e : s_e, u);
+  const float sc = fast_div((k & 1) ? -s_e : s_e, u);
   return sc * window_at(a.wpoly, k + a.half - 1, e);
 }
 
@@ -182,7 +182,7 @@ DC_DEV void tap_loop(const float2* __restrict__ w0, const float4* __restrict__ w
 DC_DEV float tap_weight_ext(const RsArgs& a, float e, float s_e, int k) {
   const float u = e - (float)k;
   if (u == 0.f) return 1.f;
-  const float sc = __fdividef((k & 1) ? -s_e : s_e, u);
+  const float sc = fast_div((k & 1) ? -s_e : s_e, u);
   const int t = k + a.half - 1;
   if (t < 0) return sc * window_at(a.wpoly, 0, e + 1.f);
   if (t >= 2 * a.half) return sc * window_at(a.wpoly, 2 * a.half - 1, e - 1.f);
