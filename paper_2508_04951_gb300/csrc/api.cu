@@ -134,11 +134,14 @@ bool apply_rows2(const dc_ctx* c, int log2L) { return log2L >= 15 && c->tune.app
 bool apply_l2(const dc_ctx* c, int log2L) {
   return log2L >= 13 && (c->tune.apply_kind == 3 || (c->tune.apply_kind == 0 && log2L == 16));
 }
-// Transforms per chunk of the two-pass apply: 8 MiB of them (256 row tasks),
-// so that the scratch (kApplyL2Slots chunks, 32 MiB) stays in L2 beside the
-// spectra and factor tables.
+// Transforms per chunk of the two-pass apply: 12 MiB of them (384 row tasks), so
+// that the scratch (kApplyL2Slots chunks, 48 MiB) stays in L2 beside the spectra
+// and factor tables.  Measured on the 256 x 16 bank at L = 65536, chunk MiB x
+// slots: 2 x 6: 2250 us, 4 x 6: 1432, 8 x 4: 1087, 12 x 4: 1048, 16 x 3: 1057, 16 x
+// 4: 1117, 32 x 3: 1238 (short blocks of rows and columns alternate more often;
+// long ones leave L2).
 int apply_l2_chunk(int log2L, size_t n_pairs) {
-  const size_t per = (size_t)8 << 20 >> (log2L + 3);
+  const size_t per = (size_t)12 << 20 >> (log2L + 3);
   return (int)std::max<size_t>(1, std::min(per, n_pairs));
 }
 

@@ -22,12 +22,17 @@
 namespace dc {
 
 // Order of the bins of a 4096-point row in stored spectra and factor tables: bin
-// k2 = s + 16 a + 256 r (nibbles r, a, s) at index 256 s + 16 r + a.  Thread
-// (s, a) of a row transform holds exactly those 16 bins (r = 0..15) after the
-// forward row and before the inverse one, so both read and write them straight
-// from registers.  Rows below 4096 points keep natural order.
-__host__ __device__ constexpr int spec_index(int k2) { return ((k2 & 15) << 8) | (k2 >> 4); }
-__host__ __device__ constexpr int spec_bin(int idx) { return ((idx & 255) << 4) | (idx >> 8); }
+// k2 = s + 16 a + 256 r (nibbles r, a, s) at index 256 s + 32 (r / 2) + 2 a + r % 2.
+// Thread (s, a) of a row transform holds exactly those 16 bins (r = 0..15) after
+// the forward row and before the inverse one, so both read and write them
+// straight from registers, two bins per 16-byte access.  Rows below 4096 points
+// keep natural order.
+__host__ __device__ constexpr int spec_index(int k2) {
+  return ((k2 & 15) << 8) | ((k2 >> 9) << 5) | (((k2 >> 4) & 15) << 1) | ((k2 >> 8) & 1);
+}
+__host__ __device__ constexpr int spec_bin(int idx) {
+  return (idx >> 8) | (((idx >> 1) & 15) << 4) | ((idx & 1) << 8) | (((idx >> 5) & 7) << 9);
+}
 
 // One transform of a launch.  64 bytes: read whole by four 16-byte loads (ldg_item).
 struct alignas(16) FftItem {

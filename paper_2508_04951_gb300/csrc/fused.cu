@@ -84,8 +84,7 @@ __global__ void __launch_bounds__(kRowThreads, 4) spec_kernel(FusedArgs a) {
     for (int r = 0; r < 16; ++r) v[r] = A[pad16(j + 256 * r)];
   }
   row_forward(v, A, j, GlobalTw{a.tw});
-#pragma unroll
-  for (int r = 0; r < 16; ++r) I.dst[(size_t)k1 * kRowN + spec_pos(j, r)] = v[r];
+  store_bins(I.dst + (size_t)k1 * kRowN, j, v);
 }
 
 template <int LOG2L1>
@@ -148,12 +147,8 @@ __global__ void __launch_bounds__(kRowThreads << LOG2G, 4 >> LOG2G) apply_kernel
   const int k1 = rank * G + h;
   float2* A = sm + h * kRowPitch;               // this row's buffer
   float2 v[16];
-  const float2* srow = I.src + (size_t)k1 * kRowN;
-  const float2* prow = I.ptab + (size_t)k1 * kRowN;
-#pragma unroll
-  for (int r = 0; r < 16; ++r) v[r] = __ldg(srow + spec_pos(jj, r));
-#pragma unroll
-  for (int r = 0; r < 16; ++r) v[r] = cmul(v[r], __ldg(prow + spec_pos(jj, r)));
+  load_bins(I.src + (size_t)k1 * kRowN, jj, v);
+  mul_bins(I.ptab + (size_t)k1 * kRowN, jj, v);
   row_inverse<(L1 > 1)>(v, A, jj, GlobalTw{a.tw});   // arrives at the cluster barrier
 
   if constexpr (L1 == 1) {
@@ -350,12 +345,8 @@ __global__ void __launch_bounds__(kRowThreads, 4) apply_l2_kernel(FusedArgs a) {
       I.n_out = T.n_out;
       if (!is_col) {
         float2 v[16];
-        const float2* srow = I.src + (size_t)rq * kRowN;
-        const float2* prow = I.ptab + (size_t)rq * kRowN;
-#pragma unroll
-        for (int r = 0; r < 16; ++r) v[r] = __ldg(srow + spec_pos(j, r));
-#pragma unroll
-        for (int r = 0; r < 16; ++r) v[r] = cmul(v[r], __ldg(prow + spec_pos(j, r)));
+        load_bins(I.src + (size_t)rq * kRowN, j, v);
+        mul_bins(I.ptab + (size_t)rq * kRowN, j, v);
         // the slot is free: the row's CTA barrier orders thread 0's wait
         // before every thread's stores (the others poll nothing)
         if (j == 0 && T.prev >= 0) wait_count(col_done + T.prev, L1, a.err);
@@ -556,8 +547,7 @@ __global__ void __launch_bounds__(kRowThreads, 4) row_4096_kernel(RowArgs a) {
   float2* dst = I.dst + (size_t)k1 * kRowN;
   float2 v[16];
   if constexpr (OP == ROW_APPLY) {
-#pragma unroll
-    for (int r = 0; r < 16; ++r) v[r] = __ldg(src + spec_pos(j, r));
+    load_bins(src, j, v);
   } else {
     // the zero-padded input itself when a row is the whole transform (L = 4096)
     const int valid = OP == ROW_SPEC && L1 == 1 ? I.n_valid : kRowN;
@@ -566,8 +556,7 @@ __global__ void __launch_bounds__(kRowThreads, 4) row_4096_kernel(RowArgs a) {
     row_forward(v, sm, j, tw);
   }
   if constexpr (OP == ROW_SPEC) {
-#pragma unroll
-    for (int r = 0; r < 16; ++r) dst[spec_pos(j, r)] = v[r];
+    store_bins(dst, j, v);
     return;
   }
   bin_factors(I, k1, a.log2L1, j, v);

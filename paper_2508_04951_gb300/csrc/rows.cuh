@@ -132,8 +132,32 @@ DC_DEV void row_inverse(float2 (&v)[16], float2* b, int j, const TW& tw, float2 
   dft16<+1>(v);                                            // over s
 }
 
-// Index of thread j's bin r in a stored row (spec_index(s + 16 t + 256 r)).
-DC_DEV int spec_pos(int j, int r) { return ((j >> 4) << 8) + (j & 15) + 16 * r; }
+// A stored row (16-byte aligned) as 16-byte pairs: thread j's bins 2 i, 2 i + 1 are
+// pair spec_pair(j) + 16 i (spec_index).
+DC_DEV int spec_pair(int j) { return ((j >> 4) << 7) + (j & 15); }
+DC_DEV void load_bins(const float2* row, int j, float2 (&v)[16]) {
+  const float4* t = reinterpret_cast<const float4*>(row) + spec_pair(j);
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const float4 q = __ldg(t + 16 * i);
+    v[2 * i] = make_float2(q.x, q.y);
+    v[2 * i + 1] = make_float2(q.z, q.w);
+  }
+}
+DC_DEV void mul_bins(const float2* row, int j, float2 (&v)[16]) {
+  const float4* t = reinterpret_cast<const float4*>(row) + spec_pair(j);
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const float4 q = __ldg(t + 16 * i);
+    v[2 * i] = cmul(v[2 * i], make_float2(q.x, q.y));
+    v[2 * i + 1] = cmul(v[2 * i + 1], make_float2(q.z, q.w));
+  }
+}
+DC_DEV void store_bins(float2* row, int j, const float2 (&v)[16]) {
+  float4* t = reinterpret_cast<float4*>(row) + spec_pair(j);
+#pragma unroll
+  for (int i = 0; i < 8; ++i) t[16 * i] = make_float4(v[2 * i].x, v[2 * i].y, v[2 * i + 1].x, v[2 * i + 1].y);
+}
 
 // v[r] *= the factor of bin k1 + L1 (s + 16 t + 256 r), r = 0..15 (L1 =
 // 2^log2L1): the item's table (exp(-i phi_k) times anything else the call
@@ -141,9 +165,7 @@ DC_DEV int spec_pos(int j, int r) { return ((j >> 4) << 8) + (j & 15) + 16 * r; 
 // replica spectrum) when there is one, else exp(-i phi_k) of Eq. 16.
 DC_DEV void bin_factors(const FftItem& I, int k1, int log2L1, int j, float2 (&v)[16]) {
   if (I.ptab) {
-    const float2* t = I.ptab + (size_t)k1 * kRowN;
-#pragma unroll
-    for (int r = 0; r < 16; ++r) v[r] = cmul(v[r], __ldg(t + spec_pos(j, r)));
+    mul_bins(I.ptab + (size_t)k1 * kRowN, j, v);
   } else if (I.ph.enabled) {
     // bins r >= 8 are the upper half of the transform: kt = k - L
     const PhaseParams& P = I.ph;
