@@ -50,15 +50,18 @@ __global__ void __launch_bounds__(kRowThreads, 4) spec_kernel(FusedArgs a) {
   const FftItem I = item_of(a, blockIdx.x >> LOG2L1);
   const int j = threadIdx.x;
   float2 v[16];
+  pdl_release();                                // the next pass may start its set-up
   if constexpr (L1 == 1) {
+    pdl_wait();                                 // the pulses' producer has finished
 #pragma unroll
     for (int r = 0; r < 16; ++r) {
       const int n = j + 256 * r;
-      v[r] = n < I.n_valid ? __ldg(I.src + n) : make_float2(0.f, 0.f);
+      v[r] = n < I.n_valid ? I.src[n] : make_float2(0.f, 0.f);
     }
   } else {
     asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");   // this CTA runs
     const float2* T = a.t4 + kT4Offset(L1);
+    pdl_wait();                                 // the pulses' producer has finished
 #pragma unroll
     for (int p = 0; p < PER; ++p) {
       const int n2 = k1 * COLS + j + 256 * p;
@@ -66,7 +69,7 @@ __global__ void __launch_bounds__(kRowThreads, 4) spec_kernel(FusedArgs a) {
 #pragma unroll
       for (int n1 = 0; n1 < L1; ++n1) {
         const int n = n2 + kRowN * n1;
-        col[n1] = n < I.n_valid ? __ldg(I.src + n) : make_float2(0.f, 0.f);
+        col[n1] = n < I.n_valid ? I.src[n] : make_float2(0.f, 0.f);   // plain: after pdl_wait
       }
       dft<L1, -1>(col);
       float2 w[4];                              // W_L^(2^b n2), conjugates of the table rows
@@ -104,13 +107,15 @@ cudaError_t launch_spec(const FusedArgs& a, cudaStream_t s) {
   cfg.blockDim = dim3(kRowThreads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = L1;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = a.pdl ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, k, a);
 }
 
@@ -147,6 +152,7 @@ __global__ void __launch_bounds__(kRowThreads << LOG2G, 4 >> LOG2G) apply_kernel
   const int k1 = rank * G + h;
   float2* A = sm + h * kRowPitch;               // this row's buffer
   float2 v[16];
+  pdl_wait();                                   // spectra and factors are written
   load_bins(I.src + (size_t)k1 * kRowN, jj, v);
   mul_bins(I.ptab + (size_t)k1 * kRowN, jj, v);
   row_inverse<(L1 > 1)>(v, A, jj, GlobalTw{a.tw});   // arrives at the cluster barrier
@@ -214,13 +220,15 @@ cudaError_t launch_apply(const FusedArgs& a, cudaStream_t s) {
   cfg.blockDim = dim3(kRowThreads * G);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = CL;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = a.pdl ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, k, a);
 }
 

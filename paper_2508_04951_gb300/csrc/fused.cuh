@@ -60,9 +60,10 @@ struct FusedArgs {
   float2* grid_dst;
   int grid_n_tec;
   int grid_n_out;
-  // FUSED_FULL: launched with programmatic serialization (set only when no
-  // item has a factor table, so that everything the kernel reads from the
-  // kernel before it -- the resampled input -- is read after pdl_wait).
+  // Launched with programmatic serialization (FUSED_FULL: set only when no
+  // item has a factor table; FUSED_SPEC, and FUSED_APPLY on clusters, always
+  // may be): everything the kernel reads from kernels before it is read after
+  // pdl_wait, by plain loads.
   int pdl;
   FftItem one;            // with items null: the single transform
 };

@@ -101,6 +101,10 @@ struct RsTcArgs {
   const float* wpoly;  // 32-tap window polynomials and their first two
                        // derivatives: [tap][3][kWCoef] (w, w', w'' in e)
   int* err;
+  // launched with programmatic serialization behind a kernel whose results it
+  // does not read; it waits for that kernel before it ends, so that work behind
+  // it in the stream finds both done
+  int pdl;
 };
 int rs_tc_max_span();
 cudaError_t launch_resample_tc(const RsTcArgs& a, cudaStream_t s);

@@ -132,14 +132,15 @@ DC_DEV void row_inverse(float2 (&v)[16], float2* b, int j, const TW& tw, float2 
   dft16<+1>(v);                                            // over s
 }
 
-// A stored row (16-byte aligned) as 16-byte pairs: thread j's bins 2 i, 2 i + 1 are
+// A stored row (16-byte aligned; plain loads: it may have been written by the kernel
+// a pdl_wait waited for) as 16-byte pairs: thread j's bins 2 i, 2 i + 1 are
 // pair spec_pair(j) + 16 i (spec_index).
 DC_DEV int spec_pair(int j) { return ((j >> 4) << 7) + (j & 15); }
 DC_DEV void load_bins(const float2* row, int j, float2 (&v)[16]) {
   const float4* t = reinterpret_cast<const float4*>(row) + spec_pair(j);
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
-    const float4 q = __ldg(t + 16 * i);
+    const float4 q = t[16 * i];
     v[2 * i] = make_float2(q.x, q.y);
     v[2 * i + 1] = make_float2(q.z, q.w);
   }
@@ -148,7 +149,7 @@ DC_DEV void mul_bins(const float2* row, int j, float2 (&v)[16]) {
   const float4* t = reinterpret_cast<const float4*>(row) + spec_pair(j);
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
-    const float4 q = __ldg(t + 16 * i);
+    const float4 q = t[16 * i];
     v[2 * i] = cmul(v[2 * i], make_float2(q.x, q.y));
     v[2 * i + 1] = cmul(v[2 * i + 1], make_float2(q.z, q.w));
   }

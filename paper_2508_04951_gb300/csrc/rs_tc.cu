@@ -129,6 +129,7 @@ __global__ void __launch_bounds__(kThreads, 2) rs_tc_kernel(RsTcArgs a) {
   __shared__ __align__(8) unsigned long long mma_bar;
   __shared__ uint32_t tmem_base;
 
+  pdl_release();                             // the transforms that follow may start their set-up
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~(uintptr_t)1023);
   uint8_t* A = smem;
@@ -349,6 +350,7 @@ __global__ void __launch_bounds__(kThreads, 2) rs_tc_kernel(RsTcArgs a) {
       }
     }
   }
+  pdl_wait();                                // see RsTcArgs::pdl
   tc_fence_before();
   __syncthreads();
   if (warp == 1) {
@@ -366,8 +368,17 @@ cudaError_t launch_resample_tc(const RsTcArgs& a, cudaStream_t s) {
   cudaError_t e = cudaFuncSetAttribute(rs_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
   if (e != cudaSuccess) return e;
   dim3 grid((a.n_out + kTile - 1) / kTile, (a.n_slots + kV - 1) / kV);
-  rs_tc_kernel<<<grid, kThreads, kSmem, s>>>(a);
-  return cudaGetLastError();
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = kSmem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = a.pdl ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, rs_tc_kernel, a);
 }
 
 }  // namespace dc
