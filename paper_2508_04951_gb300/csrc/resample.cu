@@ -190,7 +190,7 @@ DC_DEV float tap_weight_ext(const RsArgs& a, float e, float s_e, int k) {
 }
 
 template <int HALF, int LQ>
-__global__ void __launch_bounds__(kRsTile >> LQ) resample_tiled_kernel(RsArgs a) {
+__global__ void __launch_bounds__(kRsTile >> LQ, LQ == 3 ? 8 : 3) resample_tiled_kernel(RsArgs a) {
   pdl_release();                        // the transform that follows may start its set-up
   constexpr int Q = 1 << LQ;
   constexpr int NT = kRsTile / Q;          // threads
@@ -243,10 +243,15 @@ __global__ void __launch_bounds__(kRsTile >> LQ) resample_tiled_kernel(RsArgs a)
   const int G = ow + fmin - HALF + 1;
   float2* ww = win + warp * WSTRIDE;
   float2 ld[NLD];
+  if (G >= 0 && G + 32 * NLD <= I.n_in) {      // all inside the pulse
 #pragma unroll
-  for (int i = 0; i < NLD; ++i) {
-    const int gi = G + lane + 32 * i;
-    ld[i] = (lane + 32 * i < WWIN && gi >= 0 && gi < I.n_in) ? __ldg(I.x + gi) : make_float2(0.f, 0.f);
+    for (int i = 0; i < NLD; ++i) ld[i] = __ldg(I.x + G + lane + 32 * i);
+  } else {
+#pragma unroll
+    for (int i = 0; i < NLD; ++i) {
+      const int gi = G + lane + 32 * i;
+      ld[i] = gi >= 0 && gi < I.n_in ? __ldg(I.x + gi) : make_float2(0.f, 0.f);
+    }
   }
   // Quadratic weights per tap through the three nodes s = -H, 0, +H, taps
   // counted from the lower of the tile's (at most two) unit cells; a tile across
