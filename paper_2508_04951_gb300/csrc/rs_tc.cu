@@ -75,7 +75,7 @@ DC_DEV void sinc_d012(float a, float S, float C, float& s0, float& s1, float& s2
                                                                         z2 * (-1.f / 443520))));
     s2 = kPi * kPi * d2;
   } else {
-    const float ia = 1.f / a;
+    const float ia = fast_div(1.f, a);
     s0 = S * kInvPi * ia;
     s1 = (C - s0) * ia;
     s2 = (-kPi * S - 2.f * s1) * ia;
