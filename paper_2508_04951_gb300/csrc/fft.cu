@@ -215,15 +215,17 @@ __global__ void __launch_bounds__(kThreads) col_kernel_smem(ColArgs a) {
   constexpr int DIR = OP == COL_F1 ? -1 : +1;
   const int c = threadIdx.x % C, p0 = threadIdx.x / C;
   const int n2 = col0 + c;
+  pdl_release();
+  pdl_wait();                                  // plain loads below: they stay behind it
   float2 v[16];
 #pragma unroll
   for (int q = 0; q < 16; ++q) {
     const int p = p0 + R * q;
     if (OP == COL_F1) {
       const int n = n2 + L2 * p;
-      v[q] = n < I.n_valid ? __ldg(I.src + n) : make_float2(0.f, 0.f);
+      v[q] = n < I.n_valid ? I.src[n] : make_float2(0.f, 0.f);
     } else {
-      v[q] = __ldg(I.src + (size_t)p * L2 + n2);
+      v[q] = I.src[(size_t)p * L2 + n2];
     }
   }
   dft16<DIR>(v);
@@ -373,7 +375,22 @@ static cudaError_t launch_col_m(const ColArgs& a, cudaStream_t s) {
     col_kernel_reg<M, OP><<<(unsigned)grid, kThreads, 0, s>>>(a);
   } else {
     const long long grid = (long long)a.n_items * (L2 / (4096 / M));
-    col_kernel_smem<M, OP><<<(unsigned)grid, kThreads, 0, s>>>(a);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3(kThreads);
+    cfg.stream = s;
+    if (a.pdl == PDL_SPREAD) {
+      cfg.dynamicSmemBytes = kPdlColSmem - 4096 * sizeof(float2);
+      cudaError_t e = cudaFuncSetAttribute(col_kernel_smem<M, OP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           (int)cfg.dynamicSmemBytes);
+      if (e != cudaSuccess) return e;
+    }
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = a.pdl ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, col_kernel_smem<M, OP>, a);
   }
   return cudaGetLastError();
 }

@@ -82,6 +82,7 @@ struct RowArgs {
   int log2L1;      // rows per transform (0 for L <= 4096)
   const float2* tw;
   FftItem one;
+  int pdl;         // Pdl, ROW_MID: launched programmatically behind the pass before it
 };
 // The full correction (ROW_FULL) of several length classes L = 2^m, m <= 12, in
 // one launch: class m's transforms are items [first[m], first[m + 1]), its CTAs
@@ -99,7 +100,20 @@ struct ColArgs {
   int log2L1;      // column length M = L1
   const float2* tw;
   FftItem one;
+  int pdl;         // Pdl: launched programmatically behind the pass before it
 };
+// Programmatic launches of the three-pass path's second and third pass, for
+// grids of at most one CTA per SM (`pdl` below): the passes of a single pulse are
+// latency, and each one's launch and set-up then run under the one before.  A pass
+// that starts so is placed where there is room, which piles its CTAs on the few
+// SMs the first has left; above 64 CTAs (PDL_SPREAD) each therefore asks for so much
+// shared memory that two row CTAs never share an SM's 227 KiB, a row and a column
+// CTA do.  iono_correct, us, without / with / with spread: n = 2^17: 16.7 / 12.3 /
+// 12.3; 2^18: 18.2 / 12.9 / 14.3; 2^19: 18.4 / 22.5 / 14.4.
+enum Pdl : int { PDL_NONE = 0, PDL_ON = 1, PDL_SPREAD = 2 };
+constexpr int kPdlColSmem = 100 << 10, kPdlRowSmem = 120 << 10;
+inline int pdl_for(long long ctas) { return ctas <= 64 ? PDL_ON : ctas <= 152 ? PDL_SPREAD : PDL_NONE; }
+
 template <class A> DC_DEV FftItem item_of(const A& a, int i) { return a.items ? a.items[i] : a.one; }
 
 // Launchers (fft.cu).  Return cudaSuccess or the launch error.

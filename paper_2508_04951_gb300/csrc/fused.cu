@@ -554,6 +554,8 @@ __global__ void __launch_bounds__(kRowThreads, 4) row_4096_kernel(RowArgs a) {
   const float2* src = I.src + (size_t)k1 * kRowN;
   float2* dst = I.dst + (size_t)k1 * kRowN;
   float2 v[16];
+  pdl_release();
+  pdl_wait();
   if constexpr (OP == ROW_APPLY) {
     load_bins(src, j, v);
   } else {
@@ -587,12 +589,21 @@ __global__ void __launch_bounds__(kRowThreads, 4) row_4096_kernel(RowArgs a) {
 }
 
 template <int OP> cudaError_t launch_row_4096_op(const RowArgs& a, cudaStream_t s) {
-  const size_t smem = sizeof(float2) * kRowPitch;
+  const size_t smem = a.pdl == PDL_SPREAD ? kPdlRowSmem : sizeof(float2) * kRowPitch;
   auto k = row_4096_kernel<OP>;
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPdlRowSmem);
   if (e != cudaSuccess) return e;
-  k<<<(unsigned)(a.n_items << a.log2L1), kRowThreads, smem, s>>>(a);
-  return cudaGetLastError();
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(a.n_items << a.log2L1));
+  cfg.blockDim = dim3(kRowThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = a.pdl ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, k, a);
 }
 
 }  // namespace
