@@ -156,10 +156,133 @@ DC_DEV void row_pass(float2* sm, const FftItem* items, const FftItem& one, int n
   }
 }
 
+// Transforms of M = 256 A points, A = 1 .. 8, in registers: 16 A threads of 16 points
+// per transform, 16 / A transforms per CTA, one barrier in each direction (the
+// 4096-point rows of rows.cuh are A = 16).  The split n = 16 A p + 16 u + w, k =
+// s + 16 a + 16 A r (u, a < A; p, w, s, r < 16), thread (s, t) of 16 x A:
+//   forward  DFT over p in thread q = 16 u + w, W_M^(q s); exchange; DFT over u (16 / A
+//            of them, w = t + A i); transpose among the A threads of sub-problem s;
+//            W_16A^(w a) in thread a = t; DFT over w
+//   inverse  the mirror image
+// Sub-problem s keeps to its own 17 A elements except in the exchange, whose pitch
+// 17 A puts a half-warp's accesses on 16 different bank pairs throughout.  Against
+// radix-16 stages through shared memory with two barriers each and table loads per
+// element (row_pass) a lone pulse of 2048 takes 6.2 instead of 12.3 us.
+template <int A, int OP>
+DC_DEV void line_pass(float2* sm, const FftItem* items, const FftItem& one, int n_items, int block,
+                      const float2* __restrict__ tw) {
+  constexpr int M = 256 * A, T = 16 * A, P = 17 * A, NI = 16 / A;
+  const int tl = threadIdx.x % T, s = tl / A, t = tl % A;
+  const int g = block * NI + threadIdx.x / T;
+  const bool live = g < n_items;
+  const FftItem I = items ? ldg_item(items + (live ? g : 0)) : one;
+  float2* b = sm + (threadIdx.x / T) * 16 * P;
+  float2* reg = b + s * P;
+  float2 wq[4], wt[4];                          // W_M^(q 2^i), q = tl, and W_16A^(t 2^i)
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    wq[i] = __ldg(tw + (tl << i) * (4096 / M));
+    wt[i] = __ldg(tw + (t << i) * (4096 / T));
+  }
+  float2 v[16];
+  if constexpr (OP == ROW_APPLY) {
+#pragma unroll
+    for (int r = 0; r < 16; ++r) v[r] = live ? I.src[s + 16 * t + T * r] : make_float2(0.f, 0.f);
+  } else {
+#pragma unroll
+    for (int p = 0; p < 16; ++p) {
+      const int n = T * p + tl;
+      v[p] = live && n < I.n_valid ? I.src[n] : make_float2(0.f, 0.f);
+    }
+    dft16<-1>(v);                               // over p
+    apply_powers<16>(v, wq);
+#pragma unroll
+    for (int r = 0; r < 16; ++r) b[r * P + tl] = v[r];
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < NI; ++i) {
+      float2 u[A];
+#pragma unroll
+      for (int k = 0; k < A; ++k) u[k] = reg[16 * k + t + A * i];
+      dft<A, -1>(u);                            // over u
+#pragma unroll
+      for (int k = 0; k < A; ++k) v[i * A + k] = u[k];
+    }
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < NI; ++i)
+#pragma unroll
+      for (int k = 0; k < A; ++k) reg[17 * k + t + A * i] = v[i * A + k];
+    __syncwarp();
+#pragma unroll
+    for (int w = 0; w < 16; ++w) v[w] = reg[17 * t + w];
+    apply_powers<16>(v, wt);
+    dft16<-1>(v);                               // over w: v[r] = X[s + 16 t + T r]
+  }
+  if constexpr (OP == ROW_SPEC) {
+    if (live) {
+#pragma unroll
+      for (int r = 0; r < 16; ++r) I.dst[s + 16 * t + T * r] = v[r];
+    }
+    return;
+  }
+  if (I.ptab) {
+#pragma unroll
+    for (int r = 0; r < 16; ++r) v[r] = cmul(v[r], I.ptab[s + 16 * t + T * r]);
+  } else if (I.ph.enabled) {
+#pragma unroll
+    for (int r = 0; r < 16; ++r)
+      v[r] = cmul(v[r], iono_factor_kt(I.ph, (float)(s + 16 * t + T * (r < 8 ? r : r - 16))));
+  }
+  dft16<+1>(v);                                 // over r
+#pragma unroll
+  for (int i = 0; i < 4; ++i) wq[i] = conj_if<+1>(wq[i]), wt[i] = conj_if<+1>(wt[i]);
+  apply_powers<16>(v, wt);
+  __syncwarp();
+#pragma unroll
+  for (int w = 0; w < 16; ++w) reg[17 * t + w] = v[w];
+  __syncwarp();
+#pragma unroll
+  for (int i = 0; i < NI; ++i) {
+    float2 u[A];
+#pragma unroll
+    for (int k = 0; k < A; ++k) u[k] = reg[17 * k + t + A * i];
+    dft<A, +1>(u);                              // over a
+#pragma unroll
+    for (int k = 0; k < A; ++k) v[i * A + k] = u[k];
+  }
+  __syncwarp();
+#pragma unroll
+  for (int i = 0; i < NI; ++i)
+#pragma unroll
+    for (int k = 0; k < A; ++k) reg[16 * k + t + A * i] = v[i * A + k];
+  __syncthreads();
+#pragma unroll
+  for (int r = 0; r < 16; ++r) v[r] = b[r * P + tl];
+  apply_powers<16>(v, wq);
+  dft16<+1>(v);                                 // over s
+  if (live) {
+#pragma unroll
+    for (int p = 0; p < 16; ++p)
+      if (T * p + tl < I.n_out) __stcs(I.dst + T * p + tl, cscale(v[p], 1.0f / (float)M));
+  }
+}
+
+// The pass of CTA `block` for transforms of M points.
+template <int M, int OP>
+DC_DEV void short_pass(float2* sm, const FftItem* items, const FftItem& one, int n_items, int block, const float2* tw) {
+  if constexpr (M >= 256 && M <= 2048) line_pass<M / 256, OP>(sm, items, one, n_items, block, tw);
+  else row_pass<M, OP>(sm, items, one, n_items, block, tw);
+}
+// Its transforms per CTA and shared memory.
+template <int M> __host__ __device__ constexpr size_t short_smem() {
+  return sizeof(float2) * (M >= 256 && M <= 2048 ? 4352 : RowShape<M>::LINES * (M + (M >> 4) + 1));
+}
+
 template <int M, int OP>
 __global__ void __launch_bounds__(kThreads) row_kernel(RowArgs a) {
   extern __shared__ float2 sm[];
-  row_pass<M, OP>(sm, a.items, a.one, a.n_items, blockIdx.x, a.tw);
+  short_pass<M, OP>(sm, a.items, a.one, a.n_items, blockIdx.x, a.tw);
 }
 
 // Short transforms of several length classes in one launch: run one after the
@@ -167,7 +290,7 @@ __global__ void __launch_bounds__(kThreads) row_kernel(RowArgs a) {
 // chain of about 20 us on a few CTAs).
 template <int M>
 DC_DEV void class_pass(float2* sm, const RowClasses& a, int m) {
-  row_pass<M, ROW_FULL>(sm, a.items ? a.items + a.first[m] : nullptr, a.one, a.first[m + 1] - a.first[m],
+  short_pass<M, ROW_FULL>(sm, a.items ? a.items + a.first[m] : nullptr, a.one, a.first[m + 1] - a.first[m],
                         blockIdx.x - a.block[m], a.tw);
 }
 __global__ void __launch_bounds__(kThreads) row_classes_kernel(const __grid_constant__ RowClasses a) {
@@ -302,8 +425,7 @@ __global__ void __launch_bounds__(kThreads) col_kernel_reg(ColArgs a) {
 template <int M, int OP>
 static cudaError_t launch_row_m(const RowArgs& a, cudaStream_t s) {
   constexpr int LINES = RowShape<M>::LINES;
-  constexpr int LP = M + (M >> 4) + 1;
-  const size_t smem = sizeof(float2) * LINES * LP;
+  const size_t smem = short_smem<M>();
   const long long lines = (long long)a.n_items << a.log2L1;
   const long long grid = (lines + LINES - 1) / LINES;
   if (grid <= 0) return cudaSuccess;
@@ -348,8 +470,9 @@ cudaError_t launch_row_classes(RowClasses a, cudaStream_t s) {
   for (int m = 0; m <= 12; ++m) {
     const int n = a.first[m + 1] - a.first[m];
     a.block[m + 1] = a.block[m] + (n + kLines[m] - 1) / kLines[m];
-    const int M = 1 << m, line = m == 12 ? kRowPitch : M + (M >> 4) + 1;
-    if (n > 0) smem = std::max(smem, sizeof(float2) * kLines[m] * line);
+    const int M = 1 << m;
+    const size_t want = sizeof(float2) * (m >= 8 ? kRowPitch : kLines[m] * (M + (M >> 4) + 1));
+    if (n > 0) smem = std::max(smem, want);
   }
   if (a.block[13] == 0) return cudaSuccess;
   row_classes_kernel<<<(unsigned)a.block[13], kThreads, smem, s>>>(a);
