@@ -52,6 +52,12 @@ DC_DEV float fast_div(float a, float b) {
   return r;
 }
 
+DC_DEV float fast_rcp(float b) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(b));
+  return r;
+}
+
 // ------------------------------------------- programmatic dependent launch
 // A kernel launched with the programmatic-serialization attribute may start
 // while the kernel before it in the stream is still running; pdl_wait()

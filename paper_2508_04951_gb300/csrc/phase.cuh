@@ -4,7 +4,7 @@
 // radians at TEC ~ 1e2 TECU and f ~ 1 GHz, where one float ulp is ~2.4e-4 rad;
 // the double-float path keeps ~48 bits, so the reduced angle is good to float
 // rounding.  Working in cycles makes the reduction two exact subtractions of
-// an integer; a bin costs about 28 instructions with its sincos and product, so
+// an integer; a bin costs 24 to 30 instructions with its sincos and product, so
 // the transform kernels evaluate every bin where it lies in registers (bins
 // 256 rows apart) instead of regrouping runs of neighbours to step the phase
 // from one to the next.
@@ -20,8 +20,12 @@ struct PhaseParams {
   float fc_hi, fc_lo;   // carrier fc                [Hz]; 0 = RF sampling
   float d_hi, d_lo;     // bin spacing fs / L        [Hz]
   int log2L;            // transform length L = 2^log2L
-  int enabled;          // 0 when E == 0 (identity)
+  // 0 when E == 0 (identity).  kPhasePlain where every f_k > 0, |C / f_k| < 2^22
+  // and fc and fs / L are floats exactly (baseband at round frequencies): the
+  // evaluation leaves out the terms that are zero then (same results).
+  int enabled;
 };
+constexpr int kPhasePlain = 2;
 
 // kt of bin k of an L-point DFT (fftfreq order): k below L/2, else k - L.
 DC_DEV float bin_kt(const PhaseParams& P, int k) {
@@ -29,31 +33,33 @@ DC_DEV float bin_kt(const PhaseParams& P, int k) {
   return (float)(k < (L >> 1) ? k : k - L);
 }
 
-// Reduced phase in cycles, in [-1/2, 1/2], at f = fc + (fs/L) kt.  A bin at
+// Reduced phase in cycles, about [-1/2, 1/2], at f = fc + (fs/L) kt.  A bin at
 // f == 0 (DC under RF sampling) gets 0.
-DC_DEV float iono_cycles(const PhaseParams& P, float kt) {
+template <bool PLAIN> DC_DEV float iono_cycles(const PhaseParams& P, float kt) {
   // f = fh + fl: fc is 0 or above fs / 2 >= |d kt|, so the sum's rounding
   // error is exact by one subtraction each way
   const df p = two_prod(P.d_hi, kt);
   const float fh = __fadd_rn(P.fc_hi, p.hi);
   const float fe = __fsub_rn(p.hi, __fsub_rn(fh, P.fc_hi));
-  const float fl = __fadd_rn(fmaf(P.d_lo, kt, p.lo), __fadd_rn(fe, P.fc_lo));
+  const float fl = PLAIN ? __fadd_rn(p.lo, fe)
+                         : __fadd_rn(fmaf(P.d_lo, kt, p.lo), __fadd_rn(fe, P.fc_lo));
   // C / f = q1 + q2: q1 to a couple of ulps, the remainder C - q1 f formed
   // exactly, its quotient q2 to float accuracy relative to itself
-  const float rb = fast_div(1.f, fh);
+  const float rb = fast_rcp(fh);
   const float q1 = __fmul_rn(P.c_hi, rb);
   float r = fmaf(-q1, fh, P.c_hi);
   r = fmaf(-q1, fl, __fadd_rn(r, P.c_lo));
   const float q2 = __fmul_rn(r, rb);
   float x = __fadd_rn(__fsub_rn(q1, rintf(q1)), q2);   // q1 - rint(q1) is exact
+  if constexpr (PLAIN) return x;                       // |q2| below 1/4: within [-3/4, 3/4]
   x = __fsub_rn(x, rintf(x));                          // |q2| passes 1/2 for |C / f| > 2^22
   return fh == 0.f ? 0.f : x;
 }
 
 // Correction factor exp(-i phi) (Eq. 16) at kt, and at bin k.
-DC_DEV float2 iono_factor_kt(const PhaseParams& P, float kt) {
+template <bool PLAIN = false> DC_DEV float2 iono_factor_kt(const PhaseParams& P, float kt) {
   float s, c;
-  __sincosf(iono_cycles(P, kt) * 6.28318530717958648f, &s, &c);
+  __sincosf(iono_cycles<PLAIN>(P, kt) * 6.28318530717958648f, &s, &c);
   return make_float2(c, -s);
 }
 DC_DEV float2 iono_factor(const PhaseParams& P, int k) { return iono_factor_kt(P, bin_kt(P, k)); }

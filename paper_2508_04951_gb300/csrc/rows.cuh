@@ -172,9 +172,15 @@ DC_DEV void bin_factors(const FftItem& I, int k1, int log2L1, int j, float2 (&v)
     const PhaseParams& P = I.ph;
     const float kt0 = (float)(k1 + (((j >> 4) + ((j & 15) << 4)) << log2L1));
     const float step = (float)(256 << log2L1);
+    if (P.enabled == kPhasePlain) {
 #pragma unroll
-    for (int r = 0; r < 16; ++r)
-      v[r] = cmul(v[r], iono_factor_kt(P, fmaf((float)(r < 8 ? r : r - 16), step, kt0)));
+      for (int r = 0; r < 16; ++r)
+        v[r] = cmul(v[r], iono_factor_kt<true>(P, fmaf((float)(r < 8 ? r : r - 16), step, kt0)));
+    } else {
+#pragma unroll
+      for (int r = 0; r < 16; ++r)
+        v[r] = cmul(v[r], iono_factor_kt(P, fmaf((float)(r < 8 ? r : r - 16), step, kt0)));
+    }
   }
 }
 
