@@ -312,7 +312,7 @@ __global__ void __launch_bounds__(kRowThreads, 4) apply_l2_kernel(FusedArgs a) {
   int* row_done = a.ctr + 1;
   int* col_done = a.ctr + 1 + a.n_items;
   const size_t slot_elems = (size_t)L1 * kRowN;
-  // thread 0 decodes each task once (the divisions stay off the other threads)
+  // each task is decoded once (the divisions stay off the other threads)
   auto decode = [&](int t) {
     ApplyTask d = {};
     if (t >= n_tasks) {
@@ -335,13 +335,17 @@ __global__ void __launch_bounds__(kRowThreads, 4) apply_l2_kernel(FusedArgs a) {
     d.prev = d.p >= n_slots ? d.p - n_slots : -1;
     return d;
   };
-  int t_next = 0;                               // thread 0: the task taken ahead
-  if (j == 0) s_ti[0] = decode(atomicAdd(head, 1));
+  // one thread of the last warp takes tasks from the queue, one ahead, and
+  // decodes them while thread 0 counts the finished one: both chains are latency
+  // that the CTA waits for between tasks
+  const bool taker = j == kRowThreads - 32;
+  int t_next = 0;                               // the task taken ahead
+  if (taker) s_ti[0] = decode(atomicAdd(head, 1));
   for (int it = 0;; ++it) {
     __syncthreads();                            // s_ti; the last task's reads of sm are done
     const ApplyTask T = s_ti[it & 1];
     if (T.kind < 0) break;
-    if (j == 0) t_next = atomicAdd(head, 1);    // decoded at the end of this task
+    if (taker) t_next = atomicAdd(head, 1);     // decoded at the end of this task
     const int p = T.p, rq = T.rq;
     if (T.kind > 0 && DC_IN_BOUNDS(rq >= 0 && rq < L1 && p >= 0 && p < a.n_items, a.err)) {
       const bool is_col = T.kind == 2;
@@ -391,7 +395,7 @@ __global__ void __launch_bounds__(kRowThreads, 4) apply_l2_kernel(FusedArgs a) {
         if (j == 0) red_release_gpu(col_done + p, 1);   // every thread's slot reads first
       }
     }
-    if (j == 0) s_ti[(it + 1) & 1] = decode(t_next);
+    if (taker) s_ti[(it + 1) & 1] = decode(t_next);
   }
 }
 
