@@ -147,7 +147,7 @@ template <int LQ> DC_DEV int wpad(int i) { return i + (i >> LQ); }
 // |u de/ds| <= 2.06e-4 at Q = 8 and 1.77e-4 at Q = 4).
 template <int TAPS, int LQ>
 DC_DEV void tap_loop(const float2* __restrict__ w0, const float4* __restrict__ wts,
-                     float sl, float2 (&acc)[1 << LQ]) {
+                     float sl, bool step, unsigned lower, float2 (&acc)[1 << LQ]) {
   constexpr int Q = 1 << LQ;
   float2 xw[Q];
 #pragma unroll
@@ -168,6 +168,12 @@ DC_DEV void tap_loop(const float2* __restrict__ w0, const float4* __restrict__ w
     }
 #pragma unroll
     for (int q = 0; q + 1 < Q; ++q) xw[q] = xw[q + 1];
+    if (t == 0 && step) {
+      // the lowest tap has left the support of the upper cell's outputs
+#pragma unroll
+      for (int q = 0; q < Q; ++q)
+        if (!(lower >> q & 1)) acc[q] = make_float2(0.f, 0.f);
+    }
     if (t + 1 < TAPS) {
       const int m = Q + t;
       xw[Q - 1] = w0[m + (m >> LQ)];
@@ -285,23 +291,28 @@ __global__ void __launch_bounds__(kRsTile >> LQ, LQ == 3 ? 8 : 3) resample_tiled
     // Output ow + Q lane + q at tap t reads slice position Q lane + q + t,
     // padded (Q + 1) lane + m + (m >> log2 Q) with m = q + t.
     const float sl = (float)(lane * Q) + 0.5f * (float)(Q - 1) - H;   // the lane's centre
-    tap_loop<TAPS, LQ>(ww + (Q + 1) * lane, wts[warp], sl, acc);
+    unsigned lower = (1u << Q) - 1;              // outputs in the tile's lower cell
     if (step) {
-      // outputs in the upper cell: the lowest tap has left their support,
-      // one more has entered it
-      const float4 w0 = wts[warp][0], w1 = wts[warp][TAPS];
 #pragma unroll
       for (int q = 0; q < Q; ++q) {
         int fl;
         float e;
         rs_delay(I.dl_hi, I.dl_lo, (float)(ow + lane * Q + q), fl, e);
-        if (fl != fmin) {
-          const float s = (float)(lane * Q + q) - H;
-          const float h0 = fmaf(fmaf(w0.z, s, w0.y), s, w0.x), h1 = fmaf(fmaf(w1.z, s, w1.y), s, w1.x);
-          const float2 x0 = ww[wpad<LQ>(lane * Q + q)], x1 = ww[wpad<LQ>(lane * Q + q + TAPS)];
-          acc[q].x = fmaf(x1.x, h1, fmaf(-x0.x, h0, acc[q].x));
-          acc[q].y = fmaf(x1.y, h1, fmaf(-x0.y, h0, acc[q].y));
-        }
+        if (fl != fmin) lower &= ~(1u << q);
+      }
+    }
+    tap_loop<TAPS, LQ>(ww + (Q + 1) * lane, wts[warp], sl, step, lower, acc);
+    if (step) {
+      // ... and one more tap has entered it
+      const float4 w1 = wts[warp][TAPS];
+#pragma unroll
+      for (int q = 0; q < Q; ++q) {
+        if (lower >> q & 1) continue;
+        const float s = (float)(lane * Q + q) - H;
+        const float h1 = fmaf(fmaf(w1.z, s, w1.y), s, w1.x);
+        const float2 x1 = ww[wpad<LQ>(lane * Q + q + TAPS)];
+        acc[q].x = fmaf(x1.x, h1, acc[q].x);
+        acc[q].y = fmaf(x1.y, h1, acc[q].y);
       }
     }
   } else {
