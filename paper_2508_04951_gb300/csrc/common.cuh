@@ -82,6 +82,25 @@ DC_DEV df two_prod(float a, float b) {
   float p = __fmul_rn(a, b);
   return {p, fmaf(a, b, -p)};
 }
+// delta * fi = fl + e with fl integer and e in [0, 1), fi a float holding an
+// integer or half-integer output position (exact), delta a double-float.
+DC_DEV void rs_delay(float dl_hi, float dl_lo, float fi, int& fl, float& e) {
+  df p = two_prod(dl_hi, fi);
+  const float lo = fmaf(dl_lo, fi, p.lo);
+  float f = floorf(p.hi);
+  float r = __fadd_rn(__fsub_rn(p.hi, f), lo);      // p.hi - f is exact
+  if (r < 0.f) {
+    r = __fadd_rn(r, 1.f);
+    f -= 1.f;
+    if (r >= 1.f) { r = 0.f; f += 1.f; }
+  } else if (r >= 1.f) {
+    r = __fsub_rn(r, 1.f);
+    f += 1.f;
+  }
+  fl = (int)f;
+  e = r < 0x1p-100f ? 0.f : r;             // fast_div's weights need a normal fraction, or none
+}
+
 // exp(2 pi i g n) for a rotation rate g (cycles per sample) held as the
 // double-float g_hi + g_lo and an output index n < 2^24: g n is formed as a
 // double-float (two_prod, exact for the high part), its integer part removed

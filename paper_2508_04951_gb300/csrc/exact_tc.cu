@@ -136,21 +136,8 @@ template <bool FP16> DC_DEV float join1(uint16_t hi, uint16_t lo) {
 
 // a n = m_n + e_n with a - 1 a double-float (same arithmetic as the FP32 path).
 DC_DEV void position(float dl_hi, float dl_lo, int n, int& m, float& e) {
-  const float fi = (float)n;
-  df p = two_prod(dl_hi, fi);
-  const float lo = fmaf(dl_lo, fi, p.lo);
-  float f = floorf(p.hi);
-  float r = __fadd_rn(__fsub_rn(p.hi, f), lo);
-  if (r < 0.f) {
-    r = __fadd_rn(r, 1.f);
-    f -= 1.f;
-    if (r >= 1.f) { r = 0.f; f += 1.f; }
-  } else if (r >= 1.f) {
-    r = __fsub_rn(r, 1.f);
-    f += 1.f;
-  }
-  m = n + (int)f;
-  e = r;
+  rs_delay(dl_hi, dl_lo, (float)n, m, e);
+  m += n;
 }
 
 // Powers of two that keep the 16-bit moments and node values inside fp16's

@@ -60,25 +60,6 @@ DC_DEV ExItem ex_item(const ExArgs& a, int i) { return a.items ? a.items[i] : a.
 size_t exact_fp32_far_elems(long long pulses, int n);
 bool exact_fp32_far(int n_in, int n_out, int n_pulses, int n_alpha, double delta_max);
 
-// delta * fi = fl + e with fl integer and e in [0, 1), fi a float holding an
-// integer or half-integer output position (exact), delta a double-float.
-DC_DEV void rs_delay(float dl_hi, float dl_lo, float fi, int& fl, float& e) {
-  df p = two_prod(dl_hi, fi);
-  const float lo = fmaf(dl_lo, fi, p.lo);
-  float f = floorf(p.hi);
-  float r = __fadd_rn(__fsub_rn(p.hi, f), lo);      // p.hi - f is exact
-  if (r < 0.f) {
-    r = __fadd_rn(r, 1.f);
-    f -= 1.f;
-    if (r >= 1.f) { r = 0.f; f += 1.f; }
-  } else if (r >= 1.f) {
-    r = __fsub_rn(r, 1.f);
-    f += 1.f;
-  }
-  fl = (int)f;
-  e = r;
-}
-
 // v exp(2 pi i g n) (the item's carrier rotation), or v when g = 0.
 DC_DEV float2 rotate(float2 v, float g_hi, float g_lo, int n) {
   if (g_hi == 0.f && g_lo == 0.f) return v;

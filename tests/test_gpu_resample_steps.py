@@ -106,3 +106,26 @@ def test_windows_of_one_context(dcg):
                                        beta=float(beta))
         assert rel(y.cpu().numpy(), ref) <= TOL, (taps, beta)
     ctx.close()
+
+
+@pytest.mark.parametrize("v", [1e-20, -1e-20, 1e-24, 1e-27, 1e-30, -1e-30, 1e-33, 1e-36, -1e-36, 1e-300])
+def test_tiny_rates(dcg, v):
+    """Positions within a float's smallest numbers of the inputs': the pulse itself."""
+    import torch
+    x = synth.bandlimited_noise(2000, synth.rng_for(3)).astype(np.complex64)
+    for mode in (dcg.DC_WINDOWED, dcg.DC_EXACT_FP32):
+        assert rel(run(dcg, x, 2000, v, mode=mode), x) <= TOL, mode
+    ctx = dcg.Context(0)
+    xd = torch.from_numpy(x).cuda().repeat(16)
+    for mode in (dcg.DC_EXACT_FP32, dcg.DC_EXACT_BF16X3, dcg.DC_EXACT_FP16X3):
+        y = torch.empty_like(xd)
+        dcg.resample_exact_batch(ctx, xd, 2000, 16, [v], y, mode=mode)
+        dcg.dc_check(ctx)
+        assert rel(y.cpu().numpy().reshape(16, -1), np.tile(x, (16, 1))) <= 2e-5, mode   # split products
+    y = torch.empty((3, 2, 2000), dtype=torch.complex64, device="cuda")
+    dcg.correct_bank(ctx, xd[:2000], [v, 0.0, 2 * v], [50.0, 0.0], y, FS, FC)
+    dcg.dc_check(ctx)
+    ref = oracle.iono_correct(x.astype(np.complex128), FS, FC, 50.0)
+    for i in range(3):
+        assert rel(y[i, 0].cpu().numpy(), ref) <= TOL and rel(y[i, 1].cpu().numpy(), x) <= TOL
+    ctx.close()
