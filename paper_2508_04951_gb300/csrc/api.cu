@@ -257,11 +257,20 @@ dc_status ensure_ws(dc_ctx* c, size_t bytes) {
   return DC_OK;
 }
 
+// Whether work on `s` is being captured (for the null stream: whether some
+// capture forbids it): nothing may be allocated or waited for then.
+bool capturing(cudaStream_t s) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &st) == cudaSuccess) return st != cudaStreamCaptureStatusNone;
+  cudaGetLastError();
+  return true;
+}
+
 // Scratch that only a faster form of a call wants: true when the context has
 // it or can grow to it, leaving no error behind when it cannot.
-bool try_ws(dc_ctx* c, size_t bytes) {
+bool try_ws(dc_ctx* c, size_t bytes, cudaStream_t s) {
   if (bytes <= c->ws_bytes) return true;
-  if (c->rec || c->fixed_ws) return false;
+  if (c->rec || c->fixed_ws || capturing(s)) return false;
   const std::string msg = c->last_error;
   if (ensure_ws(c, bytes) == DC_OK) return true;
   c->last_error = msg;
@@ -270,13 +279,13 @@ bool try_ws(dc_ctx* c, size_t bytes) {
 
 // Near and far scratch of an FP32 exact sum, taken at offset `at` of the
 // context's scratch where the form applies and the scratch can be had.
-void exact_far(dc_ctx* c, ExArgs& a, int n_alpha, double delta_max, size_t at) {
+void exact_far(dc_ctx* c, ExArgs& a, int n_alpha, double delta_max, size_t at, cudaStream_t s) {
   if (!exact_fp32_far(a.n_in, a.n_out, a.n_pulses, n_alpha, delta_max)) return;
   const long long groups = a.shared ? 1 : n_alpha;
   at = (at + 255) & ~(size_t)255;
   const size_t mom = exact_fp32_far_elems(groups * a.n_pulses, a.n_in);
   const size_t loc = exact_fp32_far_elems(groups * a.n_pulses, a.n_out);
-  if (!try_ws(c, at + (mom + loc) * sizeof(float2))) return;
+  if (!try_ws(c, at + (mom + loc) * sizeof(float2), s)) return;
   a.mom = reinterpret_cast<float2*>(c->ws + at);
   a.loc = a.mom + mom;
 }
@@ -494,12 +503,7 @@ PolyTables poly_tables(dc_ctx* c, int taps, double beta, cudaStream_t s) {
   while (i < c->poly_keys.size() && !(c->poly_keys[i].first == taps && c->poly_keys[i].second == beta)) ++i;
   float* dev = c->poly + i * dc_ctx::kPolyFloats;
   if (i == c->poly_keys.size()) {
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (i == (size_t)dc_ctx::kPolySlots || c->rec ||
-        (s && (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone))) {
-      cudaGetLastError();
-      return {nullptr, nullptr};
-    }
+    if (i == (size_t)dc_ctx::kPolySlots || c->rec || capturing(s)) return {nullptr, nullptr};
     std::vector<float> v(dc_ctx::kPolyFloats, 0.f);
     const std::vector<float> w = window_poly(taps, beta);
     std::copy(w.begin(), w.end(), v.begin());
@@ -932,7 +936,7 @@ dc_status doppler_resample(dc_ctx* c, const dc_c64* x, long long n, dc_c64* y, d
   a.one.y = reinterpret_cast<float2*>(y);
   split(dl, a.one.dl_hi, a.one.dl_lo);
   split(rotation_rate(o, dl, fs, fc), a.one.rot_hi, a.one.rot_lo);
-  exact_far(c, a, 1, std::fabs(dl), 0);
+  exact_far(c, a, 1, std::fabs(dl), 0, s);
   enqueue(c, PH_EXACT, s, n_out, "exact launch", [=] { return launch_exact_fp32(a, 1, s); });
   return flush(c, s);
 }
@@ -1005,7 +1009,7 @@ dc_status correct_batch(dc_ctx* c, const dc_c64* in, dc_c64* out, const dc_item*
       if (exact_fp32_far((int)items[i].n, no, 1, 1, std::fabs(alpha_minus_one(items[i].v_r))))
         far = std::max(far, exact_fp32_far_elems(1, (int)items[i].n) + exact_fp32_far_elems(1, no));
     }
-    if (far) try_ws(c, ((lay.bytes + 255) & ~(size_t)255) + far * sizeof(float2));
+    if (far) try_ws(c, ((lay.bytes + 255) & ~(size_t)255) + far * sizeof(float2), s);
   }
   char* ws = c->ws;
   size_t item_at = 0;
@@ -1035,7 +1039,7 @@ dc_status correct_batch(dc_ctx* c, const dc_c64* in, dc_c64* out, const dc_item*
       a.one.y = reinterpret_cast<float2*>(ws + yoff[i]);
       split(dl, a.one.dl_hi, a.one.dl_lo);
       split(rotation_rate(o, dl, it.fs, it.fc), a.one.rot_hi, a.one.rot_lo);
-      if (lay.bytes < c->ws_bytes) exact_far(c, a, 1, std::fabs(dl), lay.bytes);
+      if (lay.bytes < c->ws_bytes) exact_far(c, a, 1, std::fabs(dl), lay.bytes, s);
       enqueue(c, PH_EXACT, s, a.n_out, "exact launch", [=] { return launch_exact_fp32(a, 1, s); });
     }
   }
@@ -1382,7 +1386,7 @@ extern "C" dc_status correct_compress(dc_ctx* c, const dc_c64* x, long long n,
   if ((st = ensure_items(c, items_bytes_for(16)))) return st;
   const double dl = alpha_minus_one(v_r);
   ExArgs ea{nullptr, (int)n, (int)n_out, 1};
-  if (o.mode == DC_EXACT_FP32) exact_far(c, ea, 1, std::fabs(dl), ar.off);   // before c->ws is read
+  if (o.mode == DC_EXACT_FP32) exact_far(c, ea, 1, std::fabs(dl), ar.off, s);   // before c->ws is read
   char* ws = c->ws;
   float2* Yr = reinterpret_cast<float2*>(ws + y_at);
   float2* H = reinterpret_cast<float2*>(ws + h_at);
@@ -1502,9 +1506,9 @@ extern "C" dc_status resample_exact_batch(dc_ctx* c, const dc_c64* x, long long 
       Arena ar;
       for (int i = 0; i < (far ? 6 : 2); ++i) at[i] = ar.take(i < 2 ? plane : i < 4 ? mom : loc);
       pl.far = far;
-      if ((st = ensure_ws(c, ar.off)) == DC_OK) break;
+      if (far ? try_ws(c, ar.off, s) : (st = ensure_ws(c, ar.off)) == DC_OK) break;
     }
-    if (st) return st;
+    if (!pl.far && st) return st;
     pl.hi = c->ws + at[0], pl.lo = c->ws + at[1];
     pl.mom_hi = c->ws + at[2], pl.mom_lo = c->ws + at[3];
     pl.loc_hi = c->ws + at[4], pl.loc_lo = c->ws + at[5];
@@ -1537,7 +1541,7 @@ extern "C" dc_status resample_exact_batch(dc_ctx* c, const dc_c64* x, long long 
   a.shared = stride == 0;
   double delta_max = 0.0;
   for (int i = 0; i < n_alpha; ++i) delta_max = std::max(delta_max, std::fabs(alpha_minus_one(v_r[i])));
-  exact_far(c, a, n_alpha, delta_max, 0);
+  exact_far(c, a, n_alpha, delta_max, 0, s);
   enqueue(c, PH_EXACT, s, (long long)n_alpha * n_pulses * n_out, "exact launch", [=] { return launch_exact_fp32(a, n_alpha, s); });
   return flush(c, s);
 }
