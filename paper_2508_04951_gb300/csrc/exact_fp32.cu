@@ -91,9 +91,14 @@ __global__ void __launch_bounds__(kFarBlock, 2) ex_moments_kernel(ExArgs a, int 
 // CTA tile: 64 outputs x PT pulses, 4 x 4 per thread, K in chunks of 16.  Input
 // chunks arrive by cp.async two chunks ahead (three buffers), the next chunk's
 // weights are formed after the current one's products (two buffers): one barrier
-// per chunk.  Weights are stored twice side by side, so that a complex
-// multiply-add is one packed FMA.  The 16 node values of the far field are one
-// more chunk, taken first (its basis evaluation then holds no accumulators).
+// per chunk.  A complex multiply-add is one packed FMA with the weight in both
+// lanes.  What bounds the products is shared memory's return path, four cycles of the
+// SM per wide load of a warp against eight for the packed FMAs of one input and
+// four weights; so four weights travel in one load and a move doubles each (stored
+// twice side by side they took two: 48 pulses x 8 rates x 4096 samples 175 us, now
+// 153).  8 x 4 per thread (4 loads for 32 FMAs, half the warps): 165.  The 16 node
+// values of the far field are one more chunk, taken first (its basis evaluation
+// then holds no accumulators).
 constexpr int kTN = 64, kTK = 16, kXS = 3;
 static_assert(kTK == kFarP, "the node values are one chunk");
 
@@ -109,7 +114,7 @@ template <int PT, int JOB>
 __global__ void __launch_bounds__(4 * PT, (PT <= 32 ? 144 : 192) / PT) ex_tile_kernel(ExArgs a) {
   constexpr int NT = 4 * PT;
   constexpr int SR = (kTK * kTN + NT - 1) / NT;        // weights per thread and chunk
-  __shared__ __align__(16) float2 Ss[2][kTK][kTN];     // {s, s}
+  __shared__ __align__(16) float Ss[2][kTK][kTN];
   __shared__ __align__(16) float2 Xs[kXS][kTK][PT + 2];
   __shared__ float s_D[JOB == EX_NEAR ? kFarP * kFarP : 1];
   const int al = blockIdx.z, n0 = blockIdx.x * kTN, p0 = blockIdx.y * PT;
@@ -150,10 +155,7 @@ __global__ void __launch_bounds__(4 * PT, (PT <= 32 ? 144 : 192) / PT) ex_tile_k
       float T[kFarP];
       far_polys(((float)(row.mn - blk * kFarBlock) - 127.5f + row.e) * (1.f / kTgtHalf), T);
 #pragma unroll 1
-      for (int k = ok; k < kTK; k += NT / kTN) {
-        const float w = row.sg * far_basis(s_D, k, T);
-        Ss[0][k][on] = make_float2(w, w);
-      }
+      for (int k = ok; k < kTK; k += NT / kTN) Ss[0][k][on] = row.sg * far_basis(s_D, k, T);
     }
   }
   const int n_chunk = (hi - lo + kTK - 1) / kTK + far;
@@ -178,7 +180,7 @@ __global__ void __launch_bounds__(4 * PT, (PT <= 32 ? 144 : 192) / PT) ex_tile_k
           w = fast_div((KS * r) & 1 ? -sgk : sgk, den);
           if (den == 0.f) w = 1.f;
         }
-        Ss[c & 1][k][on] = make_float2(w, w);
+        Ss[c & 1][k][on] = w;
       }
     }
   };
@@ -195,11 +197,10 @@ __global__ void __launch_bounds__(4 * PT, (PT <= 32 ? 144 : 192) / PT) ex_tile_k
     cp_async_commit();
   };
 
-  // a warp covers 32 outputs x 16 pulses: its four wide loads per k read 128
-  // distinct bytes at most; outputs 2 tn, + 1 and 16 more of the warp's, pulses 2 tp, + 1
-  // and 8 more
+  // a warp covers 32 outputs x 16 pulses: its three wide loads per k read 128
+  // distinct bytes at most; four consecutive outputs, pulses 2 tp, + 1 and 8 more
   const int warp = tid >> 5, lane = tid & 31;
-  const int wn = (warp & 1) * 32 + 2 * (lane & 7), wp = (warp >> 1) * 16 + 2 * (lane >> 3);
+  const int wn = (warp & 1) * 32 + 4 * (lane & 7), wp = (warp >> 1) * 16 + 2 * (lane >> 3);
   float2 acc[4][4];
 #pragma unroll
   for (int i = 0; i < 4; ++i)
@@ -219,24 +220,23 @@ __global__ void __launch_bounds__(4 * PT, (PT <= 32 ? 144 : 192) / PT) ex_tile_k
     fetch(c + 2);
     const int b = c & 1, x3 = c % kXS;
     // few warps (PT <= 32): the next k's operands are loaded ahead of this
-    // k's products; more warps hide the loads, and fewer registers fit a
-    // fourth CTA (48 pulses x 8 rates x 4096: 177 against 216 us)
+    // k's products; more warps hide the loads (48 pulses x 8 rates x 4096: 153
+    // against 165 us)
     constexpr bool AHEAD = PT <= 32;
-    float4 f[AHEAD ? 2 : 1][4];
+    float4 f[AHEAD ? 2 : 1][3];
     auto load = [&](int k) {
-      float4 (&q)[4] = f[AHEAD ? k & 1 : 0];
+      float4 (&q)[3] = f[AHEAD ? k & 1 : 0];
       q[0] = *reinterpret_cast<const float4*>(&Ss[b][k][wn]);
-      q[1] = *reinterpret_cast<const float4*>(&Ss[b][k][wn + 16]);
-      q[2] = *reinterpret_cast<const float4*>(&Xs[x3][k][wp]);
-      q[3] = *reinterpret_cast<const float4*>(&Xs[x3][k][wp + 8]);
+      q[1] = *reinterpret_cast<const float4*>(&Xs[x3][k][wp]);
+      q[2] = *reinterpret_cast<const float4*>(&Xs[x3][k][wp + 8]);
     };
     if constexpr (AHEAD) load(0);
 #pragma unroll
     for (int k = 0; k < kTK; ++k) {
       if (AHEAD ? k + 1 < kTK : true) load(AHEAD ? k + 1 : k);
-      const float4 (&q)[4] = f[AHEAD ? k & 1 : 0];
-      const float2 s[4] = {{q[0].x, q[0].y}, {q[0].z, q[0].w}, {q[1].x, q[1].y}, {q[1].z, q[1].w}};
-      const float2 x[4] = {{q[2].x, q[2].y}, {q[2].z, q[2].w}, {q[3].x, q[3].y}, {q[3].z, q[3].w}};
+      const float4 (&q)[3] = f[AHEAD ? k & 1 : 0];
+      const float2 s[4] = {{q[0].x, q[0].x}, {q[0].y, q[0].y}, {q[0].z, q[0].z}, {q[0].w, q[0].w}};
+      const float2 x[4] = {{q[1].x, q[1].y}, {q[1].z, q[1].w}, {q[2].x, q[2].y}, {q[2].z, q[2].w}};
 #pragma unroll
       for (int i = 0; i < 4; ++i)
 #pragma unroll
@@ -246,7 +246,7 @@ __global__ void __launch_bounds__(4 * PT, (PT <= 32 ? 144 : 192) / PT) ex_tile_k
   }
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-    const int n = n0 + wn + (i >> 1) * 16 + (i & 1);
+    const int n = n0 + wn + i;
     if (n >= n_out) continue;
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
