@@ -385,14 +385,18 @@ __global__ void __launch_bounds__(kRowThreads, 4) apply_l2_kernel(FusedArgs a) {
           for (int q = 0; q < L1; ++q) col[q] = __ldcg(slot + (size_t)q * kRowN + n2);
           apply_powers<L1>(col, w4[pp]);
           dft<L1, +1>(col);
+          if (pp == PER - 1) {
+            // every thread's slot reads are done; counted ahead of the output's last
+            // stores, which the release would otherwise wait for
+            __syncthreads();
+            if (j == 0) red_release_gpu(col_done + p, 1);
+          }
 #pragma unroll
           for (int n1 = 0; n1 < L1; ++n1) {
             const int n = n2 + kRowN * n1;
             if (n < I.n_out) __stcs(I.dst + n, col[n1]);
           }
         }
-        __syncthreads();
-        if (j == 0) red_release_gpu(col_done + p, 1);   // every thread's slot reads first
       }
     }
     if (taker) s_ti[(it + 1) & 1] = decode(t_next);
