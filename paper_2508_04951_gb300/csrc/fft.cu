@@ -10,149 +10,94 @@ namespace dc {
 
 constexpr int kThreads = 256;
 
-// Radix of stage s of an M-point transform: radix-16 stages, then one stage
-// of the remaining power of two.
-template <int M> __host__ __device__ constexpr int n_stages() {
-  int m = 0;
-  while ((1 << m) < M) ++m;
-  return m / 4 + (m % 4 ? 1 : 0);
-}
-template <int M> __host__ __device__ constexpr int stage_radix(int s) {
-  int m = 0;
-  while ((1 << m) < M) ++m;
-  return s < m / 4 ? 16 : (1 << (m % 4));
-}
-template <int M> __host__ __device__ constexpr int stage_ns(int s) {
-  int ns = 1;
-  for (int i = 0; i < s; ++i) ns *= stage_radix<M>(i);
-  return ns;
-}
-
-// ----------------------------------------------------------- row layout
-// Line c of the CTA at c*LP, element p at p + p/16 (breaks the stride-16
-// write pattern of the first stage across banks).
-DC_DEV int rpad(int p) { return p + (p >> 4); }
-
-template <int M> struct RowShape {
-  static constexpr int LINES = M >= 4096 ? 1 : (M >= 16 ? 4096 / M : 256);
-  static constexpr int LP = M + (M >> 4) + (M < 16 ? 0 : 0);
-  static constexpr int SMEM = LINES * (M + (M >> 4) + 1);   // +1 keeps LP odd-ish for tiny M
-};
-
-// One in-place Stockham stage over all lines of the CTA (row layout).
-template <int M, int R, int NS, int DIR, int LINES, int LP>
-DC_DEV void row_stage(float2* sm, const float2* __restrict__ tw) {
-  constexpr int NB = M / R;
-  constexpr int TOTAL = NB * LINES;
-  constexpr int PER = (TOTAL + kThreads - 1) / kThreads;
-  float2 v[PER][R];
-#pragma unroll
-  for (int q = 0; q < PER; ++q) {
-    const int b = threadIdx.x + kThreads * q;
-    if (TOTAL % kThreads == 0 || b < TOTAL) {
-      const int line = b / NB, j = b % NB;
-      const float2* s = sm + line * LP;
-#pragma unroll
-      for (int r = 0; r < R; ++r) v[q][r] = s[rpad(j + r * NB)];
-      if constexpr (NS > 1) {
-        const int k = j % NS;
-#pragma unroll
-        for (int r = 1; r < R; ++r)
-          v[q][r] = cmul(v[q][r], tw_m<DIR>(tw, (r * k) * (4096 / (NS * R))));
-      }
-      dft<R, DIR>(v[q]);
-    }
-  }
-  __syncthreads();
-#pragma unroll
-  for (int q = 0; q < PER; ++q) {
-    const int b = threadIdx.x + kThreads * q;
-    if (TOTAL % kThreads == 0 || b < TOTAL) {
-      const int line = b / NB, j = b % NB;
-      const int k = j % NS;
-      float2* s = sm + line * LP;
-      const int base = (j / NS) * NS * R + k;
-#pragma unroll
-      for (int r = 0; r < R; ++r) s[rpad(base + r * NS)] = v[q][r];
-    }
-  }
-  __syncthreads();
-}
-
-template <int M, int DIR, int LINES, int LP, int S = 0>
-DC_DEV void row_fft(float2* sm, const float2* __restrict__ tw) {
-  if constexpr (S < n_stages<M>()) {
-    row_stage<M, stage_radix<M>(S), stage_ns<M>(S), DIR, LINES, LP>(sm, tw);
-    row_fft<M, DIR, LINES, LP, S + 1>(sm, tw);
-  }
-}
-
-// Row pass of CTA `block`: its LINES transforms of length M, through shared
-// memory.  A thread's global loads are all issued before its first store to
-// shared memory, and items are read by non-coherent loads: otherwise every load
-// waits behind the store before it (a class of L <= 2048 took 20 us so).
+// Transforms of M = 16 R points, R = 2, 4 or 8, in registers: R threads of 16
+// points per transform, which exchange once in each direction behind a warp
+// barrier.  The split n = R p + t, k = s + 16 a (p, s < 16; t, a < R): DFT over p in
+// thread t, W_M^(t s); exchange; DFT over t (16 / R of them, s = t + R i, in each
+// thread); the inverse mirrored.  Point t of sub-problem s of transform q lies at
+// (t * 16 + s) * pitch + q.  With M <= 16 (R = 1) a thread holds a transform whole.
+// Latency bounds a few transforms, the accesses of 64 (R = 8) to 8 bytes many.  Radix-16
+// stages through shared memory, with two CTA barriers and table loads per element
+// each, took 8.2 us for a pulse of 128 (now 4.5), 6.2 for one of 16 (2.3), 52 for
+// 20000 transforms of 128 (22).
 template <int M, int OP>
-DC_DEV void row_pass(float2* sm, const FftItem* items, const FftItem& one, int n_items, int block,
-                     const float2* __restrict__ tw) {
-  constexpr int LINES = RowShape<M>::LINES;
-  constexpr int LP = M + (M >> 4) + 1;
-  constexpr int PER = (LINES * M + kThreads - 1) / kThreads;   // elements per thread
-  const int line0 = block * LINES;
-
-  // ---- load (coalesced along each line)
-  float2 v[PER];
+DC_DEV void tiny_pass(float2* sm, const FftItem* items, const FftItem& one, int n_items, int block,
+                      const float2* __restrict__ tw) {
+  constexpr int R = M > 16 ? M / 16 : 1, N = M > 16 ? 16 : M;      // threads, points of each
+  constexpr int NT = kThreads / R, PITCH = NT + 16 / R, NI = 16 / R;
+  const int q = threadIdx.x / R, t = threadIdx.x % R;
+  const int g = block * NT + q;
+  const bool live = g < n_items;
+  const FftItem I = items ? ldg_item(items + (live ? g : 0)) : one;
+  float2 wt[4];                                 // W_M^(t 2^i)
+  if constexpr (R > 1) {
 #pragma unroll
-  for (int q = 0; q < PER; ++q) {
-    const int idx = threadIdx.x + kThreads * q;
-    const int g = line0 + idx / M, p = idx % M;
-    v[q] = make_float2(0.f, 0.f);
-    if (g < n_items) {
-      const FftItem I = items ? ldg_item(items + g) : one;
-      if (OP == ROW_APPLY || p < I.n_valid) v[q] = I.src[p];
-      if (OP == ROW_APPLY) {
-        // the table is in the spectrum's own layout (natural below 4096)
-        if (I.ptab) v[q] = cmul(v[q], __ldg(I.ptab + p));
-        else if (I.ph.enabled) v[q] = cmul(v[q], iono_factor(I.ph, p));
+    for (int i = 0; i < 4; ++i) wt[i] = __ldg(tw + (t << i) * (4096 / M));
+  }
+  pdl_wait();                                   // the input's producer has finished
+  float2 v[N];
+  // v[i R + a] = bin t + R i + 16 a once the forward transform is done
+  auto bin = [&](int x) { return R > 1 ? t + R * (x / R) + 16 * (x % R) : x; };
+  if constexpr (OP == ROW_APPLY) {
+#pragma unroll
+    for (int x = 0; x < N; ++x) v[x] = live ? I.src[bin(x)] : make_float2(0.f, 0.f);
+  } else {
+#pragma unroll
+    for (int p = 0; p < N; ++p) v[p] = live && R * p + t < I.n_valid ? I.src[R * p + t] : make_float2(0.f, 0.f);
+    dft<N, -1>(v);                              // over p
+    if constexpr (R > 1) {
+      apply_powers<16>(v, wt);
+#pragma unroll
+      for (int s = 0; s < 16; ++s) sm[(t * 16 + s) * PITCH + q] = v[s];
+      __syncwarp();
+#pragma unroll
+      for (int i = 0; i < NI; ++i) {
+        float2 u[R];
+#pragma unroll
+        for (int k = 0; k < R; ++k) u[k] = sm[(k * 16 + t + R * i) * PITCH + q];
+        dft<R, -1>(u);                          // over t
+#pragma unroll
+        for (int k = 0; k < R; ++k) v[i * R + k] = u[k];
       }
     }
   }
+  if constexpr (OP == ROW_SPEC) {
+    if (live) {
 #pragma unroll
-  for (int q = 0; q < PER; ++q) {
-    const int idx = threadIdx.x + kThreads * q;
-    sm[(idx / M) * LP + rpad(idx % M)] = v[q];
-  }
-  __syncthreads();
-
-  if (OP != ROW_APPLY) row_fft<M, -1, LINES, LP>(sm, tw);
-
-  if (OP == ROW_FULL) {
-#pragma unroll
-    for (int q = 0; q < PER; ++q) {
-      const int idx = threadIdx.x + kThreads * q;
-      const int c = idx / M, p = idx % M;
-      if (line0 + c < n_items) {
-        const FftItem I = items ? ldg_item(items + line0 + c) : one;
-        float2 w = make_float2(1.f, 0.f);
-        if (I.ptab) w = __ldg(I.ptab + (M == 4096 ? spec_index(p) : p));
-        else if (I.ph.enabled) w = iono_factor(I.ph, p);
-        sm[c * LP + rpad(p)] = cmul(sm[c * LP + rpad(p)], w);
-      }
+      for (int x = 0; x < N; ++x) I.dst[bin(x)] = v[x];
     }
-    __syncthreads();
+    return;
   }
-
-  if (OP != ROW_SPEC) row_fft<M, +1, LINES, LP>(sm, tw);
-
-  // ---- store (scaled and truncated, or the whole spectrum)
+  if (I.ptab) {
 #pragma unroll
-  for (int q = 0; q < PER; ++q) {
-    const int idx = threadIdx.x + kThreads * q;
-    const int c = idx / M, p = idx % M;
-    if (line0 + c >= n_items) continue;
-    const FftItem I = items ? ldg_item(items + line0 + c) : one;
-    const float2 x = sm[c * LP + rpad(p)];
-    if (OP == ROW_SPEC) I.dst[p] = x;
-    else if (p < I.n_out) __stcs(I.dst + p, cscale(x, 1.0f / (float)M));
+    for (int x = 0; x < N; ++x) v[x] = cmul(v[x], I.ptab[bin(x)]);
+  } else if (I.ph.enabled) {
+#pragma unroll
+    for (int x = 0; x < N; ++x) v[x] = cmul(v[x], iono_factor(I.ph, bin(x)));
+  }
+  if constexpr (R > 1) {
+    __syncwarp();                               // the forward transform's reads
+#pragma unroll
+    for (int i = 0; i < NI; ++i) {
+      float2 u[R];
+#pragma unroll
+      for (int k = 0; k < R; ++k) u[k] = v[i * R + k];
+      dft<R, +1>(u);                            // over a
+#pragma unroll
+      for (int k = 0; k < R; ++k) sm[(k * 16 + t + R * i) * PITCH + q] = u[k];
+    }
+    __syncwarp();
+#pragma unroll
+    for (int s = 0; s < 16; ++s) v[s] = sm[(t * 16 + s) * PITCH + q];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) wt[i] = conj_if<+1>(wt[i]);
+    apply_powers<16>(v, wt);
+  }
+  dft<N, +1>(v);                                // over s
+  if (live) {
+#pragma unroll
+    for (int p = 0; p < N; ++p)
+      if (R * p + t < I.n_out) __stcs(I.dst + R * p + t, cscale(v[p], 1.0f / (float)M));
   }
 }
 
@@ -167,7 +112,7 @@ DC_DEV void row_pass(float2* sm, const FftItem* items, const FftItem& one, int n
 // Sub-problem s keeps to its own 17 A elements except in the exchange, whose pitch
 // 17 A puts a half-warp's accesses on 16 different bank pairs throughout.  Against
 // radix-16 stages through shared memory with two barriers each and table loads per
-// element (row_pass) a lone pulse of 2048 takes 6.2 instead of 12.3 us.
+// element a lone pulse of 2048 takes 6.2 instead of 12.3 us.
 template <int A, int OP>
 DC_DEV void line_pass(float2* sm, const FftItem* items, const FftItem& one, int n_items, int block,
                       const float2* __restrict__ tw) {
@@ -184,6 +129,7 @@ DC_DEV void line_pass(float2* sm, const FftItem* items, const FftItem& one, int 
     wq[i] = __ldg(tw + (tl << i) * (4096 / M));
     wt[i] = __ldg(tw + (t << i) * (4096 / T));
   }
+  pdl_wait();                                   // the input's producer has finished
   float2 v[16];
   if constexpr (OP == ROW_APPLY) {
 #pragma unroll
@@ -268,16 +214,15 @@ DC_DEV void line_pass(float2* sm, const FftItem* items, const FftItem& one, int 
   }
 }
 
-// The pass of CTA `block` for transforms of M points.
+// The pass of CTA `block` for transforms of M points, its transforms per CTA and shared memory.
 template <int M, int OP>
 DC_DEV void short_pass(float2* sm, const FftItem* items, const FftItem& one, int n_items, int block, const float2* tw) {
-  if constexpr (M >= 256 && M <= 2048) line_pass<M / 256, OP>(sm, items, one, n_items, block, tw);
-  else row_pass<M, OP>(sm, items, one, n_items, block, tw);
+  if constexpr (M == 4096) full_4096<true>(items ? ldg_item(items + block) : one, sm, threadIdx.x, tw);
+  else if constexpr (M >= 256) line_pass<M / 256, OP>(sm, items, one, n_items, block, tw);
+  else tiny_pass<M, OP>(sm, items, one, n_items, block, tw);
 }
-// Its transforms per CTA and shared memory.
-template <int M> __host__ __device__ constexpr size_t short_smem() {
-  return sizeof(float2) * (M >= 256 && M <= 2048 ? 4352 : RowShape<M>::LINES * (M + (M >> 4) + 1));
-}
+constexpr int short_lines(int M) { return M <= 16 ? kThreads : 4096 / M; }
+constexpr size_t short_smem(int M) { return M <= 16 ? 0 : sizeof(float2) * kRowPitch; }
 
 template <int M, int OP>
 __global__ void __launch_bounds__(kThreads) row_kernel(RowArgs a) {
@@ -287,7 +232,9 @@ __global__ void __launch_bounds__(kThreads) row_kernel(RowArgs a) {
 
 // Short transforms of several length classes in one launch: run one after the
 // other, the classes of a small batch leave the chip idle (each is one latency
-// chain of about 20 us on a few CTAs).
+// chain on a few CTAs).  Launched programmatically: successive calls, and the
+// resampling before it, overlap its set-up (iono_correct of 256 to 2048 samples,
+// calls back to back: 6.2 -> 4.5 us).
 template <int M>
 DC_DEV void class_pass(float2* sm, const RowClasses& a, int m) {
   short_pass<M, ROW_FULL>(sm, a.items ? a.items + a.first[m] : nullptr, a.one, a.first[m + 1] - a.first[m],
@@ -310,9 +257,7 @@ __global__ void __launch_bounds__(kThreads) row_classes_kernel(const __grid_cons
     case 9: class_pass<512>(sm, a, m); break;
     case 10: class_pass<1024>(sm, a, m); break;
     case 11: class_pass<2048>(sm, a, m); break;
-    default:
-      full_4096<false>(a.items ? ldg_item(a.items + a.first[12] + blockIdx.x - a.block[12]) : a.one, sm,
-                       threadIdx.x, a.tw);
+    default: class_pass<4096>(sm, a, m);
   }
 }
 
@@ -424,17 +369,9 @@ __global__ void __launch_bounds__(kThreads) col_kernel_reg(ColArgs a) {
 // ---------------------------------------------------------------- launchers
 template <int M, int OP>
 static cudaError_t launch_row_m(const RowArgs& a, cudaStream_t s) {
-  constexpr int LINES = RowShape<M>::LINES;
-  const size_t smem = short_smem<M>();
-  const long long lines = (long long)a.n_items << a.log2L1;
-  const long long grid = (lines + LINES - 1) / LINES;
+  const long long grid = ((long long)a.n_items + short_lines(M) - 1) / short_lines(M);
   if (grid <= 0) return cudaSuccess;
-  auto k = row_kernel<M, OP>;
-  if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
-  k<<<(unsigned)grid, kThreads, smem, s>>>(a);
+  row_kernel<M, OP><<<(unsigned)grid, kThreads, short_smem(M), s>>>(a);
   return cudaGetLastError();
 }
 
@@ -455,8 +392,7 @@ static cudaError_t launch_row_op(const RowArgs& a, cudaStream_t s) {
     case 10: return launch_row_m<1024, OP>(a, s);
     case 11: return launch_row_m<2048, OP>(a, s);
     case 12:
-      // one-pass rows of L = 4096 here; every other row of 4096 points in
-      // registers (fused.cu)
+      // one-pass rows of L = 4096 here, the four-step rows in fused.cu
       if constexpr (OP == ROW_FULL) return launch_row_m<4096, OP>(a, s);
       else return launch_row_4096(OP, a, s);
     default: return cudaErrorInvalidValue;
@@ -464,19 +400,32 @@ static cudaError_t launch_row_op(const RowArgs& a, cudaStream_t s) {
 }
 
 cudaError_t launch_row_classes(RowClasses a, cudaStream_t s) {
-  static constexpr int kLines[13] = {256, 256, 256, 256, 256, 128, 64, 32, 16, 8, 4, 2, 1};
   size_t smem = 0;
   a.block[0] = 0;
   for (int m = 0; m <= 12; ++m) {
-    const int n = a.first[m + 1] - a.first[m];
-    a.block[m + 1] = a.block[m] + (n + kLines[m] - 1) / kLines[m];
-    const int M = 1 << m;
-    const size_t want = sizeof(float2) * (m >= 8 ? kRowPitch : kLines[m] * (M + (M >> 4) + 1));
-    if (n > 0) smem = std::max(smem, want);
+    const int n = a.first[m + 1] - a.first[m], lines = short_lines(1 << m);
+    a.block[m + 1] = a.block[m] + (n + lines - 1) / lines;
+    if (n > 0) smem = std::max(smem, short_smem(1 << m));
   }
   if (a.block[13] == 0) return cudaSuccess;
-  row_classes_kernel<<<(unsigned)a.block[13], kThreads, smem, s>>>(a);
-  return cudaGetLastError();
+  // launched programmatically behind the resampling (three-pass rules)
+  const int pdl = pdl_for(a.block[13]);
+  if (pdl == PDL_SPREAD) {
+    smem = kPdlRowSmem;
+    cudaError_t e = cudaFuncSetAttribute(row_classes_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)a.block[13]);
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = pdl ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, row_classes_kernel, a);
 }
 
 cudaError_t launch_row(int op, const RowArgs& a, cudaStream_t s) {
