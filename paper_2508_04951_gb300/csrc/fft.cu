@@ -271,8 +271,10 @@ __global__ void __launch_bounds__(kThreads) row_classes_kernel(const __grid_cons
 // are rows p0 + R i: four trips through the load/store path per element, which
 // bounds this pass (with both stages and the transfers through shared memory it
 // took eight, at 85 % of that path: 128 pulses of 2^18, forward 106 us, inverse 79).
+// Four CTAs per SM: the forward pass at its own 74 registers, three, waited for its
+// loads (a batch's forward passes 538 us, now 519).
 template <int M, int OP>
-__global__ void __launch_bounds__(kThreads) col_kernel_smem(ColArgs a) {
+__global__ void __launch_bounds__(kThreads, 4) col_kernel_smem(ColArgs a) {
   constexpr int C = 4096 / M, R = M / 16, NB = 16 / R;
   __shared__ float2 sm[4096];
   const int L2 = 1 << (a.log2L - a.log2L1);
