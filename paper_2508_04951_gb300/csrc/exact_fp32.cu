@@ -88,7 +88,7 @@ __global__ void __launch_bounds__(kFarBlock, 2) ex_moments_kernel(ExArgs a, int 
 }
 
 // --------------------------------------------------------------- tiles
-// CTA tile: 64 outputs x PT pulses, 4 x 4 per thread, K in chunks of 16.  Input
+// CTA tile: TN (64 or 32) outputs x PT pulses, 4 x 4 per thread, K in chunks of 16.  Input
 // chunks arrive by cp.async two chunks ahead (three buffers), the next chunk's
 // weights are formed after the current one's products (two buffers): one barrier
 // per chunk.  A complex multiply-add is one packed FMA with the weight in both
@@ -99,7 +99,7 @@ __global__ void __launch_bounds__(kFarBlock, 2) ex_moments_kernel(ExArgs a, int 
 // 153).  8 x 4 per thread (4 loads for 32 FMAs, half the warps): 165.  The 16 node
 // values of the far field are one more chunk, taken first (its basis evaluation
 // then holds no accumulators).
-constexpr int kTN = 64, kTK = 16, kXS = 3;
+constexpr int kTK = 16, kXS = 3;
 static_assert(kTK == kFarP, "the node values are one chunk");
 
 // 8-byte copy from global to shared memory, zero where !valid.
@@ -110,14 +110,15 @@ DC_DEV void cp_async8(float2* dst, const float2* src, bool valid) {
 DC_DEV void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N> DC_DEV void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-template <int PT, int JOB>
-__global__ void __launch_bounds__(4 * PT, (PT <= 32 ? 144 : 192) / PT) ex_tile_kernel(ExArgs a) {
-  constexpr int NT = 4 * PT;
-  constexpr int SR = (kTK * kTN + NT - 1) / NT;        // weights per thread and chunk
-  __shared__ __align__(16) float Ss[2][kTK][kTN];
+template <int PT, int TN, int JOB>
+__global__ void __launch_bounds__(TN * PT / 16, (PT <= 32 ? 9216 : 12288) / (TN * PT)) ex_tile_kernel(ExArgs a) {
+  constexpr int NT = TN * PT / 16;
+  constexpr int XR = kTK * PT / NT;                    // inputs per thread and chunk
+  constexpr int SR = (kTK * TN + NT - 1) / NT;        // weights per thread and chunk
+  __shared__ __align__(16) float Ss[2][kTK][TN];
   __shared__ __align__(16) float2 Xs[kXS][kTK][PT + 2];
   __shared__ float s_D[JOB == EX_NEAR ? kFarP * kFarP : 1];
-  const int al = blockIdx.z, n0 = blockIdx.x * kTN, p0 = blockIdx.y * PT;
+  const int al = blockIdx.z, n0 = blockIdx.x * TN, p0 = blockIdx.y * PT;
   const ExItem I = ex_item(a, al);
   const int tid = threadIdx.x;
   const int blk = n0 / kFarBlock;
@@ -130,7 +131,7 @@ __global__ void __launch_bounds__(4 * PT, (PT <= 32 ? 144 : 192) / PT) ex_tile_k
   const int n_in = JOB == EX_NODES ? kb : a.n_in;
   const int n_out = JOB == EX_NODES ? ob : a.n_out;
 
-  const int on = tid % kTN, ok = tid / kTN;            // the weights this thread forms
+  const int on = tid % TN, ok = tid / TN;            // the weights this thread forms
   const ExRow row = ex_row<JOB>(I, n0 + on);
   const int xk = tid % kTK, xp = tid / kTK;            // the input it copies: 4 pulses, 16 samples a half-warp
   int lo = 0, hi = n_in, far = 0;
@@ -140,7 +141,7 @@ __global__ void __launch_bounds__(4 * PT, (PT <= 32 ? 144 : 192) / PT) ex_tile_k
     // its tile then takes every term.
     bool bad = false;
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
+    for (int r = 0; r < XR; ++r) {
       const int p = p0 + xp + NT / kTK * r;
       float2 v = make_float2(0.f, 0.f);
       if (p < a.n_pulses) v = __ldcg(L + (size_t)p * ob + blk * kFarP + xk);
@@ -155,7 +156,7 @@ __global__ void __launch_bounds__(4 * PT, (PT <= 32 ? 144 : 192) / PT) ex_tile_k
       float T[kFarP];
       far_polys(((float)(row.mn - blk * kFarBlock) - 127.5f + row.e) * (1.f / kTgtHalf), T);
 #pragma unroll 1
-      for (int k = ok; k < kTK; k += NT / kTN) Ss[0][k][on] = row.sg * far_basis(s_D, k, T);
+      for (int k = ok; k < kTK; k += NT / TN) Ss[0][k][on] = row.sg * far_basis(s_D, k, T);
     }
   }
   const int n_chunk = (hi - lo + kTK - 1) / kTK + far;
@@ -167,7 +168,7 @@ __global__ void __launch_bounds__(4 * PT, (PT <= 32 ? 144 : 192) / PT) ex_tile_k
     const float d0 = (float)(row.mn - m0 - ok);
 #pragma unroll
     for (int r = 0; r < SR; ++r) {
-      constexpr int KS = NT / kTN;
+      constexpr int KS = NT / TN;
       const int k = ok + KS * r;
       if (SR * KS == kTK || k < kTK) {
         float w;
@@ -188,7 +189,7 @@ __global__ void __launch_bounds__(4 * PT, (PT <= 32 ? 144 : 192) / PT) ex_tile_k
     if (c < n_chunk) {
       const int m = lo + (c - far) * kTK + xk;
 #pragma unroll
-      for (int r = 0; r < 4; ++r) {
+      for (int r = 0; r < XR; ++r) {
         const int p = p0 + xp + NT / kTK * r;
         const bool in = p < a.n_pulses && m < n_in;
         cp_async8(&Xs[c % kXS][xk][xp + NT / kTK * r], in ? X + (size_t)p * n_in + m : X, in);
@@ -200,7 +201,8 @@ __global__ void __launch_bounds__(4 * PT, (PT <= 32 ? 144 : 192) / PT) ex_tile_k
   // a warp covers 32 outputs x 16 pulses: its three wide loads per k read 128
   // distinct bytes at most; four consecutive outputs, pulses 2 tp, + 1 and 8 more
   const int warp = tid >> 5, lane = tid & 31;
-  const int wn = (warp & 1) * 32 + 4 * (lane & 7), wp = (warp >> 1) * 16 + 2 * (lane >> 3);
+  const int wn = (TN == 64 ? (warp & 1) * 32 : 0) + 4 * (lane & 7);
+  const int wp = (TN == 64 ? warp >> 1 : warp) * 16 + 2 * (lane >> 3);
   float2 acc[4][4];
 #pragma unroll
   for (int i = 0; i < 4; ++i)
@@ -437,20 +439,30 @@ cudaError_t launch_gemv(const ExArgs& a, int rows, int n_alpha, cudaStream_t s) 
   return launch(ex_gemv_kernel<8, JOB>, grid, 256, pdl, a, s);
 }
 
+template <int TN, int JOB>
+cudaError_t launch_tile_n(const ExArgs& a, int pt, dim3 grid, cudaStream_t s) {
+  // no programmatic launch: tiles placed while the kernel before still holds
+  // most SMs pile up on the free ones (48 pulses x 3072 samples: 138 against 76 us)
+  const bool pdl = false;
+  if (pt == 64) return launch(ex_tile_kernel<64, TN, JOB>, grid, TN * 4, pdl, a, s);
+  if (pt == 48) return launch(ex_tile_kernel<48, TN, JOB>, grid, TN * 3, pdl, a, s);
+  if (pt == 32) return launch(ex_tile_kernel<32, TN, JOB>, grid, TN * 2, pdl, a, s);
+  return launch(ex_tile_kernel<16, TN, JOB>, grid, TN, pdl, a, s);
+}
+
+// 32 instead of 64 outputs per tile while those then fill at most one CTA per SM:
+// 64 against 32, us, pulses x rates x samples: 48 x 1 x 4096: 61 / 49, 64 x 4 x 1024:
+// 62 / 43, 48 x 8 x 512: 33 / 25, 12 x 1 x 4096: 41 / 43; beyond, the inputs are
+// fetched twice as often for nothing (64 x 4 x 2048: 62 / 64, 48 x 8 x 4096: 154 / 160).
 template <int JOB>
 cudaError_t launch_tile(const ExArgs& a, int rows, int n_alpha, cudaStream_t s) {
   // the pulse tile that pads the pulses least, the widest among equals
   int pt = 64, least = (a.n_pulses + 63) / 64 * 64;
   for (int t : {48, 32, 16})
     if ((a.n_pulses + t - 1) / t * t < least) pt = t, least = (a.n_pulses + t - 1) / t * t;
-  const dim3 grid((rows + kTN - 1) / kTN, (a.n_pulses + pt - 1) / pt, n_alpha);
-  // no programmatic launch: tiles placed while the kernel before still holds
-  // most SMs pile up on the free ones (48 pulses x 3072 samples: 138 against 76 us)
-  const bool pdl = false;
-  if (pt == 64) return launch(ex_tile_kernel<64, JOB>, grid, 256, pdl, a, s);
-  if (pt == 48) return launch(ex_tile_kernel<48, JOB>, grid, 192, pdl, a, s);
-  if (pt == 32) return launch(ex_tile_kernel<32, JOB>, grid, 128, pdl, a, s);
-  return launch(ex_tile_kernel<16, JOB>, grid, 64, pdl, a, s);
+  const dim3 wide((rows + 63) / 64, (a.n_pulses + pt - 1) / pt, n_alpha);
+  if (pt <= 16 || 2LL * wide.x * wide.y * wide.z > 152) return launch_tile_n<64, JOB>(a, pt, wide, s);
+  return launch_tile_n<32, JOB>(a, pt, dim3((rows + 31) / 32, wide.y, wide.z), s);
 }
 
 // The node values of many pulses take the warp-per-output form while the
@@ -468,12 +480,12 @@ size_t exact_fp32_far_elems(long long pulses, int n) { return (size_t)pulses * k
 
 // The near and far form adds two launches and replaces n_in terms by at most 768
 // and 16.  Measured, far against dense, in us:
-//   tiles (more than 8 pulses), pulses x rates: 12 x 1: n = 1024: 62 / 49, 1536: 64 /
-//   70, 4096: 66 / 178; 48 x 8: 1024: 72 / 70, 1536: 93 / 154, 4096: 177 / 773 (the
+//   tiles (more than 8 pulses), pulses x rates: 12 x 1: n = 1024: 39 / 35, 1536: 39 /
+//   51, 4096: 41 / 129; 48 x 8: 1024: 64 / 59, 1536: 83 / 139, 4096: 154 / 670 (the
 //   dense kernel before these tiles: 1139); so from 1536 on.
-//   one warp per output: 1 x 1: 4096: 13.7 / 12.4, 6000: 14.7 / 20.1, 16384: 23 / 100;
-//   2 x 4: 1536: 16.6 / 13.5, 2048: 18.5 / 20.0; 8 x 1: 2048: 26.7 / 28.0; 8 x 8:
-//   1024: 42 / 32, 1536: 55 / 61, 4096: 117 / 327; so from 2^25 terms on.
+//   one warp per output: 1 x 1: 4096: 12.3 / 10.3, 6000: 12.4 / 16.4, 16384: 19 / 81;
+//   2 x 4: 1536: 16.4 / 12.8, 2048: 18.0 / 18.2; 8 x 1: 2048: 22.6 / 24.9; 8 x 8:
+//   1024: 36 / 31, 1536: 46 / 58, 4096: 97 / 312; so from 2^25 terms on.
 bool exact_fp32_far(int n_in, int n_out, int n_pulses, int n_alpha, double delta_max) {
   const double terms = (double)n_in * n_out * n_pulses * n_alpha;
   return n_in >= 1536 && (n_pulses > 8 || terms >= (double)(1 << 25)) &&
