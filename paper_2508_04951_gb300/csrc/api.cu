@@ -127,12 +127,15 @@ bool use_fused(const dc_ctx* c, int log2L) { return fused_L(log2L) && c->tune.ff
 // clusters, 2 CTAs per SM) ran 1.46 ms against 1.36 ms.
 bool apply_rows2(const dc_ctx* c, int log2L) { return log2L >= 15 && c->tune.apply_kind == 2; }
 // The spectrum apply in two passes through an L2-resident scratch (no
-// clusters), for 8192 <= L <= 65536.  The built-in rule takes it at
-// L = 65536, where the 16-CTA clusters' exchange costs more than the second
-// pass through L2 (256 x 16 bank: 1.19 vs 1.36 ms); below, the smaller
-// clusters win (L = 32768: 0.60 vs 0.57 ms; 16384: 0.30 vs 0.27 ms).
-bool apply_l2(const dc_ctx* c, int log2L) {
-  return log2L >= 13 && (c->tune.apply_kind == 3 || (c->tune.apply_kind == 0 && log2L == 16));
+// clusters), for 8192 <= L <= 65536.  The built-in rule takes it at L = 65536 from
+// 96 transforms on: there the 16-CTA clusters' exchange costs more than the second
+// pass through L2, while a few transforms pay for a queue, a scratch and counters
+// that they hardly use.  Whole bank, cluster against two-pass, us: L = 65536: 6
+// transforms: 34 / 40, 24: 42 / 49, 72: 61 / 62, 96: 69 / 67, 160: 90 / 86, 512: 220 /
+// 195, 4096: 1445 / 1164; below, the smaller clusters win or tie (32768: 768: 145 /
+// 149, 4096: 609 / 598; 16384: 290 / 315; 8192: 142 / 178).
+bool apply_l2(const dc_ctx* c, int log2L, size_t n_pairs) {
+  return log2L >= 13 && (c->tune.apply_kind == 3 || (c->tune.apply_kind == 0 && log2L == 16 && n_pairs >= 96));
 }
 // Transforms per chunk of the two-pass apply: 12 MiB of them (384 row tasks), so
 // that the scratch (kApplyL2Slots chunks, 48 MiB) stays in L2 beside the spectra
@@ -1207,7 +1210,7 @@ dc_status bank_impl(dc_ctx* c, const dc_c64* x, long long n, const dc_c64* rep, 
   const size_t t_at =
       ar.take(fused ? 0 : (size_t)std::max(chunk, four ? n_sp : 0) * L * sizeof(float2));
   const size_t n_pairs = (size_t)n_v * n_tec;
-  const bool l2 = fused && apply_l2(c, log2L);
+  const bool l2 = fused && apply_l2(c, log2L, n_pairs);
   const int l2_chunk = l2 ? apply_l2_chunk(log2L, n_pairs) : 0;
   const size_t q_at = ar.take(l2 ? (size_t)kApplyL2Slots * l2_chunk * L * sizeof(float2) : 0);
   const size_t k_at = ar.take(l2 ? (1 + 2 * n_pairs) * sizeof(int) : 0);
@@ -1502,7 +1505,7 @@ extern "C" dc_status resample_exact_batch(dc_ctx* c, const dc_c64* x, long long 
     size_t at[6] = {};
     for (bool far : {true, false}) {
       // the dense sum where the far field does not apply or its planes do not fit
-      if (far && !exact_tc_far((int)n, (int)n_out, delta_max)) continue;
+      if (far && !exact_tc_far(mode == DC_EXACT_FP16X3, (int)n, (int)n_out, delta_max)) continue;
       Arena ar;
       for (int i = 0; i < (far ? 6 : 2); ++i) at[i] = ar.take(i < 2 ? plane : i < 4 ? mom : loc);
       pl.far = far;

@@ -145,7 +145,7 @@ DC_DEV void position(float dl_hi, float dl_lo, int n, int& m, float& e) {
 // planes hold M / 32 and L / 32, the Cauchy elements are taken times 256.
 constexpr float kMomScale = 1.f / 32, kCauchyScale = 256.f, kLocScale = 1.f / 32;
 
-constexpr int kFarMinIn = 1536;                      // see exact_tc_far
+constexpr int kFarMinIn = 1536, kFarMinInFp16 = 1792;   // see exact_tc_far
 constexpr int kFarWideIn = 4096;                     // bf16x3 above: near = 3 blocks either side
 
 // What one launch of the tile kernel contracts.
@@ -601,13 +601,13 @@ size_t exact_tc_plane_bytes(long long rows, int n) {
 }
 
 // The near and far form replaces n_in / 32 chunks by at most 25 (bf16x3 above
-// 4096: 57) and adds two launches.  Measured, far against dense, in us (bf16x3;
-// 8 pulses x 1 rate, 512 x 1, 512 x 16): n = 1025: 62 / 63, 75 / 68, 168 / 197;
-// 1536: 62 / 86, 74 / 93, 195 / 275; 2048: 64 / 111, 76 / 119, 251 / 448; 8192 at
-// 512 x 16: 1478 / 5172.  fp16x3: 1300: 43 / 47, 56 / 51, 192 / 238; 1536: 43 / 53,
-// 56 / 59, 206 / 307; 6000: 51 / 170, 97 / 320, 761 / 3187.
-bool exact_tc_far(int n_in, int n_out, double delta_max) {
-  return n_in >= kFarMinIn && delta_max * (double)n_out <= (double)(kFarMargin - 1);
+// 4096: 57) and adds two launches.  Measured, far against dense, in us (8 pulses x 1
+// rate, 64 x 4, 512 x 1): bf16x3: n = 1025: 43 / 39, 50 / 41, 56 / 43; 1536: 43 / 51,
+// 49 / 54, 55 / 57; 2048: 45 / 63, 49 / 68, 57 / 70; 4097: 75 / 114, 83 / 121, 91 /
+// 126; 8192 at 512 x 16: 1053, dense as it was before 5172.  fp16x3: 1536: 35 / 34, 38 /
+// 37, 44 / 42; 2048: 35 / 43, 40 / 47, 46 / 49; 8192: 41 / 133, 69 / 275, 85 / 285.
+bool exact_tc_far(bool fp16, int n_in, int n_out, double delta_max) {
+  return n_in >= (fp16 ? kFarMinInFp16 : kFarMinIn) && delta_max * (double)n_out <= (double)(kFarMargin - 1);
 }
 size_t exact_tc_far_plane_bytes(long long rows, int n) {
   return (size_t)rows * kFarP * far_blocks(n) * 2;

@@ -34,7 +34,7 @@ size_t exact_tc_plane_bytes(long long rows, int n);
 // Whether blocks away from an output are summed through their moments:
 // n_in long enough, and every output within 63 samples of its own index
 // (delta_max: the largest |alpha - 1|).
-bool exact_tc_far(int n_in, int n_out, double delta_max);
+bool exact_tc_far(bool fp16, int n_in, int n_out, double delta_max);
 size_t exact_tc_far_plane_bytes(long long rows, int n);
 
 // Split x (x_rows_c complex pulses of n samples) into the planes, then run the
