@@ -66,9 +66,9 @@ UNIT = "Msamples/s"
 ALGO_BYTES_PER_SAMPLE = 8        # one complex64 corrected sample written
 # DRAM bytes (read + write) per launch of the kernel at the full workload, from
 # one ncu capture of the full-size launch (the two-pass apply kernel:
-# dram__bytes_read.sum 175,721,728 + dram__bytes_write.sum 2,207,151,872).
+# dram__bytes_read.sum 324.31 MB + dram__bytes_write.sum 2.77 GB).
 # Cleared whenever the kernel changes after the capture.
-TRAFFIC_PER_LAUNCH: dict[str, float | None] = {"fused_apply": 175721728.0 + 2207151872.0}
+TRAFFIC_PER_LAUNCH: dict[str, float | None] = {"fused_apply": 324.31e6 + 2.77e9}
 
 
 def load_peaks() -> tuple[float, str]:
