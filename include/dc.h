@@ -299,8 +299,11 @@ DC_API dc_status predistort_lfm(dc_ctx* ctx, dc_c64* y_dev, long long n, double 
                                 double bandwidth, double T, double tec_tecu, double f_mix,
                                 int kind, void* stream);
 
-/* Exact-sinc resampling of many pulses per range rate (Eq. 17 as a dense
- * contraction Y_a = X_a S_a^T, S_a[j][i] = sinc(alpha_a j - i)).
+/* Exact-sinc resampling of many pulses per range rate (Eq. 17:
+ * Y_a = X_a S_a^T, S_a[j][i] = sinc(alpha_a j - i)).  Pulses of 1536 samples
+ * and more are summed term by term near each output only, 256-sample blocks
+ * further off through 16 moments each (to FP32 accuracy), where the scratch
+ * for that is to be had.
  * x_dev: pulses [n_alpha][n_pulses][n] with x_alpha_stride samples between
  *        consecutive alpha groups (0 = every alpha uses the same pulses);
  * v_r:   host [n_alpha], 1 <= n_alpha <= 65535;
