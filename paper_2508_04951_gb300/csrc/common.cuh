@@ -1,6 +1,6 @@
 // Device-side building blocks shared by the library's kernels: complex
 // arithmetic on float2, error-free float transforms (double-float), the
-// in-register DFTs of radix 2/4/8/16 used by the Stockham stages, and the
+// in-register DFTs of radix 2/4/8/16 used by the transforms, and the
 // twiddle tables' layout.
 #pragma once
 
@@ -70,18 +70,13 @@ DC_DEV void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 DC_DEV void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // ------------------------------------------------------------ double-float
-// Dekker/Knuth error-free transforms: a value is hi + lo with |lo| <= ulp(hi)/2.
+// Dekker's error-free product: a value is hi + lo with |lo| <= ulp(hi)/2.
 struct df { float hi, lo; };
-DC_DEV df two_sum(float a, float b) {
-  float s = __fadd_rn(a, b);
-  float bb = __fsub_rn(s, a);
-  float e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
-  return {s, e};
-}
 DC_DEV df two_prod(float a, float b) {
   float p = __fmul_rn(a, b);
   return {p, fmaf(a, b, -p)};
 }
+
 // delta * fi = fl + e with fl integer and e in [0, 1), fi a float holding an
 // integer or half-integer output position (exact), delta a double-float.
 DC_DEV void rs_delay(float dl_hi, float dl_lo, float fi, int& fl, float& e) {

@@ -1,4 +1,4 @@
-// Stockham FFT passes with the fused ionospheric phase multiply.
+// FFT passes with the fused ionospheric phase multiply.
 // Index conventions and the four-step split are described in fft.cuh.
 #include <algorithm>
 

@@ -1,8 +1,8 @@
-// Stockham autosort FFT passes and the ionospheric correction built on them
+// FFT passes and the ionospheric correction built on them
 // (Sec. II-B, Eqs. 15-16: forward DFT, multiply by exp(-i phi_k), inverse DFT).
 //
 // Transform lengths L = 2^m up to 2^20.  L <= 4096 runs as one "row" pass in
-// shared memory.  Larger L uses the four-step split L = L1 x L2 with
+// registers.  Larger L uses the four-step split L = L1 x L2 with
 // L2 = 4096, n = n2 + L2 n1, k = k1 + L1 k2:
 //   F1  (column pass): DFT over n1 of x[n2 + L2 n1], times W_L^(n2 k1),
 //                      stored at T[n2 + L2 k1]

@@ -1,9 +1,8 @@
 // Cluster-fused FFT correction for 4096 <= L <= 65536 (Sec. II-B, Eq. 16).
 //
 // L = L1 x 4096 with L1 = L / 4096 <= 16 rows of 4096 points.  One thread
-// block cluster owns one transform: each CTA holds one row in shared memory,
-// 256 threads per row run the three radix-16 Stockham stages of a row with
-// the data in registers, and the column DFTs of length L1 exchange data
+// block cluster owns one transform: each CTA runs one row, 256 threads of 16
+// points (rows.cuh), and the column DFTs of length L1 exchange data
 // with the other CTAs through distributed shared memory.  The
 // four-step intermediate never leaves the SMs, so a transform reads its input
 // once and writes its output once.
