@@ -1159,6 +1159,7 @@ dc_status run_spectra(dc_ctx* c, std::vector<FftItem>& sp, int log2L, float2* T,
     RowArgs a2{nullptr, n_sp, log2L, log2L - 12, c->tw};
     if ((st = stage_items(c, f1, item_at, &a1.items, &a1.one)) || (st = stage_items(c, f2, item_at, &a2.items, &a2.one)))
       return st;
+    a2.pdl = log2L >= 17 ? pdl_for((long long)n_sp << (log2L - 12)) : PDL_NONE;
     enqueue(c, PH_COL_F1, s, samples, "F1 launch", [=] { return launch_col(COL_F1, a1, s); });
     enqueue(c, PH_ROW_SPEC, s, samples, "F2 launch", [=] { return launch_row(ROW_SPEC, a2, s); });
   }
@@ -1332,8 +1333,9 @@ dc_status bank_impl(dc_ctx* c, const dc_c64* x, long long n, const dc_c64* rep, 
   if ((st = stage_items(c, ra, item_at, &dra, &ora)) || (st = stage_items(c, cb, item_at, &dcb, &ocb))) return st;
   for (size_t j0 = 0; j0 < n_pairs; j0 += chunk) {
     const int cnt = (int)std::min<size_t>(chunk, n_pairs - j0);
-    const RowArgs a{dra ? dra + j0 : nullptr, cnt, log2L, log2L - 12, c->tw, ora};
-    const ColArgs b{dcb ? dcb + j0 : nullptr, cnt, log2L, log2L - 12, c->tw, ocb};
+    const int pdl = log2L >= 17 ? pdl_for((long long)cnt << (log2L - 12)) : PDL_NONE;
+    const RowArgs a{dra ? dra + j0 : nullptr, cnt, log2L, log2L - 12, c->tw, ora, pdl};
+    const ColArgs b{dcb ? dcb + j0 : nullptr, cnt, log2L, log2L - 12, c->tw, ocb, pdl};
     enqueue(c, PH_ROW_APPLY, s, (long long)cnt * n_out, "apply launch", [=] { return launch_row(ROW_APPLY, a, s); });
     enqueue(c, PH_COL_B, s, (long long)cnt * n_out, "B launch", [=] { return launch_col(COL_B, b, s); });
   }

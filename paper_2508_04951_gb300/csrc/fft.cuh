@@ -102,17 +102,21 @@ struct ColArgs {
   FftItem one;
   int pdl;         // Pdl: launched programmatically behind the pass before it
 };
-// Programmatic launches of the three-pass path's second and third pass, for
-// grids of at most one CTA per SM (`pdl` below): the passes of a single pulse are
-// latency, and each one's launch and set-up then run under the one before.  A pass
-// that starts so is placed where there is room, which piles its CTAs on the few
-// SMs the first has left; above 64 CTAs (PDL_SPREAD) each therefore asks for so much
-// shared memory that two row CTAs never share an SM's 227 KiB, a row and a column
-// CTA do.  iono_correct, us, without / with / with spread: n = 2^17: 16.7 / 12.3 /
-// 12.3; 2^18: 18.2 / 12.9 / 14.3; 2^19: 18.4 / 22.5 / 14.4.
+// Programmatic launches of the three-pass path's second and third pass and of the
+// short transforms (`pdl` below): a pass's launch and set-up then run under the one
+// before.  With at most one CTA per SM the passes of a single pulse are latency.
+// A pass that starts so is placed where there is room, which piles its CTAs on the
+// few SMs the first has left; above 64 CTAs (PDL_SPREAD) each therefore asks for so
+// much shared memory that two row CTAs never share an SM's 227 KiB, a row and a
+// column CTA do.  iono_correct, us, without / with / with spread: n = 2^17: 16.7 /
+// 12.3 / 12.3; 2^18: 18.2 / 12.9 / 14.3; 2^19: 18.4 / 22.5 / 14.4.  From two full
+// waves on (1216 CTAs) the next pass's CTAs only take slots that the last wave
+// leaves empty: 24 x 4 bank of 200000 samples, three chunks: 232 -> 214.
 enum Pdl : int { PDL_NONE = 0, PDL_ON = 1, PDL_SPREAD = 2 };
 constexpr int kPdlColSmem = 100 << 10, kPdlRowSmem = 120 << 10;
-inline int pdl_for(long long ctas) { return ctas <= 64 ? PDL_ON : ctas <= 152 ? PDL_SPREAD : PDL_NONE; }
+inline int pdl_for(long long ctas) {
+  return ctas <= 64 || ctas >= 1216 ? PDL_ON : ctas <= 152 ? PDL_SPREAD : PDL_NONE;
+}
 
 template <class A> DC_DEV FftItem item_of(const A& a, int i) { return a.items ? a.items[i] : a.one; }
 
