@@ -151,7 +151,7 @@ int apply_l2_chunk(int log2L, size_t n_pairs) {
 // Transforms per chunk of a three-pass class.  The tuned intermediate size
 // wins; else `dflt` bytes (0: the whole class at once -- the batch, whose
 // passes lose more to small launches than they gain from L2; the bank uses
-// 64 MiB, which also bounds its scratch).
+// 512 MiB, which also bounds its scratch).
 size_t chunk_items(const dc_ctx* c, int log2L, size_t count, size_t dflt) {
   const long long cb = c->tune.chunk[log2L] ? c->tune.chunk[log2L] : (long long)dflt;
   if (cb <= 0) return std::max<size_t>(count, 1);
@@ -1199,23 +1199,28 @@ dc_status bank_impl(dc_ctx* c, const dc_c64* x, long long n, const dc_c64* rep, 
   cudaStream_t s = S(stream);
   const bool four = log2L > 12;
   const bool fused = use_fused(c, log2L);
-  // Transforms per chunk of the inverse (four-step T kept small enough to
-  // stay in L2 between its two passes).
-  const int chunk =
-      four ? (int)chunk_items(c, log2L, (size_t)n_v * n_tec, (size_t)64 << 20) : n_v * n_tec;
-  const int n_sp = n_v + (compress ? 1 : 0);     // spectra: one per v_r, then the replica's
-  Arena ar;
-  const size_t y_at = ar.take((size_t)n_v * n_out * sizeof(float2));
-  const size_t p_at = ar.take((size_t)n_tec * L * sizeof(float2));
-  const size_t s_at = ar.take((size_t)n_sp * L * sizeof(float2));
-  const size_t t_at =
-      ar.take(fused ? 0 : (size_t)std::max(chunk, four ? n_sp : 0) * L * sizeof(float2));
   const size_t n_pairs = (size_t)n_v * n_tec;
+  const int n_sp = n_v + (compress ? 1 : 0);     // spectra: one per v_r, then the replica's
   const bool l2 = fused && apply_l2(c, log2L, n_pairs);
   const int l2_chunk = l2 ? apply_l2_chunk(log2L, n_pairs) : 0;
-  const size_t q_at = ar.take(l2 ? (size_t)kApplyL2Slots * l2_chunk * L * sizeof(float2) : 0);
-  const size_t k_at = ar.take(l2 ? (1 + 2 * n_pairs) * sizeof(int) : 0);
-  if ((st = ensure_ws(c, ar.off))) return st;
+  int chunk = 0;                                 // transforms per chunk of the inverse
+  size_t y_at = 0, p_at = 0, s_at = 0, t_at = 0, q_at = 0, k_at = 0;
+  auto layout = [&](size_t t_bytes) {
+    chunk = four ? (int)chunk_items(c, log2L, n_pairs, t_bytes) : (int)n_pairs;
+    Arena ar;
+    y_at = ar.take((size_t)n_v * n_out * sizeof(float2));
+    p_at = ar.take((size_t)n_tec * L * sizeof(float2));
+    s_at = ar.take((size_t)n_sp * L * sizeof(float2));
+    t_at = ar.take(fused ? 0 : (size_t)std::max(chunk, four ? n_sp : 0) * L * sizeof(float2));
+    q_at = ar.take(l2 ? (size_t)kApplyL2Slots * l2_chunk * L * sizeof(float2) : 0);
+    k_at = ar.take(l2 ? (1 + 2 * n_pairs) * sizeof(int) : 0);
+    return ar.off;
+  };
+  // Four-step T of 512 MiB at most, of 64 where that is not to be had: the passes
+  // of a chunk overlap only within it, and outweigh what a chunk that stays in L2
+  // saves (64 x 16 bank of 2^18: 64 MiB 1720 us, 256: 1596, 512: 1557, 2 GiB: 1519; 24 x 4 x 200000:
+  // 214, 211).
+  if (!try_ws(c, layout((size_t)512 << 20), s) && (st = ensure_ws(c, layout((size_t)64 << 20)))) return st;
   if ((st = ensure_items(c, items_bytes_for(n_pairs * 2 + n_sp * 6 + n_tec)))) return st;
   char* ws = c->ws;
   float2* Yr = reinterpret_cast<float2*>(ws + y_at);
