@@ -718,9 +718,12 @@ dc_status run_iono_class(dc_ctx* c, std::vector<FftItem>& it, int log2L, float2*
     const int cnt = (int)std::min(chunk, it.size() - j0);
     long long outs = 0;
     for (size_t i = j0; i < j0 + cnt; ++i) outs += it[i].n_out;
-    // the column passes of L1 <= 16 wait on nothing: no programmatic launch there
+    // the column passes of L1 <= 16 wait on nothing: no programmatic launch there;
+    // the first pass behind the call before it only where it spreads (iono_correct,
+    // calls back to back, without / with, us: n = 2^17: 12.3 / 12.7, 2^18: 12.3 /
+    // 14.3, 2^19: 14.6 / 13.5; batches: 3443 / 3450)
     const int pdl = log2L1 >= 5 ? pdl_for((long long)cnt << log2L1) : PDL_NONE;
-    const ColArgs a1{d1 ? d1 + j0 : nullptr, cnt, log2L, log2L1, c->tw, o1};
+    const ColArgs a1{d1 ? d1 + j0 : nullptr, cnt, log2L, log2L1, c->tw, o1, pdl == PDL_SPREAD ? pdl : PDL_NONE};
     const RowArgs a2{d2 ? d2 + j0 : nullptr, cnt, log2L, log2L1, c->tw, o2, pdl};
     const ColArgs a3{d3 ? d3 + j0 : nullptr, cnt, log2L, log2L1, c->tw, o3, pdl};
     enqueue(c, PH_COL_F1, s, outs, "col F1 launch", [=] { return launch_col(COL_F1, a1, s); });
