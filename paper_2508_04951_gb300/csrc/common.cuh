@@ -271,16 +271,21 @@ DC_DEV void apply_powers_from(float2 (&v)[16], float2 w0, const float2 (&b)[4]) 
 //   [5120, 6144)       W(2^20)^(1024 i) i in [0, 1024)
 //   [6144, 6384)       W256^(r k)   at 6144 + (r-1)*16 + k,  r in [1,16), k in [0,16)
 //   [6384, 10224)      W4096^(r j)  at 6384 + (r-1)*256 + j, r in [1,16), j in [0,256)
+//   [10224, 13584)     W_M^(r q), M = 256 A, A = 2, 4, 8, at kTwLine(A) + (r-1)*16 A + q,
+//                      r in [1,16), q in [0, 16 A) (A = 1: the W256 block)
+//   [13584, 13794)     W_(16 A)^(r t), A = 2, 4, 8, at kTwSub(A) + (r-1)*A + t, t in [0, A)
 // W_M^t for M | 4096 is W4096^(t 4096/M); W_L^t for L | 2^20 is
-// W(2^20)^s with s = t 2^20/L, split as s = 1024 i + j.  The last two blocks
-// are the per-stage twiddles of a 4096-point radix-16 row, laid out so a
-// warp's 32 consecutive butterflies read consecutive entries.
+// W(2^20)^s with s = t 2^20/L, split as s = 1024 i + j.  The last four blocks
+// are the per-stage twiddles of a 4096-point radix-16 row and of the shorter
+// transforms, laid out so a warp's consecutive butterflies read consecutive entries.
 constexpr int kTwMax = 4096;
 constexpr int kTwLo = 4096;
 constexpr int kTwHi = 5120;
 constexpr int kTwS2 = 6144;
 constexpr int kTwS3 = 6384;
-constexpr int kTwSize = 10224;
+__host__ __device__ constexpr int kTwLine(int A) { return A == 1 ? kTwS2 : 10224 + 15 * 16 * (A - 2); }
+__host__ __device__ constexpr int kTwSub(int A) { return 13584 + 15 * (A - 2); }
+constexpr int kTwSize = 13794;
 constexpr int kLog2Big = 20;
 
 template <int DIR> DC_DEV float2 tw_m(const float2* __restrict__ tw, int t4096) {

@@ -10,6 +10,21 @@ namespace dc {
 
 constexpr int kThreads = 256;
 
+// Twiddles w^1 .. w^15 of a thread from table rows of PITCH entries, and v[q] *= w^q (its
+// conjugate for DIR > 0): table values, each rounded once, in rows that a warp reads
+// consecutively.  Products of four powers of two instead, gathered from the 4096-point
+// table, round up to three times more (2048 points: 2.93e-7 from 64 bits, now 2.60e-7) and
+// gained nothing: plans of 10000 pulses of 300 samples 43.5 us, now 41.4, 4000 of 2000:
+// 82.6, 79.9, a lone pulse 8 us either way.
+template <int PITCH> DC_DEV void load_powers(float2 (&w)[16], const float2* __restrict__ row) {
+#pragma unroll
+  for (int q = 1; q < 16; ++q) w[q] = __ldg(row + (q - 1) * PITCH);
+}
+template <int DIR> DC_DEV void mul_powers(float2 (&v)[16], const float2 (&w)[16]) {
+#pragma unroll
+  for (int q = 1; q < 16; ++q) v[q] = cmul(v[q], conj_if<DIR>(w[q]));
+}
+
 // Transforms of M = 16 R points, R = 2, 4 or 8, in registers: R threads of 16
 // points per transform, which exchange once in each direction behind a warp
 // barrier.  The split n = R p + t, k = s + 16 a (p, s < 16; t, a < R): DFT over p in
@@ -29,11 +44,8 @@ DC_DEV void tiny_pass(float2* sm, const FftItem* items, const FftItem& one, int 
   const int g = block * NT + q;
   const bool live = g < n_items;
   const FftItem I = items ? ldg_item(items + (live ? g : 0)) : one;
-  float2 wt[4];                                 // W_M^(t 2^i)
-  if constexpr (R > 1) {
-#pragma unroll
-    for (int i = 0; i < 4; ++i) wt[i] = __ldg(tw + (t << i) * (4096 / M));
-  }
+  float2 wt[16];                                // W_M^(t s)
+  if constexpr (R > 1) load_powers<R>(wt, tw + kTwSub(R) + t);
   pdl_wait();                                   // the input's producer has finished
   float2 v[N];
   // v[i R + a] = bin t + R i + 16 a once the forward transform is done
@@ -46,7 +58,7 @@ DC_DEV void tiny_pass(float2* sm, const FftItem* items, const FftItem& one, int 
     for (int p = 0; p < N; ++p) v[p] = live && R * p + t < I.n_valid ? I.src[R * p + t] : make_float2(0.f, 0.f);
     dft<N, -1>(v);                              // over p
     if constexpr (R > 1) {
-      apply_powers<16>(v, wt);
+      mul_powers<-1>(v, wt);
 #pragma unroll
       for (int s = 0; s < 16; ++s) sm[(t * 16 + s) * PITCH + q] = v[s];
       __syncwarp();
@@ -89,9 +101,7 @@ DC_DEV void tiny_pass(float2* sm, const FftItem* items, const FftItem& one, int 
     __syncwarp();
 #pragma unroll
     for (int s = 0; s < 16; ++s) v[s] = sm[(t * 16 + s) * PITCH + q];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) wt[i] = conj_if<+1>(wt[i]);
-    apply_powers<16>(v, wt);
+    mul_powers<+1>(v, wt);
   }
   dft<N, +1>(v);                                // over s
   if (live) {
@@ -123,12 +133,9 @@ DC_DEV void line_pass(float2* sm, const FftItem* items, const FftItem& one, int 
   const FftItem I = items ? ldg_item(items + (live ? g : 0)) : one;
   float2* b = sm + (threadIdx.x / T) * 16 * P;
   float2* reg = b + s * P;
-  float2 wq[4], wt[4];                          // W_M^(q 2^i), q = tl, and W_16A^(t 2^i)
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    wq[i] = __ldg(tw + (tl << i) * (4096 / M));
-    wt[i] = __ldg(tw + (t << i) * (4096 / T));
-  }
+  float2 wq[16], wt[16];                        // W_M^(q r), q = tl, and W_16A^(t w)
+  load_powers<T>(wq, tw + kTwLine(A) + tl);
+  if constexpr (A > 1) load_powers<A>(wt, tw + kTwSub(A) + t);
   pdl_wait();                                   // the input's producer has finished
   float2 v[16];
   if constexpr (OP == ROW_APPLY) {
@@ -141,7 +148,7 @@ DC_DEV void line_pass(float2* sm, const FftItem* items, const FftItem& one, int 
       v[p] = live && n < I.n_valid ? I.src[n] : make_float2(0.f, 0.f);
     }
     dft16<-1>(v);                               // over p
-    apply_powers<16>(v, wq);
+    mul_powers<-1>(v, wq);
 #pragma unroll
     for (int r = 0; r < 16; ++r) b[r * P + tl] = v[r];
     __syncthreads();
@@ -162,7 +169,7 @@ DC_DEV void line_pass(float2* sm, const FftItem* items, const FftItem& one, int 
     __syncwarp();
 #pragma unroll
     for (int w = 0; w < 16; ++w) v[w] = reg[17 * t + w];
-    apply_powers<16>(v, wt);
+    if constexpr (A > 1) mul_powers<-1>(v, wt);
     dft16<-1>(v);                               // over w: v[r] = X[s + 16 t + T r]
   }
   if constexpr (OP == ROW_SPEC) {
@@ -181,9 +188,7 @@ DC_DEV void line_pass(float2* sm, const FftItem* items, const FftItem& one, int 
       v[r] = cmul(v[r], iono_factor_kt(I.ph, (float)(s + 16 * t + T * (r < 8 ? r : r - 16))));
   }
   dft16<+1>(v);                                 // over r
-#pragma unroll
-  for (int i = 0; i < 4; ++i) wq[i] = conj_if<+1>(wq[i]), wt[i] = conj_if<+1>(wt[i]);
-  apply_powers<16>(v, wt);
+  if constexpr (A > 1) mul_powers<+1>(v, wt);
   __syncwarp();
 #pragma unroll
   for (int w = 0; w < 16; ++w) reg[17 * t + w] = v[w];
@@ -205,7 +210,7 @@ DC_DEV void line_pass(float2* sm, const FftItem* items, const FftItem& one, int 
   __syncthreads();
 #pragma unroll
   for (int r = 0; r < 16; ++r) v[r] = b[r * P + tl];
-  apply_powers<16>(v, wq);
+  mul_powers<+1>(v, wq);
   dft16<+1>(v);                                 // over s
   if (live) {
 #pragma unroll
@@ -240,7 +245,7 @@ DC_DEV void class_pass(float2* sm, const RowClasses& a, int m) {
   short_pass<M, ROW_FULL>(sm, a.items ? a.items + a.first[m] : nullptr, a.one, a.first[m + 1] - a.first[m],
                         blockIdx.x - a.block[m], a.tw);
 }
-__global__ void __launch_bounds__(kThreads) row_classes_kernel(const __grid_constant__ RowClasses a) {
+__global__ void __launch_bounds__(kThreads, 2) row_classes_kernel(const __grid_constant__ RowClasses a) {
   extern __shared__ float2 sm[];
   int m = 0;
   while (m < 12 && (int)blockIdx.x >= a.block[m + 1]) ++m;

@@ -23,6 +23,10 @@ inline void fill_twiddles(float2* tw) {
   for (int r = 1; r < 16; ++r) {
     for (int k = 0; k < 16; ++k) tw[kTwS2 + (r - 1) * 16 + k] = w((r * k) % 256, 256.0);
     for (int j = 0; j < 256; ++j) tw[kTwS3 + (r - 1) * 256 + j] = w((r * j) % 4096, 4096.0);
+    for (int A = 2; A <= 8; A *= 2) {
+      for (int q = 0; q < 16 * A; ++q) tw[kTwLine(A) + (r - 1) * 16 * A + q] = w((r * q) % (256 * A), 256.0 * A);
+      for (int t = 0; t < A; ++t) tw[kTwSub(A) + (r - 1) * A + t] = w((r * t) % (16 * A), 16.0 * A);
+    }
   }
 }
 

@@ -1,0 +1,63 @@
+"""Distance of the corrections from 64 bits, over enough samples that it is steady to
+a per cent.  Bounds: what the transforms had with one table value, rounded once,
+for every twiddle and a factor angle rounded once, and 5 %.
+"""
+
+import math
+
+import numpy as np
+import pytest
+
+import oracle
+
+pytestmark = pytest.mark.gpu
+TEC = 100.0
+
+
+@pytest.fixture(scope="module")
+def dcg():
+    import paper_2508_04951_gb300 as m
+    m.build.build()
+    m.load()
+    return m
+
+
+def corrected64(x, fs, fc, tec):
+    """Eq. 16 in 64 bits for rows x [p, n]."""
+    import torch
+    n = x.shape[-1]
+    L = 1 << (n - 1).bit_length()
+    phi = torch.from_numpy(oracle.iono_phase(L, fs, fc, tec)).to(x.device)
+    return torch.fft.ifft(torch.fft.fft(x.to(torch.complex128), n=L) * torch.polar(torch.ones_like(phi), -phi))[..., :n]
+
+
+def noise(rows, n):
+    import torch
+    g = torch.Generator(device="cuda").manual_seed(n)
+    return torch.randn((rows, n), dtype=torch.complex64, device="cuda", generator=g)
+
+
+def batch_error(dcg, n, pulses, fs, fc):
+    import torch
+    ctx = dcg.Context(0)
+    x = noise(pulses, n)
+    y = torch.empty_like(x)
+    items = np.zeros(pulses, dtype=dcg.ITEM_DTYPE)
+    items["in_off"] = items["out_off"] = np.arange(pulses) * n
+    items["n"] = items["n_out"] = n
+    items["fs"], items["fc"], items["tec_tecu"] = fs, fc, TEC
+    # v_r = 0: frequency conversion copies the pulse as it is
+    dcg.correct_batch(ctx, x.view(-1), y.view(-1), items, mode=dcg.DC_FREQCONV)
+    dcg.dc_check(ctx)
+    ctx.close()
+    ref = corrected64(x, fs, fc, TEC)
+    return float((y.to(torch.complex128) - ref).norm() / ref.norm())
+
+
+# pulses of up to 2048 samples: lengths of each split (R x 16, 16 x A x 16), padded and whole
+@pytest.mark.parametrize("n,pulses,baseband,rf", [
+    (64, 2048, 2.08e-7, 2.35e-7), (100, 2048, 2.11e-7, 2.36e-7), (256, 1024, 2.33e-7, 2.44e-7),
+    (300, 1024, 2.08e-7, 2.44e-7), (700, 512, 2.20e-7, 2.53e-7), (2048, 256, 2.56e-7, 2.58e-7)])
+def test_short_pulses(dcg, n, pulses, baseband, rf):
+    assert batch_error(dcg, n, pulses, 20e6, 1e9) <= 1.05 * baseband
+    assert batch_error(dcg, n, pulses, 2.048e9, 0.0) <= 1.05 * rf
