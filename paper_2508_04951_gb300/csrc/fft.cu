@@ -185,7 +185,7 @@ DC_DEV void line_pass(float2* sm, const FftItem* items, const FftItem& one, int 
   } else if (I.ph.enabled) {
 #pragma unroll
     for (int r = 0; r < 16; ++r)
-      v[r] = cmul(v[r], iono_factor_kt(I.ph, (float)(s + 16 * t + T * (r < 8 ? r : r - 16))));
+      v[r] = cmul(v[r], iono_factor_full(I.ph, (float)(s + 16 * t + T * (r < 8 ? r : r - 16))));
   }
   dft16<+1>(v);                                 // over r
   if constexpr (A > 1) mul_powers<+1>(v, wt);

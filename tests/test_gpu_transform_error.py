@@ -61,3 +61,26 @@ def batch_error(dcg, n, pulses, fs, fc):
 def test_short_pulses(dcg, n, pulses, baseband, rf):
     assert batch_error(dcg, n, pulses, 20e6, 1e9) <= 1.05 * baseband
     assert batch_error(dcg, n, pulses, 2.048e9, 0.0) <= 1.05 * rf
+
+
+# the factors' share: nothing but a factor and a DFT in registers, and banks' tables
+@pytest.mark.parametrize("n,pulses,baseband,rf", [(16, 8192, 1.76e-7, 2.27e-7), (31, 4096, 1.98e-7, 2.53e-7)])
+def test_tiny_pulses(dcg, n, pulses, baseband, rf):
+    assert batch_error(dcg, n, pulses, 20e6, 1e9) <= 1.05 * baseband
+    assert batch_error(dcg, n, pulses, 2.048e9, 0.0) <= 1.05 * rf
+
+
+@pytest.mark.parametrize("n,n_tec,bound", [(200, 16, 2.25e-7), (1024, 16, 2.47e-7), (10001, 8, 2.83e-7),
+                                           (65536, 16, 3.30e-7), (100000, 8, 3.06e-7), (200000, 4, 3.11e-7)])
+def test_banks(dcg, n, n_tec, bound):
+    import torch
+    ctx = dcg.Context(0)
+    x = noise(1, n)
+    y = torch.empty((2, n_tec, n), dtype=torch.complex64, device="cuda")
+    tec = np.linspace(5.0, 150.0, n_tec)
+    dcg.correct_bank(ctx, x.view(-1), np.zeros(2), tec, y.view(-1), 20e6, 1e9, mode=dcg.DC_FREQCONV)
+    dcg.dc_check(ctx)
+    ctx.close()
+    ref = torch.cat([corrected64(x, 20e6, 1e9, t) for t in tec])
+    for v in range(2):
+        assert float((y[v].to(torch.complex128) - ref).norm() / ref.norm()) <= 1.05 * bound
