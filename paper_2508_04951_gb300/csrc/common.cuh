@@ -250,7 +250,16 @@ template <int N> DC_DEV void apply_powers(float2 (&v)[N], const float2 (&b)[4]) 
   for (int q = 1; q < N; ++q) v[q] = cmul(v[q], p[q]);
 }
 
-// v[q] *= w0 w^q, q = 0 .. 15, bases as above: w0 goes into the bases' first
+// The same for 16 values from b = w, w^2, w^3, w^4, w^8, w^12.
+DC_DEV void apply_powers(float2 (&v)[16], const float2 (&b)[6]) {
+#pragma unroll
+  for (int q = 1; q < 16; ++q) {
+    const int i = q >> 2, k = q & 3;
+    v[q] = cmul(v[q], i == 0 ? b[k - 1] : k == 0 ? b[i + 2] : cmul(b[i + 2], b[k - 1]));
+  }
+}
+
+// v[q] *= w0 w^q, q = 0 .. 15, bases as in either: w0 goes into the bases' first
 // products (five more complex multiplies instead of sixteen).
 DC_DEV void apply_powers_from(float2 (&v)[16], float2 w0, const float2 (&b)[4]) {
   float2 p[16];
@@ -261,6 +270,15 @@ DC_DEV void apply_powers_from(float2 (&v)[16], float2 w0, const float2 (&b)[4]) 
     for (int q = 0; q < (1 << i); ++q) p[(1 << i) + q] = cmul(b[i], p[q]);
 #pragma unroll
   for (int q = 0; q < 16; ++q) v[q] = cmul(v[q], p[q]);
+}
+DC_DEV void apply_powers_from(float2 (&v)[16], float2 w0, const float2 (&b)[6]) {
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const float2 p = i ? cmul(b[i + 2], w0) : w0;
+    v[4 * i] = cmul(v[4 * i], p);
+#pragma unroll
+    for (int k = 1; k < 4; ++k) v[4 * i + k] = cmul(v[4 * i + k], cmul(p, b[k - 1]));
+  }
 }
 
 // --------------------------------------------------------------- twiddles

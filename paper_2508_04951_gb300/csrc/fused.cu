@@ -1,6 +1,7 @@
 // Cluster-fused FFT correction kernels; see fused.cuh for the data flow.
 #include <algorithm>
 #include <cooperative_groups.h>
+#include <type_traits>
 
 #include "fused.cuh"
 #include "rows.cuh"
@@ -558,7 +559,7 @@ __global__ void __launch_bounds__(kRowThreads, 4) row_4096_kernel(RowArgs a) {
   const FftItem I = item_of(a, g >> a.log2L1);
   const int k1 = g & (L1 - 1);
   const int j = threadIdx.x;
-  const GlobalTw tw{a.tw};
+  const std::conditional_t<OP == ROW_MID, FineTw, GlobalTw> tw{a.tw};
   const float2* src = I.src + (size_t)k1 * kRowN;
   float2* dst = I.dst + (size_t)k1 * kRowN;
   float2 v[16];

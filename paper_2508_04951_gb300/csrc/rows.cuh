@@ -16,6 +16,7 @@ DC_DEV int pad16(int p) { return p + (p >> 4); }
 // 0..255 (s3), forward values.  Only the table rows r = 1, 2, 4, 8 are read;
 // the other powers are their products (apply_powers).
 struct GlobalTw {                 // the context's table (coalesced across the warp)
+  static constexpr int kBases = 4;
   const float2* __restrict__ tw;
   DC_DEV void s2(float2 (&b)[4], int k) const {
     const float2* t = tw + kTwS2 + k;             // row r at (r - 1) * 16
@@ -27,6 +28,7 @@ struct GlobalTw {                 // the context's table (coalesced across the w
   }
 };
 struct SharedTw {                 // a persistent CTA's copies of those rows, [4][16] and [4][256]
+  static constexpr int kBases = 4;
   const float2 *t2, *t3;
   DC_DEV void s2(float2 (&b)[4], int k) const {
 #pragma unroll
@@ -38,6 +40,7 @@ struct SharedTw {                 // a persistent CTA's copies of those rows, [4
   }
 };
 struct HeldTw {                   // loaded ahead by the caller, for this thread
+  static constexpr int kBases = 4;
   const float2 (&f2)[4], (&f3)[4];
   DC_DEV void s2(float2 (&b)[4], int) const {
 #pragma unroll
@@ -48,9 +51,27 @@ struct HeldTw {                   // loaded ahead by the caller, for this thread
     for (int q = 0; q < 4; ++q) b[q] = f3[q];
   }
 };
-template <int DIR> DC_DEV void orient(float2 (&b)[4]) {
+// The rows r = 1, 2, 3, 4, 8, 12, for the middle rows of long transforms: a power is one
+// product at most, of two table values, and fewer are live at a time (16 bytes spilled
+// instead of 40).  RF pulse of 2^19 samples 3.65e-7 from 64 bits, now 3.52e-7; batch of
+// 4096 uneven pulses 3435 us, now 3417.  All 15 rows of both tables: 3.42e-7, but the batch takes
+// 3481 us; the cluster kernels, whose error is no larger with four rows, lose 1 to 3 %.
+struct FineTw {
+  static constexpr int kBases = 6;
+  const float2* __restrict__ tw;
+  static __host__ __device__ constexpr int row(int q) { return q < 3 ? q + 1 : 4 * (q - 2); }
+  DC_DEV void s2(float2 (&b)[6], int k) const {
 #pragma unroll
-  for (int q = 0; q < 4; ++q) b[q] = conj_if<DIR>(b[q]);
+    for (int q = 0; q < 6; ++q) b[q] = __ldg(tw + kTwS2 + (row(q) - 1) * 16 + k);
+  }
+  DC_DEV void s3(float2 (&b)[6], int j) const {
+#pragma unroll
+    for (int q = 0; q < 6; ++q) b[q] = __ldg(tw + kTwS3 + (row(q) - 1) * 256 + j);
+  }
+};
+template <int DIR, int N> DC_DEV void orient(float2 (&b)[N]) {
+#pragma unroll
+  for (int q = 0; q < N; ++q) b[q] = conj_if<DIR>(b[q]);
 }
 
 // 4096-point rows, thread j = 16 s + t of 256, with one CTA barrier each.  The
@@ -76,10 +97,10 @@ template <int DIR> DC_DEV void orient(float2 (&b)[4]) {
 template <class TW>
 DC_DEV void row_forward(float2 (&v)[16], float2* b, int j, const TW& tw) {
   const int s = j >> 4, t = j & 15;
-  float2 w[4];
+  float2 w[TW::kBases];
   tw.s3(w, j);                                             // issued ahead of the DFT
   dft16<-1>(v);                                            // over p
-  apply_powers<16>(v, w);                                  // W4096^(q s), q = j
+  apply_powers(v, w);                                       // W4096^(q s), q = j
 #pragma unroll
   for (int r = 0; r < 16; ++r) b[pad16(256 * r + j)] = v[r];
   tw.s2(w, t);
@@ -88,7 +109,7 @@ DC_DEV void row_forward(float2 (&v)[16], float2* b, int j, const TW& tw) {
 #pragma unroll
   for (int u = 0; u < 16; ++u) v[u] = reg[17 * u + t];     // q = 16 u + t
   dft16<-1>(v);                                            // over u
-  apply_powers<16>(v, w);                                  // W256^(w a)
+  apply_powers(v, w);                                       // W256^(w a)
   __syncwarp();                                            // its reads of the region are done
 #pragma unroll
   for (int a = 0; a < 16; ++a) reg[17 * a + t] = v[a];     // V[w = t][a]
@@ -105,11 +126,11 @@ DC_DEV void row_forward(float2 (&v)[16], float2* b, int j, const TW& tw) {
 template <bool ARRIVE, bool FROM = false, class TW>
 DC_DEV void row_inverse(float2 (&v)[16], float2* b, int j, const TW& tw, float2 from = float2{1.f, 0.f}) {
   const int s = j >> 4, t = j & 15;
-  float2 w[4];
+  float2 w[TW::kBases];
   tw.s2(w, t);
   dft16<+1>(v);                                            // over r
   orient<+1>(w);
-  apply_powers<16>(v, w);                                  // W256^(-w a), a = t
+  apply_powers(v, w);                                       // W256^(-w a), a = t
   float2* reg = b + 272 * s;
   __syncwarp();                                            // a forward row's reads of the region
 #pragma unroll
@@ -128,7 +149,7 @@ DC_DEV void row_inverse(float2 (&v)[16], float2* b, int j, const TW& tw, float2 
   if constexpr (ARRIVE) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
   orient<+1>(w);
   if constexpr (FROM) apply_powers_from(v, from, w);       // W4096^(-q s), q = j
-  else apply_powers<16>(v, w);
+  else apply_powers(v, w);
   dft16<+1>(v);                                            // over s
 }
 
