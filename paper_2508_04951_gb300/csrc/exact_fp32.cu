@@ -415,6 +415,8 @@ __global__ void __launch_bounds__(256) ex_gemv_kernel(ExArgs a) {
 }
 
 // -------------------------------------------------------------- launches
+constexpr int kMaxGrid = 65535;                        // CTAs of a grid in y and z
+
 template <class K>
 cudaError_t launch(K k, dim3 grid, int threads, bool pdl, const ExArgs& a, cudaStream_t s) {
   cudaLaunchConfig_t cfg = {};
@@ -456,10 +458,13 @@ cudaError_t launch_tile_n(const ExArgs& a, int pt, dim3 grid, cudaStream_t s) {
 // fetched twice as often for nothing (64 x 4 x 2048: 62 / 64, 48 x 8 x 4096: 154 / 160).
 template <int JOB>
 cudaError_t launch_tile(const ExArgs& a, int rows, int n_alpha, cudaStream_t s) {
-  // the pulse tile that pads the pulses least, the widest among equals
+  // the pulse tile that pads the pulses least, the widest among equals, of those
+  // whose tiles a grid takes
   int pt = 64, least = (a.n_pulses + 63) / 64 * 64;
-  for (int t : {48, 32, 16})
-    if ((a.n_pulses + t - 1) / t * t < least) pt = t, least = (a.n_pulses + t - 1) / t * t;
+  for (int t : {48, 32, 16}) {
+    const int tiles = (a.n_pulses + t - 1) / t;
+    if (tiles <= kMaxGrid && tiles * t < least) pt = t, least = tiles * t;
+  }
   const dim3 wide((rows + 63) / 64, (a.n_pulses + pt - 1) / pt, n_alpha);
   if (pt <= 16 || 2LL * wide.x * wide.y * wide.z > 152) return launch_tile_n<64, JOB>(a, pt, wide, s);
   return launch_tile_n<32, JOB>(a, pt, dim3((rows + 31) / 32, wide.y, wide.z), s);
@@ -470,7 +475,8 @@ cudaError_t launch_tile(const ExArgs& a, int rows, int n_alpha, cudaStream_t s) 
 constexpr int kNodesGemvMax = 1024;                    // moments per pulse
 template <int JOB>
 cudaError_t launch_sum(const ExArgs& a, int rows, int n_alpha, cudaStream_t s) {
-  const bool gemv = a.n_pulses <= 8 || (JOB == EX_NODES && kFarP * far_blocks(a.n_in) <= kNodesGemvMax);
+  const bool gemv = a.n_pulses <= 8 || (JOB == EX_NODES && kFarP * far_blocks(a.n_in) <= kNodesGemvMax &&
+                                        (a.n_pulses + 7) / 8 <= kMaxGrid);
   return gemv ? launch_gemv<JOB>(a, rows, n_alpha, s) : launch_tile<JOB>(a, rows, n_alpha, s);
 }
 
@@ -494,6 +500,7 @@ bool exact_fp32_far(int n_in, int n_out, int n_pulses, int n_alpha, double delta
 
 cudaError_t launch_exact_fp32(const ExArgs& a, int n_alpha, cudaStream_t s) {
   if (n_alpha <= 0 || a.n_out <= 0 || a.n_pulses <= 0) return cudaSuccess;
+  if (a.n_pulses > 64 * kMaxGrid) return cudaErrorInvalidConfiguration;   // before the first launch
   if (!a.mom) return launch_sum<EX_DENSE>(a, a.n_out, n_alpha, s);
   const int groups = a.shared ? 1 : n_alpha;
   const long long pairs = (long long)groups * a.n_pulses * ((far_blocks(a.n_in) + 1) / 2);
