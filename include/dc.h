@@ -136,7 +136,8 @@ DC_API long long dc_launch_count(const dc_ctx* ctx);
 
 /* Per-phase kernel timing.  With profiling on, every kernel launch of later
  * calls is bracketed by CUDA events recorded on the call's stream (so the
- * times are device times of exactly that launch).  dc_profile_enable resets
+ * times are device times of exactly that launch; the kernels of an exact sum
+ * or a cubic predistortion are bracketed together, each counted).  dc_profile_enable resets
  * the totals (waiting for events still pending).  dc_profile_read waits for
  * pending events, folds them into the totals and writes up to `max` phases
  * (name, launches, samples covered, total ms) to `out`; returns the number

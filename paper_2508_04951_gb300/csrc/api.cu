@@ -65,7 +65,7 @@ struct dc_ctx {
   bool fixed_ws = false;      // the scratch is the caller's (a server's pool block): never grown
   // per-phase CUDA-event timing (dc_profile_enable / dc_profile_read)
   bool profiling = false;
-  struct Rec { int phase; cudaEvent_t a, b; long long samples; };
+  struct Rec { int phase, kernels; cudaEvent_t a, b; long long samples; };
   std::vector<cudaEvent_t> pool;
   std::vector<Rec> pending;
   static constexpr int kMaxPhases = 24;
@@ -170,17 +170,18 @@ cudaEvent_t take_event(dc_ctx* c) {
   return e;
 }
 
-// Counts one kernel launch; with profiling on, brackets it with events on
-// the launching stream.
+// Counts the launch of a phase's kernels; with profiling on, brackets them with
+// events on the launching stream.
 struct Phase {
   dc_ctx* c;
   int id;
   cudaStream_t s;
   long long samples;
+  int kernels;
   cudaEvent_t a = nullptr;
-  Phase(dc_ctx* c_, int id_, cudaStream_t s_, long long samples_)
-      : c(c_), id(id_), s(s_), samples(samples_) {
-    ++c->launches;
+  Phase(dc_ctx* c_, int id_, cudaStream_t s_, long long samples_, int kernels_ = 1)
+      : c(c_), id(id_), s(s_), samples(samples_), kernels(kernels_) {
+    c->launches += kernels;
     nvtxRangePushA(kPhaseName[id]);   // host-side range per phase (profilers; no cost without one)
     if (c->profiling && !c->rec) {
       a = take_event(c);
@@ -191,7 +192,7 @@ struct Phase {
     if (a) {
       cudaEvent_t b = take_event(c);
       cudaEventRecord(b, s);
-      c->pending.push_back({id, a, b, samples});
+      c->pending.push_back({id, kernels, a, b, samples});
     }
     nvtxRangePop();
   }
@@ -459,9 +460,9 @@ dc_status stage_items(dc_ctx* c, const std::vector<T>& v, size_t& at, const T** 
 }
 
 template <class F>
-void enqueue(dc_ctx* c, int phase, cudaStream_t s, long long samples, const char* what, F&& launch) {
+void enqueue(dc_ctx* c, int phase, cudaStream_t s, long long samples, const char* what, F&& launch, int kernels = 1) {
   c->todo.emplace_back([=]() -> dc_status {
-    Phase ph(c, phase, s, samples);
+    Phase ph(c, phase, s, samples, kernels);
     const cudaError_t e = launch();
     return e == cudaSuccess ? DC_OK : cuda_fail(c, e, what);
   });
@@ -858,7 +859,7 @@ int dc_profile_read(dc_ctx* c, dc_phase_time* out, int max) {
     float ms = 0.f;
     cudaEventElapsedTime(&ms, r.a, r.b);
     c->acc_ms[r.phase] += ms;
-    c->acc_launches[r.phase] += 1;
+    c->acc_launches[r.phase] += r.kernels;
     c->acc_samples[r.phase] += r.samples;
     c->pool.push_back(r.a);
     c->pool.push_back(r.b);
@@ -943,7 +944,7 @@ dc_status doppler_resample(dc_ctx* c, const dc_c64* x, long long n, dc_c64* y, d
   split(dl, a.one.dl_hi, a.one.dl_lo);
   split(rotation_rate(o, dl, fs, fc), a.one.rot_hi, a.one.rot_lo);
   exact_far(c, a, 1, std::fabs(dl), 0, s);
-  enqueue(c, PH_EXACT, s, n_out, "exact launch", [=] { return launch_exact_fp32(a, 1, s); });
+  enqueue(c, PH_EXACT, s, n_out, "exact launch", [=] { return launch_exact_fp32(a, 1, s); }, exact_fp32_kernels(a));
   return flush(c, s);
 }
 
@@ -1046,7 +1047,7 @@ dc_status correct_batch(dc_ctx* c, const dc_c64* in, dc_c64* out, const dc_item*
       split(dl, a.one.dl_hi, a.one.dl_lo);
       split(rotation_rate(o, dl, it.fs, it.fc), a.one.rot_hi, a.one.rot_lo);
       if (lay.bytes < c->ws_bytes) exact_far(c, a, 1, std::fabs(dl), lay.bytes, s);
-      enqueue(c, PH_EXACT, s, a.n_out, "exact launch", [=] { return launch_exact_fp32(a, 1, s); });
+      enqueue(c, PH_EXACT, s, a.n_out, "exact launch", [=] { return launch_exact_fp32(a, 1, s); }, exact_fp32_kernels(a));
     }
   }
   // 2. ionospheric correction per L class; the classes below 4096, with that of
@@ -1413,7 +1414,7 @@ extern "C" dc_status correct_compress(dc_ctx* c, const dc_c64* x, long long n,
     ea.one.y = Yr;
     split(dl, ea.one.dl_hi, ea.one.dl_lo);
     split(rotation_rate(o, dl, fs, fc), ea.one.rot_hi, ea.one.rot_lo);
-    enqueue(c, PH_EXACT, s, n_out, "exact launch", [=] { return launch_exact_fp32(ea, 1, s); });
+    enqueue(c, PH_EXACT, s, n_out, "exact launch", [=] { return launch_exact_fp32(ea, 1, s); }, exact_fp32_kernels(ea));
   } else {
     std::vector<RsItem> rs(1);
     rs[0] = RsItem{};
@@ -1478,7 +1479,7 @@ extern "C" dc_status predistort_lfm(dc_ctx* c, dc_c64* y, long long n, double fs
   if (kind == DC_LFM_CUBIC && (st = ensure_ws(c, predist_scratch_bytes(n)))) return st;
   const PredistParams p =
       predist_params(kind, fs, f0, bandwidth, T, kKappa * tec * 1e16, kC, f_mix);
-  Phase ph(c, PH_PREDIST, s, n);
+  Phase ph(c, PH_PREDIST, s, n, kind == DC_LFM_CUBIC ? 3 : 1);
   cudaError_t e = launch_predist(p, reinterpret_cast<float2*>(y), n, c->ws, s);
   if (e != cudaSuccess) return cuda_fail(c, e, "predistortion launch");
   return DC_OK;
@@ -1533,7 +1534,7 @@ extern "C" dc_status resample_exact_batch(dc_ctx* c, const dc_c64* x, long long 
     if ((st = upload(c, dl, 0, &ddl)) || (st = flush(c, s))) return st;
     ExTcArgs a{(int)n, (int)n_out, n_pulses, stride ? 2 * n_pulses : 0,
                reinterpret_cast<float2*>(y), ddl, c->err};
-    Phase ph(c, PH_EXACT_TC, s, (long long)n_alpha * n_pulses * n_out);
+    Phase ph(c, PH_EXACT_TC, s, (long long)n_alpha * n_pulses * n_out, exact_tc_kernels(pl));
     cudaError_t e = launch_exact_tc(mode == DC_EXACT_FP16X3, reinterpret_cast<const float2*>(x), rows_c,
                                     (int)n, pl, a, n_alpha, s);
     if (e != cudaSuccess) return cuda_fail(c, e, "tensor-core exact launch");
@@ -1555,7 +1556,8 @@ extern "C" dc_status resample_exact_batch(dc_ctx* c, const dc_c64* x, long long 
   double delta_max = 0.0;
   for (int i = 0; i < n_alpha; ++i) delta_max = std::max(delta_max, std::fabs(alpha_minus_one(v_r[i])));
   exact_far(c, a, n_alpha, delta_max, 0, s);
-  enqueue(c, PH_EXACT, s, (long long)n_alpha * n_pulses * n_out, "exact launch", [=] { return launch_exact_fp32(a, n_alpha, s); });
+  enqueue(c, PH_EXACT, s, (long long)n_alpha * n_pulses * n_out, "exact launch", [=] { return launch_exact_fp32(a, n_alpha, s); },
+          exact_fp32_kernels(a));
   return flush(c, s);
 }
 

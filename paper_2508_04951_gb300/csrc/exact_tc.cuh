@@ -41,5 +41,6 @@ size_t exact_tc_far_plane_bytes(long long rows, int n);
 // contraction.
 cudaError_t launch_exact_tc(bool fp16, const float2* x, long long x_rows_c, int n, const ExTcPlanes& planes,
                             const ExTcArgs& args, int n_alpha, cudaStream_t s);
+inline int exact_tc_kernels(const ExTcPlanes& p) { return p.far ? 3 : 2; }   // launched by it
 
 }  // namespace dc

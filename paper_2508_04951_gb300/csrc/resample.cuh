@@ -105,5 +105,6 @@ cudaError_t launch_resample_tiled32(const RsArgs& a, int q, cudaStream_t s);
 cudaError_t launch_freqconv(const RsArgs& a, cudaStream_t s);
 cudaError_t launch_resample_direct(const RsArgs& a, cudaStream_t s);
 cudaError_t launch_exact_fp32(const ExArgs& a, int n_alpha, cudaStream_t s);
+inline int exact_fp32_kernels(const ExArgs& a) { return a.mom ? 3 : 1; }   // launched by it
 
 }  // namespace dc
