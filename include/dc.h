@@ -26,6 +26,10 @@
  *    enqueued asynchronously on it; results are ready when the stream is.
  *    Host arrays passed in (item lists, v_r/TEC lists) are read before the
  *    call returns and may be reused afterwards.
+ *  - A call may be captured into a graph of the caller's.  Its lists are kept
+ *    with the graph, so that later calls on the context do not change what a
+ *    replay does; the context must outlive the graph, and its scratch and item
+ *    buffer are not grown while capturing (make the call once before).
  *  - A context serialises its own scratch memory: do not run calls on one
  *    context from several host threads or streams at the same time.
  *  - Arguments are validated before anything is launched; a bad argument

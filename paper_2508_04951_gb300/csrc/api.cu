@@ -480,15 +480,41 @@ struct Call {
   }
 };
 
+// A copy of n bytes that lives as long as the graph that `s` is being captured into and
+// what is instantiated from it; null if that cannot be had.
+void* keep_with_graph(const void* p, size_t n, cudaStream_t s) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  cudaGraph_t graph = nullptr;
+  cudaUserObject_t obj = nullptr;
+  void* q = malloc(n);
+  if (!q) return nullptr;
+  memcpy(q, p, n);
+  if (cudaStreamGetCaptureInfo(s, &st, nullptr, &graph) != cudaSuccess || st != cudaStreamCaptureStatusActive ||
+      cudaUserObjectCreate(&obj, q, free, 1, cudaUserObjectNoDestructorSync) != cudaSuccess) {
+    cudaGetLastError();
+    free(q);
+    return nullptr;
+  }
+  if (cudaGraphRetainUserObject(graph, obj, 1, cudaGraphUserObjectMove) != cudaSuccess) {
+    cudaGetLastError();
+    cudaUserObjectRelease(obj, 1);                     // frees q
+    return nullptr;
+  }
+  return q;
+}
+
 dc_status flush(dc_ctx* c, cudaStream_t s) {
   if (c->stage_hi) {
     const size_t n = c->stage_hi - c->stage_lo;
+    const void* src = c->stage.data() + c->stage_lo;
     if (c->rec) {
-      memcpy(c->rec->data() + c->stage_lo, c->stage.data() + c->stage_lo, n);
+      memcpy(c->rec->data() + c->stage_lo, src, n);
     } else {
-      // the pageable source may be reused as soon as this returns
-      const cudaError_t e = cudaMemcpyAsync(c->items + c->stage_lo, c->stage.data() + c->stage_lo, n,
-                                            cudaMemcpyHostToDevice, s);
+      // the pageable source may be reused as soon as this returns, except that a
+      // graph's copy reads it at every replay: its lists stay with the graph
+      if (capturing(s) && !(src = keep_with_graph(src, n, s)))
+        return fail(c, DC_ECUDA, "item lists of a captured call: no capture to keep them with");
+      const cudaError_t e = cudaMemcpyAsync(c->items + c->stage_lo, src, n, cudaMemcpyHostToDevice, s);
       if (e != cudaSuccess) return cuda_fail(c, e, "item upload");
     }
   }
