@@ -242,7 +242,9 @@ DC_API dc_status correct_batch(dc_ctx* ctx, const dc_c64* in_dev, dc_c64* out_de
  *          inverse-transform kernel then stores the results straight into
  *          it over the host link, overlapping the transfer with the work.
  * Resampling and the forward transform run once per v_r, the phase multiply
- * and inverse transform once per pair. */
+ * and inverse transform once per pair.  Scratch: the resampled pulses, spectra and
+ * factor tables, and beyond 65536 points 512 MiB at most for the transforms
+ * between their passes (64 MiB where that cannot be had). */
 DC_API dc_status correct_bank(dc_ctx* ctx, const dc_c64* x_dev, long long n, const double* v_r,
                        int n_v, const double* tec_tecu, int n_tec, dc_c64* out_dev,
                        double fs, double fc, const dc_opts* opts, void* stream);
@@ -321,7 +323,8 @@ DC_API dc_status resample_exact_batch(dc_ctx* ctx, const dc_c64* x_dev, long lon
 
 /* Plans: a correct_batch or correct_bank call recorded once into a CUDA
  * graph and replayed.  Creating a plan runs the call once on a private stream
- * (the outputs are written), then records it with plan-owned scratch and item
+ * (the outputs are written), then records it with plan-owned scratch (as much as
+ * the call takes, less where that cannot be had) and item
  * lists (uploaded once) and instantiates the graph.  The buffers and host
  * lists the call was given must stay valid while the plan is used; every
  * execution recomputes the outputs from the current contents of the input

@@ -50,6 +50,8 @@ struct dc_ctx {
   int* err = nullptr;         // device error flag
   char* ws = nullptr;         // scratch
   size_t ws_bytes = 0;
+  size_t ws_need = 0;         // most scratch that a call was granted since make_plan cleared this
+  bool lean = false;          // optional scratch (try_ws) is not taken
   std::vector<void*> retired; // outgrown scratch, freed at destroy
   char* items = nullptr;      // device item arrays
   size_t items_bytes = 0;
@@ -242,7 +244,10 @@ PhaseParams phase_params(double fs, double fc, double tec_tecu, int log2L) {
 // Make sure the context has `bytes` of scratch (stream-ordered: the old
 // block stays allocated until destroy, since queued work may still use it).
 dc_status ensure_ws(dc_ctx* c, size_t bytes) {
-  if (bytes <= c->ws_bytes) return DC_OK;
+  if (bytes <= c->ws_bytes) {
+    c->ws_need = std::max(c->ws_need, bytes);
+    return DC_OK;
+  }
   if (c->rec) return fail(c, DC_ENOMEM, "plan scratch too small");
   if (c->budget && bytes > c->budget)
     return fail(c, DC_EBUSY, "scratch of %zu bytes exceeds the context budget of %zu", bytes,
@@ -258,6 +263,7 @@ dc_status ensure_ws(dc_ctx* c, size_t bytes) {
   if (c->ws) c->retired.push_back(c->ws);
   c->ws = (char*)p;
   c->ws_bytes = want;
+  c->ws_need = std::max(c->ws_need, bytes);
   return DC_OK;
 }
 
@@ -273,8 +279,8 @@ bool capturing(cudaStream_t s) {
 // Scratch that only a faster form of a call wants: true when the context has
 // it or can grow to it, leaving no error behind when it cannot.
 bool try_ws(dc_ctx* c, size_t bytes, cudaStream_t s) {
-  if (bytes <= c->ws_bytes) return true;
-  if (c->rec || c->fixed_ws || capturing(s)) return false;
+  if (c->lean) return false;
+  if (bytes > c->ws_bytes && (c->rec || c->fixed_ws || capturing(s))) return false;
   const std::string msg = c->last_error;
   if (ensure_ws(c, bytes) == DC_OK) return true;
   c->last_error = msg;
@@ -1590,7 +1596,8 @@ extern "C" dc_status resample_exact_batch(dc_ctx* c, const dc_c64* x, long long 
 // ================================================================ plans
 // A plan is one of the calls above recorded once into a CUDA graph: the call
 // runs once on a private stream (sizing the context's scratch and warming
-// up), then again with the plan's own scratch and item buffers swapped in,
+// up), then again with the plan's own scratch (as much as the call was granted) and
+// item buffers swapped in,
 // item uploads staged on the host and every kernel launch captured.  The
 // staged items are copied to the plan's device buffer and the graph is
 // instantiated; dc_plan_execute replays it with one cudaGraphLaunch.
@@ -1612,21 +1619,29 @@ dc_status make_plan(dc_ctx* c, F&& call, dc_plan** out) {
   cudaStream_t cs = nullptr;
   cudaError_t e = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking);
   if (e != cudaSuccess) return cuda_fail(c, e, "plan stream");
-  dc_status st = call(cs);
-  if (!st && (e = cudaStreamSynchronize(cs)) != cudaSuccess) st = cuda_fail(c, e, "plan warm-up");
-  dc_plan* p = nullptr;
-  if (!st) {
-    p = new dc_plan();
-    p->c = c;
-    if (cudaMalloc(&p->ws, std::max<size_t>(c->ws_bytes, 256)) != cudaSuccess ||
-        cudaMalloc(&p->items, c->items_bytes) != cudaSuccess) {
-      cudaGetLastError();
-      st = fail(c, DC_ENOMEM, "plan buffers");
-    }
+  dc_plan* p = new dc_plan();
+  p->c = c;
+  // the plan's scratch is what the call was granted; where a second block of that
+  // size cannot be had, the form of the call without optional scratch is recorded
+  dc_status st = DC_OK;
+  for (bool lean : {false, true}) {
+    c->lean = lean;
+    c->ws_need = 256;
+    st = call(cs);
+    if (!st && (e = cudaStreamSynchronize(cs)) != cudaSuccess) st = cuda_fail(c, e, "plan warm-up");
+    if (st || cudaMalloc(&p->ws, c->ws_need) == cudaSuccess) break;
+    cudaGetLastError();
+    p->ws = nullptr;
+  }
+  if (!st && (!p->ws || cudaMalloc(&p->items, c->items_bytes) != cudaSuccess)) {
+    cudaGetLastError();
+    st = fail(c, DC_ENOMEM, "plan buffers");
   }
   if (!st) {
     char* ws0 = c->ws;
+    const size_t b0 = c->ws_bytes;
     char* it0 = c->items;
+    c->ws_bytes = c->ws_need;
     std::vector<char> staging(c->items_bytes, 0);
     c->ws = p->ws;
     c->items = p->items;
@@ -1643,6 +1658,7 @@ dc_status make_plan(dc_ctx* c, F&& call, dc_plan** out) {
     }
     c->rec = nullptr;
     c->ws = ws0;
+    c->ws_bytes = b0;
     c->items = it0;
     p->launches = c->launches - l0;
     c->launches = l0;
@@ -1653,14 +1669,13 @@ dc_status make_plan(dc_ctx* c, F&& call, dc_plan** out) {
       st = cuda_fail(c, e, "graph instantiate");
     if (graph) cudaGraphDestroy(graph);
   }
+  c->lean = false;
   cudaStreamDestroy(cs);
   if (st) {
-    if (p) {
-      if (p->exec) cudaGraphExecDestroy(p->exec);
-      if (p->ws) cudaFree(p->ws);
-      if (p->items) cudaFree(p->items);
-      delete p;
-    }
+    if (p->exec) cudaGraphExecDestroy(p->exec);
+    if (p->ws) cudaFree(p->ws);
+    if (p->items) cudaFree(p->items);
+    delete p;
     return st;
   }
   *out = p;
