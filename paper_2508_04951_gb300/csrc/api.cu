@@ -52,6 +52,11 @@ struct dc_ctx {
   size_t ws_bytes = 0;
   size_t ws_need = 0;         // most scratch that a call was granted since make_plan cleared this
   bool lean = false;          // optional scratch (try_ws) is not taken
+  // Optional scratch that could not be had: not asked for again in the next kTryAgain
+  // calls that want as much (a failing allocation costs more than a short call).
+  static constexpr int kTryAgain = 64;
+  size_t refused = 0;
+  int refusals = 0;
   std::vector<void*> retired; // outgrown scratch, freed at destroy
   char* items = nullptr;      // device item arrays
   size_t items_bytes = 0;
@@ -280,10 +285,18 @@ bool capturing(cudaStream_t s) {
 // it or can grow to it, leaving no error behind when it cannot.
 bool try_ws(dc_ctx* c, size_t bytes, cudaStream_t s) {
   if (c->lean) return false;
-  if (bytes > c->ws_bytes && (c->rec || c->fixed_ws || capturing(s))) return false;
+  if (bytes > c->ws_bytes) {
+    if (c->rec || c->fixed_ws || capturing(s)) return false;
+    if (c->refusals > 0 && bytes >= c->refused) {
+      --c->refusals;
+      return false;
+    }
+  }
   const std::string msg = c->last_error;
   if (ensure_ws(c, bytes) == DC_OK) return true;
   c->last_error = msg;
+  c->refused = bytes;
+  c->refusals = dc_ctx::kTryAgain;
   return false;
 }
 

@@ -76,3 +76,30 @@ def test_plan_with_less_scratch(dcg):
     plan.close()
     ctx.close()
     free_bytes()
+
+
+def test_refused_scratch_is_not_asked_for_on_every_call(dcg):
+    # a bank whose passes would take 512 MiB with 500 MiB left: it runs in the 64 MiB
+    # form, and the next 64 calls do not ask for the 512 again (seen from the memory that
+    # they leave alone when it has become free); then it is taken
+    import torch
+    m = dcg
+    n, v, tec = 1 << 18, np.linspace(-5000.0, 5000.0, 8), np.linspace(5.0, 100.0, 33)
+    x = torch.randn(n, dtype=torch.complex64, device="cuda")
+    a, b, c = (torch.empty((8, 33, n), dtype=torch.complex64, device="cuda") for _ in range(3))
+    ctx = m.Context(0)
+    m.correct_bank(ctx, x[:1000], v, tec, a, 20e6, 1e9)
+    filler = torch.empty(free_bytes() - 500 * MIB, dtype=torch.uint8, device="cuda")
+    m.correct_bank(ctx, x, v, tec, a, 20e6, 1e9)
+    m.dc_check(ctx)
+    del filler
+    before = free_bytes()
+    for _ in range(64):
+        m.correct_bank(ctx, x, v, tec, b, 20e6, 1e9)
+    assert before - free_bytes() < 64 * MIB
+    m.correct_bank(ctx, x, v, tec, c, 20e6, 1e9)
+    assert before - free_bytes() > 400 * MIB
+    m.dc_check(ctx)
+    for y in (b, c):
+        assert torch.equal(torch.view_as_real(a), torch.view_as_real(y))
+    ctx.close()
