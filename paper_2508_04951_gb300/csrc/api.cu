@@ -240,8 +240,9 @@ PhaseParams phase_params(double fs, double fc, double tec_tecu, int log2L) {
   split(fs / (double)(1LL << log2L), p.d_hi, p.d_lo);
   p.log2L = log2L;
   p.enabled = tec_tecu != 0.0;
+  const double f_min = fc - 0.5 * fs;
   if (p.enabled && fc > 0.0 && p.fc_lo == 0.f && p.d_lo == 0.f &&
-      2.0 * kKappa * std::fabs(tec_tecu) * 1e16 / kC / (fc - 0.5 * fs) < (double)(1 << 22))
+      2.0 * kKappa * std::fabs(tec_tecu) * 1e16 / kC / f_min * std::max(1.0, 0.5 * fs / f_min) < kPlainCycles)
     p.enabled = kPhasePlain;
   return p;
 }

@@ -20,12 +20,18 @@ struct PhaseParams {
   float fc_hi, fc_lo;   // carrier fc                [Hz]; 0 = RF sampling
   float d_hi, d_lo;     // bin spacing fs / L        [Hz]
   int log2L;            // transform length L = 2^log2L
-  // 0 when E == 0 (identity).  kPhasePlain where every f_k > 0, |C / f_k| < 2^22
-  // and fc and fs / L are floats exactly (baseband at round frequencies): the
-  // evaluation leaves out the terms that are zero then (same results).
+  // 0 when E == 0 (identity).  kPhasePlain where every f_k > 0, fc and fs / L are
+  // floats exactly (baseband at round frequencies) and |C / f| max(1, fs / 2f) <
+  // kPlainCycles at the lowest f: the evaluation leaves out the terms that are zero then
+  // and the second reduction.
   int enabled;
 };
 constexpr int kPhasePlain = 2;
+// q2 below is at most 2.75 ulps of C / f (2^-23 each: the reciprocal one, its product 1/2, f's
+// low part 1/2 and as much times fs / 2f, C's low part 1/4): 0.086 cycles here, so that the
+// phase stays within 0.59 cycles, where the approximate sine is specified (to 2^-20.5
+// within a cycle).  1e4 TECU at a carrier of 300 MHz are 9e4 cycles.
+constexpr double kPlainCycles = 1 << 18;
 
 // kt of bin k of an L-point DFT (fftfreq order): k below L/2, else k - L.
 DC_DEV float bin_kt(const PhaseParams& P, int k) {
@@ -51,7 +57,7 @@ template <bool PLAIN> DC_DEV float iono_cycles(const PhaseParams& P, float kt) {
   r = fmaf(-q1, fl, __fadd_rn(r, P.c_lo));
   const float q2 = __fmul_rn(r, rb);
   float x = __fadd_rn(__fsub_rn(q1, rintf(q1)), q2);   // q1 - rint(q1) is exact
-  if constexpr (PLAIN) return x;                       // |q2| below 1/4: within [-3/4, 3/4]
+  if constexpr (PLAIN) return x;                       // within [-0.59, 0.59]: kPlainCycles
   x = __fsub_rn(x, rintf(x));                          // |q2| passes 1/2 for |C / f| > 2^22
   return fh == 0.f ? 0.f : x;
 }
