@@ -222,7 +222,10 @@ typedef struct {
  * carrier_shift, freq_ref; opts->n_out is ignored, items carry n_out), then
  * apply Eq. 16 with its TEC.  in_dev and out_dev hold all items at the given
  * offsets; output ranges must not overlap each other or the inputs.  Each
- * item's result does not depend on the other items of the batch. */
+ * item's result does not depend on the other items of the batch.  (Exact sums
+ * leave out the far field of resample_exact_batch in contexts with a scratch
+ * budget, in a server and while a caller's graph is captured: there the batch
+ * would decide whether an item has room for it.) */
 DC_API dc_status correct_batch(dc_ctx* ctx, const dc_c64* in_dev, dc_c64* out_dev,
                         const dc_item* items, int n_items, const dc_opts* opts,
                         void* stream);

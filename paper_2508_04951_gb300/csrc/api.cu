@@ -1053,16 +1053,19 @@ dc_status correct_batch(dc_ctx* c, const dc_c64* in, dc_c64* out, const dc_item*
   const std::vector<size_t>& class_chunk = lay.class_chunk;
   if ((st = ensure_ws(c, lay.bytes))) return st;
   if ((st = ensure_items(c, items_bytes_for((size_t)n_items * 4)))) return st;
-  if (o.mode == DC_EXACT_FP32) {
-    // the near and far scratch lies behind the batch's, one item's at a time;
-    // grown to the largest first, as the layout's pointers come from c->ws
-    size_t far = 0;
+  // Exact sums: near and far scratch behind the batch's, one item's at a time, grown to
+  // the largest before c->ws is read.  Every item's form follows from its own sizes: where
+  // the batch would decide whether there is room (a budget, the caller's scratch, a
+  // caller's capture), all are dense.
+  bool far = false;
+  if (o.mode == DC_EXACT_FP32 && !c->budget && !c->fixed_ws && (c->rec || !capturing(s))) {
+    size_t elems = 0;
     for (int i = 0; i < n_items; ++i) {
       const int no = (int)(items[i].n_out ? items[i].n_out : items[i].n);
       if (exact_fp32_far((int)items[i].n, no, 1, 1, std::fabs(alpha_minus_one(items[i].v_r))))
-        far = std::max(far, exact_fp32_far_elems(1, (int)items[i].n) + exact_fp32_far_elems(1, no));
+        elems = std::max(elems, exact_fp32_far_elems(1, (int)items[i].n) + exact_fp32_far_elems(1, no));
     }
-    if (far) try_ws(c, ((lay.bytes + 255) & ~(size_t)255) + far * sizeof(float2), s);
+    far = elems && try_ws(c, ((lay.bytes + 255) & ~(size_t)255) + elems * sizeof(float2), s);
   }
   char* ws = c->ws;
   size_t item_at = 0;
@@ -1092,7 +1095,7 @@ dc_status correct_batch(dc_ctx* c, const dc_c64* in, dc_c64* out, const dc_item*
       a.one.y = reinterpret_cast<float2*>(ws + yoff[i]);
       split(dl, a.one.dl_hi, a.one.dl_lo);
       split(rotation_rate(o, dl, it.fs, it.fc), a.one.rot_hi, a.one.rot_lo);
-      if (lay.bytes < c->ws_bytes) exact_far(c, a, 1, std::fabs(dl), lay.bytes, s);
+      if (far) exact_far(c, a, 1, std::fabs(dl), lay.bytes, s);
       enqueue(c, PH_EXACT, s, a.n_out, "exact launch", [=] { return launch_exact_fp32(a, 1, s); }, exact_fp32_kernels(a));
     }
   }
