@@ -1561,13 +1561,14 @@ extern "C" dc_status resample_exact_batch(dc_ctx* c, const dc_c64* x, long long 
     const size_t plane = exact_tc_plane_bytes(2 * rows_c, (int)n);
     const size_t mom = exact_tc_far_plane_bytes(2 * rows_c, (int)n);
     const size_t loc = exact_tc_far_plane_bytes(2 * rows_c, (int)n_out);
+    const size_t peak = exact_tc_peak_bytes(mode == DC_EXACT_FP16X3, stride ? n_alpha : 1, n_pulses, (int)n);
     ExTcPlanes pl{};
-    size_t at[6] = {};
+    size_t at[7] = {};
     for (bool far : {true, false}) {
       // the dense sum where the far field does not apply or its planes do not fit
       if (far && !exact_tc_far(mode == DC_EXACT_FP16X3, (int)n, (int)n_out, delta_max)) continue;
       Arena ar;
-      for (int i = 0; i < (far ? 6 : 2); ++i) at[i] = ar.take(i < 2 ? plane : i < 4 ? mom : loc);
+      for (int i = 0; i < (far ? 7 : 2); ++i) at[i] = ar.take(i < 2 ? plane : i < 4 ? mom : i < 6 ? loc : peak);
       pl.far = far;
       if (far ? try_ws(c, ar.off, s) : (st = ensure_ws(c, ar.off)) == DC_OK) break;
     }
@@ -1575,6 +1576,7 @@ extern "C" dc_status resample_exact_batch(dc_ctx* c, const dc_c64* x, long long 
     pl.hi = c->ws + at[0], pl.lo = c->ws + at[1];
     pl.mom_hi = c->ws + at[2], pl.mom_lo = c->ws + at[3];
     pl.loc_hi = c->ws + at[4], pl.loc_lo = c->ws + at[5];
+    pl.peak = c->ws + at[6];
     if ((st = ensure_items(c, items_bytes_for(n_alpha)))) return st;
     std::vector<float> dl(2 * (size_t)n_alpha);
     for (int i = 0; i < n_alpha; ++i) split(alpha_minus_one(v_r[i]), dl[2 * i], dl[2 * i + 1]);

@@ -142,8 +142,18 @@ DC_DEV void position(float dl_hi, float dl_lo, int n, int& m, float& e) {
 
 // Powers of two that keep the 16-bit moments and node values inside fp16's
 // range for any pulse inside it (|M| <= 32 max|x|, |L| <= 17 max|x|):
-// planes hold M / 32 and L / 32, the Cauchy elements are taken times 256.
-constexpr float kMomScale = 1.f / 32, kCauchyScale = 256.f, kLocScale = 1.f / 32;
+// planes hold M / 32 and L times loc_scale, the Cauchy elements are taken times 256.
+constexpr float kMomScale = 1.f / 32, kCauchyScale = 256.f;
+// 2^-e, e the exponent of the largest component of the tile's pulses, in [1/32, 1]: 1/32
+// throughout left node values of pulses below 1e-4 32 times coarser than their
+// samples, as fp16's spacing ends at 2^-24 (pulses of 1e-6 x 2000 samples: up to 3.0 times
+// the dense sum's distance from 64 bits, now below it; 512 pulses x 16 rates x 8192:
+// 542 us, now 546).  bf16, with FP32's range, keeps 1/32.
+constexpr float kLocScale = 1.f / 32;
+DC_DEV float loc_scale(uint32_t peak_bits) {
+  const int e = (int)(peak_bits >> 23) - 127;                   // 128 for inf and NaN
+  return __uint_as_float((uint32_t)(127 - min(max(e, 0), 5)) << 23);
+}
 
 constexpr int kFarMinIn = 1536, kFarMinInFp16 = 1792;   // see exact_tc_far
 constexpr int kFarWideIn = 4096;                     // bf16x3 above: near = 3 blocks either side
@@ -168,6 +178,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   __shared__ float s_sig[C::BM], s_e[C::BM];
   __shared__ int s_m[C::BM];
   __shared__ float s_far[JOB == JOB_DENSE ? 1 : kFarP * kFarP];   // basis table, or source nodes
+  constexpr bool PEAK = FP16 && JOB == JOB_FAR;
+  __shared__ uint32_t s_peak[PEAK ? kThreads / 32 : 1];   // the warps' shares of the pulses' peak
 
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~(uintptr_t)1023);
@@ -228,9 +240,28 @@ __global__ void __launch_bounds__(kThreads, 1)
   if constexpr (JOB == JOB_FAR) {
     if (threadIdx.x < kFarP) s_far[threadIdx.x] = kSrcHalf * far_node(threadIdx.x);
   }
+  if constexpr (PEAK) {
+    // non-negative floats (inf and NaN above all) in the order of their bits
+    const long long first = (long long)alpha * (a.rows_per_alpha / 2) + c0 / 2;
+    const int count = min(BN / 2, a.n_pulses - c0 / 2) * a.n_peaks;
+    uint32_t m = 0;
+    for (int i = threadIdx.x; i < count; i += kThreads)
+      m = max(m, __float_as_uint(__ldg(a.peak + first * a.n_peaks + i)));
+    m = __reduce_max_sync(0xffffffffu, m);
+    if (lane == 0) s_peak[warp] = m;
+  }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  // node values' scale: formed where they are, read where they are used
+  float* const tile_inv = a.loc_inv + (a.rows_per_alpha ? alpha : 0) * gridDim.y + blockIdx.y;
+  float loc = kLocScale;
+  if constexpr (PEAK) {
+    uint32_t m = 0;
+    for (int i = 0; i < kThreads / 32; ++i) m = max(m, s_peak[i]);
+    loc = loc_scale(m);
+    if (blockIdx.x == 0 && threadIdx.x == 0) *tile_inv = 1.f / loc;
+  }
   const uint32_t tmem = tmem_base;
   bool ok = true;
 
@@ -301,6 +332,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int h = nl >> 7, r = nl & 127;       // half and row inside it
     const int mn = s_m[nl];
     const float en = s_e[nl], sg = s_sig[nl];
+    const float loc_inv = FP16 && JOB == JOB_NEAR ? __ldg(tile_inv) : 1.f / kLocScale;
     for (int kc = 0; kc < nk && ok; ++kc) {
       const int s = kc % C::STAGES;
       const uint32_t ph = (kc / C::STAGES) & 1;
@@ -317,7 +349,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           if (k8 >= kFarP / 8) continue;       // the MMA reads 16 columns of this chunk
           float T[kFarP];
           far_polys(((float)(mn - blk * kFarBlock) - 127.5f + en) * (1.f / kTgtHalf), T);
-          const float sc = sg * (1.f / kLocScale);
+          const float sc = sg * loc_inv;
 #pragma unroll
           for (int i = 0; i < 8; ++i) v[i] = sc * far_basis(s_far, k8 * 8 + i, T);
         } else if (JOB == JOB_FAR) {
@@ -381,7 +413,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 const int col = c0 + cc * 16 + i;
                 if (col >= 2 * a.n_pulses) break;
                 uint16_t hi, lo;
-                split1<FP16>(f[i] * (kLocScale / (kMomScale * kCauchyScale)), hi, lo);
+                split1<FP16>(f[i] * (loc / (kMomScale * kCauchyScale)), hi, lo);
                 const size_t o = ((size_t)alpha * 2 * a.n_pulses + col) * a.n_out + n;
                 a.loc_hi[o] = hi;
                 a.loc_lo[o] = lo;
@@ -439,7 +471,7 @@ constexpr int kFsWarps = 8;
 template <bool FP16>
 __global__ void __launch_bounds__(32 * kFsWarps, 2)
     far_split_kernel(const float2* __restrict__ x, int n, long long rows_c, int ld, uint16_t* hi,
-                     uint16_t* lo, int ld_mom, uint16_t* mom_hi, uint16_t* mom_lo) {
+                     uint16_t* lo, int ld_mom, uint16_t* mom_hi, uint16_t* mom_lo, float* peak) {
   __shared__ float s_w[kFarP * kFarBlock];             // l_j(m) (-1)^m kMomScale at [j][m]
   __shared__ float s_D[kFarP * kFarP];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -473,6 +505,18 @@ __global__ void __launch_bounds__(32 * kFsWarps, 2)
           if (m + 1 < n) v[b][q][1] = __ldcs(xp + m + 1);
         }
       }
+    if constexpr (FP16) {                              // g = pr * n_pair + pair
+      uint32_t top = 0;
+#pragma unroll
+      for (int b = 0; b < 2; ++b)
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+#pragma unroll
+          for (int i = 0; i < 2; ++i)
+            top = max(top, max(__float_as_uint(v[b][q][i].x) & 0x7fffffffu, __float_as_uint(v[b][q][i].y) & 0x7fffffffu));
+      top = __reduce_max_sync(0xffffffffu, top);
+      if (lane == 0) peak[g] = __uint_as_float(top);
+    }
 #pragma unroll
     for (int b = 0; b < 2; ++b)
 #pragma unroll
@@ -577,12 +621,15 @@ cudaError_t run_exact_tc(const float2* x, long long x_rows_c, int n, const ExTcP
   const long long pairs = x_rows_c * ((far_blocks(n) + 1) / 2);
   const int grid_c = (int)std::min<long long>((pairs + kFsWarps - 1) / kFsWarps, 152LL * 2);
   far_split_kernel<FP16><<<grid_c, 32 * kFsWarps, 0, s>>>(x, n, x_rows_c, ld, (uint16_t*)pl.hi, (uint16_t*)pl.lo, kb,
-                                                          (uint16_t*)pl.mom_hi, (uint16_t*)pl.mom_lo);
+                                                          (uint16_t*)pl.mom_hi, (uint16_t*)pl.mom_lo, (float*)pl.peak);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   ExTcArgs g = args;
   g.near = !FP16 && n > kFarWideIn ? 3 : 1;
   g.own_first = g.near > 1;
+  g.peak = (const float*)pl.peak;
+  g.n_peaks = (far_blocks(n) + 1) / 2;
+  g.loc_inv = (float*)pl.peak + x_rows_c * g.n_peaks;
   ExTcArgs f = g;
   f.n_in = kb;
   f.n_out = ob;
@@ -611,6 +658,11 @@ bool exact_tc_far(bool fp16, int n_in, int n_out, double delta_max) {
 }
 size_t exact_tc_far_plane_bytes(long long rows, int n) {
   return (size_t)rows * kFarP * far_blocks(n) * 2;
+}
+
+size_t exact_tc_peak_bytes(bool fp16, long long groups, int n_pulses, int n) {
+  const size_t tiles = (2 * (size_t)n_pulses + BN - 1) / BN;
+  return fp16 ? (size_t)groups * (n_pulses * (size_t)((far_blocks(n) + 1) / 2) + tiles) * sizeof(float) : 0;
 }
 
 cudaError_t launch_exact_tc(bool fp16, const float2* x, long long x_rows_c, int n, const ExTcPlanes& pl,

@@ -17,15 +17,21 @@ struct ExTcArgs {
   // near and far field: blocks either side taken term by term; whether the
   // output's own block is summed first
   int near, own_first;
+  // fp16x3 with far field: largest |component| of each two blocks, [pulses][n_peaks],
+  // and the inverse of the node values' scale, one per alpha group and column tile
+  const float* peak;
+  int n_peaks;
+  float* loc_inv;
 };
 
 // Device scratch of one call: the split planes (exact_tc_plane_bytes each)
 // and, with `far`, the planes of block moments (exact_tc_far_plane_bytes of
-// n) and of node values (exact_tc_far_plane_bytes of n_out).
+// n), of node values (exact_tc_far_plane_bytes of n_out) and the pulses' peaks with
+// the scales from them (exact_tc_peak_bytes; `groups` of n_pulses).
 struct ExTcPlanes {
   void *hi, *lo;
   bool far;
-  void *mom_hi, *mom_lo, *loc_hi, *loc_lo;
+  void *mom_hi, *mom_lo, *loc_hi, *loc_lo, *peak;
 };
 
 // Bytes of one 16-bit split plane for `rows` real rows of n samples.
@@ -36,6 +42,7 @@ size_t exact_tc_plane_bytes(long long rows, int n);
 // (delta_max: the largest |alpha - 1|).
 bool exact_tc_far(bool fp16, int n_in, int n_out, double delta_max);
 size_t exact_tc_far_plane_bytes(long long rows, int n);
+size_t exact_tc_peak_bytes(bool fp16, long long groups, int n_pulses, int n);
 
 // Split x (x_rows_c complex pulses of n samples) into the planes, then run the
 // contraction.
