@@ -80,7 +80,7 @@ DC_DEV void tiny_pass(float2* sm, const FftItem* items, const FftItem& one, int 
     }
     return;
   }
-  if (I.ptab) {
+  if (OP == ROW_APPLY || I.ptab) {
 #pragma unroll
     for (int x = 0; x < N; ++x) v[x] = cmul(v[x], I.ptab[bin(x)]);
   } else if (I.ph.enabled) {
@@ -179,7 +179,7 @@ DC_DEV void line_pass(float2* sm, const FftItem* items, const FftItem& one, int 
     }
     return;
   }
-  if (I.ptab) {
+  if (OP == ROW_APPLY || I.ptab) {
 #pragma unroll
     for (int r = 0; r < 16; ++r) v[r] = cmul(v[r], I.ptab[s + 16 * t + T * r]);
   } else if (I.ph.enabled) {
@@ -222,7 +222,7 @@ DC_DEV void line_pass(float2* sm, const FftItem* items, const FftItem& one, int 
 // The pass of CTA `block` for transforms of M points, its transforms per CTA and shared memory.
 template <int M, int OP>
 DC_DEV void short_pass(float2* sm, const FftItem* items, const FftItem& one, int n_items, int block, const float2* tw) {
-  if constexpr (M == 4096) full_4096<true>(items ? ldg_item(items + block) : one, sm, threadIdx.x, tw);
+  if constexpr (M == 4096) full_4096(items ? ldg_item(items + block) : one, sm, threadIdx.x, tw);
   else if constexpr (M >= 256) line_pass<M / 256, OP>(sm, items, one, n_items, block, tw);
   else tiny_pass<M, OP>(sm, items, one, n_items, block, tw);
 }

@@ -18,10 +18,8 @@ template <int CL> DC_DEV void cluster_wait() {
   if constexpr (CL > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-// Transform p of a FUSED_APPLY launch: from the item list, or formed from
-// the grid description (FusedArgs::grid_src).
+// Transform p of a FUSED_APPLY launch, formed from the grid description.
 DC_DEV FftItem apply_item(const FusedArgs& a, int p) {
-  if (!a.grid_src) return item_of(a, p);
   FftItem I = {};
   const int i = p / a.grid_n_tec, t = p - i * a.grid_n_tec;
   const size_t L = (size_t)1 << a.log2L;
@@ -447,7 +445,7 @@ __global__ void __launch_bounds__(kRowThreads, LOG2L1 == 0 ? 2 : 4) full_kernel(
   const FftItem I = item_of(a, blockIdx.x >> LOG2L1);
   const int j = threadIdx.x;
   if constexpr (L1 == 1) {
-    full_4096<true>(I, A, j, a.tw);
+    full_4096(I, A, j, a.tw);
   } else {
     asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");   // this CTA runs
     float2 v[16];
@@ -578,7 +576,8 @@ __global__ void __launch_bounds__(kRowThreads, 4) row_4096_kernel(RowArgs a) {
     store_bins(dst, j, v);
     return;
   }
-  bin_factors(I, k1, a.log2L1, j, v);
+  if constexpr (OP == ROW_APPLY) mul_bins(I.ptab + (size_t)k1 * kRowN, j, v);
+  else bin_factors(I, k1, a.log2L1, j, v);
   if (OP == ROW_APPLY && L1 == 1) {
     row_inverse<false>(v, sm, j, tw);
     const float invL = 1.0f / (float)kRowN;

@@ -50,10 +50,9 @@ struct FusedArgs {
   float2* scratch;
   int* ctr;
   int chunk;
-  // FUSED_APPLY over a grid of transforms (the bank): with grid_src set,
-  // transform p = i * grid_n_tec + t reads the spectrum grid_src + i L and
-  // the factors grid_ptab + t L and writes grid_n_out samples to
-  // grid_dst + p grid_n_out; `items` is not read.
+  // FUSED_APPLY, a grid of transforms (the bank): transform p = i * grid_n_tec + t
+  // reads the spectrum grid_src + i L and the factors grid_ptab + t L and writes
+  // grid_n_out samples to grid_dst + p grid_n_out; `items` is not read.
   const float2* grid_src;
   const float2* grid_ptab;
   float2* grid_dst;

@@ -208,14 +208,13 @@ DC_DEV void bin_factors(const FftItem& I, int k1, int log2L1, int j, float2 (&v)
 // The whole correction of one L = 4096 transform: zero-padded input, forward row,
 // factors, inverse row, 1 / L, truncation.  Every stage base of both rows is loaded up
 // front, beside the input: one CTA per transform leaves nothing to hide a load issued
-// per stage.  PDL: the input is read after pdl_wait, by plain loads (a
-// non-coherent load may be scheduled ahead of the wait).
-template <bool PDL>
+// per stage.  The input is read after pdl_wait, by plain loads (a non-coherent load may
+// be scheduled ahead of the wait).
 DC_DEV void full_4096(const FftItem& I, float2* b, int j, const float2* tw) {
   float2 f2[4], f3[4];
   GlobalTw{tw}.s2(f2, j & 15);
   GlobalTw{tw}.s3(f3, j);
-  if constexpr (PDL) pdl_wait();                // the input's producer has finished
+  pdl_wait();                                   // the input's producer has finished
   float2 v[16];
 #pragma unroll
   for (int r = 0; r < 16; ++r) {
