@@ -310,10 +310,14 @@ DC_API dc_status predistort_lfm(dc_ctx* ctx, dc_c64* y_dev, long long n, double 
                                 int kind, void* stream);
 
 /* Exact-sinc resampling of many pulses per range rate (Eq. 17:
- * Y_a = X_a S_a^T, S_a[j][i] = sinc(alpha_a j - i)).  Pulses of 1536 samples
- * and more are summed term by term near each output only, 256-sample blocks
- * further off through 16 moments each (to FP32 accuracy), where the scratch
- * for that is to be had.
+ * Y_a = X_a S_a^T, S_a[j][i] = sinc(alpha_a j - i)).  Long pulses are summed
+ * term by term near each output only, 256-sample blocks further off through 16
+ * moments each (the far field), where the scratch for that is to be had and
+ * no output lies more than 63 samples from its own index: from 1536
+ * samples on in FP32 (8 pulses and fewer per rate: from 2^25 terms of all
+ * outputs) and bf16x3, from 1792 in fp16x3.  Moments and node values are held
+ * in FP32, or as hi/lo pairs of 16 bits as the samples are in the tensor-core
+ * modes; each mode is no further from the sum than term by term throughout.
  * x_dev: pulses [n_alpha][n_pulses][n] with x_alpha_stride samples between
  *        consecutive alpha groups (0 = every alpha uses the same pulses);
  * v_r:   host [n_alpha], 1 <= n_alpha <= 65535;

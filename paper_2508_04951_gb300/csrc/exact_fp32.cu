@@ -487,8 +487,8 @@ size_t exact_fp32_far_elems(long long pulses, int n) { return (size_t)pulses * k
 // The near and far form adds two launches and replaces n_in terms by at most 768
 // and 16.  Measured, far against dense, in us:
 //   tiles (more than 8 pulses), pulses x rates: 12 x 1: n = 1024: 39 / 35, 1536: 39 /
-//   51, 4096: 41 / 129; 48 x 8: 1024: 64 / 59, 1536: 83 / 139, 4096: 154 / 670 (the
-//   dense kernel before these tiles: 1139); so from 1536 on.
+//   51, 4096: 41 / 129; 48 x 8: 1024: 64 / 59, 1536: 83 / 139, 4096: 154 /
+//   670; so from 1536 on.
 //   one warp per output: 1 x 1: 4096: 12.3 / 10.3, 6000: 12.4 / 16.4, 16384: 19 / 81;
 //   2 x 4: 1536: 16.4 / 12.8, 2048: 18.0 / 18.2; 8 x 1: 2048: 22.6 / 24.9; 8 x 8:
 //   1024: 36 / 31, 1536: 46 / 58, 4096: 97 / 312; so from 2^25 terms on.

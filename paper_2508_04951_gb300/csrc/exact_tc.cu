@@ -651,7 +651,7 @@ size_t exact_tc_plane_bytes(long long rows, int n) {
 // 4096: 57) and adds two launches.  Measured, far against dense, in us (8 pulses x 1
 // rate, 64 x 4, 512 x 1): bf16x3: n = 1025: 43 / 39, 50 / 41, 56 / 43; 1536: 43 / 51,
 // 49 / 54, 55 / 57; 2048: 45 / 63, 49 / 68, 57 / 70; 4097: 75 / 114, 83 / 121, 91 /
-// 126; 8192 at 512 x 16: 1053, dense as it was before 5172.  fp16x3: 1536: 35 / 34, 38 /
+// 126; 8192 at 512 x 16: 1023 / 3383.  fp16x3: 1536: 35 / 34, 38 /
 // 37, 44 / 42; 2048: 35 / 43, 40 / 47, 46 / 49; 8192: 41 / 133, 69 / 275, 85 / 285.
 bool exact_tc_far(bool fp16, int n_in, int n_out, double delta_max) {
   return n_in >= (fp16 ? kFarMinInFp16 : kFarMinIn) && delta_max * (double)n_out <= (double)(kFarMargin - 1);

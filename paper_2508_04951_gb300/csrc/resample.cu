@@ -16,8 +16,8 @@
 //    weight is then the quadratic through its exact values at the warp tile's
 //    first, middle and last output (error <= 2e-7), with one more tap where
 //    floor(delta n) steps inside the tile.  Other warp tiles use exact
-//    per-output weights read against the same slice (Q = 8 used to take them at
-//    every step: 18.4 instead of 6.2 us for a short pulse).
+//    per-output weights read against the same slice (taken at every step
+//    they cost a short pulse 18.4 instead of 6.2 us).
 #include "resample.cuh"
 
 namespace dc {
@@ -242,9 +242,8 @@ __global__ void __launch_bounds__(kRsTile >> LQ, LQ == 3 ? 8 : 3) resample_tiled
   // the pulse -- goes from global memory into a private, bank-spread region of
   // shared memory (compile-time tap offsets, no CTA barrier; the region then
   // stages the warp's outputs).  Its loads are in flight while the weights are
-  // formed.  (Staged for the whole CTA by one bulk copy first, as this kernel had
-  // it, the slice waited for the copy, a barrier and a second pass through
-  // shared memory.)
+  // formed.  (Staged for the whole CTA by one bulk copy first, the slice waits for
+  // the copy, a barrier and a second pass through shared memory.)
   const int fmin = min(f0, f2);
   const int G = ow + fmin - HALF + 1;
   float2* ww = win + warp * WSTRIDE;
